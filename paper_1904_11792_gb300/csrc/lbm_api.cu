@@ -24,6 +24,27 @@ dim3 default_block(const Geom& g) {
   const unsigned bx = ux >= 256 ? 256 : (ux >= 128 ? 128 : (ux >= 64 ? 64 : 32));
   return dim3(bx, 256 / bx, 1);
 }
+
+// The block a collide-stream kernel launches with where no shape was asked
+// for: the default, but rows shorter than a warp are not padded to one - the
+// block takes whole rows of several y and z, so a warp's lanes all hold nodes -
+// and lattices too small to give every SM two blocks take smaller blocks,
+// down to one warp.  (4x49x49 FP64, whose pipe a warp instruction occupies
+// for 16 clocks whatever its live lanes: 68 us per step in 32 x 8 blocks, 2 of
+// 32 lanes live, 10.3 us in 4 x 8 x 1.)
+dim3 auto_block(const Geom& g, bool pairs) {
+  const unsigned ux = pairs ? g.nx / 2 : g.nx;
+  const long long units = (long long)ux * g.ny * g.nz;
+  unsigned threads = 256;
+  while (threads > 32 && units < (long long)threads * 2 * kSmCount) threads /= 2;
+  if (ux >= 32) {
+    const unsigned bx = std::min(threads, default_block(g).x);
+    return dim3(bx, threads / bx, 1);
+  }
+  const unsigned by = std::min<unsigned>(g.ny, std::max(1u, threads / ux));
+  const unsigned bz = std::min<unsigned>(std::min(g.nz, 64), std::max(1u, threads / (ux * by)));
+  return dim3(ux, by, bz);
+}
 }  // namespace lbm
 
 namespace {
@@ -149,6 +170,7 @@ int salt_word(const lbm_ctx* h, long long step, int cur) {
 // 9.11 ms against 9.84); 2 for the A-B step's two-node kernel (no spills at
 // <= 128 registers).
 int auto_minb(bool vec, int mode, int precision) {
+  if (precision == LBM_F64) return 2;   // 988 us per launch on 256x128x128 against 1013 with 3 (spills)
   if (!vec || mode == MODE_AA_EVEN) return 3;
   if (mode == MODE_AA_ODD && (precision == LBM_F16DEV || precision == LBM_BF16DEV)) return 3;
   return 2;
@@ -213,7 +235,7 @@ int enqueue_step(lbm_ctx* h, cudaStream_t s, long long step, int cur, bool timed
   }
   if (diag_step) {
     CK(launch_diagnostics(prec, layout, h->g, h->ph, src, h->rho_l, h->rho_v, h->d_scratch, h->d_ring,
-                          h->psi, h->d_flag, h->d_ring_count, lbm_ctx::kRing, s));
+                          h->psi, h->d_flag, h->d_ring_count, lbm_ctx::kRing, s, aa ? nullptr : dst));
     if (h->diag_ccl) {
       long long* d4 = (long long*)(h->d_small + 32);
       CK(launch_ccl(prec, layout, h->g, h->ph, src, 0.5 * (h->rho_l + h->rho_v), h->d_labels,
@@ -221,15 +243,16 @@ int enqueue_step(lbm_ctx* h, cudaStream_t s, long long step, int cur, bool timed
       CK(launch_ccl_ring(d4, h->d_ring, h->d_ring_count, lbm_ctx::kRing, s));
     }
   } else {
-    CK(launch_psi(prec, layout, h->vec, h->g, h->ph, src, h->psi, h->d_flag, s));
+    CK(launch_psi(prec, layout, h->vec, h->g, h->ph, src, h->psi, h->d_flag, s, aa ? nullptr : dst));
   }
   if (timed) CK(cudaEventRecord(e1, s));
-  const bool vec = h->vec && (h->g.nx % 2 == 0);
+  const bool vec = node_pairs(prec, h->vec, h->g);
   const int minb = h->minb ? h->minb : auto_minb(vec, mode, prec);
+  const dim3 block = h->block_asked ? h->block : auto_block(h->g, vec);
   if (h->ph.coll == COLL_MRT)
-    CK(launch_collide_mrt(prec, mode, vec, h->g, ph, src, dst, h->psi, h->block, s));
+    CK(launch_collide_mrt(prec, mode, vec, h->g, ph, src, dst, h->psi, block, s));
   else
-    CK(launch_collide(prec, mode, minb, vec, h->g, ph, src, dst, h->psi, h->block, s));
+    CK(launch_collide(prec, mode, minb, vec, h->g, ph, src, dst, h->psi, block, s));
   if (timed) {
     CK(cudaEventRecord(e2, s));
     h->pending.push_back({0, e0, e1});
@@ -443,6 +466,7 @@ void lbm_destroy(lbm_handle h) {
   if (h->own_state) dev_free(h->state, h->state_bytes);
   if (h->own_psi) dev_free(h->psi, h->psi_bytes);
   dev_free(h->d_flag, sizeof(int) * 4);
+  dev_free(h->d_psi_tab, sizeof(double2) * kPsiTab);
   dev_free(h->d_small, sizeof(double) * 64);
   dev_free(h->d_scratch, h->scratch_doubles * sizeof(double));
   dev_free(h->d_labels, (size_t)h->g.N * 2 * sizeof(int));
@@ -467,9 +491,8 @@ lbm_handle lbm_create_ex(const lbm_config* cfg) {
                cfg->precision >= LBM_F16DEV ? 1 : 0, COLL_SRT, 1.19, 1.4, 1.2, 1.4, 1.98};
   h->ph.inv_rho0 = 1.0 / cfg->rho0;
   phys_finalize(h->ph, cfg->precision);
-  h->block = (cfg->block_x && cfg->block_y && cfg->block_z)
-                 ? dim3(cfg->block_x, cfg->block_y, cfg->block_z)
-                 : default_block(h->g);
+  h->block_asked = cfg->block_x && cfg->block_y && cfg->block_z;
+  h->block = h->block_asked ? dim3(cfg->block_x, cfg->block_y, cfg->block_z) : default_block(h->g);
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) {
@@ -518,6 +541,14 @@ lbm_handle lbm_create_ex(const lbm_config* cfg) {
   }
   if (rc == LBM_OK) rc = dev_alloc((void**)&h->d_flag, sizeof(int) * 4, "flag");
   if (rc == LBM_OK) h->ph.salt = (const unsigned*)(h->d_flag + 2);
+  if (rc == LBM_OK && cfg->precision == LBM_F64) {
+    rc = dev_alloc((void**)&h->d_psi_tab, sizeof(double2) * kPsiTab, "psi table");
+    if (rc == LBM_OK) {
+      e = psi_table_launch(h->d_psi_tab, h->stream);
+      if (e != cudaSuccess) rc = cuda_fail(e, "psi table");
+    }
+    h->ph.psi_tab = h->d_psi_tab;
+  }
   if (rc == LBM_OK) rc = dev_alloc((void**)&h->d_small, sizeof(double) * 64, "results");
   if (rc == LBM_OK) {
     e = cudaMemsetAsync(h->d_flag, 0, sizeof(int) * 4, h->stream);
@@ -663,6 +694,7 @@ int lbm_set_option(lbm_handle h, const char* key, double v) {
     if ((long long)nb.x * nb.y * nb.z > 256 || nb.z > 64)
       return fail(LBM_ERR_ARG, "block shape has more than 256 threads");
     h->block = nb;
+    h->block_asked = true;
     drop_graphs(h);
   } else {
     return fail(LBM_ERR_ARG, "unknown option " + k);
@@ -682,7 +714,7 @@ int lbm_get_option(lbm_handle h, const char* key, double* v) {
   else if (k == "diag_ccl") *v = h->diag_ccl;
   else if (k == "occupancy")
     *v = h->minb ? h->minb
-                 : auto_minb(h->vec && h->g.nx % 2 == 0, h->cfg.pattern == LBM_AA ? MODE_AA_ODD : MODE_AB,
+                 : auto_minb(node_pairs(h->cfg.precision, h->vec, h->g), h->cfg.pattern == LBM_AA ? MODE_AA_ODD : MODE_AB,
                              h->cfg.precision);
   else if (k == "vector") *v = h->vec && (h->g.nx % 2 == 0);
   else if (k == "stochastic_rounding") *v = h->ph.sr;

@@ -178,7 +178,8 @@ __global__ void __launch_bounds__(DX* DY, 2) diag_partial_kernel(Geom g, Phys ph
                                                               const typename Prec<P>::T* f,
                                                               double rho_l, double rho_v,
                                                               double* slices, double* blocks,
-                                                              typename Prec<P>::C* psi, int* flag) {
+                                                              typename Prec<P>::C* psi, int* flag,
+                                                              double* rho_out) {
   using C = typename Prec<P>::C;
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int x = blockIdx.x * DX + tx;
@@ -212,7 +213,10 @@ __global__ void __launch_bounds__(DX* DY, 2) diag_partial_kernel(Geom g, Phys ph
       const C rho = rho_of_x(fv, rho_lo);   // rho_of bitwise, plus its rounding error
       C jx, jy, jz;
       mom_of<C>(fv, jx, jy, jz);
-      if constexpr (WRITE_PSI) psi[i] = psi_of<C>(rho, ph);
+      if constexpr (WRITE_PSI) {
+        psi[i] = psi_of<C>(rho, ph);
+        if (P == LBM_F64 && rho_out) rho_out[i] = rho;
+      }
       s_mass.add(rho, rho_lo);
       s_jx.add(jx);
       s_jy.add(jy);
@@ -653,7 +657,7 @@ cudaError_t moments_t(int layout, const Geom& g, const Phys& ph, const void* f, 
 template <int P>
 cudaError_t diag_t(int layout, const Geom& g, const Phys& ph, const void* f, double rho_l,
                    double rho_v, double* scratch, double* out, void* psi, int* flag,
-                   unsigned long long* ring_count, int ring_cap, cudaStream_t s) {
+                   unsigned long long* ring_count, int ring_cap, cudaStream_t s, double* rho_out) {
   const int rb = diag_row_blocks(g);
   const int gx = (g.nx + DX - 1) / DX;
   double* slices = scratch;
@@ -665,17 +669,17 @@ cudaError_t diag_t(int layout, const Geom& g, const Phys& ph, const void* f, dou
   if (psi) {
     if (layout == LAYOUT_LOCAL)
       diag_partial_kernel<P, true, LAYOUT_LOCAL><<<grid, block, 0, s>>>(
-          g, ph, (const T*)f, rho_l, rho_v, slices, blocks, (C*)psi, flag);
+          g, ph, (const T*)f, rho_l, rho_v, slices, blocks, (C*)psi, flag, rho_out);
     else
       diag_partial_kernel<P, true, LAYOUT_GATHER><<<grid, block, 0, s>>>(
-          g, ph, (const T*)f, rho_l, rho_v, slices, blocks, (C*)psi, flag);
+          g, ph, (const T*)f, rho_l, rho_v, slices, blocks, (C*)psi, flag, rho_out);
   } else {
     if (layout == LAYOUT_LOCAL)
       diag_partial_kernel<P, false, LAYOUT_LOCAL><<<grid, block, 0, s>>>(
-          g, ph, (const T*)f, rho_l, rho_v, slices, blocks, nullptr, nullptr);
+          g, ph, (const T*)f, rho_l, rho_v, slices, blocks, nullptr, nullptr, nullptr);
     else
       diag_partial_kernel<P, false, LAYOUT_GATHER><<<grid, block, 0, s>>>(
-          g, ph, (const T*)f, rho_l, rho_v, slices, blocks, nullptr, nullptr);
+          g, ph, (const T*)f, rho_l, rho_v, slices, blocks, nullptr, nullptr, nullptr);
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
@@ -716,6 +720,17 @@ cudaError_t droplets_t(int layout, const Geom& g, const Phys& ph, const void* f,
 }
 
 }  // namespace
+
+// The table of psi_of<double>: exp(-k/256) and 1 - exp(-k/256), k < kPsiTab.
+__global__ void psi_table_kernel(double2* tab) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k < kPsiTab) tab[k] = make_double2(exp(-k / 256.0), -expm1(-k / 256.0));
+}
+
+cudaError_t psi_table_launch(double2* tab, cudaStream_t s) {
+  psi_table_kernel<<<(kPsiTab + 127) / 128, 128, 0, s>>>(tab);
+  return cudaGetLastError();
+}
 
 // Stochastic-rounding step salt: set it (mode 1), advance it by one (mode
 // 0, after each time step's collision) or by `value` (mode 2, after a launch
@@ -830,16 +845,20 @@ size_t diag_scratch_doubles(const Geom& g) {
 cudaError_t launch_diagnostics(int precision, int layout, const Geom& g, const Phys& ph, const void* f,
                                double rho_l, double rho_v, double* scratch, double* out, void* psi,
                                int* flag, unsigned long long* ring_count, int ring_cap,
-                               cudaStream_t s) {
+                               cudaStream_t s, void* dst) {
   switch (precision) {
     case LBM_F64:
-      return diag_t<LBM_F64>(layout, g, ph, f, rho_l, rho_v, scratch, out, psi, flag, ring_count, ring_cap, s);
+      return diag_t<LBM_F64>(layout, g, ph, f, rho_l, rho_v, scratch, out, psi, flag, ring_count, ring_cap, s,
+                             (double*)dst);
     case LBM_F32:
-      return diag_t<LBM_F32>(layout, g, ph, f, rho_l, rho_v, scratch, out, psi, flag, ring_count, ring_cap, s);
+      return diag_t<LBM_F32>(layout, g, ph, f, rho_l, rho_v, scratch, out, psi, flag, ring_count, ring_cap, s,
+                             nullptr);
     case LBM_F16DEV:
-      return diag_t<LBM_F16DEV>(layout, g, ph, f, rho_l, rho_v, scratch, out, psi, flag, ring_count, ring_cap, s);
+      return diag_t<LBM_F16DEV>(layout, g, ph, f, rho_l, rho_v, scratch, out, psi, flag, ring_count, ring_cap, s,
+                             nullptr);
     case LBM_BF16DEV:
-      return diag_t<LBM_BF16DEV>(layout, g, ph, f, rho_l, rho_v, scratch, out, psi, flag, ring_count, ring_cap, s);
+      return diag_t<LBM_BF16DEV>(layout, g, ph, f, rho_l, rho_v, scratch, out, psi, flag, ring_count, ring_cap, s,
+                             nullptr);
   }
   return cudaErrorInvalidValue;
 }

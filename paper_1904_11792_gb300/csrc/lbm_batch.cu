@@ -58,19 +58,22 @@ __device__ __forceinline__ int find_inst(const BatchInst* __restrict__ inst, int
 
 template <int P>
 __global__ void __launch_bounds__(256) batch_psi_kernel(const BatchInst* __restrict__ inst, int count,
-                                                        const typename Prec<P>::T* pool_f, int cur,
+                                                        typename Prec<P>::T* pool_f, int cur,
                                                         typename Prec<P>::C* pool_psi, int* flag) {
   const int k = find_inst(inst, count, blockIdx.x, true);
   const BatchInst I = inst[k];
   const long long t = (long long)(blockIdx.x - I.psi_block0) * blockDim.x + threadIdx.x;
   const typename Prec<P>::T* f = pool_f + I.off_f + (long long)cur * Q * I.g.N;
-  if (I.vec) {
-    if (2 * t >= I.g.N) return;
-    psi_pair<P, LAYOUT_LOCAL>(I.g, I.ph, f, pool_psi + I.off_psi, flag, 2 * t);
-  } else {
-    if (t >= I.g.N) return;
-    psi_node<P, LAYOUT_LOCAL>(I.g, I.ph, f, pool_psi + I.off_psi, flag, t);
+  double* rho_out = nullptr;
+  if constexpr (P == LBM_F64) rho_out = pool_f + I.off_f + (long long)(cur ^ 1) * Q * I.g.N;
+  if constexpr (P != LBM_F64) {
+    if (I.vec) {
+      if (2 * t < I.g.N) psi_pair<P, LAYOUT_LOCAL>(I.g, I.ph, f, pool_psi + I.off_psi, flag, 2 * t);
+      return;
+    }
   }
+  if (t >= I.g.N) return;
+  psi_node<P, LAYOUT_LOCAL>(I.g, I.ph, f, pool_psi + I.off_psi, flag, t, rho_out);
 }
 
 // Collide-stream over the batch.  A block covers kChunks x blockDim.x
@@ -101,10 +104,13 @@ __global__ void __launch_bounds__(256, MINB) batch_collide_kernel(const BatchIns
     const int x = ii - row * I.g.nx;
     const int z = row / I.g.ny, y = row - z * I.g.ny;
     // the branch is uniform over a block (one instance per block)
-    if (I.vec)
-      collide_pair<P, MODE_AB>(I.g, I.ph, src, dst, pool_psi + I.off_psi, x, y, z);
-    else
-      collide_node<P, MODE_AB>(I.g, I.ph, src, dst, pool_psi + I.off_psi, x, y, z);
+    if constexpr (P != LBM_F64) {
+      if (I.vec) {
+        collide_pair<P, MODE_AB>(I.g, I.ph, src, dst, pool_psi + I.off_psi, x, y, z);
+        continue;
+      }
+    }
+    collide_node<P, MODE_AB>(I.g, I.ph, src, dst, pool_psi + I.off_psi, x, y, z);
   }
 }
 
@@ -113,7 +119,7 @@ cudaError_t batch_launch_t(const BatchInst* d_inst, int count, int psi_blocks, i
                            int cur, void* pool_psi, int* flag, dim3 block, int minb, cudaStream_t s) {
   using T = typename Prec<P>::T;
   using C = typename Prec<P>::C;
-  batch_psi_kernel<P><<<psi_blocks, 256, 0, s>>>(d_inst, count, (const T*)pool_f, cur, (C*)pool_psi, flag);
+  batch_psi_kernel<P><<<psi_blocks, 256, 0, s>>>(d_inst, count, (T*)pool_f, cur, (C*)pool_psi, flag);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const unsigned threads = block.x * block.y * block.z;
@@ -270,6 +276,7 @@ struct lbm_batch_ctx {
   void* pool_psi = nullptr;
   size_t pool_psi_bytes = 0;
   int* d_flag = nullptr;
+  double2* d_psi_tab = nullptr;    // FP64: table of psi_of<double>
   double* d_small = nullptr;
   double* d_scratch = nullptr;
   size_t scratch_doubles = 0;
@@ -324,7 +331,7 @@ int layout_tiles(lbm_batch_ctx* b) {
   long long tiles = 0, psi_blocks = 0;
   const int threads = (int)(b->block.x * b->block.y * b->block.z);
   for (auto& I : b->inst) {
-    I.vec = (b->vec && I.g.nx % 2 == 0) ? 1 : 0;
+    I.vec = node_pairs(b->precision, b->vec, I.g) ? 1 : 0;
     const long long units = I.vec ? I.g.N / 2 : I.g.N;
     I.tile0 = (int)tiles;
     tiles += (units + (long long)threads * kChunks - 1) / ((long long)threads * kChunks);
@@ -602,6 +609,7 @@ void lbm_batch_destroy(lbm_batch b) {
   cudaFree(b->d_tickets);
   cudaFree(b->pool_p);
   cudaFree(b->d_ttable);
+  cudaFree(b->d_psi_tab);
   cudaFree(b->d_small);
   cudaFree(b->d_scratch);
   cudaFree(b->d_labels);
@@ -684,6 +692,11 @@ lbm_batch lbm_batch_create(const lbm_instance* inst, int count, int precision, i
   // d_flag[2] is the stochastic-rounding step salt of every instance
   if (err == cudaSuccess)
     for (auto& I : b->inst) I.ph.salt = (const unsigned*)(b->d_flag + 2);
+  if (err == cudaSuccess && precision == LBM_F64) {
+    err = cudaMalloc(&b->d_psi_tab, sizeof(double2) * kPsiTab);
+    if (err == cudaSuccess) err = psi_table_launch(b->d_psi_tab, b->stream);
+    for (auto& I : b->inst) I.ph.psi_tab = b->d_psi_tab;
+  }
   if (err == cudaSuccess) err = cudaMemsetAsync(b->pool_f, 0, b->pool_f_bytes, b->stream);
   if (err != cudaSuccess) {
     bcuda(err, "lbm_batch_create");
@@ -867,9 +880,9 @@ int lbm_batch_step_sequential(lbm_batch b, int n) {
       View v = view_of(b, k);
       void* dst = (char*)v.f + (b->cur ? -1 : 1) * (long long)Q * v.g.N * (long long)e;
       const bool vec = b->inst[k].vec != 0;
-      BCK(launch_psi(b->precision, LAYOUT_LOCAL, vec, v.g, v.ph, v.f, v.psi, b->d_flag, b->stream));
+      BCK(launch_psi(b->precision, LAYOUT_LOCAL, vec, v.g, v.ph, v.f, v.psi, b->d_flag, b->stream, dst));
       // as a standalone lattice of this size runs by default
-      BCK(launch_collide(b->precision, MODE_AB, 0, vec, v.g, v.ph, v.f, dst, v.psi, default_block(v.g),
+      BCK(launch_collide(b->precision, MODE_AB, 0, vec, v.g, v.ph, v.f, dst, v.psi, auto_block(v.g, vec),
                          b->stream));
     }
     if (batch_sr(b)) BCK(launch_salt((unsigned*)(b->d_flag + 2), false, 0u, b->stream));

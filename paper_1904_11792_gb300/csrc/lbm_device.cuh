@@ -386,6 +386,12 @@ struct Phys {
   float G_f, tau_f, omega_f;   // G, tau, 1 / tau (FP32 division)
   float rho0_f, ninv_rho0_f;   // rho0, -(1 / rho0)
   float shift_f[3];            // storage shifts of the rest, axis and diagonal classes (deviation forms)
+  // FP64 arithmetic: 1 / tau, 1 - 1 / tau and -G tau / 36 (the force enters
+  // through tau F only; phys_finalize), whether rho0 is 1, and the table of
+  // psi_of<double> in device memory (psi_table_launch; nullptr: exp)
+  double omega, om1, gtau;
+  int unit_rho0;
+  const double2* psi_tab;
 };
 enum Collision { COLL_SRT = 0, COLL_MRT = 1 };
 // Sets the FP32 fields of ph from its doubles, for storage `precision`.
@@ -395,6 +401,10 @@ __host__ inline void phys_finalize(Phys& ph, int precision) {
   ph.omega_f = 1.0f / ph.tau_f;
   ph.rho0_f = (float)ph.rho0;
   ph.ninv_rho0_f = -(float)ph.inv_rho0;
+  ph.omega = 1.0 / ph.tau;
+  ph.om1 = 1.0 - ph.omega;
+  ph.gtau = -(ph.G * ph.tau) / 36.0;
+  ph.unit_rho0 = ph.rho0 == 1.0;
   const int lead[3] = {0, 1, 7};
   for (int c = 0; c < 3; ++c) {
     const float v = (float)(wgt(lead[c]) * ph.rho_ref);
@@ -450,12 +460,47 @@ __device__ __forceinline__ void raise_flag(bool bad, int* flag) {
   }
 }
 
+// 1 - exp(-r) in FP64 from a table: for 0 <= r < 8, X the multiple of 1/256
+// nearest r (0 below 1/256), k = 256 X and d = r - X (exact, |d| <= 1/256),
+//   1 - exp(-r) = (1 - T_k) + T_k d q(d),  T_k = exp(-X),
+//   q(d) = 1 - d/2 + d^2/6 - d^3/24 + d^4/120  (Taylor; d^6/720 < 5e-18),
+// which keeps the relative error near 1e-16 where 1 - exp(-r) loses digits
+// for small r.  GB300's FP64 pipe issues about two lanes per clock and SM, so
+// an FP64 step costs what its FP64 instructions cost (the psi pass of
+// 256x128x128: 371 us with exp and the division, 222 us with the table): 7
+// here against about 22 of exp and, for rho0 = 1, no division by rho0; X and k come from the exponent and mantissa
+// bits in integer instructions, which run beside them.  The table (33 KB) sits
+// in L1; the bulk phases read a few entries of it.
+constexpr int kPsiTab = 8 * 256 + 1;   // entries (T_k, 1 - T_k)
+__device__ __forceinline__ double psi_exp_tab(double r, const double2* __restrict__ tab) {
+  const int hi = __double2hiint(r);
+  if (tab == nullptr || (unsigned)hi >= 0x40200000u) return 1.0 - exp(-r);   // r >= 8, negative or NaN
+  // r = m 2^(e - 20) with m the high 21 mantissa bits; one unit of X is 2^s
+  // units of m.  Rounding to nearest carries into the exponent field.
+  const int s = 12 + 1023 - (hi >> 20);
+  int k = 0;
+  double x = 0.0;
+  if (s <= 20) {
+    const int hx = (hi + (1 << (s - 1))) & ~((1 << s) - 1);
+    k = ((hx & 0xFFFFF) | 0x100000) >> (12 + 1023 - (hx >> 20));
+    x = __hiloint2double(hx, 0);
+  }
+  const double d = r - x;
+  const double2 t = __ldg(tab + k);
+  double q = __fma_rn(d, 1.0 / 120.0, -1.0 / 24.0);
+  q = __fma_rn(d, q, 1.0 / 6.0);
+  q = __fma_rn(d, q, -0.5);
+  q = __fma_rn(d, q, 1.0);
+  return __fma_rn(__dmul_rn(t.x, d), q, t.y);
+}
+
 // psi(rho) (definition after Eq. 5).
 template <typename C>
 __device__ __forceinline__ C psi_of(C rho, const Phys& ph) {
   if (ph.psi_form == LBM_PSI_RHO) return rho;
   if constexpr (sizeof(C) == 8) {
-    return ph.rho0 * (1.0 - exp(-rho / ph.rho0));
+    if (ph.unit_rho0) return psi_exp_tab(rho, ph.psi_tab);
+    return __dmul_rn(ph.rho0, psi_exp_tab(rho / ph.rho0, ph.psi_tab));
   } else {
     // products and the difference through the non-contracted forms: the
     // bits of psi_of2 below (a product fused into 1 - e would differ)

@@ -25,13 +25,21 @@ enum Mode {
 enum Layout { LAYOUT_LOCAL = 0, LAYOUT_GATHER = 1 };
 
 size_t elem_size(int precision);
+// Whether the two-kernel step updates two neighbouring nodes per thread
+// (vec: option "vector").
+bool node_pairs(int precision, bool vec, const Geom& g);
 
 // ---- launchers (lbm_step.cu) ---------------------------------------------
 // psi pass: psi[i] = psi(rho_i) for all nodes; flag |= 1 on a non-positive
 // or non-finite density.
 // vec: two nodes per thread with vector accesses (used when nx is even).
+// dst: the destination array of an A-B step, whose slot 0 FP64 storage uses
+// to hand the densities to the step's collide kernel (required before a FP64
+// A-B launch_collide; nullptr otherwise).
 cudaError_t launch_psi(int precision, int layout, bool vec, const Geom& g, const Phys& ph,
-                       const void* f, void* psi, int* flag, cudaStream_t s);
+                       const void* f, void* psi, int* flag, cudaStream_t s, void* dst = nullptr);
+// Fills the table of psi_of<double> (kPsiTab entries in device memory).
+cudaError_t psi_table_launch(double2* tab, cudaStream_t s);
 // fused force + collision + streaming of one step; block has at most 256
 // threads (with vec, block.x counts node pairs); minb (2, 3, 4) = blocks per
 // SM the register budget must allow.
@@ -39,8 +47,14 @@ cudaError_t launch_collide(int precision, int mode, int minb, bool vec, const Ge
                            const Phys& ph, const void* src, void* dst, const void* psi, dim3 block,
                            cudaStream_t s);
 
-// Default collide-stream block shape of a lattice (lbm_api.cu).
+// SMs of a GB300: lattices with little work split it to reach them all.
+constexpr int kSmCount = 152;
+
+// Default collide-stream block shape of a lattice, as the block_x .. block_z
+// options start from, and the shape launched where none was asked for
+// (lbm_api.cu).
 dim3 default_block(const Geom& g);
+dim3 auto_block(const Geom& g, bool pairs);
 
 // force + collision + streaming with the MRT collision (lbm_mrt.cu); the
 // same modes and layouts as launch_collide
@@ -108,11 +122,13 @@ constexpr int DIAG_CCL = 14;
 constexpr int DIAG_STRIDE = 20;
 // psi (nullable): also write psi of every node and raise flag on a bad
 // density (the psi pass of a diagnostic step).  ring_count (nullable):
-// append the record to the ring at out instead of writing out[0..12].
+// append the record to the ring at out instead of writing out[0..12].  dst:
+// as launch_psi (with psi).
 cudaError_t launch_diagnostics(int precision, int layout, const Geom& g, const Phys& ph,
                                const void* f, double rho_l, double rho_v, double* scratch,
                                double* out, void* psi, int* flag,
-                               unsigned long long* ring_count, int ring_cap, cudaStream_t s);
+                               unsigned long long* ring_count, int ring_cap, cudaStream_t s,
+                               void* dst = nullptr);
 
 // Stochastic-rounding step salt (Phys::salt): set to value, or advance by one.
 cudaError_t launch_salt(unsigned* salt, bool set, unsigned value, cudaStream_t s);
@@ -211,6 +227,7 @@ struct lbm_ctx {
   double rho_l = 1.0, rho_v = 0.0;
 
   int* d_flag = nullptr;          // [0] numeric / timeout flag, [2] stochastic-rounding step salt
+  double2* d_psi_tab = nullptr;   // FP64: table of psi_of<double>
   double* d_small = nullptr;      // small result buffer (diagnostics out etc.)
   double* d_scratch = nullptr;    // diagnostics partials
   size_t scratch_doubles = 0;
@@ -225,6 +242,7 @@ struct lbm_ctx {
   int graph_chunk = 0;            // steps per captured chunk
   bool use_graph = true;
   dim3 block{0, 0, 0};
+  bool block_asked = false;       // block was given (else auto_block is launched)
   int minb = 0;                   // collide kernel register budget variant (0 = auto)
   bool vec = true;                // two nodes per thread (when nx is even)
   bool fused = true;              // single-pass fused step on non-diagnostic A-B steps (where it applies)

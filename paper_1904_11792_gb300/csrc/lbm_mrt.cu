@@ -45,18 +45,18 @@ cudaError_t mrt_dispatch(int mode, bool vec, const Geom& g, const Phys& ph, cons
   const C* ps = (const C*)psi;
   const int ux = vec ? g.nx / 2 : g.nx;
   const dim3 grid((ux + block.x - 1) / block.x, (g.ny + block.y - 1) / block.y, (g.nz + block.z - 1) / block.z);
-  if (vec) {
+  if constexpr (P != LBM_F64) if (vec) {
     switch (mode) {
       case MODE_AB: collide_pair_mrt_kernel<P, MODE_AB><<<grid, block, 0, s>>>(g, ph, in, out, ps); break;
       case MODE_AA_EVEN: collide_pair_mrt_kernel<P, MODE_AA_EVEN><<<grid, block, 0, s>>>(g, ph, in, out, ps); break;
       default: collide_pair_mrt_kernel<P, MODE_AA_ODD><<<grid, block, 0, s>>>(g, ph, in, out, ps); break;
     }
-  } else {
-    switch (mode) {
-      case MODE_AB: collide_mrt_kernel<P, MODE_AB><<<grid, block, 0, s>>>(g, ph, in, out, ps); break;
-      case MODE_AA_EVEN: collide_mrt_kernel<P, MODE_AA_EVEN><<<grid, block, 0, s>>>(g, ph, in, out, ps); break;
-      default: collide_mrt_kernel<P, MODE_AA_ODD><<<grid, block, 0, s>>>(g, ph, in, out, ps); break;
-    }
+    return cudaGetLastError();
+  }
+  switch (mode) {
+    case MODE_AB: collide_mrt_kernel<P, MODE_AB><<<grid, block, 0, s>>>(g, ph, in, out, ps); break;
+    case MODE_AA_EVEN: collide_mrt_kernel<P, MODE_AA_EVEN><<<grid, block, 0, s>>>(g, ph, in, out, ps); break;
+    default: collide_mrt_kernel<P, MODE_AA_ODD><<<grid, block, 0, s>>>(g, ph, in, out, ps); break;
   }
   return cudaGetLastError();
 }
@@ -66,10 +66,9 @@ cudaError_t mrt_dispatch(int mode, bool vec, const Geom& g, const Phys& ph, cons
 cudaError_t launch_collide_mrt(int precision, int mode, bool vec, const Geom& g, const Phys& ph, const void* src,
                                void* dst, const void* psi, dim3 block, cudaStream_t s) {
   if ((long long)block.x * block.y * block.z > 256) return cudaErrorInvalidConfiguration;
-  vec = vec && (g.nx % 2 == 0);
+  vec = node_pairs(precision, vec, g);
   switch (precision) {
-    // FP64: one node per thread (two nodes' moments in doubles spill)
-    case LBM_F64: return mrt_dispatch<LBM_F64>(mode, false, g, ph, src, dst, psi, block, s);
+    case LBM_F64: return mrt_dispatch<LBM_F64>(mode, vec, g, ph, src, dst, psi, block, s);
     case LBM_F32: return mrt_dispatch<LBM_F32>(mode, vec, g, ph, src, dst, psi, block, s);
     case LBM_F16DEV: return mrt_dispatch<LBM_F16DEV>(mode, vec, g, ph, src, dst, psi, block, s);
     case LBM_BF16DEV: return mrt_dispatch<LBM_BF16DEV>(mode, vec, g, ph, src, dst, psi, block, s);

@@ -12,8 +12,8 @@
 //                 relaxation (Eq. 3) and streaming to x + c_a.
 //
 // Each comes in a one-node form and a two-node form (x and x + 1, x even)
-// that loads and stores pairs of populations as one 2-element vector where
-// the addresses allow it.  Both forms call the same arithmetic
+// (4- and 2-byte storage) that loads and stores pairs of populations as one
+// 2-element vector where the addresses allow it.  Both forms call the same arithmetic
 // (collide_math, psi_math), so their results are identical.
 #pragma once
 
@@ -36,12 +36,6 @@ __device__ __forceinline__ typename Prec<P>::C shift_of(int a, const Phys& ph) {
 
 // Two adjacent stored populations (x, x + 1) as one vector access.
 template <int P> struct Pair;
-template <> struct Pair<LBM_F64> {
-  using V = double2;
-  __device__ static __forceinline__ void unpack(V v, double& a, double& b) { a = v.x; b = v.y; }
-  __device__ static __forceinline__ V pack(double a, double b) { return make_double2(a, b); }
-  __device__ static __forceinline__ V pack_sr(double a, double b, unsigned, unsigned) { return make_double2(a, b); }
-};
 template <> struct Pair<LBM_F32> {
   using V = float2;
   __device__ static __forceinline__ void unpack(V v, float& a, float& b) { a = v.x; b = v.y; }
@@ -179,7 +173,6 @@ __device__ __forceinline__ void store_pop(const Phys& ph, typename Prec<P>::T* p
 // Correctly rounded reciprocal: the bits of 1 / x (IEEE division) without
 // the division's general path.
 __device__ __forceinline__ float rcp_rn(float x) { return __frcp_rn(x); }
-__device__ __forceinline__ double rcp_rn(double x) { return __drcp_rn(x); }
 
 // Lane-wise correctly rounded reciprocal of a pair.
 __device__ __forceinline__ float2 rcp_rn(float2 x) { return make_float2(__frcp_rn(x.x), __frcp_rn(x.y)); }
@@ -216,14 +209,9 @@ __device__ __forceinline__ void collide_math_ls(const Phys& ph, const C f[Q], C 
   // only where written), so every kernel that inlines this function computes
   // the same bits whatever the compiler's contraction choices around it.
   const C w1 = splat<C>((S)(1.0 / 18.0)), w2 = splat<C>((S)(1.0 / 36.0));
-  // the constants in the arithmetic's precision (FP32: the host's
-  // conversions, read from the kernel parameters)
-  S G_s, tau_s, omega_s;
-  if constexpr (sizeof(S) == 4) {
-    G_s = ph.G_f, tau_s = ph.tau_f, omega_s = ph.omega_f;
-  } else {
-    G_s = (S)ph.G, tau_s = (S)ph.tau, omega_s = (S)1 / tau_s;
-  }
+  // the constants in FP32 (the host's conversions, read from the kernel
+  // parameters)
+  const S G_s = ph.G_f, tau_s = ph.tau_f, omega_s = ph.omega_f;
   const C gp = xmul(splat<C>(-G_s), pc);
   const C Fx = xmul(gp, xfma(w1, ax, xmul(w2, dx)));
   const C Fy = xmul(gp, xfma(w1, ay, xmul(w2, dy)));
@@ -267,6 +255,56 @@ __device__ __forceinline__ void collide_math_ls(const Phys& ph, const C f[Q], C 
     fs[b] = xfma(om1, f[b], vsub(A, B));
   }
   fs[0] = xfma(om1, f[0], xfma(splat<C>((S)-2), sumA, orho));
+}
+
+// 1 / x in FP64 by one third-order (Halley) iteration, y (1 + e + e^2) with e
+// = 1 - x y, on the seed of the PTX instruction rcp.approx.ftz.f64 (relative
+// error below 2^-20, so e^3 is below 2^-60): 3 FP64 instructions.  x = 0, inf
+// and NaN give NaN, where the caller's product with 1 / x is NaN or void
+// anyway (rho = 0 has zero momentum and force).
+__device__ __forceinline__ double rcp_f64(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  double e = __fma_rn(-x, y, 1.0);
+  e = __fma_rn(e, e, e);
+  return __fma_rn(y, e, y);
+}
+
+// The FP64 form (the same equations in fewer
+// operations, since every one occupies GB300's narrow FP64 pipe for 16 clocks
+// per warp): the force enters as tau F = -(G tau / 36) psi (2 a + d), with the
+// constant from the host; of the pair a, b = opp(a) each f* takes om1 f + A
+// +- T cu as two fused multiply-adds; and the rest population takes omega rho
+// minus the closed sum of the other equilibria, 2 sum_pairs A = 12 q + 9 q
+// u'.u' (q = omega w_1 rho; from the lattice's isotropy), so that a rounded
+// w_1 creates no mass.  About 130 FP64 instructions against 190 of the
+// general form with its division by tau and, in the A-B step, the density
+// summed again (load from slot 0, see psi_node): the collide kernel on
+// 256x128x128 1358 -> 988 us.
+template <>
+__device__ __forceinline__ void collide_math_ls<double>(const Phys& ph, const double f[Q], double rho, double jx,
+                                                        double jy, double jz, double pc, double ax, double ay,
+                                                        double az, double dx, double dy, double dz, double fs[Q]) {
+  const double gp = xmul(ph.gtau, pc);
+  const double ir = rcp_f64(rho);
+  const double ux = xmul(xfma(gp, xfma(2.0, ax, dx), jx), ir);
+  const double uy = xmul(xfma(gp, xfma(2.0, ay, dy), jy), ir);
+  const double uz = xmul(xfma(gp, xfma(2.0, az, dz), jz), ir);
+  const double u2 = xfma(uz, uz, xfma(uy, uy, xmul(ux, ux)));
+  const double om1 = ph.om1, orho = xmul(ph.omega, rho);
+  const double q1 = xmul(orho, 1.0 / 18.0), v = xmul(q1, u2);
+  const double E1 = xfma(-1.5, v, q1), M1 = xmul(4.5, q1), T1 = xmul(3.0, q1);
+  const double E2 = xmul(0.5, E1), M2 = xmul(2.25, q1), T2 = xmul(1.5, q1);
+#pragma unroll
+  for (int a = 1; a < Q; a += 2) {
+    const int b = a + 1;  // opp(a)
+    const bool axis = a <= 6;
+    const double cu = cdotu<double>(a, ux, uy, uz);
+    const double A = xfma(xmul(axis ? M1 : M2, cu), cu, axis ? E1 : E2), T = axis ? T1 : T2;
+    fs[a] = xfma(T, cu, xfma(om1, f[a], A));
+    fs[b] = xfma(-T, cu, xfma(om1, f[b], A));
+  }
+  fs[0] = xfma(om1, f[0], xfma(-9.0, v, xfma(-12.0, q1, orho)));
 }
 
 // The same from the neighbour values pn[a] = psi(x + c_a) (a = 1..18).
@@ -329,11 +367,16 @@ __device__ __forceinline__ void psi_math(const Phys& ph, C rho, C* out, int* fla
 
 // LAYOUT_LOCAL reads slot a at x; LAYOUT_GATHER (AA before an odd step)
 // reads slot opp(a) at x - c_a.
+// rho_out (FP64 storage; nullable): where the densities go as well.  The
+// A-B step passes the start of its destination array: the rest population of
+// a node streams nowhere, so slot 0 of the destination holds the node's
+// density from the psi pass until the collision of that node overwrites it,
+// which saves the FP64 collision its 18 additions (kRhoFromDst).
 template <int P, int LAYOUT>
 __device__ __forceinline__ void psi_node(const Geom& g, const Phys& ph,
                                          const typename Prec<P>::T* f,
                                          typename Prec<P>::C* __restrict__ psi,
-                                         int* __restrict__ flag, long long i) {
+                                         int* __restrict__ flag, long long i, double* rho_out = nullptr) {
   using C = typename Prec<P>::C;
   const C s0 = shift_of<P>(0, ph), s1 = shift_of<P>(1, ph),
           s2 = shift_of<P>(7, ph);
@@ -353,7 +396,9 @@ __device__ __forceinline__ void psi_node(const Geom& g, const Phys& ph,
       fv[a] = Prec<P>::load(f + (long long)opp(a) * g.N + nb.idx(-cx(a), -cy(a), -cz(a)),
                             a == 0 ? s0 : (a <= 6 ? s1 : s2));
   }
-  psi_math<C>(ph, rho_of<C>(fv), psi + i, flag);
+  const C rho = rho_of<C>(fv);
+  psi_math<C>(ph, rho, psi + i, flag);
+  if (P == LBM_F64 && rho_out) rho_out[i] = rho;
 }
 
 // Two nodes i, i + 1 (i even, nx even), vector loads where the addresses
@@ -363,6 +408,7 @@ template <int P, int LAYOUT>
 __device__ __forceinline__ void psi_pair(const Geom& g, const Phys& ph, const typename Prec<P>::T* f,
                                          typename Prec<P>::C* __restrict__ psi,
                                          int* __restrict__ flag, long long i) {
+  static_assert(P != LBM_F64, "two-node psi pass is for 4- and 2-byte storage");
   using C = typename Prec<P>::C;
   const C s0 = shift_of<P>(0, ph), s1 = shift_of<P>(1, ph),
           s2 = shift_of<P>(7, ph);
@@ -396,21 +442,14 @@ __device__ __forceinline__ void psi_pair(const Geom& g, const Phys& ph, const ty
       }
     }
   }
-  if constexpr (sizeof(C) == 4) {
-    // the two nodes as float2 lanes (paired FP32 instructions, the bits of
-    // the scalar form)
-    float2 fp[Q];
+  // the two nodes as float2 lanes (paired FP32 instructions, the bits of
+  // the scalar form)
+  float2 fp[Q];
 #pragma unroll
-    for (int a = 0; a < Q; ++a) fp[a] = make_float2(f0[a], f1[a]);
-    const float2 rho = rho_of<float2>(fp);
-    raise_flag(bad_rho(rho.x) | bad_rho(rho.y), flag);
-    *reinterpret_cast<float2*>(psi + i) = psi_of2(rho, ph);
-  } else {
-    C p0, p1;
-    psi_math<C>(ph, rho_of<C>(f0), &p0, flag);
-    psi_math<C>(ph, rho_of<C>(f1), &p1, flag);
-    *reinterpret_cast<double2*>(psi + i) = make_double2(p0, p1);
-  }
+  for (int a = 0; a < Q; ++a) fp[a] = make_float2(f0[a], f1[a]);
+  const float2 rho = rho_of<float2>(fp);
+  raise_flag(bad_rho(rho.x) | bad_rho(rho.y), flag);
+  *reinterpret_cast<float2*>(psi + i) = psi_of2(rho, ph);
 }
 
 // The four populations of slot `a` at x0 .. x0 + 3 of a row (x0 % 4 == 0,
@@ -529,6 +568,11 @@ __device__ __forceinline__ void psi_quad_gather(const Geom& g, const Phys& ph, c
 // collide + stream
 // ---------------------------------------------------------------------------
 
+// Whether the collision takes the density the psi pass left in slot 0 of the
+// destination (psi_node, rho_out): every FP64 A-B step of the paper's collision.
+template <int P, int MODE, int COLL>
+constexpr bool kRhoFromDst = P == LBM_F64 && MODE == MODE_AB && COLL == COLL_SRT;
+
 // One node.
 template <int P, int MODE, int COLL = COLL_SRT>
 __device__ __forceinline__ void collide_node(const Geom& g, const Phys& ph,
@@ -561,6 +605,8 @@ __device__ __forceinline__ void collide_node(const Geom& g, const Phys& ph,
   C fs[Q];
   if constexpr (COLL == COLL_MRT)
     collide_math_mrt<C>(ph, f, __ldg(psi + i), pn, fs);
+  else if constexpr (kRhoFromDst<P, MODE, COLL>)
+    collide_math_r<C>(ph, f, dst[i], __ldg(psi + i), pn, fs);
   else
     collide_math<C>(ph, f, __ldg(psi + i), pn, fs);
   const unsigned seed = (Prec<P>::dev && ph.sr) ? sr_seed(i, fs[0], salt_of(ph)) : 0u;
@@ -585,6 +631,7 @@ __device__ __forceinline__ void collide_pair(const Geom& g, const Phys& ph,
                                              typename Prec<P>::T* dst,
                                              const typename Prec<P>::C* __restrict__ psi, int x0,
                                              int y, int z) {
+  static_assert(P != LBM_F64, "two-node collision is for 4- and 2-byte storage");
   using C = typename Prec<P>::C;
   const int xm = x0 == 0 ? g.nx - 1 : x0 - 1;      // left of node 0
   const int xp = x0 + 2 == g.nx ? 0 : x0 + 2;      // right of node 1
@@ -634,18 +681,9 @@ __device__ __forceinline__ void collide_pair(const Geom& g, const Phys& ph,
 #pragma unroll
     for (int dz = -1; dz <= 1; ++dz) {
       const C* row = psi + rows[dy + 1][dz + 1];
-      C c0, c1;
-      if constexpr (sizeof(C) == 4) {
-        const float2 v = __ldg(reinterpret_cast<const float2*>(row + x0));
-        c0 = v.x;
-        c1 = v.y;
-      } else {
-        const double2 v = __ldg(reinterpret_cast<const double2*>(row + x0));
-        c0 = v.x;
-        c1 = v.y;
-      }
-      q[dy + 1][dz + 1][1] = c0;
-      q[dy + 1][dz + 1][2] = c1;
+      const float2 v = __ldg(reinterpret_cast<const float2*>(row + x0));
+      q[dy + 1][dz + 1][1] = v.x;
+      q[dy + 1][dz + 1][2] = v.y;
       // rows holding a direction with c_x != 0: (0,0), (+-1,0), (0,+-1)
       if (dy == 0 || dz == 0) {
         q[dy + 1][dz + 1][0] = __ldg(row + xm);
@@ -655,27 +693,24 @@ __device__ __forceinline__ void collide_pair(const Geom& g, const Phys& ph,
         q[dy + 1][dz + 1][3] = 0;
       }
     }
-  C pn0[Q], pn1[Q];
-  pn0[0] = pn1[0] = 0;
-#pragma unroll
-  for (int a = 1; a < Q; ++a) {
-    pn0[a] = q[cy(a) + 1][cz(a) + 1][1 + cx(a)];
-    pn1[a] = q[cy(a) + 1][cz(a) + 1][2 + cx(a)];
-  }
   C fs0[Q], fs1[Q];
   if constexpr (COLL == COLL_MRT) {
+    C pn0[Q], pn1[Q];
+    pn0[0] = pn1[0] = 0;
+#pragma unroll
+    for (int a = 1; a < Q; ++a) {
+      pn0[a] = q[cy(a) + 1][cz(a) + 1][1 + cx(a)];
+      pn1[a] = q[cy(a) + 1][cz(a) + 1][2 + cx(a)];
+    }
     collide_math_mrt<C>(ph, f0, q[1][1][1], pn0, fs0);
     collide_math_mrt<C>(ph, f1, q[1][1][2], pn1, fs1);
-  } else if constexpr (sizeof(C) == 4) {
+  } else {
     float2 fp[Q], fs[Q];
 #pragma unroll
     for (int a = 0; a < Q; ++a) fp[a] = make_float2(f0[a], f1[a]);
     collide_pair_math(ph, fp, rho_of<float2>(fp), q, fs);
 #pragma unroll
     for (int a = 0; a < Q; ++a) fs0[a] = fs[a].x, fs1[a] = fs[a].y;
-  } else {
-    collide_math<C>(ph, f0, q[1][1][1], pn0, fs0);
-    collide_math<C>(ph, f1, q[1][1][2], pn1, fs1);
   }
   const bool sr = Prec<P>::dev && ph.sr;
   const unsigned salt = sr ? salt_of(ph) : 0u;

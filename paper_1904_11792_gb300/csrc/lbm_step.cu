@@ -15,10 +15,10 @@ namespace {
 template <int P, int LAYOUT>
 __global__ void __launch_bounds__(256) psi_kernel(Geom g, Phys ph, const typename Prec<P>::T* f,
                                                   typename Prec<P>::C* __restrict__ psi,
-                                                  int* __restrict__ flag) {
+                                                  int* __restrict__ flag, double* rho_out) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= g.N) return;
-  psi_node<P, LAYOUT>(g, ph, f, psi, flag, i);
+  psi_node<P, LAYOUT>(g, ph, f, psi, flag, i, rho_out);
 }
 
 // Fused force + collision + streaming.  One thread per node.  MINB is the
@@ -81,13 +81,21 @@ __global__ void __launch_bounds__(256, MINB) collide_pair_kernel(Geom g, Phys ph
   collide_pair<P, MODE>(g, ph, src, dst, psi, x0, y, z);
 }
 
+// Threads per block of the psi pass: 256, fewer (to one warp) where that
+// leaves less than two blocks per SM.
+int psi_threads(long long units) {
+  int threads = 256;
+  while (threads > 32 && units < (long long)threads * 2 * kSmCount) threads /= 2;
+  return threads;
+}
+
 template <int P>
 cudaError_t psi_dispatch(int layout, bool vec, const Geom& g, const Phys& ph, const void* f,
-                         void* psi, int* flag, cudaStream_t s) {
+                         void* psi, int* flag, cudaStream_t s, double* rho_out) {
   using T = typename Prec<P>::T;
   using C = typename Prec<P>::C;
-  const int threads = 256;
   if constexpr (P != LBM_F64) {
+    const int threads = psi_threads(g.N / 4);
     const long long blocks = (g.N / 4 + threads - 1) / threads;
     if (vec && g.nx % 4 == 0 && layout == LAYOUT_LOCAL) {
       psi_quad_kernel<P><<<(unsigned)blocks, threads, 0, s>>>(g, ph, (const T*)f, (C*)psi, flag);
@@ -102,7 +110,8 @@ cudaError_t psi_dispatch(int layout, bool vec, const Geom& g, const Phys& ph, co
       }
     }
   }
-  if (vec) {
+  const int threads = psi_threads(vec ? g.N / 2 : g.N);
+  if constexpr (P != LBM_F64) if (vec) {
     const long long blocks = (g.N / 2 + threads - 1) / threads;
     if (layout == LAYOUT_LOCAL)
       psi_pair_kernel<P, LAYOUT_LOCAL><<<(unsigned)blocks, threads, 0, s>>>(g, ph, (const T*)f, (C*)psi, flag);
@@ -112,9 +121,11 @@ cudaError_t psi_dispatch(int layout, bool vec, const Geom& g, const Phys& ph, co
   }
   const long long blocks = (g.N + threads - 1) / threads;
   if (layout == LAYOUT_LOCAL)
-    psi_kernel<P, LAYOUT_LOCAL><<<(unsigned)blocks, threads, 0, s>>>(g, ph, (const T*)f, (C*)psi, flag);
+    psi_kernel<P, LAYOUT_LOCAL><<<(unsigned)blocks, threads, 0, s>>>(g, ph, (const T*)f, (C*)psi, flag,
+                rho_out);
   else
-    psi_kernel<P, LAYOUT_GATHER><<<(unsigned)blocks, threads, 0, s>>>(g, ph, (const T*)f, (C*)psi, flag);
+    psi_kernel<P, LAYOUT_GATHER><<<(unsigned)blocks, threads, 0, s>>>(g, ph, (const T*)f, (C*)psi, flag,
+                rho_out);
   return cudaGetLastError();
 }
 
@@ -149,7 +160,7 @@ cudaError_t collide_dispatch(int mode, int minb, bool vec, const Geom& g, const 
   const int ux = vec ? g.nx / 2 : g.nx;  // threads needed along x
   dim3 grid((ux + block.x - 1) / block.x, (g.ny + block.y - 1) / block.y,
             (g.nz + block.z - 1) / block.z);
-  if (vec) {
+  if constexpr (P != LBM_F64) if (vec) {
     switch (minb) {
       case 2: return collide_mode<P, 2, true>(mode, g, ph, src, dst, psi, grid, block, s);
       case 3: return collide_mode<P, 3, true>(mode, g, ph, src, dst, psi, grid, block, s);
@@ -166,13 +177,13 @@ cudaError_t collide_dispatch(int mode, int minb, bool vec, const Geom& g, const 
 }  // namespace
 
 cudaError_t launch_psi(int precision, int layout, bool vec, const Geom& g, const Phys& ph,
-                       const void* f, void* psi, int* flag, cudaStream_t s) {
-  vec = vec && (g.nx % 2 == 0);
+                       const void* f, void* psi, int* flag, cudaStream_t s, void* dst) {
+  vec = node_pairs(precision, vec, g);
   switch (precision) {
-    case LBM_F64: return psi_dispatch<LBM_F64>(layout, vec, g, ph, f, psi, flag, s);
-    case LBM_F32: return psi_dispatch<LBM_F32>(layout, vec, g, ph, f, psi, flag, s);
-    case LBM_F16DEV: return psi_dispatch<LBM_F16DEV>(layout, vec, g, ph, f, psi, flag, s);
-    case LBM_BF16DEV: return psi_dispatch<LBM_BF16DEV>(layout, vec, g, ph, f, psi, flag, s);
+    case LBM_F64: return psi_dispatch<LBM_F64>(layout, vec, g, ph, f, psi, flag, s, (double*)dst);
+    case LBM_F32: return psi_dispatch<LBM_F32>(layout, vec, g, ph, f, psi, flag, s, nullptr);
+    case LBM_F16DEV: return psi_dispatch<LBM_F16DEV>(layout, vec, g, ph, f, psi, flag, s, nullptr);
+    case LBM_BF16DEV: return psi_dispatch<LBM_BF16DEV>(layout, vec, g, ph, f, psi, flag, s, nullptr);
   }
   return cudaErrorInvalidValue;
 }
@@ -181,7 +192,7 @@ cudaError_t launch_collide(int precision, int mode, int minb, bool vec, const Ge
                            const Phys& ph, const void* src, void* dst, const void* psi, dim3 block,
                            cudaStream_t s) {
   if ((long long)block.x * block.y * block.z > 256) return cudaErrorInvalidConfiguration;
-  vec = vec && (g.nx % 2 == 0);
+  vec = node_pairs(precision, vec, g);
   switch (precision) {
     case LBM_F64: return collide_dispatch<LBM_F64>(mode, minb, vec, g, ph, src, dst, psi, block, s);
     case LBM_F32: return collide_dispatch<LBM_F32>(mode, minb, vec, g, ph, src, dst, psi, block, s);
@@ -190,6 +201,12 @@ cudaError_t launch_collide(int precision, int mode, int minb, bool vec, const Ge
   }
   return cudaErrorInvalidValue;
 }
+
+// FP64 kernels take one node per thread: the FP64 pipe bounds them either way
+// (256x128x128: 222 + 988 us per step with one node, 222 + 982 us with two),
+// and lattices of a few warps per SM reach more SMs (4x49x49: 10.3 us per step
+// against 16.5 us).
+bool node_pairs(int precision, bool vec, const Geom& g) { return precision != LBM_F64 && vec && g.nx % 2 == 0; }
 
 size_t elem_size(int precision) {
   switch (precision) {

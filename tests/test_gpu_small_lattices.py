@@ -1,0 +1,75 @@
+"""Small and thin lattices: the launch shapes chosen for rows shorter than a
+warp, and the FP64 pseudo-potential's table at the edges of its ranges."""
+import numpy as np
+import pytest
+
+import lbm_inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def L():
+    from paper_1904_11792_gb300 import build, lbm
+    build.build()
+    lbm.load()
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    return lbm
+
+
+@pytest.mark.parametrize("precision,pattern", [("f64", "ab"), ("f64", "aa"), ("f32", "aa"), ("f16dev", "ab")])
+@pytest.mark.parametrize("shape", [(4, 49, 49), (3, 5, 70), (31, 9, 8), (62, 7, 3), (10, 3, 200), (66, 40, 9)])
+def test_automatic_block_equals_explicit_block(L, shape, precision, pattern):
+    f0 = lbm_inputs.random_populations(*shape, seed=71)
+    out = []
+    for block in (None, (32, 8, 1), (1, 1, 1)):
+        with L.Lattice(*shape, 0.9, -5.5, precision=precision, pattern=pattern, block=block, rho_ref=0.1) as lat:
+            lat.set_option("fused", 0)
+            lat.set_populations(f0)
+            lat.step(5)
+            out.append(lat.populations())
+    np.testing.assert_array_equal(out[0], out[1])
+    np.testing.assert_array_equal(out[0], out[2])
+
+
+def test_block_options_start_from_the_default_shape(L):
+    with L.Lattice(4, 49, 49, 0.9, -5.5, precision="f32") as lat:
+        assert [lat.get_option("block_" + k) for k in "xyz"] == [32, 8, 1]
+        lat.set_option("block_x", 16)
+        assert [lat.get_option("block_" + k) for k in "xyz"] == [16, 8, 1]
+
+
+@pytest.mark.parametrize("rho0", [1.0, 1.7])
+def test_f64_psi_against_expm1(L, rho0):
+    """psi = rho0 (1 - exp(-rho / rho0)) within 2e-15 relative.  The table's
+    Taylor series to the fourth power leaves d^5/720 of d, at most 1.3e-15 for
+    d <= 1/256; three roundings and the entries' own (half a unit in the last
+    place each) add at most 4.5e-16; from r = 8 on 1 - exp(-r) rounds once."""
+    import torch
+    k = np.arange(0, 2050) / 256.0
+    edges = np.concatenate([k + s * e for e in (0.0, 1e-17, 1e-9, 1 / 512, 1 / 512 - 1e-12) for s in (-1, 1)])
+    r = np.concatenate([edges, np.linspace(1e-6, 12.0, 5000), 2.0 ** -np.arange(1, 60), [8.0, np.nextafter(8.0, 0), 30.0]])
+    r = np.unique(r[r > 0])
+    shape = (12, 23, -(-r.size // (12 * 23)))     # x, y, z
+    n = 12 * 23 * shape[2]
+    rho = np.full(n, 1.0)
+    rho[:r.size] = r * rho0
+    f = np.zeros((19, n))
+    f[0] = rho
+    cfg = L.lbm_config_default()
+    cfg.nx, cfg.ny, cfg.nz = shape
+    cfg.G, cfg.rho0, cfg.precision = -5.5, rho0, L.LBM_F64
+    sb, pb = L.lbm_required_bytes(cfg)
+    psi = torch.empty(pb // 8, dtype=torch.float64, device="cuda")
+    cfg.ext_psi, cfg.ext_psi_bytes = psi.data_ptr(), pb
+    h = L.lbm_create_ex(cfg)
+    try:
+        L.lbm_set_populations(h, f)
+        got_rho = L.lbm_moments(h, shape[::-1], ("rho",))["rho"].ravel()
+        got = psi.cpu().numpy()
+    finally:
+        L.lbm_destroy(h)
+    np.testing.assert_array_equal(got_rho, rho)
+    want = -rho0 * np.expm1(-rho / rho0)
+    assert np.max(np.abs(got - want) / want) <= 2e-15
