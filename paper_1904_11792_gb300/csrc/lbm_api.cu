@@ -137,11 +137,12 @@ int cur_layout(const lbm_ctx* h) {
 }
 
 void drop_graphs(lbm_ctx* h) {
-  for (auto& ge : h->graph)
-    if (ge) {
-      cudaGraphExecDestroy(ge);
-      ge = nullptr;
-    }
+  for (auto& pair : h->graph)
+    for (auto& ge : pair)
+      if (ge) {
+        cudaGraphExecDestroy(ge);
+        ge = nullptr;
+      }
 }
 
 cudaEvent_t take_event(lbm_ctx* h) {
@@ -178,8 +179,9 @@ int auto_minb(bool vec, int mode, int precision) {
 
 // Enqueues one time step on stream s.  `phase` is the step parity (AA) or
 // the index of the current array (A-B).  With timing on, each kernel is
-// bracketed by events on s.
-int enqueue_step(lbm_ctx* h, cudaStream_t s, long long step, int cur, bool timed) {
+// bracketed by events on s.  side (captures): where the diagnostics'
+// reduction runs beside the following steps.
+int enqueue_step(lbm_ctx* h, cudaStream_t s, long long step, int cur, bool timed, ReduceSide* side = nullptr) {
   const int prec = h->cfg.precision;
   const bool aa = h->cfg.pattern == LBM_AA;
   const int layout = (aa && (step & 1)) ? LAYOUT_GATHER : LAYOUT_LOCAL;
@@ -189,6 +191,13 @@ int enqueue_step(lbm_ctx* h, cudaStream_t s, long long step, int cur, bool timed
   cudaEvent_t e0 = nullptr, e1 = nullptr, e2 = nullptr;
   const bool diag_step = h->diag_interval > 0 && step % h->diag_interval == 0;
   const bool fused = h->fused && !aa && fused_applicable(h->g, prec);
+  Geom g = h->g;
+  if (h->diag_ccl) side = nullptr;   // the labelling appends to the record of its own step
+  if (side && side->open && diag_step) {
+    CK(cudaStreamWaitEvent(s, side->join, 0));
+    side->open = false;
+    g.chain = 0;   // a kernel with two predecessors
+  }
   // stochastic-rounding salt: a pair of words, read and advanced by the
   // step's collision kernel; the word a step reads follows the A-B array
   // (AA: the step parity), so graph replays and eager steps agree
@@ -200,7 +209,7 @@ int enqueue_step(lbm_ctx* h, cudaStream_t s, long long step, int cur, bool timed
   }
   // a diagnostic step runs fused too when the scratch holds its partials
   const bool fused_diag =
-      fused && diag_step && h->d_scratch && fused_diag_scratch_doubles(h->g, prec, h->fused_fz) <= h->scratch_doubles;
+      fused && diag_step && h->d_scratch && fused_diag_scratch_doubles(g, prec, h->fused_fz) <= h->scratch_doubles;
   if (fused && (!diag_step || fused_diag)) {
     // single pass: psi of each tile is computed from the staged populations
     if (timed) {
@@ -211,9 +220,10 @@ int enqueue_step(lbm_ctx* h, cudaStream_t s, long long step, int cur, bool timed
     if (diag_step) {
       const FusedDiag fd{h->rho_l, h->rho_v, h->d_scratch, h->scratch_doubles, h->d_ring, h->d_ring_count,
                          lbm_ctx::kRing};
-      CK(launch_fused(prec, h->g, ph, src, dst, h->d_flag, h->fused_fz, h->fused_group, &fd, h->fused_stall_test_ns, s));
+      CK(launch_fused(prec, g, ph, src, dst, h->d_flag, h->fused_fz, h->fused_group, &fd,
+                      h->fused_stall_test_ns, s, side));
     } else {
-      CK(launch_fused(prec, h->g, ph, src, dst, h->d_flag, h->fused_fz, h->fused_group, nullptr, h->fused_stall_test_ns, s));
+      CK(launch_fused(prec, g, ph, src, dst, h->d_flag, h->fused_fz, h->fused_group, nullptr, h->fused_stall_test_ns, s));
     }
     if (timed) {
       CK(cudaEventRecord(e1, s));
@@ -234,8 +244,9 @@ int enqueue_step(lbm_ctx* h, cudaStream_t s, long long step, int cur, bool timed
     CK(cudaEventRecord(e0, s));
   }
   if (diag_step) {
-    CK(launch_diagnostics(prec, layout, h->g, h->ph, src, h->rho_l, h->rho_v, h->d_scratch, h->d_ring,
-                          h->psi, h->d_flag, h->d_ring_count, lbm_ctx::kRing, s, aa ? nullptr : dst));
+    CK(launch_diagnostics(prec, layout, g, h->ph, src, h->rho_l, h->rho_v, h->d_scratch, h->d_ring,
+                          h->psi, h->d_flag, h->d_ring_count, lbm_ctx::kRing, s,
+                          aa ? nullptr : dst, side));
     if (h->diag_ccl) {
       long long* d4 = (long long*)(h->d_small + 32);
       CK(launch_ccl(prec, layout, h->g, h->ph, src, 0.5 * (h->rho_l + h->rho_v), h->d_labels,
@@ -243,16 +254,16 @@ int enqueue_step(lbm_ctx* h, cudaStream_t s, long long step, int cur, bool timed
       CK(launch_ccl_ring(d4, h->d_ring, h->d_ring_count, lbm_ctx::kRing, s));
     }
   } else {
-    CK(launch_psi(prec, layout, h->vec, h->g, h->ph, src, h->psi, h->d_flag, s, aa ? nullptr : dst));
+    CK(launch_psi(prec, layout, h->vec, g, h->ph, src, h->psi, h->d_flag, s, aa ? nullptr : dst));
   }
   if (timed) CK(cudaEventRecord(e1, s));
   const bool vec = node_pairs(prec, h->vec, h->g);
   const int minb = h->minb ? h->minb : auto_minb(vec, mode, prec);
   const dim3 block = h->block_asked ? h->block : auto_block(h->g, vec);
   if (h->ph.coll == COLL_MRT)
-    CK(launch_collide_mrt(prec, mode, vec, h->g, ph, src, dst, h->psi, block, s));
+    CK(launch_collide_mrt(prec, mode, vec, g, ph, src, dst, h->psi, block, s));
   else
-    CK(launch_collide(prec, mode, minb, vec, h->g, ph, src, dst, h->psi, block, s));
+    CK(launch_collide(prec, mode, minb, vec, g, ph, src, dst, h->psi, block, s));
   if (timed) {
     CK(cudaEventRecord(e2, s));
     h->pending.push_back({0, e0, e1});
@@ -295,37 +306,53 @@ int chunk_len(const lbm_ctx* h) {
   return k;
 }
 
-// Captures chunk_len() consecutive steps starting at array `phase` (A-B; 0
-// for AA) into an executable graph.  Capture runs on a private stream
+// Steps of the longer graph that small lattices replay while enough steps are
+// left: the multiple of chunk_len() from 16 on.  A graph launch costs about
+// 2.7 us between two replays (64x32x32 FP32 and 4x49x49 FP64, 2-step against
+// 50- and 100-step graphs), as much as a kernel of such a step; larger
+// lattices do not feel it and keep the shorter capture.
+int long_chunk_len(const lbm_ctx* h) {
+  const int c = chunk_len(h);
+  return h->g.chain ? (16 + c - 1) / c * c : c;
+}
+
+// Captures `steps` consecutive steps (a multiple of chunk_len()) starting at
+// array `phase` (A-B; 0 for AA) into an executable graph.  Capture runs on a private stream
 // (capture is not allowed on the legacy default stream); the graph is
 // launched on the handle's stream.
-int capture_chunk(lbm_ctx* h, int phase) {
-  cudaStream_t cs;
-  CK(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
+int capture_chunk(lbm_ctx* h, int phase, int steps, cudaGraphExec_t* exec) {
+  cudaStream_t cs = nullptr;
+  ReduceSide side{nullptr, nullptr, nullptr, false};
   cudaGraph_t graph = nullptr;
   int rc = LBM_OK;
-  cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
-  if (e != cudaSuccess) {
-    cudaStreamDestroy(cs);
-    return cuda_fail(e, "cudaStreamBeginCapture");
+  cudaError_t e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
+  if (e == cudaSuccess && h->diag_interval > 0) {
+    e = cudaStreamCreateWithFlags(&side.stream, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&side.fork, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&side.join, cudaEventDisableTiming);
   }
-  const int C = chunk_len(h);
-  for (int k = 0; k < C && rc == LBM_OK; ++k) {
-    // step numbers relative to a chunk start (a multiple of C): the same
+  if (e == cudaSuccess) e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
+  if (e == cudaSuccess) {
+    // step numbers relative to a chunk start (a multiple of chunk_len()): the same
     // parity and the same diagnostic steps as every replay
-    rc = enqueue_step(h, cs, k, phase ^ (k & 1), false);
+    for (int k = 0; k < steps && rc == LBM_OK; ++k)
+      rc = enqueue_step(h, cs, k, phase ^ (k & 1), false, side.join ? &side : nullptr);
+    if (side.open) e = cudaStreamWaitEvent(cs, side.join, 0);
+    const cudaError_t e2 = cudaStreamEndCapture(cs, &graph);
+    if (e == cudaSuccess) e = e2;
   }
-  e = cudaStreamEndCapture(cs, &graph);
-  cudaStreamDestroy(cs);
-  if (rc != LBM_OK) {
+  if (side.join) cudaEventDestroy(side.join);
+  if (side.fork) cudaEventDestroy(side.fork);
+  if (side.stream) cudaStreamDestroy(side.stream);
+  if (cs) cudaStreamDestroy(cs);
+  if (rc != LBM_OK || e != cudaSuccess) {
     if (graph) cudaGraphDestroy(graph);
-    return rc;
+    return rc != LBM_OK ? rc : cuda_fail(e, "graph capture of the steps");
   }
-  if (e != cudaSuccess) return cuda_fail(e, "cudaStreamEndCapture");
-  e = cudaGraphInstantiate(&h->graph[phase], graph, 0);
+  e = cudaGraphInstantiate(exec, graph, 0);
   cudaGraphDestroy(graph);
   if (e != cudaSuccess) {
-    h->graph[phase] = nullptr;
+    *exec = nullptr;
     return cuda_fail(e, "cudaGraphInstantiate");
   }
   return LBM_OK;
@@ -485,7 +512,8 @@ lbm_handle lbm_create_ex(const lbm_config* cfg) {
     return nullptr;
   }
   h->cfg = *cfg;
-  h->g = Geom{cfg->nx, cfg->ny, cfg->nz, (long long)cfg->nx * cfg->ny * cfg->nz};
+  const long long N = (long long)cfg->nx * cfg->ny * cfg->nz;
+  h->g = Geom{cfg->nx, cfg->ny, cfg->nz, N, N <= kChainNodes ? 1 : 0};
   // stochastic rounding is on by default for the reduced-precision forms
   h->ph = Phys{cfg->tau, cfg->G, cfg->rho0, cfg->rho_ref, cfg->psi_form,
                cfg->precision >= LBM_F16DEV ? 1 : 0, COLL_SRT, 1.19, 1.4, 1.2, 1.4, 1.98};
@@ -808,20 +836,22 @@ int lbm_step(lbm_handle h, int n) {
   if (n < 0) return fail(LBM_ERR_ARG, "negative step count");
   if (!h->initialized) return fail(LBM_ERR_STATE, "lattice not initialised");
   const bool aa = h->cfg.pattern == LBM_AA;
-  const int C = chunk_len(h);
+  const int base = chunk_len(h), longer = long_chunk_len(h);
   const int k = h->diag_interval;
-  if (h->graph_chunk != C) {
+  if (h->graph_chunk != base) {
     drop_graphs(h);
-    h->graph_chunk = C;
+    h->graph_chunk = base;
   }
   while (n > 0) {
-    if (h->use_graph && !h->kernel_timing && n >= C && h->step % C == 0) {
+    if (h->use_graph && !h->kernel_timing && n >= base && h->step % base == 0) {
       const int phase = aa ? 0 : h->cur;
-      if (!h->graph[phase]) {
-        int rc = capture_chunk(h, phase);
+      const int C = n >= longer ? longer : base;
+      cudaGraphExec_t& ge = h->graph[phase][C != base];
+      if (!ge) {
+        int rc = capture_chunk(h, phase, C, &ge);
         if (rc) return rc;
       }
-      CK(cudaGraphLaunch(h->graph[phase], h->stream));
+      CK(cudaGraphLaunch(ge, h->stream));
       if (k > 0)
         for (long long t = h->step; t < h->step + C; t += k) h->diag_steps.push_back(t);
       if (!aa && (C & 1)) h->cur ^= 1;

@@ -2,6 +2,7 @@
 // population export/import, macroscopic fields, FP64 diagnostics and the
 // connected-component labelling of the liquid (droplet count).
 #include "lbm_internal.h"
+#include "lbm_launch.cuh"
 
 namespace lbm {
 
@@ -35,7 +36,7 @@ __device__ __forceinline__ void node_rho_j(const Geom& g, const Phys& ph, int la
   using C = typename Prec<P>::C;
   C v[Q];
 #pragma unroll
-  for (int a = 0; a < Q; ++a) v[a] = Prec<P>::load(f + slot_index(g, layout, a, nb), (C)shift_d<P>(a, ph.rho_ref));
+  for (int a = 0; a < Q; ++a) v[a] = Prec<P>::template load<true>(f + slot_index(g, layout, a, nb), (C)shift_d<P>(a, ph.rho_ref));
   rho = rho_of<C>(v);
   mom_of<C>(v, j[0], j[1], j[2]);
 }
@@ -86,7 +87,7 @@ __global__ void get_plane_kernel(Geom g, Phys ph, int layout, const typename Pre
   Nbr nb;
   nb.make(g, x, y, z);
   using C = typename Prec<P>::C;
-  out[i] = (double)Prec<P>::load(f + slot_index(g, layout, a, nb), (C)shift_d<P>(a, ph.rho_ref));
+  out[i] = (double)Prec<P>::template load<true>(f + slot_index(g, layout, a, nb), (C)shift_d<P>(a, ph.rho_ref));
 }
 
 template <int P>
@@ -200,13 +201,13 @@ __global__ void __launch_bounds__(DX* DY, 2) diag_partial_kernel(Geom g, Phys ph
       if constexpr (LAYOUT == LAYOUT_LOCAL) {
 #pragma unroll
         for (int a = 0; a < Q; ++a)
-          fv[a] = Prec<P>::load(f + (long long)a * g.N + i, a == 0 ? s0 : (a <= 6 ? s1 : s2));
+          fv[a] = Prec<P>::template load<true>(f + (long long)a * g.N + i, a == 0 ? s0 : (a <= 6 ? s1 : s2));
       } else {
         Nbr nb;
         nb.make(g, x, (int)(r % g.ny), (int)(r / g.ny));
 #pragma unroll
         for (int a = 0; a < Q; ++a)
-          fv[a] = Prec<P>::load(f + (long long)opp(a) * g.N + nb.idx(-cx(a), -cy(a), -cz(a)),
+          fv[a] = Prec<P>::template load<true>(f + (long long)opp(a) * g.N + nb.idx(-cx(a), -cy(a), -cz(a)),
                                 a == 0 ? s0 : (a <= 6 ? s1 : s2));
       }
       C rho_lo;
@@ -301,8 +302,8 @@ constexpr int FT = 256;
 // ... with four independent accumulators (loads in flight), then a fixed
 // shuffle tree.  tot[2x] = liquid area A_w(x), tot[2x + 1] = liquid nodes.
 __global__ void __launch_bounds__(256) diag_slices_kernel(Geom g, int row_blocks,
-                                                         const double* __restrict__ slices,
-                                                         double* __restrict__ tot) {
+                                                         const double* slices, double* tot) {
+  if (g.chain) chain_wait();
   const int lane = threadIdx.x & 31;
   const int x = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (x >= g.nx) return;
@@ -380,6 +381,7 @@ __global__ void __launch_bounds__(FT) diag_final_kernel(Geom g, int nblocks, int
   __shared__ double sg[NG][FT];
   __shared__ double smin_w[FT], smin_n[FT];
   __shared__ int smin_x[FT];
+  if (g.chain) chain_wait();
   const int t = threadIdx.x;
   double acc[NG];
 #pragma unroll
@@ -657,7 +659,7 @@ cudaError_t moments_t(int layout, const Geom& g, const Phys& ph, const void* f, 
 template <int P>
 cudaError_t diag_t(int layout, const Geom& g, const Phys& ph, const void* f, double rho_l,
                    double rho_v, double* scratch, double* out, void* psi, int* flag,
-                   unsigned long long* ring_count, int ring_cap, cudaStream_t s, double* rho_out) {
+                   unsigned long long* ring_count, int ring_cap, cudaStream_t s, double* rho_out, ReduceSide* side) {
   const int rb = diag_row_blocks(g);
   const int gx = (g.nx + DX - 1) / DX;
   double* slices = scratch;
@@ -681,13 +683,9 @@ cudaError_t diag_t(int layout, const Geom& g, const Phys& ph, const void* f, dou
       diag_partial_kernel<P, false, LAYOUT_GATHER><<<grid, block, 0, s>>>(
           g, ph, (const T*)f, rho_l, rho_v, slices, blocks, nullptr, nullptr, nullptr);
   }
-  cudaError_t e = cudaGetLastError();
+  const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  diag_slices_kernel<<<(g.nx + 7) / 8, 256, 0, s>>>(g, rb, slices, slice_tot);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  diag_final_kernel<<<1, FT, 0, s>>>(g, gx * rb, 1, slice_tot, blocks, out, ring_count, ring_cap);
-  return cudaGetLastError();
+  return launch_diag_reduce(g, rb, gx * rb, slices, blocks, slice_tot, out, ring_count, ring_cap, s, side);
 }
 template <int P>
 cudaError_t ccl_t(int layout, const Geom& g, const Phys& ph, const void* f, double thr, int* L,
@@ -751,24 +749,35 @@ cudaError_t launch_salt_add(unsigned* salt, unsigned n, cudaStream_t s) {
 
 cudaError_t launch_diag_reduce(const Geom& g, int row_blocks, int nblocks, const double* slices,
                                double* blocks, double* slice_tot, double* out,
-                               unsigned long long* ring_count, int ring_cap, cudaStream_t s) {
-  diag_slices_kernel<<<(g.nx + 7) / 8, 256, 0, s>>>(g, row_blocks, slices, slice_tot);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+                               unsigned long long* ring_count, int ring_cap, cudaStream_t s, ReduceSide* side) {
+  cudaError_t e = cudaSuccess;
+  int chain = g.chain;
+  if (side) {
+    e = cudaEventRecord(side->fork, s);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(side->stream, side->fork, 0);
+    if (e != cudaSuccess) return e;
+    s = side->stream;
+    chain = 0;
+  }
+  e = chain_launch(chain, diag_slices_kernel, (g.nx + 7) / 8, 256, 0, s, g, row_blocks, slices, slice_tot);
   // many records (one per block of the fused step): a parallel first stage
   // folds runs of kChunk records in place (a single block reading 131072
   // records of the 1024x512x512 lattice took 0.44 ms)
   constexpr int kChunk = 256;
   int stride = 1, n = nblocks;
-  if (nblocks > 4 * kChunk) {
+  if (e == cudaSuccess && nblocks > 4 * kChunk) {
     n = (nblocks + kChunk - 1) / kChunk;
     diag_blocks_kernel<<<n, FT, 0, s>>>(nblocks, kChunk, blocks);
     e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
     stride = kChunk;
   }
-  diag_final_kernel<<<1, FT, 0, s>>>(g, n, stride, slice_tot, blocks, out, ring_count, ring_cap);
-  return cudaGetLastError();
+  if (e == cudaSuccess)
+    e = chain_launch(chain, diag_final_kernel, 1, FT, 0, s, g, n, stride, slice_tot, blocks, out, ring_count, ring_cap);
+  if (e == cudaSuccess && side) {
+    e = cudaEventRecord(side->join, s);
+    side->open = true;
+  }
+  return e;
 }
 
 cudaError_t launch_ccl_ring(const long long* out4, double* ring, const unsigned long long* ring_count,
@@ -845,20 +854,20 @@ size_t diag_scratch_doubles(const Geom& g) {
 cudaError_t launch_diagnostics(int precision, int layout, const Geom& g, const Phys& ph, const void* f,
                                double rho_l, double rho_v, double* scratch, double* out, void* psi,
                                int* flag, unsigned long long* ring_count, int ring_cap,
-                               cudaStream_t s, void* dst) {
+                               cudaStream_t s, void* dst, ReduceSide* side) {
   switch (precision) {
     case LBM_F64:
       return diag_t<LBM_F64>(layout, g, ph, f, rho_l, rho_v, scratch, out, psi, flag, ring_count, ring_cap, s,
-                             (double*)dst);
+                             (double*)dst, side);
     case LBM_F32:
       return diag_t<LBM_F32>(layout, g, ph, f, rho_l, rho_v, scratch, out, psi, flag, ring_count, ring_cap, s,
-                             nullptr);
+                             nullptr, side);
     case LBM_F16DEV:
       return diag_t<LBM_F16DEV>(layout, g, ph, f, rho_l, rho_v, scratch, out, psi, flag, ring_count, ring_cap, s,
-                             nullptr);
+                             nullptr, side);
     case LBM_BF16DEV:
       return diag_t<LBM_BF16DEV>(layout, g, ph, f, rho_l, rho_v, scratch, out, psi, flag, ring_count, ring_cap, s,
-                             nullptr);
+                             nullptr, side);
   }
   return cudaErrorInvalidValue;
 }

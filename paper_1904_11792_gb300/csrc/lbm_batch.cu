@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "lbm_gfused.cuh"
+#include "lbm_launch.cuh"
 #include "lbm_node.cuh"
 
 namespace lbm {
@@ -68,12 +69,12 @@ __global__ void __launch_bounds__(256) batch_psi_kernel(const BatchInst* __restr
   if constexpr (P == LBM_F64) rho_out = pool_f + I.off_f + (long long)(cur ^ 1) * Q * I.g.N;
   if constexpr (P != LBM_F64) {
     if (I.vec) {
-      if (2 * t < I.g.N) psi_pair<P, LAYOUT_LOCAL>(I.g, I.ph, f, pool_psi + I.off_psi, flag, 2 * t);
+      if (2 * t < I.g.N) psi_pair<P, LAYOUT_LOCAL, true>(I.g, I.ph, f, pool_psi + I.off_psi, flag, 2 * t);
       return;
     }
   }
   if (t >= I.g.N) return;
-  psi_node<P, LAYOUT_LOCAL>(I.g, I.ph, f, pool_psi + I.off_psi, flag, t, rho_out);
+  psi_node<P, LAYOUT_LOCAL, true>(I.g, I.ph, f, pool_psi + I.off_psi, flag, t, rho_out);
 }
 
 // Collide-stream over the batch.  A block covers kChunks x blockDim.x
@@ -106,11 +107,11 @@ __global__ void __launch_bounds__(256, MINB) batch_collide_kernel(const BatchIns
     // the branch is uniform over a block (one instance per block)
     if constexpr (P != LBM_F64) {
       if (I.vec) {
-        collide_pair<P, MODE_AB>(I.g, I.ph, src, dst, pool_psi + I.off_psi, x, y, z);
+        collide_pair<P, MODE_AB, true>(I.g, I.ph, src, dst, pool_psi + I.off_psi, x, y, z);
         continue;
       }
     }
-    collide_node<P, MODE_AB>(I.g, I.ph, src, dst, pool_psi + I.off_psi, x, y, z);
+    collide_node<P, MODE_AB, true>(I.g, I.ph, src, dst, pool_psi + I.off_psi, x, y, z);
   }
 }
 
@@ -203,24 +204,21 @@ cudaError_t batch_persist_launch(int precision, const GInst* d_ginst, int count,
 
 // The single-pass step of the whole batch: one launch.
 cudaError_t batch_fused_launch(int precision, const GInst* d_ginst, int count, int blocks, void* pool_f, int cur,
-                               int* flag, cudaStream_t s) {
+                               int* flag, int chain, cudaStream_t s) {
   switch (precision) {
     case LBM_F64:
-      gfused_kernel<LBM_F64><<<blocks, GNT, GShape<LBM_F64>::smem, s>>>(d_ginst, count, (double*)pool_f, cur, flag);
-      break;
+      return chain_launch(chain, gfused_kernel<LBM_F64>, blocks, GNT, GShape<LBM_F64>::smem, s, d_ginst, count,
+                          (double*)pool_f, cur, flag);
     case LBM_F32:
-      gfused_kernel<LBM_F32><<<blocks, GNT, GShape<LBM_F32>::smem, s>>>(d_ginst, count, (float*)pool_f, cur, flag);
-      break;
+      return chain_launch(chain, gfused_kernel<LBM_F32>, blocks, GNT, GShape<LBM_F32>::smem, s, d_ginst, count,
+                          (float*)pool_f, cur, flag);
     case LBM_F16DEV:
-      gfused_kernel<LBM_F16DEV><<<blocks, GNT, GShape<LBM_F16DEV>::smem, s>>>(d_ginst, count, (__half*)pool_f,
-                                                                              cur, flag);
-      break;
+      return chain_launch(chain, gfused_kernel<LBM_F16DEV>, blocks, GNT, GShape<LBM_F16DEV>::smem, s, d_ginst, count,
+                          (__half*)pool_f, cur, flag);
     default:
-      gfused_kernel<LBM_BF16DEV><<<blocks, GNT, GShape<LBM_BF16DEV>::smem, s>>>(
-          d_ginst, count, (__nv_bfloat16*)pool_f, cur, flag);
-      break;
+      return chain_launch(chain, gfused_kernel<LBM_BF16DEV>, blocks, GNT, GShape<LBM_BF16DEV>::smem, s, d_ginst, count,
+                          (__nv_bfloat16*)pool_f, cur, flag);
   }
-  return cudaGetLastError();
 }
 
 cudaError_t batch_launch(int precision, const BatchInst* d_inst, int count, int psi_blocks, int tiles,
@@ -479,7 +477,8 @@ int enqueue_batch_step(lbm_batch_ctx* b, cudaStream_t s, int cur) {
     BCK(batch_tma_launch(b->precision, b->d_ttable, b->tplan, b->pool_p, cur, b->d_flag, s));
   // (the caller marks the unpadded copies stale: lbm_batch_step)
   else if (b->fused && fused_fits)
-    BCK(batch_fused_launch(b->precision, b->d_ginst, b->count, b->gblocks, b->pool_f, cur, b->d_flag, s));
+    BCK(batch_fused_launch(b->precision, b->d_ginst, b->count, b->gblocks, b->pool_f, cur, b->d_flag,
+                           b->inst[0].g.chain, s));
   else
     BCK(batch_launch(b->precision, b->d_inst, b->count, b->psi_blocks, b->tiles, b->pool_f, cur, b->pool_psi,
                      b->d_flag, b->block, b->minb, s));
@@ -649,7 +648,7 @@ lbm_batch lbm_batch_create(const lbm_instance* inst, int count, int precision, i
     }
     BatchInst I;
     std::memset(&I, 0, sizeof(I));
-    I.g = Geom{s.nx, s.ny, s.nz, N};
+    I.g = Geom{s.nx, s.ny, s.nz, N, 1};
     I.ph = Phys{s.tau, s.G, rho0, precision >= LBM_F16DEV ? s.rho_v : 0.0, psi_form,
                 precision >= LBM_F16DEV ? 1 : 0};
     I.ph.inv_rho0 = 1.0 / rho0;

@@ -273,16 +273,28 @@ __device__ __forceinline__ void link_sums(const C p[Q], C& ax, C& ay, C& az, C& 
 }
 
 // Storage traits.  T = stored type, C = compute type.  The *DEV forms store
-// the deviation g_a = f_a - w_a rho_ref and add it back on load.  load()
-// goes through the read-only data path and is only used on arrays the kernel
-// does not write; load_rw() is a plain load for in-place (AA) updates.
+// the deviation g_a = f_a - w_a rho_ref and add it back on load.
+//
+// ld: a load through the read-only path (NC) or a plain one.  The read-only
+// path assumes memory that nothing writes while the kernel is resident: it is
+// for arrays the kernel does not write, in kernels that are not launched
+// chained (a chained kernel is resident before its predecessor has finished
+// writing, lbm_launch.cuh).  The two-kernel step keeps it there: with plain
+// loads its register-bound forms are slower (FP16 AA step 4 %).
+template <bool NC, typename T>
+__device__ __forceinline__ T ld(const T* p) {
+  if constexpr (NC)
+    return __ldg(p);
+  else
+    return *p;
+}
 template <int P> struct Prec;
 template <> struct Prec<LBM_F64> {
   using T = double;
   using C = double;
   static constexpr bool dev = false;
-  __device__ static __forceinline__ C load(const T* p, C) { return __ldg(p); }
-  __device__ static __forceinline__ C load_rw(const T* p, C) { return *p; }
+  template <bool NC = false>
+  __device__ static __forceinline__ C load(const T* p, C) { return ld<NC>(p); }
   __device__ static __forceinline__ void store(T* p, C v, C) { *p = v; }
   __device__ static __forceinline__ void store_sr(T* p, C v, C, unsigned) { *p = v; }
 };
@@ -290,8 +302,8 @@ template <> struct Prec<LBM_F32> {
   using T = float;
   using C = float;
   static constexpr bool dev = false;
-  __device__ static __forceinline__ C load(const T* p, C) { return __ldg(p); }
-  __device__ static __forceinline__ C load_rw(const T* p, C) { return *p; }
+  template <bool NC = false>
+  __device__ static __forceinline__ C load(const T* p, C) { return ld<NC>(p); }
   __device__ static __forceinline__ void store(T* p, C v, C) { *p = v; }
   __device__ static __forceinline__ void store_sr(T* p, C v, C, unsigned) { *p = v; }
 };
@@ -299,11 +311,9 @@ template <> struct Prec<LBM_F16DEV> {
   using T = __half;
   using C = float;
   static constexpr bool dev = true;
+  template <bool NC = false>
   __device__ static __forceinline__ C load(const T* p, C shift) {
-    return __half2float(__ldg(p)) + shift;
-  }
-  __device__ static __forceinline__ C load_rw(const T* p, C shift) {
-    return __half2float(*p) + shift;
+    return __half2float(ld<NC>(p)) + shift;
   }
   __device__ static __forceinline__ void store(T* p, C v, C shift) {
     *p = __float2half_rn(v - shift);
@@ -316,11 +326,9 @@ template <> struct Prec<LBM_BF16DEV> {
   using T = __nv_bfloat16;
   using C = float;
   static constexpr bool dev = true;
+  template <bool NC = false>
   __device__ static __forceinline__ C load(const T* p, C shift) {
-    return __bfloat162float(__ldg(p)) + shift;
-  }
-  __device__ static __forceinline__ C load_rw(const T* p, C shift) {
-    return __bfloat162float(*p) + shift;
+    return __bfloat162float(ld<NC>(p)) + shift;
   }
   __device__ static __forceinline__ void store(T* p, C v, C shift) {
     *p = __float2bfloat16_rn(v - shift);
@@ -353,6 +361,7 @@ __device__ __forceinline__ float storage_shift(int a, double rho_ref) {
 struct Geom {
   int nx, ny, nz;
   long long N;  // nx * ny * nz
+  int chain;    // the step's kernels overlap their starts (lbm_launch.cuh)
 };
 
 struct Phys {
@@ -413,7 +422,7 @@ __host__ inline void phys_finalize(Phys& ph, int precision) {
                                                : 0.0f;
   }
 }
-__device__ __forceinline__ unsigned salt_of(const Phys& ph) { return ph.salt ? __ldg(ph.salt) : 0u; }
+__device__ __forceinline__ unsigned salt_of(const Phys& ph) { return ph.salt ? *ph.salt : 0u; }
 // One thread of a step's collision kernel writes salt + 1 for the next step
 // into the other word of the pair, which nothing of this step reads.
 __device__ __forceinline__ void advance_salt(const Phys& ph) {

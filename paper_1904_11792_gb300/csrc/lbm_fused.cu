@@ -188,7 +188,8 @@ cudaError_t fused_grid(const Geom& g, int fz_req, int grp_req, int* fz, int* nch
 
 template <int P>
 cudaError_t fused_t(const Geom& g, const Phys& ph, const void* src, void* dst, int* flag, int fz_req,
-                    int grp_req, const FusedDiag* diag, unsigned long long stall_ns, cudaStream_t s) {
+                    int grp_req, const FusedDiag* diag, unsigned long long stall_ns, cudaStream_t s,
+                    ReduceSide* side) {
   using S = FusedShape<P>;
   int fz = 0, nchunks = 0, grp = 0;
   long long blocks = 0;
@@ -203,13 +204,8 @@ cudaError_t fused_t(const Geom& g, const Phys& ph, const void* src, void* dst, i
   for (int a = 0; a < Q; ++a) db.p[a] = (T*)dst + (long long)a * g.N;
   if (!diag) {
     const DiagOut none = diag_out(0.0, 0.0, nullptr, nullptr, stall_ns);
-    if (ph.coll == COLL_MRT)
-      fused_kernel<P, false, COLL_MRT><<<(unsigned)blocks, S::NT, S::smem, s>>>(m, g, ph, (T*)dst, flag, ntx, nchunks,
-                                                                             fz, grp, none, db);
-    else
-      fused_kernel<P, false, COLL_SRT><<<(unsigned)blocks, S::NT, S::smem, s>>>(m, g, ph, (T*)dst, flag, ntx, nchunks,
-                                                                             fz, grp, none, db);
-    return cudaGetLastError();
+    return chain_launch(g.chain, ph.coll == COLL_MRT ? fused_kernel<P, false, COLL_MRT> : fused_kernel<P, false, COLL_SRT>,
+                        (unsigned)blocks, S::NT, S::smem, s, m, g, ph, (T*)dst, flag, ntx, nchunks, fz, grp, none, db);
   }
   const long long row_blocks = (long long)(g.ny / S::TY) * nchunks;
   const size_t need = (size_t)row_blocks * g.nx * 2 + (size_t)blocks * DIAG_NG + (size_t)g.nx * 2;
@@ -218,16 +214,11 @@ cudaError_t fused_t(const Geom& g, const Phys& ph, const void* src, void* dst, i
   double* bl = slices + (size_t)row_blocks * g.nx * 2;
   double* slice_tot = bl + (size_t)blocks * DIAG_NG;
   const DiagOut dg = diag_out(diag->rho_l, diag->rho_v, slices, bl, stall_ns);
-  if (ph.coll == COLL_MRT)
-    fused_kernel<P, true, COLL_MRT><<<(unsigned)blocks, S::NT, S::smem, s>>>(m, g, ph, (T*)dst, flag, ntx, nchunks,
-                                                                          fz, grp, dg, db);
-  else
-    fused_kernel<P, true, COLL_SRT><<<(unsigned)blocks, S::NT, S::smem, s>>>(m, g, ph, (T*)dst, flag, ntx, nchunks,
-                                                                          fz, grp, dg, db);
-  e = cudaGetLastError();
+  e = chain_launch(g.chain, ph.coll == COLL_MRT ? fused_kernel<P, true, COLL_MRT> : fused_kernel<P, true, COLL_SRT>,
+                   (unsigned)blocks, S::NT, S::smem, s, m, g, ph, (T*)dst, flag, ntx, nchunks, fz, grp, dg, db);
   if (e != cudaSuccess) return e;
   return launch_diag_reduce(g, (int)row_blocks, (int)blocks, slices, bl, slice_tot, diag->out, diag->ring_count,
-                            diag->ring_cap, s);
+                            diag->ring_cap, s, side);
 }
 
 template <int P>
@@ -256,12 +247,13 @@ bool fused_applicable(const Geom& g, int precision) {
 }
 
 cudaError_t launch_fused(int precision, const Geom& g, const Phys& ph, const void* src, void* dst, int* flag,
-                         int fz, int grp, const FusedDiag* diag, unsigned long long stall_ns, cudaStream_t s) {
+                         int fz, int grp, const FusedDiag* diag, unsigned long long stall_ns, cudaStream_t s,
+                         ReduceSide* side) {
   if (!fused_applicable(g, precision)) return cudaErrorInvalidValue;
   switch (precision) {
-    case LBM_F32: return fused_t<LBM_F32>(g, ph, src, dst, flag, fz, grp, diag, stall_ns, s);
-    case LBM_F16DEV: return fused_t<LBM_F16DEV>(g, ph, src, dst, flag, fz, grp, diag, stall_ns, s);
-    case LBM_BF16DEV: return fused_t<LBM_BF16DEV>(g, ph, src, dst, flag, fz, grp, diag, stall_ns, s);
+    case LBM_F32: return fused_t<LBM_F32>(g, ph, src, dst, flag, fz, grp, diag, stall_ns, s, side);
+    case LBM_F16DEV: return fused_t<LBM_F16DEV>(g, ph, src, dst, flag, fz, grp, diag, stall_ns, s, side);
+    case LBM_BF16DEV: return fused_t<LBM_BF16DEV>(g, ph, src, dst, flag, fz, grp, diag, stall_ns, s, side);
   }
   return cudaErrorInvalidValue;
 }
@@ -291,6 +283,7 @@ cudaError_t batch_tma_build_t(const BatchTmaInst* in, int count, int fz_req, int
     BTInst& t = ti[k];
     std::memset(&t, 0, sizeof(t));
     t.g = b.g;
+    plan->chain = b.g.chain;   // the same for all instances
     t.ph = b.ph;
     t.off_f = b.off_f;
     t.px = b.px;
@@ -332,23 +325,19 @@ cudaError_t batch_tma_build_w(int tile_w, const BatchTmaInst* insts, int count, 
 }
 
 template <int P, int W>
-void batch_tma_launch_t(const void* d_table, const BatchTmaPlan& plan, void* pool, int cur, int* flag,
-                        cudaStream_t s) {
+cudaError_t batch_tma_launch_t(const void* d_table, const BatchTmaPlan& plan, void* pool, int cur, int* flag,
+                               cudaStream_t s) {
   using S = FusedShape<P, W>;
-  bfused_kernel<P, W><<<plan.blocks, S::NT, S::smem, s>>>(reinterpret_cast<const BTInst*>(d_table), plan.count,
-                                                          (typename Prec<P>::T*)pool, cur, flag);
+  return chain_launch(plan.chain, bfused_kernel<P, W>, plan.blocks, S::NT, S::smem, s, reinterpret_cast<const BTInst*>(d_table),
+                      plan.count, (typename Prec<P>::T*)pool, cur, flag);
 }
 
 template <int P>
 cudaError_t batch_tma_launch_w(const void* d_table, const BatchTmaPlan& plan, void* pool, int cur, int* flag,
                                cudaStream_t s) {
-  if (plan.width == 32)
-    batch_tma_launch_t<P, 32>(d_table, plan, pool, cur, flag, s);
-  else if (plan.width == TX)
-    batch_tma_launch_t<P, TX>(d_table, plan, pool, cur, flag, s);
-  else
-    return cudaErrorInvalidValue;
-  return cudaGetLastError();
+  if (plan.width == 32) return batch_tma_launch_t<P, 32>(d_table, plan, pool, cur, flag, s);
+  if (plan.width == TX) return batch_tma_launch_t<P, TX>(d_table, plan, pool, cur, flag, s);
+  return cudaErrorInvalidValue;
 }
 
 template <int P, int W>

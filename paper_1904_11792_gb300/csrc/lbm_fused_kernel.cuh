@@ -42,6 +42,7 @@
 
 #include <cuda.h>
 
+#include "lbm_launch.cuh"
 #include "lbm_node.cuh"
 
 namespace lbm {
@@ -236,6 +237,7 @@ __device__ __forceinline__ void fused_body(const Maps& maps, const Geom& g, cons
   unsigned long long* full = reinterpret_cast<unsigned long long*>(smem + S::off_bar);
   C* ring = reinterpret_cast<C*>(smem + S::off_ring);
 
+  if (g.chain) chain_wait();
   advance_salt(ph);
   // Block order: z runs in groups of grp consecutive runs; inside a group
   // the run index varies fastest, then the tile x, then the tile y.  Blocks

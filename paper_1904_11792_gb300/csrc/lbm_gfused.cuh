@@ -24,6 +24,7 @@
 // paper's SRT collision, any storage precision.
 #pragma once
 
+#include "lbm_launch.cuh"
 #include "lbm_node.cuh"
 
 namespace lbm {
@@ -268,6 +269,7 @@ template <int P>
 __global__ void __launch_bounds__(GNT, gfused_minb<P>())
     gfused_kernel(const GInst* __restrict__ inst, int count, typename Prec<P>::T* pool_f, int cur, int* flag) {
   extern __shared__ __align__(16) unsigned char gsm[];
+  if (inst[0].g.chain) chain_wait();
   const Phys& ph = inst[0].ph;   // every instance shares the salt word
   const unsigned salt = (Prec<P>::dev && ph.sr) ? salt_of(ph) : 0u;
   gfused_item<P>(inst, count, pool_f, cur, flag, blockIdx.x, salt, gsm);

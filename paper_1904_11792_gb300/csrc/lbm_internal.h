@@ -29,6 +29,19 @@ size_t elem_size(int precision);
 // (vec: option "vector").
 bool node_pairs(int precision, bool vec, const Geom& g);
 
+// Where the last stages of a diagnostics reduction run while a graph is
+// captured: on a second stream, forked after the kernel that wrote the
+// partials, so that the next steps need not wait for these small kernels (two
+// or three single launches of a few blocks: 17 us per diagnostic step of
+// 64x32x32 FP32 in the steps' own chain, 6 us beside it).  The
+// caller waits for `join` (where open) before the next use of the partials and
+// at the end of the capture.
+struct ReduceSide {
+  cudaStream_t stream;
+  cudaEvent_t fork, join;
+  bool open;
+};
+
 // ---- launchers (lbm_step.cu) ---------------------------------------------
 // psi pass: psi[i] = psi(rho_i) for all nodes; flag |= 1 on a non-positive
 // or non-finite density.
@@ -47,6 +60,9 @@ cudaError_t launch_collide(int precision, int mode, int minb, bool vec, const Ge
                            const Phys& ph, const void* src, void* dst, const void* psi, dim3 block,
                            cudaStream_t s);
 
+// Lattices up to this many nodes launch their steps chained (lbm_launch.cuh)
+// and replay longer graphs: their kernels take a few microseconds each.
+constexpr long long kChainNodes = 1 << 20;
 // SMs of a GB300: lattices with little work split it to reach them all.
 constexpr int kSmCount = 152;
 
@@ -86,7 +102,7 @@ cudaError_t fused_launch_shape(int precision, const Geom& g, int fz_req, int grp
 // block order (0 = automatic).
 cudaError_t launch_fused(int precision, const Geom& g, const Phys& ph, const void* src, void* dst,
                          int* flag, int fz, int grp, const FusedDiag* diag, unsigned long long stall_ns,
-                         cudaStream_t s);
+                         cudaStream_t s, ReduceSide* side = nullptr);
 size_t fused_diag_scratch_doubles(const Geom& g, int precision, int fz);
 
 // ---- auxiliary kernels (lbm_aux.cu) ---------------------------------------
@@ -123,12 +139,13 @@ constexpr int DIAG_STRIDE = 20;
 // psi (nullable): also write psi of every node and raise flag on a bad
 // density (the psi pass of a diagnostic step).  ring_count (nullable):
 // append the record to the ring at out instead of writing out[0..12].  dst:
-// as launch_psi (with psi).
+// as launch_psi (with psi).  side (nullable): where the stages after the pass
+// over the populations run.
 cudaError_t launch_diagnostics(int precision, int layout, const Geom& g, const Phys& ph,
                                const void* f, double rho_l, double rho_v, double* scratch,
                                double* out, void* psi, int* flag,
                                unsigned long long* ring_count, int ring_cap, cudaStream_t s,
-                               void* dst = nullptr);
+                               void* dst = nullptr, ReduceSide* side = nullptr);
 
 // Stochastic-rounding step salt (Phys::salt): set to value, or advance by one.
 cudaError_t launch_salt(unsigned* salt, bool set, unsigned value, cudaStream_t s);
@@ -141,7 +158,8 @@ cudaError_t launch_salt_add(unsigned* salt, unsigned n, cudaStream_t s);
 // blocks is overwritten); arguments after slice_tot as launch_diagnostics.
 cudaError_t launch_diag_reduce(const Geom& g, int row_blocks, int nblocks, const double* slices,
                                double* blocks, double* slice_tot, double* out,
-                               unsigned long long* ring_count, int ring_cap, cudaStream_t s);
+                               unsigned long long* ring_count, int ring_cap, cudaStream_t s,
+                               ReduceSide* side = nullptr);
 
 // Connected components of the liquid mask.  labels: N ints; sizes: N ints;
 // out3 (device, 4 long long): components, components with >= 8 nodes,
@@ -178,9 +196,10 @@ struct BatchTmaInst {
   int px;
 };
 int batch_tma_row_align(int precision);
-// The launch of one step: tile width (32 or 64), instance records, blocks.
+// The launch of one step: tile width (32 or 64), instance records, blocks,
+// chained launches.
 struct BatchTmaPlan {
-  int width, count, blocks;
+  int width, count, blocks, chain;
 };
 // Bytes of the device table (instance records and their tensor maps).
 size_t batch_tma_table_bytes(int count);
@@ -238,8 +257,8 @@ struct lbm_ctx {
 
   // CUDA graphs of one chunk of steps, keyed by the A-B array they start on
   // (AA chunks always start on an even step)
-  cudaGraphExec_t graph[2] = {nullptr, nullptr};
-  int graph_chunk = 0;            // steps per captured chunk
+  cudaGraphExec_t graph[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};   // [phase][longer chunk]
+  int graph_chunk = 0;            // steps per captured chunk (the shorter one)
   bool use_graph = true;
   dim3 block{0, 0, 0};
   bool block_asked = false;       // block was given (else auto_block is launched)

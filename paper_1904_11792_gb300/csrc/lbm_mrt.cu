@@ -13,26 +13,26 @@ namespace {
 template <int P, int MODE>
 __global__ void __launch_bounds__(256, 2) collide_mrt_kernel(Geom g, Phys ph, const typename Prec<P>::T* src,
                                                              typename Prec<P>::T* dst,
-                                                             const typename Prec<P>::C* __restrict__ psi) {
+                                                             const typename Prec<P>::C* psi) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int z = blockIdx.z * blockDim.z + threadIdx.z;
   if (x >= g.nx || y >= g.ny || z >= g.nz) return;
   advance_salt(ph);
-  collide_node<P, MODE, COLL_MRT>(g, ph, src, dst, psi, x, y, z);
+  collide_node<P, MODE, true, COLL_MRT>(g, ph, src, dst, psi, x, y, z);
 }
 
 template <int P, int MODE>
 __global__ void __launch_bounds__(256, 2) collide_pair_mrt_kernel(Geom g, Phys ph,
                                                                   const typename Prec<P>::T* src,
                                                                   typename Prec<P>::T* dst,
-                                                                  const typename Prec<P>::C* __restrict__ psi) {
+                                                                  const typename Prec<P>::C* psi) {
   const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int z = blockIdx.z * blockDim.z + threadIdx.z;
   if (x0 >= g.nx || y >= g.ny || z >= g.nz) return;
   advance_salt(ph);
-  collide_pair<P, MODE, COLL_MRT>(g, ph, src, dst, psi, x0, y, z);
+  collide_pair<P, MODE, true, COLL_MRT>(g, ph, src, dst, psi, x0, y, z);
 }
 
 template <int P>

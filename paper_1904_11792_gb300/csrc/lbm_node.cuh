@@ -119,19 +119,14 @@ __device__ __forceinline__ float load_shifted(const typename Prec<P>::T* p, floa
     return *p;
 }
 
-// Loads populations x and x + 1 (RO: read-only path; else a plain load for
-// in-place updates) and adds the deviation shift.  Full-precision storage has
+// Loads populations x and x + 1 and adds the deviation shift.  Full-precision storage has
 // no shift and skips the add (x + 0 is not x for x = -0, so the compiler
 // keeps it otherwise), as Prec<P>::load does.
-template <int P, bool RO>
+template <int P, bool NC>
 __device__ __forceinline__ void load_pair(const typename Prec<P>::T* p, typename Prec<P>::C sh,
                                           typename Prec<P>::C& a, typename Prec<P>::C& b) {
   using V = typename Pair<P>::V;
-  V v;
-  if constexpr (RO)
-    v = __ldg(reinterpret_cast<const V*>(p));
-  else
-    v = *reinterpret_cast<const V*>(p);
+  const V v = ld<NC>(reinterpret_cast<const V*>(p));
   Pair<P>::unpack(v, a, b);
   if constexpr (Prec<P>::dev) {
     a += sh;
@@ -372,7 +367,7 @@ __device__ __forceinline__ void psi_math(const Phys& ph, C rho, C* out, int* fla
 // a node streams nowhere, so slot 0 of the destination holds the node's
 // density from the psi pass until the collision of that node overwrites it,
 // which saves the FP64 collision its 18 additions (kRhoFromDst).
-template <int P, int LAYOUT>
+template <int P, int LAYOUT, bool NC>
 __device__ __forceinline__ void psi_node(const Geom& g, const Phys& ph,
                                          const typename Prec<P>::T* f,
                                          typename Prec<P>::C* __restrict__ psi,
@@ -384,7 +379,7 @@ __device__ __forceinline__ void psi_node(const Geom& g, const Phys& ph,
   if constexpr (LAYOUT == LAYOUT_LOCAL) {
 #pragma unroll
     for (int a = 0; a < Q; ++a)
-      fv[a] = Prec<P>::load(f + (long long)a * g.N + i, a == 0 ? s0 : (a <= 6 ? s1 : s2));
+      fv[a] = Prec<P>::template load<NC>(f + (long long)a * g.N + i, a == 0 ? s0 : (a <= 6 ? s1 : s2));
   } else {
     const int x = (int)(i % g.nx);
     const long long r = i / g.nx;
@@ -393,7 +388,7 @@ __device__ __forceinline__ void psi_node(const Geom& g, const Phys& ph,
     nb.make(g, x, y, z);
 #pragma unroll
     for (int a = 0; a < Q; ++a)
-      fv[a] = Prec<P>::load(f + (long long)opp(a) * g.N + nb.idx(-cx(a), -cy(a), -cz(a)),
+      fv[a] = Prec<P>::template load<NC>(f + (long long)opp(a) * g.N + nb.idx(-cx(a), -cy(a), -cz(a)),
                             a == 0 ? s0 : (a <= 6 ? s1 : s2));
   }
   const C rho = rho_of<C>(fv);
@@ -404,7 +399,7 @@ __device__ __forceinline__ void psi_node(const Geom& g, const Phys& ph,
 // Two nodes i, i + 1 (i even, nx even), vector loads where the addresses
 // allow (all of LAYOUT_LOCAL; the c_x = 0 slots of LAYOUT_GATHER) and a
 // vector store of the two psi values.
-template <int P, int LAYOUT>
+template <int P, int LAYOUT, bool NC>
 __device__ __forceinline__ void psi_pair(const Geom& g, const Phys& ph, const typename Prec<P>::T* f,
                                          typename Prec<P>::C* __restrict__ psi,
                                          int* __restrict__ flag, long long i) {
@@ -416,7 +411,7 @@ __device__ __forceinline__ void psi_pair(const Geom& g, const Phys& ph, const ty
   if constexpr (LAYOUT == LAYOUT_LOCAL) {
 #pragma unroll
     for (int a = 0; a < Q; ++a)
-      load_pair<P, true>(f + (long long)a * g.N + i, a == 0 ? s0 : (a <= 6 ? s1 : s2), f0[a], f1[a]);
+      load_pair<P, NC>(f + (long long)a * g.N + i, a == 0 ? s0 : (a <= 6 ? s1 : s2), f0[a], f1[a]);
   } else {
     const int x0 = (int)(i % g.nx);
     const long long r = i / g.nx;
@@ -432,13 +427,13 @@ __device__ __forceinline__ void psi_pair(const Geom& g, const Phys& ph, const ty
       const typename Prec<P>::T* base = f + (long long)opp(a) * g.N + row;
       const C sh = a == 0 ? s0 : (a <= 6 ? s1 : s2);
       if (cx(a) == 0) {
-        load_pair<P, true>(base + x0, sh, f0[a], f1[a]);
+        load_pair<P, NC>(base + x0, sh, f0[a], f1[a]);
       } else if (cx(a) > 0) {  // from x0 - 1 and x0
-        f0[a] = Prec<P>::load(base + xm, sh);
-        f1[a] = Prec<P>::load(base + x0, sh);
+        f0[a] = Prec<P>::template load<NC>(base + xm, sh);
+        f1[a] = Prec<P>::template load<NC>(base + x0, sh);
       } else {                 // from x0 + 1 and x0 + 2
-        f0[a] = Prec<P>::load(base + x0 + 1, sh);
-        f1[a] = Prec<P>::load(base + xp, sh);
+        f0[a] = Prec<P>::template load<NC>(base + x0 + 1, sh);
+        f1[a] = Prec<P>::template load<NC>(base + xp, sh);
       }
     }
   }
@@ -454,16 +449,16 @@ __device__ __forceinline__ void psi_pair(const Geom& g, const Phys& ph, const ty
 
 // The four populations of slot `a` at x0 .. x0 + 3 of a row (x0 % 4 == 0,
 // 16-byte (FP32) or 8-byte (2-byte) aligned), unpacked and shifted.
-template <int P>
+template <int P, bool NC>
 __device__ __forceinline__ void load_quad(const typename Prec<P>::T* p, float sh, float v[4]) {
   if constexpr (P == LBM_F32) {
-    const float4 w = __ldg(reinterpret_cast<const float4*>(p));
+    const float4 w = ld<NC>(reinterpret_cast<const float4*>(p));
     v[0] = w.x;
     v[1] = w.y;
     v[2] = w.z;
     v[3] = w.w;
   } else {
-    const uint2 raw = __ldg(reinterpret_cast<const uint2*>(p));
+    const uint2 raw = ld<NC>(reinterpret_cast<const uint2*>(p));
     typename Pair<P>::V lo, hi;
     memcpy(&lo, &raw.x, 4);
     memcpy(&hi, &raw.y, 4);
@@ -478,7 +473,7 @@ __device__ __forceinline__ void load_quad(const typename Prec<P>::T* p, float sh
 
 // Four nodes i .. i + 3 (i % 4 == 0, nx % 4 == 0, LAYOUT_LOCAL): one 16-byte
 // (FP32) or 8-byte (FP16/BF16) load per population, one 16-byte psi store.
-template <int P>
+template <int P, bool NC>
 __device__ __forceinline__ void psi_quad(const Geom& g, const Phys& ph, const typename Prec<P>::T* f,
                                          typename Prec<P>::C* __restrict__ psi,
                                          int* __restrict__ flag, long long i) {
@@ -489,7 +484,7 @@ __device__ __forceinline__ void psi_quad(const Geom& g, const Phys& ph, const ty
 #pragma unroll
   for (int a = 0; a < Q; ++a) {
     float v[4];
-    load_quad<P>(f + (long long)a * g.N + i, a == 0 ? s0 : (a <= 6 ? s1 : s2), v);
+    load_quad<P, NC>(f + (long long)a * g.N + i, a == 0 ? s0 : (a <= 6 ? s1 : s2), v);
 #pragma unroll
     for (int k = 0; k < 4; ++k) fv[k][a] = v[k];
   }
@@ -512,7 +507,7 @@ __device__ __forceinline__ void psi_quad(const Geom& g, const Phys& ph, const ty
 // node), for c_x = -1 the node x0 + 4 from the lane above (its first),
 // except where that lane holds another row or none (lanes 0 and 31, row
 // ends), which load it.  The same values, and psi, as psi_pair.
-template <int P>
+template <int P, bool NC>
 __device__ __forceinline__ void psi_quad_gather(const Geom& g, const Phys& ph, const typename Prec<P>::T* f,
                                                 typename Prec<P>::C* __restrict__ psi, int* __restrict__ flag,
                                                 long long i, bool live) {
@@ -534,7 +529,7 @@ __device__ __forceinline__ void psi_quad_gather(const Geom& g, const Phys& ph, c
     const float sh = a == 0 ? s0 : (a <= 6 ? s1 : s2);
     const typename Prec<P>::T* base = f + (long long)opp(a) * g.N + (long long)g.nx * (yv[1 - cy(a)] + g.ny * zv[1 - cz(a)]);
     float v[4];
-    load_quad<P>(base + x0, sh, v);
+    load_quad<P, NC>(base + x0, sh, v);
     if (cx(a) == 0) {
 #pragma unroll
       for (int k = 0; k < 4; ++k) fv[k][a] = v[k];
@@ -574,11 +569,11 @@ template <int P, int MODE, int COLL>
 constexpr bool kRhoFromDst = P == LBM_F64 && MODE == MODE_AB && COLL == COLL_SRT;
 
 // One node.
-template <int P, int MODE, int COLL = COLL_SRT>
+template <int P, int MODE, bool NC, int COLL = COLL_SRT>
 __device__ __forceinline__ void collide_node(const Geom& g, const Phys& ph,
                                              const typename Prec<P>::T* src,
                                              typename Prec<P>::T* dst,
-                                             const typename Prec<P>::C* __restrict__ psi, int x,
+                                             const typename Prec<P>::C* psi, int x,
                                              int y, int z) {
   using C = typename Prec<P>::C;
   Nbr nb;
@@ -591,24 +586,22 @@ __device__ __forceinline__ void collide_node(const Geom& g, const Phys& ph,
 #pragma unroll
   for (int a = 0; a < Q; ++a) {
     const C sh = a == 0 ? s0 : (a <= 6 ? s1 : s2);
-    if constexpr (MODE == MODE_AB)
-      f[a] = Prec<P>::load(src + (long long)a * N + i, sh);
-    else if constexpr (MODE == MODE_AA_EVEN)
-      f[a] = Prec<P>::load_rw(src + (long long)a * N + i, sh);
+    if constexpr (MODE == MODE_AB || MODE == MODE_AA_EVEN)
+      f[a] = Prec<P>::template load<NC && MODE == MODE_AB>(src + (long long)a * N + i, sh);
     else
-      f[a] = Prec<P>::load_rw(src + (long long)opp(a) * N + nb.idx(-cx(a), -cy(a), -cz(a)), sh);
+      f[a] = Prec<P>::template load<NC && MODE == MODE_AB>(src + (long long)opp(a) * N + nb.idx(-cx(a), -cy(a), -cz(a)), sh);
   }
   C pn[Q];
   pn[0] = 0;
 #pragma unroll
-  for (int a = 1; a < Q; ++a) pn[a] = __ldg(psi + nb.idx(cx(a), cy(a), cz(a)));
+  for (int a = 1; a < Q; ++a) pn[a] = ld<NC>(psi + nb.idx(cx(a), cy(a), cz(a)));
   C fs[Q];
   if constexpr (COLL == COLL_MRT)
-    collide_math_mrt<C>(ph, f, __ldg(psi + i), pn, fs);
+    collide_math_mrt<C>(ph, f, ld<NC>(psi + i), pn, fs);
   else if constexpr (kRhoFromDst<P, MODE, COLL>)
-    collide_math_r<C>(ph, f, dst[i], __ldg(psi + i), pn, fs);
+    collide_math_r<C>(ph, f, dst[i], ld<NC>(psi + i), pn, fs);
   else
-    collide_math<C>(ph, f, __ldg(psi + i), pn, fs);
+    collide_math<C>(ph, f, ld<NC>(psi + i), pn, fs);
   const unsigned seed = (Prec<P>::dev && ph.sr) ? sr_seed(i, fs[0], salt_of(ph)) : 0u;
 #pragma unroll
   for (int a = 0; a < Q; ++a) {
@@ -625,11 +618,11 @@ __device__ __forceinline__ void collide_node(const Geom& g, const Phys& ph,
 // Two nodes x0, x0 + 1 of one row (x0 even, nx even).  Populations whose
 // address pair is contiguous and aligned (x unchanged) move as one vector;
 // those shifted along x (c_x != 0 on a gather or scatter) move one by one.
-template <int P, int MODE, int COLL = COLL_SRT>
+template <int P, int MODE, bool NC, int COLL = COLL_SRT>
 __device__ __forceinline__ void collide_pair(const Geom& g, const Phys& ph,
                                              const typename Prec<P>::T* src,
                                              typename Prec<P>::T* dst,
-                                             const typename Prec<P>::C* __restrict__ psi, int x0,
+                                             const typename Prec<P>::C* psi, int x0,
                                              int y, int z) {
   static_assert(P != LBM_F64, "two-node collision is for 4- and 2-byte storage");
   using C = typename Prec<P>::C;
@@ -656,18 +649,16 @@ __device__ __forceinline__ void collide_pair(const Geom& g, const Phys& ph,
 #pragma unroll
   for (int a = 0; a < Q; ++a) {
     const C sh = a == 0 ? s0 : (a <= 6 ? s1 : s2);
-    if constexpr (MODE == MODE_AB) {
-      load_pair<P, true>(src + (long long)a * N + i0, sh, f0[a], f1[a]);
-    } else if constexpr (MODE == MODE_AA_EVEN) {
-      load_pair<P, false>(src + (long long)a * N + i0, sh, f0[a], f1[a]);
+    if constexpr (MODE == MODE_AB || MODE == MODE_AA_EVEN) {
+      load_pair<P, NC && MODE == MODE_AB>(src + (long long)a * N + i0, sh, f0[a], f1[a]);
     } else {
       const int r = rows[1 - cy(a)][1 - cz(a)];
       const typename Prec<P>::T* base = src + (long long)opp(a) * N + r;
       if (cx(a) == 0) {
-        load_pair<P, false>(base + x0, sh, f0[a], f1[a]);
+        load_pair<P, NC && MODE == MODE_AB>(base + x0, sh, f0[a], f1[a]);
       } else {
-        f0[a] = Prec<P>::load_rw(base + xof(0, -cx(a)), sh);
-        f1[a] = Prec<P>::load_rw(base + xof(1, -cx(a)), sh);
+        f0[a] = Prec<P>::template load<NC && MODE == MODE_AB>(base + xof(0, -cx(a)), sh);
+        f1[a] = Prec<P>::template load<NC && MODE == MODE_AB>(base + xof(1, -cx(a)), sh);
       }
     }
   }
@@ -681,13 +672,13 @@ __device__ __forceinline__ void collide_pair(const Geom& g, const Phys& ph,
 #pragma unroll
     for (int dz = -1; dz <= 1; ++dz) {
       const C* row = psi + rows[dy + 1][dz + 1];
-      const float2 v = __ldg(reinterpret_cast<const float2*>(row + x0));
+      const float2 v = ld<NC>(reinterpret_cast<const float2*>(row + x0));
       q[dy + 1][dz + 1][1] = v.x;
       q[dy + 1][dz + 1][2] = v.y;
       // rows holding a direction with c_x != 0: (0,0), (+-1,0), (0,+-1)
       if (dy == 0 || dz == 0) {
-        q[dy + 1][dz + 1][0] = __ldg(row + xm);
-        q[dy + 1][dz + 1][3] = __ldg(row + xp);
+        q[dy + 1][dz + 1][0] = ld<NC>(row + xm);
+        q[dy + 1][dz + 1][3] = ld<NC>(row + xp);
       } else {
         q[dy + 1][dz + 1][0] = 0;
         q[dy + 1][dz + 1][3] = 0;

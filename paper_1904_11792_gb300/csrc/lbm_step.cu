@@ -5,6 +5,9 @@
 // fastest, so a warp's 32 threads touch 32 consecutive x of one plane per
 // load or store.  Both kernels are bound by HBM bandwidth (about 1 flop per
 // byte); no tensor-core work exists on this path.
+#include <type_traits>
+
+#include "lbm_launch.cuh"
 #include "lbm_node.cuh"
 
 namespace lbm {
@@ -12,73 +15,79 @@ namespace lbm {
 namespace {
 
 // psi pass over all nodes of one lattice.
-template <int P, int LAYOUT>
+template <int P, int LAYOUT, bool CHAIN>
 __global__ void __launch_bounds__(256) psi_kernel(Geom g, Phys ph, const typename Prec<P>::T* f,
                                                   typename Prec<P>::C* __restrict__ psi,
                                                   int* __restrict__ flag, double* rho_out) {
+  if constexpr (CHAIN) chain_wait();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= g.N) return;
-  psi_node<P, LAYOUT>(g, ph, f, psi, flag, i, rho_out);
+  psi_node<P, LAYOUT, !CHAIN>(g, ph, f, psi, flag, i, rho_out);
 }
 
 // Fused force + collision + streaming.  One thread per node.  MINB is the
 // number of 256-thread blocks per SM the register allocation must allow
 // (4: <= 64 registers, 3: <= 80, 2: <= 128); the autotuner picks it.
-template <int P, int MODE, int MINB>
+template <int P, int MODE, int MINB, bool CHAIN>
 __global__ void __launch_bounds__(256, MINB) collide_kernel(Geom g, Phys ph,
                                                             const typename Prec<P>::T* src,
                                                             typename Prec<P>::T* dst,
-                                                            const typename Prec<P>::C* __restrict__ psi) {
+                                                            const typename Prec<P>::C* psi) {
+  if constexpr (CHAIN) chain_wait();
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int z = blockIdx.z * blockDim.z + threadIdx.z;
   if (x >= g.nx || y >= g.ny || z >= g.nz) return;
   advance_salt(ph);
-  collide_node<P, MODE>(g, ph, src, dst, psi, x, y, z);
+  collide_node<P, MODE, !CHAIN>(g, ph, src, dst, psi, x, y, z);
 }
 
 // Two-node forms (x even, nx even): one thread per node pair.
-template <int P, int LAYOUT>
+template <int P, int LAYOUT, bool CHAIN>
 __global__ void __launch_bounds__(256) psi_pair_kernel(Geom g, Phys ph, const typename Prec<P>::T* f,
                                                        typename Prec<P>::C* __restrict__ psi,
                                                        int* __restrict__ flag) {
+  if constexpr (CHAIN) chain_wait();
   const long long i = 2 * ((long long)blockIdx.x * blockDim.x + threadIdx.x);
   if (i >= g.N) return;
-  psi_pair<P, LAYOUT>(g, ph, f, psi, flag, i);
+  psi_pair<P, LAYOUT, !CHAIN>(g, ph, f, psi, flag, i);
 }
 
-template <int P>
+template <int P, bool CHAIN>
 __global__ void __launch_bounds__(256) psi_quad_kernel(Geom g, Phys ph, const typename Prec<P>::T* f,
                                                        typename Prec<P>::C* __restrict__ psi,
                                                        int* __restrict__ flag) {
+  if constexpr (CHAIN) chain_wait();
   const long long i = 4 * ((long long)blockIdx.x * blockDim.x + threadIdx.x);
   if (i >= g.N) return;
-  psi_quad<P>(g, ph, f, psi, flag, i);
+  psi_quad<P, !CHAIN>(g, ph, f, psi, flag, i);
 }
 
 // Gather layout, four nodes per thread; every thread of the last block takes
 // part in the warp shuffles (those past the lattice on its last quad).
-template <int P>
+template <int P, bool CHAIN>
 __global__ void __launch_bounds__(256) psi_quad_gather_kernel(Geom g, Phys ph, const typename Prec<P>::T* f,
                                                               typename Prec<P>::C* __restrict__ psi,
                                                               int* __restrict__ flag) {
+  if constexpr (CHAIN) chain_wait();
   long long i = 4 * ((long long)blockIdx.x * blockDim.x + threadIdx.x);
   const bool live = i < g.N;
   if (!live) i = g.N - 4;
-  psi_quad_gather<P>(g, ph, f, psi, flag, i, live);
+  psi_quad_gather<P, !CHAIN>(g, ph, f, psi, flag, i, live);
 }
 
-template <int P, int MODE, int MINB>
+template <int P, int MODE, int MINB, bool CHAIN>
 __global__ void __launch_bounds__(256, MINB) collide_pair_kernel(Geom g, Phys ph,
                                                                  const typename Prec<P>::T* src,
                                                                  typename Prec<P>::T* dst,
-                                                                 const typename Prec<P>::C* __restrict__ psi) {
+                                                                 const typename Prec<P>::C* psi) {
+  if constexpr (CHAIN) chain_wait();
   const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int z = blockIdx.z * blockDim.z + threadIdx.z;
   if (x0 >= g.nx || y >= g.ny || z >= g.nz) return;
   advance_salt(ph);
-  collide_pair<P, MODE>(g, ph, src, dst, psi, x0, y, z);
+  collide_pair<P, MODE, !CHAIN>(g, ph, src, dst, psi, x0, y, z);
 }
 
 // Threads per block of the psi pass: 256, fewer (to one warp) where that
@@ -89,7 +98,7 @@ int psi_threads(long long units) {
   return threads;
 }
 
-template <int P>
+template <int P, bool CHAIN>
 cudaError_t psi_dispatch(int layout, bool vec, const Geom& g, const Phys& ph, const void* f,
                          void* psi, int* flag, cudaStream_t s, double* rho_out) {
   using T = typename Prec<P>::T;
@@ -98,15 +107,14 @@ cudaError_t psi_dispatch(int layout, bool vec, const Geom& g, const Phys& ph, co
     const int threads = psi_threads(g.N / 4);
     const long long blocks = (g.N / 4 + threads - 1) / threads;
     if (vec && g.nx % 4 == 0 && layout == LAYOUT_LOCAL) {
-      psi_quad_kernel<P><<<(unsigned)blocks, threads, 0, s>>>(g, ph, (const T*)f, (C*)psi, flag);
-      return cudaGetLastError();
+      return chain_launch(CHAIN, psi_quad_kernel<P, CHAIN>, (unsigned)blocks, threads, 0, s, g, ph, (const T*)f, (C*)psi, flag);
     }
     // the gather layout in four-node form for 2-byte storage only (FP32:
     // 10.28 ms against 9.84 ms per AA step on 1024x512x512 with node pairs)
     if constexpr (Prec<P>::dev) {
       if (vec && g.nx % 4 == 0) {
-        psi_quad_gather_kernel<P><<<(unsigned)blocks, threads, 0, s>>>(g, ph, (const T*)f, (C*)psi, flag);
-        return cudaGetLastError();
+        return chain_launch(CHAIN, psi_quad_gather_kernel<P, CHAIN>, (unsigned)blocks, threads, 0, s, g, ph, (const T*)f, (C*)psi,
+                            flag);
       }
     }
   }
@@ -114,22 +122,22 @@ cudaError_t psi_dispatch(int layout, bool vec, const Geom& g, const Phys& ph, co
   if constexpr (P != LBM_F64) if (vec) {
     const long long blocks = (g.N / 2 + threads - 1) / threads;
     if (layout == LAYOUT_LOCAL)
-      psi_pair_kernel<P, LAYOUT_LOCAL><<<(unsigned)blocks, threads, 0, s>>>(g, ph, (const T*)f, (C*)psi, flag);
+      return chain_launch(CHAIN, psi_pair_kernel<P, LAYOUT_LOCAL, CHAIN>, (unsigned)blocks, threads, 0, s, g, ph, (const T*)f,
+                          (C*)psi, flag);
     else
-      psi_pair_kernel<P, LAYOUT_GATHER><<<(unsigned)blocks, threads, 0, s>>>(g, ph, (const T*)f, (C*)psi, flag);
-    return cudaGetLastError();
+      return chain_launch(CHAIN, psi_pair_kernel<P, LAYOUT_GATHER, CHAIN>, (unsigned)blocks, threads, 0, s, g, ph, (const T*)f,
+                          (C*)psi, flag);
   }
   const long long blocks = (g.N + threads - 1) / threads;
   if (layout == LAYOUT_LOCAL)
-    psi_kernel<P, LAYOUT_LOCAL><<<(unsigned)blocks, threads, 0, s>>>(g, ph, (const T*)f, (C*)psi, flag,
-                rho_out);
+    return chain_launch(CHAIN, psi_kernel<P, LAYOUT_LOCAL, CHAIN>, (unsigned)blocks, threads, 0, s, g, ph, (const T*)f, (C*)psi,
+                        flag, rho_out);
   else
-    psi_kernel<P, LAYOUT_GATHER><<<(unsigned)blocks, threads, 0, s>>>(g, ph, (const T*)f, (C*)psi, flag,
-                rho_out);
-  return cudaGetLastError();
+    return chain_launch(CHAIN, psi_kernel<P, LAYOUT_GATHER, CHAIN>, (unsigned)blocks, threads, 0, s, g, ph, (const T*)f, (C*)psi,
+                        flag, rho_out);
 }
 
-template <int P, int MINB, bool VEC>
+template <int P, bool CHAIN, int MINB, bool VEC>
 cudaError_t collide_mode(int mode, const Geom& g, const Phys& ph, const void* src, void* dst,
                          const void* psi, dim3 grid, dim3 block, cudaStream_t s) {
   using T = typename Prec<P>::T;
@@ -139,21 +147,22 @@ cudaError_t collide_mode(int mode, const Geom& g, const Phys& ph, const void* sr
   const C* ps = (const C*)psi;
   if constexpr (VEC) {
     switch (mode) {
-      case MODE_AB: collide_pair_kernel<P, MODE_AB, MINB><<<grid, block, 0, s>>>(g, ph, in, out, ps); break;
-      case MODE_AA_EVEN: collide_pair_kernel<P, MODE_AA_EVEN, MINB><<<grid, block, 0, s>>>(g, ph, in, out, ps); break;
-      default: collide_pair_kernel<P, MODE_AA_ODD, MINB><<<grid, block, 0, s>>>(g, ph, in, out, ps); break;
+      case MODE_AB: return chain_launch(CHAIN, collide_pair_kernel<P, MODE_AB, MINB, CHAIN>, grid, block, 0, s, g, ph, in, out, ps);
+      case MODE_AA_EVEN: return chain_launch(CHAIN, collide_pair_kernel<P, MODE_AA_EVEN, MINB, CHAIN>, grid, block, 0, s, g, ph, in,
+                                             out, ps);
+      default: return chain_launch(CHAIN, collide_pair_kernel<P, MODE_AA_ODD, MINB, CHAIN>, grid, block, 0, s, g, ph, in, out, ps);
     }
   } else {
     switch (mode) {
-      case MODE_AB: collide_kernel<P, MODE_AB, MINB><<<grid, block, 0, s>>>(g, ph, in, out, ps); break;
-      case MODE_AA_EVEN: collide_kernel<P, MODE_AA_EVEN, MINB><<<grid, block, 0, s>>>(g, ph, in, out, ps); break;
-      default: collide_kernel<P, MODE_AA_ODD, MINB><<<grid, block, 0, s>>>(g, ph, in, out, ps); break;
+      case MODE_AB: return chain_launch(CHAIN, collide_kernel<P, MODE_AB, MINB, CHAIN>, grid, block, 0, s, g, ph, in, out, ps);
+      case MODE_AA_EVEN: return chain_launch(CHAIN, collide_kernel<P, MODE_AA_EVEN, MINB, CHAIN>, grid, block, 0, s, g, ph, in, out,
+                                             ps);
+      default: return chain_launch(CHAIN, collide_kernel<P, MODE_AA_ODD, MINB, CHAIN>, grid, block, 0, s, g, ph, in, out, ps);
     }
   }
-  return cudaGetLastError();
 }
 
-template <int P>
+template <int P, bool CHAIN>
 cudaError_t collide_dispatch(int mode, int minb, bool vec, const Geom& g, const Phys& ph,
                              const void* src, void* dst, const void* psi, dim3 block,
                              cudaStream_t s) {
@@ -162,15 +171,15 @@ cudaError_t collide_dispatch(int mode, int minb, bool vec, const Geom& g, const 
             (g.nz + block.z - 1) / block.z);
   if constexpr (P != LBM_F64) if (vec) {
     switch (minb) {
-      case 2: return collide_mode<P, 2, true>(mode, g, ph, src, dst, psi, grid, block, s);
-      case 3: return collide_mode<P, 3, true>(mode, g, ph, src, dst, psi, grid, block, s);
-      default: return collide_mode<P, 4, true>(mode, g, ph, src, dst, psi, grid, block, s);
+      case 2: return collide_mode<P, CHAIN, 2, true>(mode, g, ph, src, dst, psi, grid, block, s);
+      case 3: return collide_mode<P, CHAIN, 3, true>(mode, g, ph, src, dst, psi, grid, block, s);
+      default: return collide_mode<P, CHAIN, 4, true>(mode, g, ph, src, dst, psi, grid, block, s);
     }
   }
   switch (minb) {
-    case 2: return collide_mode<P, 2, false>(mode, g, ph, src, dst, psi, grid, block, s);
-    case 3: return collide_mode<P, 3, false>(mode, g, ph, src, dst, psi, grid, block, s);
-    default: return collide_mode<P, 4, false>(mode, g, ph, src, dst, psi, grid, block, s);
+    case 2: return collide_mode<P, CHAIN, 2, false>(mode, g, ph, src, dst, psi, grid, block, s);
+    case 3: return collide_mode<P, CHAIN, 3, false>(mode, g, ph, src, dst, psi, grid, block, s);
+    default: return collide_mode<P, CHAIN, 4, false>(mode, g, ph, src, dst, psi, grid, block, s);
   }
 }
 
@@ -179,13 +188,17 @@ cudaError_t collide_dispatch(int mode, int minb, bool vec, const Geom& g, const 
 cudaError_t launch_psi(int precision, int layout, bool vec, const Geom& g, const Phys& ph,
                        const void* f, void* psi, int* flag, cudaStream_t s, void* dst) {
   vec = node_pairs(precision, vec, g);
-  switch (precision) {
-    case LBM_F64: return psi_dispatch<LBM_F64>(layout, vec, g, ph, f, psi, flag, s, (double*)dst);
-    case LBM_F32: return psi_dispatch<LBM_F32>(layout, vec, g, ph, f, psi, flag, s, nullptr);
-    case LBM_F16DEV: return psi_dispatch<LBM_F16DEV>(layout, vec, g, ph, f, psi, flag, s, nullptr);
-    case LBM_BF16DEV: return psi_dispatch<LBM_BF16DEV>(layout, vec, g, ph, f, psi, flag, s, nullptr);
-  }
-  return cudaErrorInvalidValue;
+  auto run = [&](auto chain) {
+    constexpr bool CHAIN = decltype(chain)::value;
+    switch (precision) {
+      case LBM_F64: return psi_dispatch<LBM_F64, CHAIN>(layout, vec, g, ph, f, psi, flag, s, (double*)dst);
+      case LBM_F32: return psi_dispatch<LBM_F32, CHAIN>(layout, vec, g, ph, f, psi, flag, s, nullptr);
+      case LBM_F16DEV: return psi_dispatch<LBM_F16DEV, CHAIN>(layout, vec, g, ph, f, psi, flag, s, nullptr);
+      case LBM_BF16DEV: return psi_dispatch<LBM_BF16DEV, CHAIN>(layout, vec, g, ph, f, psi, flag, s, nullptr);
+    }
+    return cudaErrorInvalidValue;
+  };
+  return g.chain ? run(std::true_type{}) : run(std::false_type{});
 }
 
 cudaError_t launch_collide(int precision, int mode, int minb, bool vec, const Geom& g,
@@ -193,13 +206,17 @@ cudaError_t launch_collide(int precision, int mode, int minb, bool vec, const Ge
                            cudaStream_t s) {
   if ((long long)block.x * block.y * block.z > 256) return cudaErrorInvalidConfiguration;
   vec = node_pairs(precision, vec, g);
-  switch (precision) {
-    case LBM_F64: return collide_dispatch<LBM_F64>(mode, minb, vec, g, ph, src, dst, psi, block, s);
-    case LBM_F32: return collide_dispatch<LBM_F32>(mode, minb, vec, g, ph, src, dst, psi, block, s);
-    case LBM_F16DEV: return collide_dispatch<LBM_F16DEV>(mode, minb, vec, g, ph, src, dst, psi, block, s);
-    case LBM_BF16DEV: return collide_dispatch<LBM_BF16DEV>(mode, minb, vec, g, ph, src, dst, psi, block, s);
-  }
-  return cudaErrorInvalidValue;
+  auto run = [&](auto chain) {
+    constexpr bool CHAIN = decltype(chain)::value;
+    switch (precision) {
+      case LBM_F64: return collide_dispatch<LBM_F64, CHAIN>(mode, minb, vec, g, ph, src, dst, psi, block, s);
+      case LBM_F32: return collide_dispatch<LBM_F32, CHAIN>(mode, minb, vec, g, ph, src, dst, psi, block, s);
+      case LBM_F16DEV: return collide_dispatch<LBM_F16DEV, CHAIN>(mode, minb, vec, g, ph, src, dst, psi, block, s);
+      case LBM_BF16DEV: return collide_dispatch<LBM_BF16DEV, CHAIN>(mode, minb, vec, g, ph, src, dst, psi, block, s);
+    }
+    return cudaErrorInvalidValue;
+  };
+  return g.chain ? run(std::true_type{}) : run(std::false_type{});
 }
 
 // FP64 kernels take one node per thread: the FP64 pipe bounds them either way

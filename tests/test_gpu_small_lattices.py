@@ -73,3 +73,32 @@ def test_f64_psi_against_expm1(L, rho0):
     np.testing.assert_array_equal(got_rho, rho)
     want = -rho0 * np.expm1(-rho / rho0)
     assert np.max(np.abs(got - want) / want) <= 2e-15
+
+
+@pytest.mark.parametrize("shape,precision,pattern,fused", [((64, 8, 12), "f32", "ab", 1), ((64, 8, 12), "f16dev", "ab", 1),
+                                                           ((10, 9, 8), "f64", "ab", 0), ((12, 9, 8), "f16dev", "aa", 0)])
+@pytest.mark.parametrize("interval", [0, 1, 3, 10])
+def test_long_graphs_and_side_reductions_equal_eager_steps(L, shape, precision, pattern, fused, interval):
+    """Small lattices replay longer graphs of chained launches, whose
+    diagnostics are reduced beside the following steps: the state and every
+    record equal those of single launches, over calls that mix both graph
+    lengths and single steps."""
+    f0 = lbm_inputs.random_populations(*shape, seed=72)
+    out = []
+    for graph in (1, 0):
+        with L.Lattice(*shape, 0.9, -5.5, precision=precision, pattern=pattern, rho_ref=0.1) as lat:
+            lat.set_option("fused", fused)
+            lat.set_option("graph", graph)
+            lat.set_option("rho_l", 2.0)
+            lat.set_option("rho_v", 0.2)
+            lat.set_option("diag_interval", interval)
+            lat.set_populations(f0)
+            recs = []
+            for n in (40, 7, 23, 60):
+                lat.step(n)
+                recs += lat.diag_history()
+            lat.sync()
+            out.append((lat.populations(), recs))
+    np.testing.assert_array_equal(out[0][0], out[1][0])
+    assert out[0][1] == out[1][1]
+    assert [r["step"] for r in out[0][1]] == ([] if not interval else list(range(0, 130, interval)))
