@@ -409,9 +409,23 @@ void fill_diag(lbm_diag* out, const double* r, long long step) {
   out->largest_droplet = -1;
 }
 
-// One FP64 plane of N doubles for host transfers (moments, populations).
-int with_plane(lbm_ctx* h, double** plane) {
-  return dev_alloc((void**)plane, (size_t)h->g.N * sizeof(double), "transfer plane");
+// Room for `planes` FP64 planes on their way to or from the host (fewer where
+// they exceed 64 MiB); end_transfer gives back what is larger than that.
+int begin_transfer(lbm_ctx* h, int planes) {
+  const size_t need = transfer_doubles(h->g.N, planes);
+  if (h->transfer_n >= need) return LBM_OK;
+  dev_free(h->d_transfer, h->transfer_n * sizeof(double));
+  h->d_transfer = nullptr;
+  h->transfer_n = 0;
+  const int rc = dev_alloc((void**)&h->d_transfer, need * sizeof(double), "transfer planes");
+  if (rc == LBM_OK) h->transfer_n = need;
+  return rc;
+}
+void end_transfer(lbm_ctx* h) {
+  if (h->transfer_n <= ((size_t)8 << 20)) return;
+  dev_free(h->d_transfer, h->transfer_n * sizeof(double));
+  h->d_transfer = nullptr;
+  h->transfer_n = 0;
 }
 
 struct StateHeader {
@@ -496,6 +510,7 @@ void lbm_destroy(lbm_handle h) {
   dev_free(h->d_psi_tab, sizeof(double2) * kPsiTab);
   dev_free(h->d_small, sizeof(double) * 64);
   dev_free(h->d_scratch, h->scratch_doubles * sizeof(double));
+  dev_free(h->d_transfer, h->transfer_n * sizeof(double));
   dev_free(h->d_labels, (size_t)h->g.N * 2 * sizeof(int));
   dev_free(h->d_drop, h->drop_bytes);
   dev_free(h->d_ring, sizeof(double) * DIAG_STRIDE * lbm_ctx::kRing);
@@ -877,24 +892,29 @@ int lbm_diag_history(lbm_handle h, lbm_diag* out, int max_records, int* count) {
     CK(cudaStreamSynchronize(h->stream));
     return LBM_OK;
   }
-  unsigned long long dev_total = 0;
-  CK(cudaMemcpyAsync(&dev_total, h->d_ring_count, sizeof(dev_total), cudaMemcpyDeviceToHost, h->stream));
-  CK(cudaStreamSynchronize(h->stream));
-  if ((long long)dev_total != total) return fail(LBM_ERR_STATE, "diagnostics ring out of step with the host log");
   long long first = h->diag_fetched;
   if (total - first > lbm_ctx::kRing) first = total - lbm_ctx::kRing;  // older records were overwritten
   if (total - first > max_records) first = total - max_records;
-  std::vector<double> rec(DIAG_STRIDE);
+  // the records' slots are one or two runs of the ring; one wait for all
+  std::vector<double> rec((size_t)(total - first) * DIAG_STRIDE);
+  unsigned long long dev_total = 0;
+  CK(cudaMemcpyAsync(&dev_total, h->d_ring_count, sizeof(dev_total), cudaMemcpyDeviceToHost, h->stream));
+  for (long long r = first; r < total;) {
+    const long long slot = r % lbm_ctx::kRing, run = std::min(total - r, (long long)lbm_ctx::kRing - slot);
+    CK(cudaMemcpyAsync(&rec[(size_t)(r - first) * DIAG_STRIDE], h->d_ring + slot * DIAG_STRIDE,
+                       sizeof(double) * DIAG_STRIDE * run, cudaMemcpyDeviceToHost, h->stream));
+    r += run;
+  }
+  CK(cudaStreamSynchronize(h->stream));
+  if ((long long)dev_total != total) return fail(LBM_ERR_STATE, "diagnostics ring out of step with the host log");
   int n = 0;
   for (long long r = first; r < total; ++r) {
-    const long long slot = r % lbm_ctx::kRing;
-    CK(cudaMemcpy(rec.data(), h->d_ring + slot * DIAG_STRIDE, sizeof(double) * DIAG_STRIDE,
-                  cudaMemcpyDeviceToHost));
-    fill_diag(&out[n], rec.data(), h->diag_steps[(size_t)r]);
-    if (rec[DIAG_CCL + 3] != 0.0) return fail(LBM_ERR_TIMEOUT, "connected-component labelling guard tripped");
-    out[n].droplets = (int)rec[DIAG_CCL];
-    out[n].droplets_min8 = (int)rec[DIAG_CCL + 1];
-    out[n].largest_droplet = (long long)rec[DIAG_CCL + 2];
+    const double* v = &rec[(size_t)(r - first) * DIAG_STRIDE];
+    fill_diag(&out[n], v, h->diag_steps[(size_t)r]);
+    if (v[DIAG_CCL + 3] != 0.0) return fail(LBM_ERR_TIMEOUT, "connected-component labelling guard tripped");
+    out[n].droplets = (int)v[DIAG_CCL];
+    out[n].droplets_min8 = (int)v[DIAG_CCL + 1];
+    out[n].largest_droplet = (long long)v[DIAG_CCL + 2];
     ++n;
   }
   h->diag_fetched = total;
@@ -922,23 +942,31 @@ int lbm_moments(lbm_handle h, double* rho, double* ux, double* uy, double* uz) {
   const int layout = cur_layout(h);
   const void* f = cur_array(h);
   CK(launch_psi(h->cfg.precision, layout, h->vec, h->g, h->ph, f, h->psi, h->d_flag, h->stream));
-  double* plane = nullptr;
-  int rc = with_plane(h, &plane);
-  if (rc) return rc;
   double* outs[4] = {rho, ux, uy, uz};
-  for (int k = 0; k < 4 && rc == LBM_OK; ++k) {
+  int want = 0;
+  for (double* o : outs) want += o != nullptr;
+  int rc = begin_transfer(h, want > 0 ? want : 1);
+  if (rc) return rc;
+  // the requested fields together where the planes hold them, else one by one
+  const long long N = h->g.N;
+  const bool together = h->transfer_n >= (size_t)want * N;
+  cudaError_t e = cudaSuccess;
+  double* dev[4] = {nullptr, nullptr, nullptr, nullptr};
+  for (int k = 0, n = 0; k < 4; ++k)
+    if (outs[k]) dev[k] = h->d_transfer + (together ? (n++) * N : 0);
+  if (together)
+    e = launch_moments(h->cfg.precision, layout, h->g, h->ph, f, h->psi, dev[0], dev[1], dev[2], dev[3], h->stream);
+  for (int k = 0; k < 4 && e == cudaSuccess; ++k) {
     if (!outs[k]) continue;
-    cudaError_t e = launch_moments(h->cfg.precision, layout, h->g, h->ph, f, h->psi, k == 0 ? plane : nullptr,
-                                   k == 1 ? plane : nullptr, k == 2 ? plane : nullptr,
-                                   k == 3 ? plane : nullptr, h->stream);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(outs[k], plane, sizeof(double) * h->g.N, cudaMemcpyDeviceToHost, h->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    if (e != cudaSuccess) rc = cuda_fail(e, "moments");
+    if (!together)
+      e = launch_moments(h->cfg.precision, layout, h->g, h->ph, f, h->psi, k == 0 ? dev[0] : nullptr,
+                         k == 1 ? dev[1] : nullptr, k == 2 ? dev[2] : nullptr, k == 3 ? dev[3] : nullptr, h->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(outs[k], dev[k], sizeof(double) * N, cudaMemcpyDeviceToHost, h->stream);
   }
-  cudaStreamSynchronize(h->stream);
-  dev_free(plane, sizeof(double) * h->g.N);
-  return rc;
+  const cudaError_t e2 = cudaStreamSynchronize(h->stream);
+  end_transfer(h);
+  if (e == cudaSuccess) e = e2;
+  return e == cudaSuccess ? LBM_OK : cuda_fail(e, "moments");
 }
 
 int lbm_diagnostics(lbm_handle h, lbm_diag* out, int want_ccl) {
@@ -1047,41 +1075,24 @@ int lbm_droplets(lbm_handle h, lbm_droplet* out, int max_droplets, int* count) {
 
 int lbm_get_populations(lbm_handle h, double* host) {
   if (!h || !host) return fail(LBM_ERR_ARG, "null argument");
-  double* plane = nullptr;
-  int rc = with_plane(h, &plane);
+  int rc = begin_transfer(h, Q);
   if (rc) return rc;
-  const int layout = cur_layout(h);
-  for (int a = 0; a < Q && rc == LBM_OK; ++a) {
-    cudaError_t e = launch_get_plane(h->cfg.precision, layout, h->g, h->ph, cur_array(h), a, plane, h->stream);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(host + (size_t)a * h->g.N, plane, sizeof(double) * h->g.N, cudaMemcpyDeviceToHost,
-                          h->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    if (e != cudaSuccess) rc = cuda_fail(e, "get_populations");
-  }
-  cudaStreamSynchronize(h->stream);
-  dev_free(plane, sizeof(double) * h->g.N);
-  return rc;
+  const cudaError_t e = export_populations(h->cfg.precision, cur_layout(h), h->g, h->ph, cur_array(h), h->d_transfer,
+                                           h->transfer_n, host, h->stream);
+  end_transfer(h);
+  return e == cudaSuccess ? LBM_OK : cuda_fail(e, "get_populations");
 }
 
 int lbm_set_populations(lbm_handle h, const double* host) {
   if (!h || !host) return fail(LBM_ERR_ARG, "null argument");
-  double* plane = nullptr;
-  int rc = with_plane(h, &plane);
+  int rc = begin_transfer(h, Q);
   if (rc) return rc;
-  const int layout = cur_layout(h);
-  for (int a = 0; a < Q && rc == LBM_OK; ++a) {
-    cudaError_t e = cudaMemcpyAsync(plane, host + (size_t)a * h->g.N, sizeof(double) * h->g.N,
-                                    cudaMemcpyHostToDevice, h->stream);
-    if (e == cudaSuccess)
-      e = launch_set_plane(h->cfg.precision, layout, h->g, h->ph, cur_array(h), a, plane, h->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    if (e != cudaSuccess) rc = cuda_fail(e, "set_populations");
-  }
-  cudaStreamSynchronize(h->stream);
-  dev_free(plane, sizeof(double) * h->g.N);
-  if (rc == LBM_OK) h->initialized = true;
-  return rc;
+  const cudaError_t e = import_populations(h->cfg.precision, cur_layout(h), h->g, h->ph, cur_array(h), h->d_transfer,
+                                           h->transfer_n, host, h->stream);
+  end_transfer(h);
+  if (e != cudaSuccess) return cuda_fail(e, "set_populations");
+  h->initialized = true;
+  return LBM_OK;
 }
 
 int lbm_state_bytes(lbm_handle h, size_t* bytes) {

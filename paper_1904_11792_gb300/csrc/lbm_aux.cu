@@ -1,6 +1,8 @@
 // Kernels around the time step: ligament initial condition, canonical
 // population export/import, macroscopic fields, FP64 diagnostics and the
 // connected-component labelling of the liquid (droplet count).
+#include <algorithm>
+
 #include "lbm_internal.h"
 #include "lbm_launch.cuh"
 
@@ -75,32 +77,36 @@ __global__ void init_kernel(Geom g, Phys ph, InitSpec sp, typename Prec<P>::T* f
 }
 
 // ---------------------------------------------------------------------------
-// Canonical FP64 plane a <-> storage.
+// Canonical FP64 planes a0 + blockIdx.y <-> storage.
 // ---------------------------------------------------------------------------
 template <int P>
-__global__ void get_plane_kernel(Geom g, Phys ph, int layout, const typename Prec<P>::T* f, int a,
-                                 double* out) {
+__global__ void get_planes_kernel(Geom g, Phys ph, int layout, const typename Prec<P>::T* f, int a0,
+                                  double* out) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= g.N) return;
+  const int a = a0 + blockIdx.y;
   int x, y, z;
   coords(g, i, x, y, z);
   Nbr nb;
   nb.make(g, x, y, z);
   using C = typename Prec<P>::C;
-  out[i] = (double)Prec<P>::template load<true>(f + slot_index(g, layout, a, nb), (C)shift_d<P>(a, ph.rho_ref));
+  out[(long long)blockIdx.y * g.N + i] =
+      (double)Prec<P>::template load<true>(f + slot_index(g, layout, a, nb), (C)shift_d<P>(a, ph.rho_ref));
 }
 
 template <int P>
-__global__ void set_plane_kernel(Geom g, Phys ph, int layout, typename Prec<P>::T* f, int a,
-                                 const double* in) {
+__global__ void set_planes_kernel(Geom g, Phys ph, int layout, typename Prec<P>::T* f, int a0,
+                                  const double* in) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= g.N) return;
+  const int a = a0 + blockIdx.y;
   int x, y, z;
   coords(g, i, x, y, z);
   Nbr nb;
   nb.make(g, x, y, z);
   using C = typename Prec<P>::C;
-  Prec<P>::store(f + slot_index(g, layout, a, nb), (C)in[i], (C)shift_d<P>(a, ph.rho_ref));
+  Prec<P>::store(f + slot_index(g, layout, a, nb), (C)in[(long long)blockIdx.y * g.N + i],
+                 (C)shift_d<P>(a, ph.rho_ref));
 }
 
 // ---------------------------------------------------------------------------
@@ -636,17 +642,16 @@ cudaError_t init_t(const Geom& g, const Phys& ph, const InitSpec& sp, void* f, c
   return cudaGetLastError();
 }
 template <int P>
-cudaError_t get_t(int layout, const Geom& g, const Phys& ph, const void* f, int a, double* out,
+cudaError_t get_t(int layout, const Geom& g, const Phys& ph, const void* f, int a0, int n, double* out,
                   cudaStream_t s) {
-  get_plane_kernel<P><<<blocks_for(g.N, 256), 256, 0, s>>>(g, ph, layout,
-                                                           (const typename Prec<P>::T*)f, a, out);
+  get_planes_kernel<P><<<dim3(blocks_for(g.N, 256), n), 256, 0, s>>>(g, ph, layout, (const typename Prec<P>::T*)f, a0,
+                                                                     out);
   return cudaGetLastError();
 }
 template <int P>
-cudaError_t set_t(int layout, const Geom& g, const Phys& ph, void* f, int a, const double* in,
+cudaError_t set_t(int layout, const Geom& g, const Phys& ph, void* f, int a0, int n, const double* in,
                   cudaStream_t s) {
-  set_plane_kernel<P><<<blocks_for(g.N, 256), 256, 0, s>>>(g, ph, layout,
-                                                           (typename Prec<P>::T*)f, a, in);
+  set_planes_kernel<P><<<dim3(blocks_for(g.N, 256), n), 256, 0, s>>>(g, ph, layout, (typename Prec<P>::T*)f, a0, in);
   return cudaGetLastError();
 }
 template <int P>
@@ -811,26 +816,53 @@ cudaError_t launch_init(int precision, const Geom& g, const Phys& ph, const Init
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_get_plane(int precision, int layout, const Geom& g, const Phys& ph, const void* f,
-                             int a, double* out, cudaStream_t s) {
+cudaError_t launch_get_planes(int precision, int layout, const Geom& g, const Phys& ph, const void* f,
+                              int a0, int n, double* out, cudaStream_t s) {
   switch (precision) {
-    case LBM_F64: return get_t<LBM_F64>(layout, g, ph, f, a, out, s);
-    case LBM_F32: return get_t<LBM_F32>(layout, g, ph, f, a, out, s);
-    case LBM_F16DEV: return get_t<LBM_F16DEV>(layout, g, ph, f, a, out, s);
-    case LBM_BF16DEV: return get_t<LBM_BF16DEV>(layout, g, ph, f, a, out, s);
+    case LBM_F64: return get_t<LBM_F64>(layout, g, ph, f, a0, n, out, s);
+    case LBM_F32: return get_t<LBM_F32>(layout, g, ph, f, a0, n, out, s);
+    case LBM_F16DEV: return get_t<LBM_F16DEV>(layout, g, ph, f, a0, n, out, s);
+    case LBM_BF16DEV: return get_t<LBM_BF16DEV>(layout, g, ph, f, a0, n, out, s);
   }
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_set_plane(int precision, int layout, const Geom& g, const Phys& ph, void* f, int a,
-                             const double* in, cudaStream_t s) {
+cudaError_t launch_set_planes(int precision, int layout, const Geom& g, const Phys& ph, void* f, int a0,
+                              int n, const double* in, cudaStream_t s) {
   switch (precision) {
-    case LBM_F64: return set_t<LBM_F64>(layout, g, ph, f, a, in, s);
-    case LBM_F32: return set_t<LBM_F32>(layout, g, ph, f, a, in, s);
-    case LBM_F16DEV: return set_t<LBM_F16DEV>(layout, g, ph, f, a, in, s);
-    case LBM_BF16DEV: return set_t<LBM_BF16DEV>(layout, g, ph, f, a, in, s);
+    case LBM_F64: return set_t<LBM_F64>(layout, g, ph, f, a0, n, in, s);
+    case LBM_F32: return set_t<LBM_F32>(layout, g, ph, f, a0, n, in, s);
+    case LBM_F16DEV: return set_t<LBM_F16DEV>(layout, g, ph, f, a0, n, in, s);
+    case LBM_BF16DEV: return set_t<LBM_BF16DEV>(layout, g, ph, f, a0, n, in, s);
   }
   return cudaErrorInvalidValue;
+}
+
+cudaError_t export_populations(int precision, int layout, const Geom& g, const Phys& ph, const void* f, double* work,
+                               size_t work_doubles, double* host, cudaStream_t s) {
+  const int per = (int)std::min<size_t>(Q, work_doubles / g.N);
+  cudaError_t e = per < 1 ? cudaErrorInvalidValue : cudaSuccess;
+  for (int a = 0; a < Q && e == cudaSuccess; a += per) {
+    const int n = std::min(per, Q - a);
+    e = launch_get_planes(precision, layout, g, ph, f, a, n, work, s);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(host + (size_t)a * g.N, work, sizeof(double) * n * g.N, cudaMemcpyDeviceToHost, s);
+  }
+  const cudaError_t e2 = cudaStreamSynchronize(s);
+  return e != cudaSuccess ? e : e2;
+}
+
+cudaError_t import_populations(int precision, int layout, const Geom& g, const Phys& ph, void* f, double* work,
+                               size_t work_doubles, const double* host, cudaStream_t s) {
+  const int per = (int)std::min<size_t>(Q, work_doubles / g.N);
+  cudaError_t e = per < 1 ? cudaErrorInvalidValue : cudaSuccess;
+  for (int a = 0; a < Q && e == cudaSuccess; a += per) {
+    const int n = std::min(per, Q - a);
+    e = cudaMemcpyAsync(work, host + (size_t)a * g.N, sizeof(double) * n * g.N, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = launch_set_planes(precision, layout, g, ph, f, a, n, work, s);
+  }
+  const cudaError_t e2 = cudaStreamSynchronize(s);
+  return e != cudaSuccess ? e : e2;
 }
 
 cudaError_t launch_moments(int precision, int layout, const Geom& g, const Phys& ph, const void* f,

@@ -908,14 +908,10 @@ int lbm_batch_sync(lbm_batch b) {
 int lbm_batch_get_populations(lbm_batch b, int k, double* host) {
   if (!b || !host || k < 0 || k >= b->count) return bfail(LBM_ERR_ARG, "bad batch, instance or buffer");
   if (int rc = ensure_contig_instance(b, k)) return rc;
-  if (!b->d_plane) BCK(cudaMalloc(&b->d_plane, sizeof(double) * b->max_nodes));
+  const size_t room = transfer_doubles(b->max_nodes, Q);
+  if (!b->d_plane) BCK(cudaMalloc(&b->d_plane, sizeof(double) * room));
   View v = view_of(b, k);
-  for (int a = 0; a < Q; ++a) {
-    BCK(launch_get_plane(b->precision, LAYOUT_LOCAL, v.g, v.ph, v.f, a, b->d_plane, b->stream));
-    BCK(cudaMemcpyAsync(host + (size_t)a * v.g.N, b->d_plane, sizeof(double) * v.g.N, cudaMemcpyDeviceToHost,
-                        b->stream));
-  }
-  BCK(cudaStreamSynchronize(b->stream));
+  BCK(export_populations(b->precision, LAYOUT_LOCAL, v.g, v.ph, v.f, b->d_plane, room, host, b->stream));
   return LBM_OK;
 }
 

@@ -114,11 +114,22 @@ struct InitSpec {
 };
 cudaError_t launch_init(int precision, const Geom& g, const Phys& ph, const InitSpec& spec,
                         void* f, cudaStream_t s);
-// canonical FP64 plane a <-> storage (layout-aware)
-cudaError_t launch_get_plane(int precision, int layout, const Geom& g, const Phys& ph,
-                             const void* f, int a, double* out, cudaStream_t s);
-cudaError_t launch_set_plane(int precision, int layout, const Geom& g, const Phys& ph, void* f,
-                             int a, const double* in, cudaStream_t s);
+// Canonical FP64 populations to and from a host array of 19 N doubles, through
+// `work` (device), which takes as many whole planes at a time as it holds (at
+// least one).  Both wait for the stream.  Copies of a few MB into host pages
+// that nothing has touched yet cost more than 1 ms each whatever their size,
+// so the planes of small lattices cross together (48x48x96, 19 planes of 1.8
+// MB one by one: 22 ms; together: 2 ms).
+cudaError_t export_populations(int precision, int layout, const Geom& g, const Phys& ph, const void* f, double* work,
+                               size_t work_doubles, double* host, cudaStream_t s);
+cudaError_t import_populations(int precision, int layout, const Geom& g, const Phys& ph, void* f, double* work,
+                               size_t work_doubles, const double* host, cudaStream_t s);
+// Doubles of `work` for a lattice of N nodes and `planes` planes: all of them
+// up to 64 MiB, at least one.
+inline size_t transfer_doubles(long long N, int planes) {
+  const size_t cap = (size_t)8 << 20, all = (size_t)planes * N;
+  return all <= cap ? all : ((size_t)N > cap ? (size_t)N : cap);
+}
 // rho and u = (j + F/2)/rho into four FP64 device arrays (psi must be current)
 cudaError_t launch_moments(int precision, int layout, const Geom& g, const Phys& ph,
                            const void* f, const void* psi, double* rho, double* ux, double* uy,
@@ -249,6 +260,8 @@ struct lbm_ctx {
   double2* d_psi_tab = nullptr;   // FP64: table of psi_of<double>
   double* d_small = nullptr;      // small result buffer (diagnostics out etc.)
   double* d_scratch = nullptr;    // diagnostics partials
+  double* d_transfer = nullptr;   // FP64 planes on their way to or from the host (kept up to 64 MiB)
+  size_t transfer_n = 0;
   size_t scratch_doubles = 0;
   int* d_labels = nullptr;        // CCL labels and sizes (2 N ints)
   bool diag_ccl = false;          // label droplets at every in-loop diagnostic step

@@ -102,3 +102,35 @@ def test_long_graphs_and_side_reductions_equal_eager_steps(L, shape, precision, 
     np.testing.assert_array_equal(out[0][0], out[1][0])
     assert out[0][1] == out[1][1]
     assert [r["step"] for r in out[0][1]] == ([] if not interval else list(range(0, 130, interval)))
+
+
+@pytest.mark.parametrize("shape", [(37, 11, 9), (96, 96, 64), (160, 128, 110)])   # 19, 14 and 3 planes cross at a time
+def test_host_transfers_in_groups_of_planes(L, shape):
+    nx, ny, nz = shape
+    rng = np.random.default_rng(73)
+    f0 = rng.uniform(0.01, 0.1, (19, nz, ny, nx))
+    with L.Lattice(*shape, 0.9, -5.5, precision="f64") as lat:
+        lat.set_populations(f0)
+        np.testing.assert_array_equal(lat.populations(), f0)
+        every = lat.moments()      # all four fields together, except on the largest shape
+        for k, v in every.items():
+            np.testing.assert_array_equal(lat.moments((k,))[k], v)
+    np.testing.assert_allclose(every["rho"], f0.sum(axis=0), rtol=1e-14)
+
+
+def test_diag_history_across_the_ring_end(L):
+    """More records than the ring's 1024 slots, read in two calls: the second
+    one's slots wrap around the ring's end."""
+    f0 = lbm_inputs.random_populations(8, 5, 4, seed=74)
+    with L.Lattice(8, 5, 4, 0.9, -5.5, precision="f64") as lat:
+        lat.set_option("diag_interval", 1)
+        lat.set_populations(f0)
+        lat.step(1000)
+        a = lat.diag_history()
+        lat.step(100)
+        b = lat.diag_history()
+        lat.step(30)
+        c = lat.diag_history(7)
+        d = lat.diagnostics()
+    assert [r["step"] for r in a + b] == list(range(1100)) and [r["step"] for r in c] == list(range(1123, 1130))
+    assert all(abs(r["mass"] / d["mass"] - 1) < 1e-11 for r in a + b + c)
