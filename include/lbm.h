@@ -159,14 +159,20 @@ int lbm_set_stream(lbm_handle h, void *stream);
  * the A-B step's value),
  * "vector" (0/1, default 1: when nx is even each thread updates two
  * neighbouring nodes with 2-element vector loads and stores; block_x then
- * counts node pairs), "fused" (0/1, default 1: A-B steps run as one
+ * counts node pairs), "fused" (0, 1 or 2, default 1: A-B steps run as one
  * single-pass kernel that computes psi per tile in shared memory, reading
  * the populations once per step, with a variant that also reduces the
  * in-loop diagnostics on diagnostic steps; applies to FP32,
  * FP16-dev and BF16-dev storage when nx % 64 == 0 and ny % 4 == 0 (FP32) or
- * ny % 8 == 0 (2-byte storage), other
- * lattices take the two-kernel step; results equal the two-kernel step
- * bitwise; lbm_get_option answers whether it applies), "fused_fz" (z planes
+ * ny % 8 == 0 (2-byte storage); lbm_get_option answers whether it applies.
+ * Of the other lattices of these storage forms, larger ones (more than 1 M
+ * nodes in FP32, 2.6 M in 2-byte storage, nx >= 32; with the value 2 all of
+ * them) run plain SRT steps as a single pass on tiles cut at their edges: every
+ * step where rows are a multiple of 16 bytes; otherwise the steps inside a
+ * replayed graph but its first one, on two private arrays with padded rows
+ * (allocated on the first such call if they take at most a quarter of the
+ * free device memory, else not at all).  Everything else is the two-kernel
+ * step; results equal it bitwise), "fused_fz" (z planes
  * each block of the fused step marches through; 0 = chosen from the lattice
  * size and the GPU, the default), "fused_group" (the fused step launches
  * its blocks in groups of this many consecutive z runs, the run varying

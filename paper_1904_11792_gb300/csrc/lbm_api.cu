@@ -177,6 +177,8 @@ int auto_minb(bool vec, int mode, int precision) {
   return 2;
 }
 
+bool ragged_direct(const lbm_ctx* h);
+
 // Enqueues one time step on stream s.  `phase` is the step parity (AA) or
 // the index of the current array (A-B).  With timing on, each kernel is
 // bracketed by events on s.  side (captures): where the diagnostics'
@@ -237,6 +239,19 @@ int enqueue_step(lbm_ctx* h, cudaStream_t s, long long step, int cur, bool timed
     }
     return LBM_OK;
   }
+  if (!diag_step && ragged_direct(h)) {
+    if (timed) {
+      e0 = take_event(h);
+      e1 = take_event(h);
+      CK(cudaEventRecord(e0, s));
+    }
+    CK(launch_ragged(prec, g, ph, src, g.nx, dst, g.nx, h->d_flag, h->fused_fz, h->fused_group, s));
+    if (timed) {
+      CK(cudaEventRecord(e1, s));
+      h->pending.push_back({2, e0, e1});
+    }
+    return LBM_OK;
+  }
   if (timed) {
     e0 = take_event(h);
     e1 = take_event(h);
@@ -269,6 +284,80 @@ int enqueue_step(lbm_ctx* h, cudaStream_t s, long long step, int cur, bool timed
     h->pending.push_back({0, e0, e1});
     h->pending.push_back({1, e1, e2});
   }
+  return LBM_OK;
+}
+
+// Whether plain steps run as the ragged single pass between the lattice's own
+// arrays (its rows are 16-byte multiples), and whether the steps inside a
+// captured chunk run on padded copies (they are not, and there is room).
+bool ragged_form(const lbm_ctx* h) {
+  const long long least = Prec_dev(h->cfg.precision) ? kRaggedNodesDev : kRaggedNodes;
+  return h->fused && (h->fused == 2 || (h->g.N > least && h->g.nx >= kRaggedMinNx)) &&
+         h->cfg.pattern == LBM_AB && h->ph.coll == COLL_SRT && ragged_applicable(h->g, h->cfg.precision);
+}
+bool ragged_direct(const lbm_ctx* h) {
+  return ragged_form(h) && ragged_row(h->g, h->cfg.precision) == h->g.nx && ((uintptr_t)h->state & 15) == 0;
+}
+bool padded_form(const lbm_ctx* h) { return ragged_form(h) && !ragged_direct(h) && h->pad[1]; }
+
+// Allocates the padded arrays where they take at most a quarter of the free
+// memory; without them the steps stay on the two kernels.
+void ensure_padded(lbm_ctx* h) {
+  if (h->pad[1] || h->pad_failed || !ragged_form(h) || ragged_direct(h)) return;
+  const size_t bytes =
+      (size_t)Q * ragged_row(h->g, h->cfg.precision) * h->g.ny * h->g.nz * elem_size(h->cfg.precision);
+  size_t free_b = 0, total_b = 0;
+  const std::string msg = g_last_error;
+  h->pad_failed = cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || 8 * bytes > free_b ||
+                  dev_alloc(&h->pad[0], bytes, "padded rows") != LBM_OK;
+  if (!h->pad_failed) {
+    h->pad_bytes = bytes;
+    h->pad_failed = dev_alloc(&h->pad[1], bytes, "padded rows") != LBM_OK;
+  }
+  if (!h->pad_failed) return;
+  (void)cudaGetLastError();
+  g_last_error = msg;
+  dev_free(h->pad[0], h->pad_bytes);
+  h->pad[0] = h->pad[1] = nullptr;
+  h->pad_bytes = 0;
+}
+
+// Step k of a captured chunk of `steps` that starts on array `phase`, on
+// padded rows: the first step (the chunk's diagnostic step, if any) is the
+// two-kernel one and writes its collision's result to the first padded array,
+// the others are single passes between the two, the last one back into the
+// lattice's own array.  20 FP32 steps on 251x112x112 with
+// a diagnostic step in ten: 2843 -> 2208 us.
+int enqueue_padded_step(lbm_ctx* h, cudaStream_t s, int k, int steps, int phase, ReduceSide* side) {
+  const int prec = h->cfg.precision, px = ragged_row(h->g, prec);
+  const Geom& g = h->g;
+  Phys ph = h->ph;
+  if (Prec_dev(prec) && ph.sr) {
+    const int w = salt_word(h, k, phase ^ (k & 1));
+    ph.salt = (const unsigned*)(h->d_flag + 2 + w);
+    ph.salt_next = (unsigned*)(h->d_flag + 2 + (w ^ 1));
+  }
+  if (k == 0) {
+    const void* src = array_ptr(h, phase);
+    if (h->diag_interval > 0) {
+      if (h->diag_ccl) side = nullptr;
+      CK(launch_diagnostics(prec, LAYOUT_LOCAL, g, h->ph, src, h->rho_l, h->rho_v, h->d_scratch, h->d_ring, h->psi,
+                            h->d_flag, h->d_ring_count, lbm_ctx::kRing, s, nullptr, side));
+      if (h->diag_ccl) {
+        long long* d4 = (long long*)(h->d_small + 32);
+        CK(launch_ccl(prec, LAYOUT_LOCAL, g, h->ph, src, 0.5 * (h->rho_l + h->rho_v), h->d_labels,
+                      h->d_labels + g.N, d4, s));
+        CK(launch_ccl_ring(d4, h->d_ring, h->d_ring_count, lbm_ctx::kRing, s));
+      }
+    } else {
+      CK(launch_psi(prec, LAYOUT_LOCAL, h->vec, g, h->ph, src, h->psi, h->d_flag, s));
+    }
+    CK(launch_collide_padded(prec, g, ph, src, h->pad[0], px, h->psi, auto_block(g, false), s));
+    return LBM_OK;
+  }
+  const bool last = k == steps - 1;
+  CK(launch_ragged(prec, g, ph, h->pad[(k - 1) & 1], px, last ? array_ptr(h, phase ^ (steps & 1)) : h->pad[k & 1],
+                   last ? g.nx : px, h->d_flag, h->fused_fz, h->fused_group, s));
   return LBM_OK;
 }
 
@@ -306,14 +395,16 @@ int chunk_len(const lbm_ctx* h) {
   return k;
 }
 
-// Steps of the longer graph that small lattices replay while enough steps are
-// left: the multiple of chunk_len() from 16 on.  A graph launch costs about
+// Steps of the longer graph that small lattices, and plain steps on padded
+// rows (whose first step is the slow one), replay while enough steps are left:
+// the multiple of chunk_len() from 16 on.  A graph launch costs about
 // 2.7 us between two replays (64x32x32 FP32 and 4x49x49 FP64, 2-step against
 // 50- and 100-step graphs), as much as a kernel of such a step; larger
 // lattices do not feel it and keep the shorter capture.
 int long_chunk_len(const lbm_ctx* h) {
   const int c = chunk_len(h);
-  return h->g.chain ? (16 + c - 1) / c * c : c;
+  const bool longer = padded_form(h) ? h->diag_interval == 0 : h->g.chain != 0;
+  return longer ? (16 + c - 1) / c * c : c;
 }
 
 // Captures `steps` consecutive steps (a multiple of chunk_len()) starting at
@@ -335,8 +426,10 @@ int capture_chunk(lbm_ctx* h, int phase, int steps, cudaGraphExec_t* exec) {
   if (e == cudaSuccess) {
     // step numbers relative to a chunk start (a multiple of chunk_len()): the same
     // parity and the same diagnostic steps as every replay
+    const bool padded = padded_form(h) && steps > 1;
     for (int k = 0; k < steps && rc == LBM_OK; ++k)
-      rc = enqueue_step(h, cs, k, phase ^ (k & 1), false, side.join ? &side : nullptr);
+      rc = padded ? enqueue_padded_step(h, cs, k, steps, phase, side.join ? &side : nullptr)
+                  : enqueue_step(h, cs, k, phase ^ (k & 1), false, side.join ? &side : nullptr);
     if (side.open) e = cudaStreamWaitEvent(cs, side.join, 0);
     const cudaError_t e2 = cudaStreamEndCapture(cs, &graph);
     if (e == cudaSuccess) e = e2;
@@ -510,6 +603,7 @@ void lbm_destroy(lbm_handle h) {
   dev_free(h->d_psi_tab, sizeof(double2) * kPsiTab);
   dev_free(h->d_small, sizeof(double) * 64);
   dev_free(h->d_scratch, h->scratch_doubles * sizeof(double));
+  for (void* p : h->pad) dev_free(p, h->pad_bytes);
   dev_free(h->d_transfer, h->transfer_n * sizeof(double));
   dev_free(h->d_labels, (size_t)h->g.N * 2 * sizeof(int));
   dev_free(h->d_drop, h->drop_bytes);
@@ -668,7 +762,7 @@ int lbm_set_option(lbm_handle h, const char* key, double v) {
     if (k == "mrt_s_m") h->ph.s_m = v;
     drop_graphs(h);
   } else if (k == "fused") {
-    h->fused = v != 0.0;
+    h->fused = v == 0.0 ? 0 : (v == 2.0 ? 2 : 1);
     drop_graphs(h);
     if (h->diag_interval > 0) {
       int rc = ensure_scratch(h);
@@ -851,6 +945,7 @@ int lbm_step(lbm_handle h, int n) {
   if (n < 0) return fail(LBM_ERR_ARG, "negative step count");
   if (!h->initialized) return fail(LBM_ERR_STATE, "lattice not initialised");
   const bool aa = h->cfg.pattern == LBM_AA;
+  if (h->use_graph && !h->kernel_timing && n > 1) ensure_padded(h);
   const int base = chunk_len(h), longer = long_chunk_len(h);
   const int k = h->diag_interval;
   if (h->graph_chunk != base) {

@@ -440,11 +440,15 @@ struct Nbr {
   int rows[3][3];
   __device__ __forceinline__ void make(const Geom& g, int x, int y, int z) {
     const int xm = x == 0 ? g.nx - 1 : x - 1, xp = x == g.nx - 1 ? 0 : x + 1;
-    const int ym = y == 0 ? g.ny - 1 : y - 1, yp = y == g.ny - 1 ? 0 : y + 1;
-    const int zm = z == 0 ? g.nz - 1 : z - 1, zp = z == g.nz - 1 ? 0 : z + 1;
     xs[0] = xm;
     xs[1] = x;
     xs[2] = xp;
+    make_rows(g, y, z);
+  }
+  // the row offsets alone (rows g.nx apart)
+  __device__ __forceinline__ void make_rows(const Geom& g, int y, int z) {
+    const int ym = y == 0 ? g.ny - 1 : y - 1, yp = y == g.ny - 1 ? 0 : y + 1;
+    const int zm = z == 0 ? g.nz - 1 : z - 1, zp = z == g.nz - 1 ? 0 : z + 1;
     const int yv[3] = {ym, y, yp}, zv[3] = {zm, z, zp};
 #pragma unroll
     for (int i = 0; i < 3; ++i)

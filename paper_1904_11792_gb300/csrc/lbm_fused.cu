@@ -87,41 +87,117 @@ cudaError_t maps_for(int precision, const Geom& g, const void* base, Maps* out) 
   return cudaSuccess;
 }
 
-// z planes per block.  Each block also loads the two planes around its run,
-// and a grid that leaves SMs idle in its last wave wastes their bandwidth:
-// the cost of a run length is waves x planes loaded per block, times
-// (1 + fz/256) for long runs.  On grids of many waves long runs cost more
-// than that (measured on GB300, 1024x512x512 in groups of runs: 12-, 16-,
-// 19-, 24- and 32-plane runs take 6.5, 6.4-7.8, 7.0, 7.7 and 8.2 ms per
-// step: the longer a block lives, the further apart in time neighbouring
-// tiles read the rows they share; with the current kernel, 8-plane runs in
-// groups of 4 take 6.44 ms and 12-plane runs 6.99 ms), so on lattices with
-// more tiles than resident blocks runs stop at 8 planes (cap); small grids (256x128x128:
-// 1.96 waves of 19-plane runs, 0.114 ms, against 0.126 ms for 16-plane runs
-// in 2.25 waves) keep the wave count low instead.  2-byte storage, bound by
-// instruction issue and with half the bytes per plane in L2, has no cap, and
-// on lattices with more tiles than resident blocks long runs cost it little
-// (1 + fz/2048: 1024x512x512 FP16, 1 run per group, 27-, 32-, 48-, 64-,
-// 86-, 128-, 256- and 512-plane runs take 4.598, 4.567, 4.524, 4.485, 4.506,
-// 4.491, 4.614 and 4.700 ms; BF16 is best at 64 too, 4.519 ms); on smaller
-// lattices 1 + fz/256 keeps the best shape (512x256x256: 20-plane runs
-// 0.5975 ms, 32 0.604, 64 0.604; 256x128x128: 15-plane runs 0.0894 ms, 32
-// 0.0933).
-int choose_fz(const Geom& g, long long tiles, long long slots, bool cap) {
-  int best = g.nz;
+// Tile width of the ragged step, as for batches: 64 for FP32, 32 for 2-byte
+// storage (fewer idle lanes at the x end).
+template <int P> constexpr int kRaggedW = Prec<P>::dev ? 32 : TX;
+
+// Predicted time of a launch with z runs of fz planes on `tiles` tiles.  Unit:
+// a plane collided by one block while every slot is taken.  Both forms were
+// fitted to the times of 38 run lengths on 14 lattices of 0.5 to 34 M nodes.
+//
+// FP32 (bound by HBM): whole waves take their blocks' mean cost, where the two
+// planes a run loads but does not collide count 0.6 each; the last wave what
+// its blocks cost at full bandwidth, but at least 0.75 of its planes' latency;
+// times 1 + fz / 80, because the longer a run, the further apart in time
+// neighbouring tiles read the rows they share.  The chosen length is 3.1 %
+// slower than the best one on average, at most 11 %; whole waves x (fz + 2) x
+// (1 + fz / 256), the rule before, 6.6 %, at most 20 % (256x110x112: 28 planes
+// 104.7 us, 10 planes 87.1 us).
+double run_cost_f32(long long tiles, long long slots, int nz, int fz) {
+  const long long blocks = tiles * ((nz + fz - 1) / fz), waves = blocks / slots, last = blocks - waves * slots;
+  const double mean = (double)tiles * nz / blocks + 1.2;
+  double cost = waves * mean;
+  if (last) cost += std::max(mean * last / slots, 0.75 * (fz + 2));
+  return cost * (1.0 + fz / 80.0);
+}
+
+// 2-byte storage (bound by instruction issue): a small simulation of how the
+// blocks run.  They start in launch order (the short last runs last) as slots
+// come free, and all resident blocks progress at the same rate, a plane taking
+// max(R, 0.9 slots) / slots while R blocks are resident; the two planes a run
+// does not collide count 0.8 each; times 1 + fz / 300.  The chosen length is
+// 0.8 % slower than the best one on average, at most 3 %; the rule before 2.6 %,
+// at most 6 % (256x128x128 FP16: 15 planes 88.3 us, 29 planes 84.1 us).
+double run_cost_dev(long long tiles, long long slots, int nz, int fz) {
+  constexpr double h = 0.8;
+  struct Group {
+    double left;
+    long long count;
+  };
+  const int full = nz / fz, rem = nz - full * fz;
+  Group queue[2] = {{fz + 2 * h, tiles * full}, {rem + 2 * h, rem ? tiles : 0}};
+  std::vector<Group> run;
+  double t = 0.0;
+  long long resident = 0;
+  for (int q = 0;;) {
+    while (q < 2 && resident < slots) {
+      const long long n = std::min(queue[q].count, slots - resident);
+      if (n) run.push_back({queue[q].left, n});
+      resident += n;
+      queue[q].count -= n;
+      if (!queue[q].count) ++q;
+    }
+    if (run.empty()) break;
+    double step = run[0].left;
+    for (const Group& g : run) step = std::min(step, g.left);
+    t += step * std::max((double)resident, 0.9 * slots);
+    size_t keep = 0;
+    for (Group& g : run) {
+      g.left -= step;
+      if (g.left < 1e-9)
+        resident -= g.count;
+      else
+        run[keep++] = g;
+    }
+    run.resize(keep);
+  }
+  return t / slots * (1.0 + fz / 300.0);
+}
+
+// z planes per block.  Lattices with more than twice as many tiles as slots
+// have many waves whatever the run: FP32 runs of 8 planes (1024x512x512, in
+// groups of 4: 6.44 ms, 12-plane runs 6.99 ms), 2-byte storage by whole waves x
+// (fz + 2) x (1 + fz / 2048) (1024x512x512 FP16, 27-, 32-, 48-, 64-, 86-, 128-,
+// 256- and 512-plane runs take 4.598, 4.567, 4.524, 4.485, 4.506, 4.491, 4.614
+// and 4.700 ms).  Others take the run length of the least predicted time, kept
+// per shape (a pure function of its arguments).
+template <int P>
+int choose_fz(const Geom& g, long long tiles, long long slots) {
+  constexpr bool dev = Prec<P>::dev;
+  const bool many = tiles > 2 * slots;
+  if (!dev && many) return std::min(g.nz, 8);
+  static std::mutex mu;
+  static std::map<std::tuple<long long, long long, int>, int> kept;
+  const auto key = std::make_tuple(tiles, slots, g.nz);
+  std::lock_guard<std::mutex> lock(mu);
+  const auto it = kept.find(key);
+  if (it != kept.end()) return it->second;
+  int best = std::min(g.nz, 4);
   double best_cost = -1.0;
-  const double k = (!cap && tiles > slots) ? 2048.0 : 256.0;   // the long-run factor 1 + fz / k
-  for (int fz = 4; fz <= g.nz; ++fz) {
-    const long long chunks = (g.nz + fz - 1) / fz;
-    const long long waves = (tiles * chunks + slots - 1) / slots;
-    if (cap && fz > 8 && tiles > slots) continue;
-    const double cost = (double)waves * (fz + 2) * (1.0 + fz / k);
+  for (int fz = best; fz <= (many ? g.nz : std::min(g.nz, 64)); ++fz) {
+    const long long waves = (tiles * ((g.nz + fz - 1) / fz) + slots - 1) / slots;
+    const double cost = many ? (double)waves * (fz + 2) * (1.0 + fz / 2048.0)
+                             : (dev ? run_cost_dev : run_cost_f32)(tiles, slots, g.nz, fz);
     if (best_cost < 0.0 || cost < best_cost) {
       best_cost = cost;
       best = fz;
     }
   }
+  if (kept.size() >= 1024) kept.clear();
+  kept[key] = best;
   return best;
+}
+
+// Runs per group of the block order (a tile's y neighbours are ntx x grp
+// blocks apart in the launch order; blocks of a group share the planes at
+// their runs' ends).  FP32: 4 on lattices at least 8 tiles wide (512x256x256:
+// 819 us against 833 us with 2; 1024x512x512: 6.42 ms, 8 take 6.53 ms), one
+// on narrower ones (256x128x128 within 1 % for 1 to 4, 304x150x150 1 %
+// slower with 2); 2-byte storage: one (1024x512x512 FP16 6.20 ms against 6.33
+// ms in pairs).
+template <int P>
+int choose_grp(int ntx) {
+  return !Prec<P>::dev && ntx >= 8 ? 4 : 1;
 }
 
 // Per device and storage type: the kernels' shared-memory limit is set and
@@ -145,6 +221,9 @@ cudaError_t fused_device_info(int* slots_per_sm, int* sms) {
       if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem);
     for (const void* k : {(const void*)bfused_kernel<P, TX>, (const void*)bpersist_kernel<P, TX>})
       if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem);
+    for (const void* k : {(const void*)ragged_kernel<P, kRaggedW<P>, false>, (const void*)ragged_kernel<P, kRaggedW<P>, true>})
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FusedShape<P, kRaggedW<P>>::smem);
     for (const void* k : {(const void*)bfused_kernel<P, 32>, (const void*)bpersist_kernel<P, 32>})
       if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FusedShape<P, 32>::smem);
@@ -170,19 +249,10 @@ cudaError_t fused_grid(const Geom& g, int fz_req, int grp_req, int* fz, int* nch
   cudaError_t e = fused_device_info<P>(&slots_per_sm, &sms);
   if (e != cudaSuccess) return e;
   const long long tiles = (long long)(g.nx / TX) * (g.ny / FusedShape<P>::TY);
-  *fz = fz_req > 0 ? std::min(fz_req, g.nz) : choose_fz(g, tiles, (long long)slots_per_sm * sms, !Prec<P>::dev);
+  *fz = fz_req > 0 ? std::min(fz_req, g.nz) : choose_fz<P>(g, tiles, (long long)slots_per_sm * sms);
   *nchunks = (g.nz + *fz - 1) / *fz;
   *blocks = tiles * *nchunks;
-  // runs per group (a tile's y neighbours are ntx x grp blocks apart in the
-  // launch order).  Measured on GB300 (FP32, A-B): 256x128x128 is fastest
-  // with one run per group (0.117 ms against 0.127 ms with all 7 runs of a
-  // tile together), 512x256x256 within 2 % for 1 to 4, 1024x512x512 with
-  // 12-plane runs in groups of 4 (6.5 ms and 21.8 GB of DRAM reads in every
-  // launch; 16-plane runs in pairs took 6.4 to 7.8 ms, reading 22 to 29 GB):
-  // one run per 4 tile columns (2-byte storage: one run per group, 32-plane
-  // runs in ones 6.20 ms on 1024x512x512 FP16, in pairs 6.33 ms)
-  const int ntx = g.nx / TX;
-  *grp = std::min(grp_req > 0 ? grp_req : (Prec<P>::dev ? 1 : std::max(1, ntx / 4)), *nchunks);
+  *grp = std::min(grp_req > 0 ? grp_req : choose_grp<P>(g.nx / TX), *nchunks);
   return *blocks > 0x7fffffffLL ? cudaErrorInvalidConfiguration : cudaSuccess;
 }
 
@@ -229,7 +299,61 @@ size_t fused_scratch_t(const Geom& g, int fz_req) {
   return (size_t)(g.ny / FusedShape<P>::TY) * nchunks * g.nx * 2 + (size_t)blocks * DIAG_NG + (size_t)g.nx * 2;
 }
 
+template <int P>
+cudaError_t ragged_t(const Geom& g, const Phys& ph, const void* src, int src_px, void* dst, int dst_px, int* flag,
+                     int fz_req, int grp_req, cudaStream_t s) {
+  constexpr int W = kRaggedW<P>;
+  using S = FusedShape<P, W>;
+  using T = typename Prec<P>::T;
+  int slots_per_sm = 0, sms = 0;
+  cudaError_t e = fused_device_info<P>(&slots_per_sm, &sms);
+  if (e != cudaSuccess) return e;
+  const int cw = 16 / (int)sizeof(T);
+  Maps m;
+  e = make_map(&m.interior, P, g, src, W, S::TY, src_px);
+  if (e == cudaSuccess) e = make_map(&m.row, P, g, src, W, 1, src_px);
+  if (e == cudaSuccess) e = make_map(&m.col, P, g, src, cw, S::TY, src_px);
+  if (e == cudaSuccess) e = make_map(&m.cor, P, g, src, cw, 1, src_px);
+  if (e != cudaSuccess) return e;
+  const int ntx = (g.nx + W - 1) / W;
+  const long long tiles = (long long)ntx * ((g.ny + S::TY - 1) / S::TY);
+  const int fz =
+      fz_req > 0 ? std::min(fz_req, g.nz) : choose_fz<P>(g, tiles, (long long)slots_per_sm * sms);
+  const int nchunks = (g.nz + fz - 1) / fz;
+  if (tiles * nchunks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+  const int grp = std::min(grp_req > 0 ? grp_req : choose_grp<P>(ntx), nchunks);
+  const long long dstride = (long long)dst_px * g.ny * g.nz;
+  DirBases<T> db;
+  for (int a = 0; a < Q; ++a) db.p[a] = (T*)dst + a * dstride;
+  // pairs of nodes are stored as one 2-element vector where every row starts
+  // at such a vector's boundary
+  const bool odd = dst_px % 2 != 0 || (uintptr_t)dst % (2 * sizeof(T)) != 0;
+  return chain_launch(g.chain, odd ? ragged_kernel<P, W, true> : ragged_kernel<P, W, false>, (unsigned)(tiles * nchunks),
+                      S::NT, S::smem, s, m, g, ph, flag, ntx, nchunks, fz, grp, dst_px, dstride, db);
+}
+
 }  // namespace
+
+int ragged_row(const Geom& g, int precision) {
+  const int al = 16 / (int)elem_size(precision);
+  return (g.nx + al - 1) / al * al;
+}
+
+bool ragged_applicable(const Geom& g, int precision) {
+  return precision != LBM_F64 && !fused_applicable(g, precision) &&
+         (long long)ragged_row(g, precision) * g.ny * g.nz <= 0x7fffffffLL;
+}
+
+cudaError_t launch_ragged(int precision, const Geom& g, const Phys& ph, const void* src, int src_px, void* dst,
+                          int dst_px, int* flag, int fz, int grp, cudaStream_t s) {
+  if (src_px % (16 / (int)elem_size(precision)) || ((uintptr_t)src & 15)) return cudaErrorInvalidValue;
+  switch (precision) {
+    case LBM_F32: return ragged_t<LBM_F32>(g, ph, src, src_px, dst, dst_px, flag, fz, grp, s);
+    case LBM_F16DEV: return ragged_t<LBM_F16DEV>(g, ph, src, src_px, dst, dst_px, flag, fz, grp, s);
+    case LBM_BF16DEV: return ragged_t<LBM_BF16DEV>(g, ph, src, src_px, dst, dst_px, flag, fz, grp, s);
+  }
+  return cudaErrorInvalidValue;
+}
 
 cudaError_t fused_launch_shape(int precision, const Geom& g, int fz_req, int grp_req, int* fz, int* grp) {
   int nchunks = 0;

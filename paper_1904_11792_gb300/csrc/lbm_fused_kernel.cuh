@@ -30,9 +30,10 @@
 // instructions (float2 lanes, each rounded like the scalar instruction), and
 // the stores are those of collide_pair, so the results equal the two-kernel
 // step bitwise.  A-B streaming, 4- and 2-byte storage, lattices with
-// nx % 64 == 0 and ny % 4 == 0 (8 for 2-byte storage); bfused_kernel runs
-// the same body over the instances of a batch, of any size, whose rows the
-// batch pads to 16-byte multiples, on 64-wide tiles or on 32-wide ones (two
+// nx % 64 == 0 and ny % 4 == 0 (8 for 2-byte storage); ragged_kernel runs the
+// same body on one lattice of any size whose source rows start on 16-byte
+// boundaries, bfused_kernel over the instances of a batch, of any size, whose
+// rows the batch pads to 16-byte multiples, on 64-wide tiles or on 32-wide ones (two
 // rows of 16 lanes x two nodes per warp, twice as many rows per tile).
 //
 // This header holds the kernel and its device helpers; lbm_fused.cu holds
@@ -219,7 +220,12 @@ constexpr int fused_minb() {
 // store nor write psi), its rows are padded to a 16-byte multiple, and the
 // halo column at x = nx - 1 comes from the 16-byte box that contains it.
 // W: the tile width (32 only for BATCH).
-template <int P, bool DIAG, int COLL, bool BATCH, int W = TX, bool SALT_GIVEN = false>
+// TABLE: the destination belongs to an instance of a table (the batched
+// step); else the direction bases are kernel parameters (db).  ODD: the
+// destination's rows may start at odd elements, so that node pairs are stored
+// one node at a time.
+template <int P, bool DIAG, int COLL, bool BATCH, int W = TX, bool SALT_GIVEN = false, bool TABLE = BATCH,
+          bool ODD = false>
 __device__ __forceinline__ void fused_body(const Maps& maps, const Geom& g, const Phys& ph,
                                            typename Prec<P>::T* dst, int* flag, int ntx, int nchunks, int fz,
                                            int grp, const DiagOut& dg, int u, int px, long long dstride,
@@ -320,7 +326,7 @@ __device__ __forceinline__ void fused_body(const Maps& maps, const Geom& g, cons
   // which saves the 64-bit arithmetic per direction and plane (measured: 1.4 %
   // faster; a latency-bound FP32 step was 3 % slower this way).
   __shared__ T* s_dir[Q];
-  if (BATCH && Prec<P>::dev && tid < Q) s_dir[tid] = dst + (long long)tid * N;
+  if (TABLE && Prec<P>::dev && tid < Q) s_dir[tid] = dst + (long long)tid * N;
   __shared__ int s_abort;
   // the deviation shifts, staged through shared memory so that they live in
   // registers: the widening adds of the 2-byte loads take no constant-bank
@@ -530,12 +536,13 @@ __device__ __forceinline__ void fused_body(const Maps& maps, const Geom& g, cons
         const C sh = a == 0 ? s0 : (a <= 6 ? s1 : s2);
         const int row = rowp * (yv[1 + cy(a)] + g.ny * zv[1 + cz(a)]);
         if constexpr (Prec<P>::dev) {
-          T* const base = BATCH ? s_dir[a] : db->p[a];
+          T* const base = TABLE ? s_dir[a] : db->p[a];
           // the shift comes off both nodes in one paired difference
           const float2 sh2 = splat<float2>(sh);
           if (cx(a) == 0) {
-            if (BATCH && !act1) {
+            if (ODD || (BATCH && !act1)) {
               store_pop<P>(ph, base + (row + x), fs0[a], sh, seed0, a);   // alone: its bits as in the pair
+              if (ODD && act1) store_pop<P>(ph, base + (row + x + 1), fs1[a], sh, seed1, a);
             } else if (sr) {
               const float2 d = vsub(make_float2(fs0[a], fs1[a]), sh2);   // node x low, x + 1 high
               *reinterpret_cast<unsigned*>(base + (row + x)) =
@@ -551,7 +558,7 @@ __device__ __forceinline__ void fused_body(const Maps& maps, const Geom& g, cons
             // one conversion per node rounds both with the bits sr_bits gives
             // them (the high half a, the low half a + 1), so the stored values
             // equal those of the one-value conversions of the two-kernel step
-            T* const base_b = BATCH ? s_dir[a + 1] : db->p[a + 1];
+            T* const base_b = TABLE ? s_dir[a + 1] : db->p[a + 1];
             const int row_b = rowp * (yv[1 + cy(a + 1)] + g.ny * zv[1 + cz(a + 1)]);
             const unsigned j = (unsigned)(a + 1) >> 1;
             const float2 da = vsub(make_float2(fs0[a], fs1[a]), sh2);
@@ -567,12 +574,14 @@ __device__ __forceinline__ void fused_body(const Maps& maps, const Geom& g, cons
           }
           // even a with c_x != 0 under stochastic rounding: stored with a - 1
         } else {
-          T* base = (BATCH ? dst + (long long)a * N : db->p[a]) + row;
+          T* base = (TABLE ? dst + (long long)a * N : db->p[a]) + row;
           if (cx(a) == 0) {
-            if (act1)
+            if (!ODD && act1) {
               store_pair<P>(base + x, fs0[a], fs1[a], sh);
-            else
+            } else {
               store_pop<P>(ph, base + x, fs0[a], sh, seed0, a);
+              if (ODD && act1) store_pop<P>(ph, base + x + 1, fs1[a], sh, seed1, a);
+            }
           } else {
             store_pop<P>(ph, base + (cx(a) > 0 ? xr0 : xm), fs0[a], sh, seed0, a);
             if (act1) store_pop<P>(ph, base + (cx(a) > 0 ? xp : x), fs1[a], sh, seed1, a);
@@ -670,6 +679,18 @@ __global__ void __launch_bounds__(FusedShape<P>::NT, fused_minb<P, DIAG, COLL>()
     fused_kernel(const __grid_constant__ Maps maps, Geom g, Phys ph, typename Prec<P>::T* dst, int* flag, int ntx,
                  int nchunks, int fz, int grp, DiagOut dg, const __grid_constant__ DirBases<typename Prec<P>::T> db) {
   fused_body<P, DIAG, COLL, false>(maps, g, ph, dst, flag, ntx, nchunks, fz, grp, dg, blockIdx.x, g.nx, g.N, &db);
+}
+
+// The single-pass step of one lattice of any size (tiles cut at its edges):
+// its source rows start on 16-byte boundaries (maps), its destination has
+// rows of px elements and dstride elements per direction (db).
+template <int P, int W, bool ODD>
+__global__ void __launch_bounds__(FusedShape<P, W>::NT, fused_minb<P, false, COLL_SRT>())
+    ragged_kernel(const __grid_constant__ Maps maps, Geom g, Phys ph, int* flag, int ntx, int nchunks, int fz, int grp,
+                  int px, long long dstride, const __grid_constant__ DirBases<typename Prec<P>::T> db) {
+  const DiagOut none{0.0, 0.0, nullptr, nullptr, 0ull, 0.0f, 0.0f, 0.0f};
+  fused_body<P, false, COLL_SRT, true, W, false, false, ODD>(maps, g, ph, nullptr, flag, ntx, nchunks, fz, grp, none,
+                                                             blockIdx.x, px, dstride, &db);
 }
 
 // One instance of the batched TMA step (device table built by the host).

@@ -60,6 +60,12 @@ cudaError_t launch_collide(int precision, int mode, int minb, bool vec, const Ge
                            const Phys& ph, const void* src, void* dst, const void* psi, dim3 block,
                            cudaStream_t s);
 
+// force + collision + streaming of an A-B step into an array with rows px
+// elements apart (the first step of a run on padded rows; 4- and 2-byte
+// storage, SRT, one node per thread).
+cudaError_t launch_collide_padded(int precision, const Geom& g, const Phys& ph, const void* src, void* dst, int px,
+                                  const void* psi, dim3 block, cudaStream_t s);
+
 // Lattices up to this many nodes launch their steps chained (lbm_launch.cuh)
 // and replay longer graphs: their kernels take a few microseconds each.
 constexpr long long kChainNodes = 1 << 20;
@@ -104,6 +110,26 @@ cudaError_t launch_fused(int precision, const Geom& g, const Phys& ph, const voi
                          int* flag, int fz, int grp, const FusedDiag* diag, unsigned long long stall_ns,
                          cudaStream_t s, ReduceSide* side = nullptr);
 size_t fused_diag_scratch_doubles(const Geom& g, int precision, int fz);
+
+// The single-pass step for lattices that the fused step does not take (any nx
+// and ny, 4- and 2-byte storage, SRT), on tiles cut at the lattice's edges;
+// bitwise the two-kernel step.  TMA needs source rows that start on 16-byte
+// boundaries (src_px elements apart; src 16-byte aligned, Q px ny nz
+// elements): ragged_row is nx where the lattice's own rows do, else the pitch
+// of a padded copy.  dst_px: row pitch of the destination, any.  fz, grp: as
+// launch_fused.
+// Smaller lattices keep the two kernels by default: they live in L2, where the
+// two short passes are as fast or faster (plain steps, two-kernel against
+// single pass: FP32 181x56x56 20.8 / 20.4 us, 172x80x80 42.2 / 37.5, 201x100x100
+// 90.5 / 71.3, 303x150x150 295 / 199; FP16 201x100x100 78 / 70, 200x100x100 68 /
+// 71, 251x112x112 111 / 101, 303x150x150 264 / 194); so do rows of less than
+// half a tile.
+constexpr long long kRaggedNodes = 1 << 20, kRaggedNodesDev = 5 << 19;
+constexpr int kRaggedMinNx = 32;
+bool ragged_applicable(const Geom& g, int precision);
+int ragged_row(const Geom& g, int precision);
+cudaError_t launch_ragged(int precision, const Geom& g, const Phys& ph, const void* src, int src_px, void* dst,
+                          int dst_px, int* flag, int fz, int grp, cudaStream_t s);
 
 // ---- auxiliary kernels (lbm_aux.cu) ---------------------------------------
 struct InitSpec {
@@ -248,6 +274,12 @@ struct lbm_ctx {
   void* state = nullptr;  // populations: A-B = two arrays, AA = one
   size_t state_bytes = 0;
   bool own_state = false;
+  // two private arrays with rows padded to 16 bytes, between which the steps
+  // inside a captured chunk run where the lattice's own rows are not 16-byte
+  // multiples; pad_failed: there was no room for them
+  void* pad[2] = {nullptr, nullptr};
+  size_t pad_bytes = 0;           // of each
+  bool pad_failed = false;
   void* psi = nullptr;
   size_t psi_bytes = 0;
   bool own_psi = false;
@@ -277,7 +309,7 @@ struct lbm_ctx {
   bool block_asked = false;       // block was given (else auto_block is launched)
   int minb = 0;                   // collide kernel register budget variant (0 = auto)
   bool vec = true;                // two nodes per thread (when nx is even)
-  bool fused = true;              // single-pass fused step on non-diagnostic A-B steps (where it applies)
+  int fused = 1;                  // single-pass A-B steps: 0 never, 1 where they apply and pay, 2 where they apply
   int fused_fz = 0;               // z planes per block of the fused step (0 = automatic)
   int fused_group = 0;            // z runs per group of its block order (0 = automatic)
   unsigned long long fused_stall_test_ns = 0;   // test hook of the fused step's timeout path

@@ -568,13 +568,13 @@ __device__ __forceinline__ void psi_quad_gather(const Geom& g, const Phys& ph, c
 template <int P, int MODE, int COLL>
 constexpr bool kRhoFromDst = P == LBM_F64 && MODE == MODE_AB && COLL == COLL_SRT;
 
-// One node.
+// One node.  px > 0: the destination's rows are px elements apart (A-B only).
 template <int P, int MODE, bool NC, int COLL = COLL_SRT>
 __device__ __forceinline__ void collide_node(const Geom& g, const Phys& ph,
                                              const typename Prec<P>::T* src,
                                              typename Prec<P>::T* dst,
                                              const typename Prec<P>::C* psi, int x,
-                                             int y, int z) {
+                                             int y, int z, int px = 0) {
   using C = typename Prec<P>::C;
   Nbr nb;
   nb.make(g, x, y, z);
@@ -603,6 +603,14 @@ __device__ __forceinline__ void collide_node(const Geom& g, const Phys& ph,
   else
     collide_math<C>(ph, f, ld<NC>(psi + i), pn, fs);
   const unsigned seed = (Prec<P>::dev && ph.sr) ? sr_seed(i, fs[0], salt_of(ph)) : 0u;
+  Nbr nd = nb;
+  long long Nd = N;
+  if (MODE == MODE_AB && px > 0) {
+    Geom gd = g;
+    gd.nx = px;
+    nd.make_rows(gd, y, z);
+    Nd = (long long)px * g.ny * g.nz;
+  }
 #pragma unroll
   for (int a = 0; a < Q; ++a) {
     const C sh = a == 0 ? s0 : (a <= 6 ? s1 : s2);
@@ -610,7 +618,7 @@ __device__ __forceinline__ void collide_node(const Geom& g, const Phys& ph,
     if constexpr (MODE == MODE_AA_EVEN)
       d = (long long)opp(a) * N + i;
     else
-      d = (long long)a * N + nb.idx(cx(a), cy(a), cz(a));
+      d = (long long)a * Nd + nd.idx(cx(a), cy(a), cz(a));
     store_pop<P>(ph, dst + d, fs[a], sh, seed, a);
   }
 }

@@ -90,6 +90,29 @@ __global__ void __launch_bounds__(256, MINB) collide_pair_kernel(Geom g, Phys ph
   collide_pair<P, MODE, !CHAIN>(g, ph, src, dst, psi, x0, y, z);
 }
 
+// The one-node A-B kernel into an array with rows px elements apart.
+template <int P>
+__global__ void __launch_bounds__(256, 3) collide_padded_kernel(Geom g, Phys ph, const typename Prec<P>::T* src,
+                                                                typename Prec<P>::T* dst, int px,
+                                                                const typename Prec<P>::C* psi) {
+  const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  const int y = blockIdx.y * blockDim.y + threadIdx.y;
+  const int z = blockIdx.z * blockDim.z + threadIdx.z;
+  if (x >= g.nx || y >= g.ny || z >= g.nz) return;
+  advance_salt(ph);
+  collide_node<P, MODE_AB, true>(g, ph, src, dst, psi, x, y, z, px);
+}
+
+template <int P>
+cudaError_t collide_padded(const Geom& g, const Phys& ph, const void* src, void* dst, int px, const void* psi,
+                           dim3 block, cudaStream_t s) {
+  using T = typename Prec<P>::T;
+  using C = typename Prec<P>::C;
+  const dim3 grid((g.nx + block.x - 1) / block.x, (g.ny + block.y - 1) / block.y, (g.nz + block.z - 1) / block.z);
+  collide_padded_kernel<P><<<grid, block, 0, s>>>(g, ph, (const T*)src, (T*)dst, px, (const C*)psi);
+  return cudaGetLastError();
+}
+
 // Threads per block of the psi pass: 256, fewer (to one warp) where that
 // leaves less than two blocks per SM.
 int psi_threads(long long units) {
@@ -217,6 +240,16 @@ cudaError_t launch_collide(int precision, int mode, int minb, bool vec, const Ge
     return cudaErrorInvalidValue;
   };
   return g.chain ? run(std::true_type{}) : run(std::false_type{});
+}
+
+cudaError_t launch_collide_padded(int precision, const Geom& g, const Phys& ph, const void* src, void* dst, int px,
+                                  const void* psi, dim3 block, cudaStream_t s) {
+  switch (precision) {
+    case LBM_F32: return collide_padded<LBM_F32>(g, ph, src, dst, px, psi, block, s);
+    case LBM_F16DEV: return collide_padded<LBM_F16DEV>(g, ph, src, dst, px, psi, block, s);
+    case LBM_BF16DEV: return collide_padded<LBM_BF16DEV>(g, ph, src, dst, px, psi, block, s);
+  }
+  return cudaErrorInvalidValue;
 }
 
 // FP64 kernels take one node per thread: the FP64 pipe bounds them either way
