@@ -167,7 +167,7 @@ int lbm_set_stream(lbm_handle h, void *stream);
  * ny % 8 == 0 (2-byte storage); lbm_get_option answers whether it applies.
  * Of the other lattices of these storage forms, larger ones (more than 1 M
  * nodes in FP32, 2.6 M in 2-byte storage, nx >= 32; with the value 2 all of
- * them) run plain SRT steps as a single pass on tiles cut at their edges: every
+ * them) run plain steps as a single pass on tiles cut at their edges: every
  * step where rows are a multiple of 16 bytes; otherwise the steps inside a
  * replayed graph but its first one, on two private arrays with padded rows
  * (allocated on the first such call if they take at most a quarter of the

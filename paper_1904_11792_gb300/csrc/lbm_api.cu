@@ -293,7 +293,7 @@ int enqueue_step(lbm_ctx* h, cudaStream_t s, long long step, int cur, bool timed
 bool ragged_form(const lbm_ctx* h) {
   const long long least = Prec_dev(h->cfg.precision) ? kRaggedNodesDev : kRaggedNodes;
   return h->fused && (h->fused == 2 || (h->g.N > least && h->g.nx >= kRaggedMinNx)) &&
-         h->cfg.pattern == LBM_AB && h->ph.coll == COLL_SRT && ragged_applicable(h->g, h->cfg.precision);
+         h->cfg.pattern == LBM_AB && ragged_applicable(h->g, h->cfg.precision);
 }
 bool ragged_direct(const lbm_ctx* h) {
   return ragged_form(h) && ragged_row(h->g, h->cfg.precision) == h->g.nx && ((uintptr_t)h->state & 15) == 0;
@@ -760,6 +760,7 @@ int lbm_set_option(lbm_handle h, const char* key, double v) {
     if (k == "mrt_s_q") h->ph.s_q = v;
     if (k == "mrt_s_pi") h->ph.s_pi = v;
     if (k == "mrt_s_m") h->ph.s_m = v;
+    phys_finalize(h->ph, h->cfg.precision);
     drop_graphs(h);
   } else if (k == "fused") {
     h->fused = v == 0.0 ? 0 : (v == 2.0 ? 2 : 1);

@@ -146,6 +146,31 @@ __device__ __forceinline__ C splat(typename Lane<C>::S x) {
     return x;
 }
 
+// Correctly rounded reciprocal: the bits of 1 / x (IEEE division) without
+// the division's general path.
+__device__ __forceinline__ float rcp_rn(float x) { return __frcp_rn(x); }
+
+// Lane-wise correctly rounded reciprocal of a pair.
+__device__ __forceinline__ float2 rcp_rn(float2 x) { return make_float2(__frcp_rn(x.x), __frcp_rn(x.y)); }
+
+// 1 / x in FP64 by one third-order (Halley) iteration, y (1 + e + e^2) with e
+// = 1 - x y, on the seed of the PTX instruction rcp.approx.ftz.f64 (relative
+// error below 2^-20, so e^3 is below 2^-60): 3 FP64 instructions.  x = 0, inf
+// and NaN give NaN, where the caller's product with 1 / x is NaN or void
+// anyway (rho = 0 has zero momentum and force).
+__device__ __forceinline__ double rcp_f64(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  double e = __fma_rn(-x, y, 1.0);
+  e = __fma_rn(e, e, e);
+  return __fma_rn(y, e, y);
+}
+
+// The reciprocal of a density in the arithmetic's own form.
+__device__ __forceinline__ float rcp_node(float x) { return rcp_rn(x); }
+__device__ __forceinline__ float2 rcp_node(float2 x) { return rcp_rn(x); }
+__device__ __forceinline__ double rcp_node(double x) { return rcp_f64(x); }
+
 // Moments of one node's populations, and the link sums of the force, in one
 // fixed order shared by every kernel: opposite populations a, a + 1 (a odd)
 // are combined first, then short trees, so the dependency chains are 5 adds
@@ -401,6 +426,9 @@ struct Phys {
   double omega, om1, gtau;
   int unit_rho0;
   const double2* psi_tab;
+  // FP32 MRT rates s_e, s_eps, s_q, s_pi, s_m, and 1 - s/2 of the first four
+  // and of the shear rate 1/tau (phys_finalize)
+  float mrt_sf[5], mrt_hf[5];
 };
 enum Collision { COLL_SRT = 0, COLL_MRT = 1 };
 // Sets the FP32 fields of ph from its doubles, for storage `precision`.
@@ -414,6 +442,11 @@ __host__ inline void phys_finalize(Phys& ph, int precision) {
   ph.om1 = 1.0 - ph.omega;
   ph.gtau = -(ph.G * ph.tau) / 36.0;
   ph.unit_rho0 = ph.rho0 == 1.0;
+  const double rates[5] = {ph.s_e, ph.s_eps, ph.s_q, ph.s_pi, ph.s_m};
+  for (int c = 0; c < 5; ++c) {
+    ph.mrt_sf[c] = (float)rates[c];
+    ph.mrt_hf[c] = fmaf(-0.5f, c < 4 ? ph.mrt_sf[c] : ph.omega_f, 1.0f);
+  }
   const int lead[3] = {0, 1, 7};
   for (int c = 0; c < 3; ++c) {
     const float v = (float)(wgt(lead[c]) * ph.rho_ref);

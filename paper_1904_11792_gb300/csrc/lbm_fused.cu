@@ -221,9 +221,12 @@ cudaError_t fused_device_info(int* slots_per_sm, int* sms) {
       if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem);
     for (const void* k : {(const void*)bfused_kernel<P, TX>, (const void*)bpersist_kernel<P, TX>})
       if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem);
-    for (const void* k : {(const void*)ragged_kernel<P, kRaggedW<P>, false>, (const void*)ragged_kernel<P, kRaggedW<P>, true>})
+    constexpr int RW = kRaggedW<P>;
+    for (const void* k :
+         {(const void*)ragged_kernel<P, COLL_SRT, RW, false>, (const void*)ragged_kernel<P, COLL_SRT, RW, true>,
+          (const void*)ragged_kernel<P, COLL_MRT, RW, false>, (const void*)ragged_kernel<P, COLL_MRT, RW, true>})
       if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FusedShape<P, kRaggedW<P>>::smem);
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FusedShape<P, RW>::smem);
     for (const void* k : {(const void*)bfused_kernel<P, 32>, (const void*)bpersist_kernel<P, 32>})
       if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FusedShape<P, 32>::smem);
@@ -328,8 +331,11 @@ cudaError_t ragged_t(const Geom& g, const Phys& ph, const void* src, int src_px,
   // pairs of nodes are stored as one 2-element vector where every row starts
   // at such a vector's boundary
   const bool odd = dst_px % 2 != 0 || (uintptr_t)dst % (2 * sizeof(T)) != 0;
-  return chain_launch(g.chain, odd ? ragged_kernel<P, W, true> : ragged_kernel<P, W, false>, (unsigned)(tiles * nchunks),
-                      S::NT, S::smem, s, m, g, ph, flag, ntx, nchunks, fz, grp, dst_px, dstride, db);
+  const auto kernel = ph.coll == COLL_MRT
+                          ? (odd ? ragged_kernel<P, COLL_MRT, W, true> : ragged_kernel<P, COLL_MRT, W, false>)
+                          : (odd ? ragged_kernel<P, COLL_SRT, W, true> : ragged_kernel<P, COLL_SRT, W, false>);
+  return chain_launch(g.chain, kernel, (unsigned)(tiles * nchunks), S::NT, S::smem, s, m, g, ph, flag, ntx, nchunks, fz,
+                      grp, dst_px, dstride, db);
 }
 
 }  // namespace

@@ -237,7 +237,7 @@ __device__ __forceinline__ void fused_body(const Maps& maps, const Geom& g, cons
   constexpr int TY = S::TY, RH = S::RH, RW = S::RWW;
   static_assert(!DIAG || 2 * TY * TX * sizeof(double) + 10 * TY * sizeof(double) <= S::ring_bytes,
                 "the diagnostics reduction reuses the psi ring");
-  static_assert(!(BATCH && (DIAG || COLL != COLL_SRT)), "the batched step is the plain SRT step");
+  static_assert(!(BATCH && DIAG) && !(TABLE && COLL != COLL_SRT), "cut tiles run plain steps, the batched step SRT");
   static_assert(W == TX || BATCH, "32-wide tiles for the batched step only");
   extern __shared__ __align__(128) unsigned char smem[];
   unsigned long long* full = reinterpret_cast<unsigned long long*>(smem + S::off_bar);
@@ -510,24 +510,10 @@ __device__ __forceinline__ void fused_body(const Maps& maps, const Geom& g, cons
         unpack_shifted<P>(prev[a], a == 0 ? s0 : (a <= 6 ? s1 : s2), g2[a].x, g2[a].y);
       }
       C fs0[Q], fs1[Q];
-      if constexpr (COLL == COLL_MRT) {
-        C g0[Q], g1[Q], pn0[Q], pn1[Q];
-        pn0[0] = pn1[0] = 0;
+      float2 fs2[Q];
+      collide_pair_math<COLL>(ph, g2, make_float2(prho[0], prho[1]), q, fs2);
 #pragma unroll
-        for (int a = 0; a < Q; ++a) g0[a] = g2[a].x, g1[a] = g2[a].y;
-#pragma unroll
-        for (int a = 1; a < Q; ++a) {
-          pn0[a] = q[cy(a) + 1][cz(a) + 1][1 + cx(a)];
-          pn1[a] = q[cy(a) + 1][cz(a) + 1][2 + cx(a)];
-        }
-        collide_math_mrt<C>(ph, g0, q[1][1][1], pn0, fs0);
-        collide_math_mrt<C>(ph, g1, q[1][1][2], pn1, fs1);
-      } else {
-        float2 fs2[Q];
-        collide_pair_math(ph, g2, make_float2(prho[0], prho[1]), q, fs2);
-#pragma unroll
-        for (int a = 0; a < Q; ++a) fs0[a] = fs2[a].x, fs1[a] = fs2[a].y;
-      }
+      for (int a = 0; a < Q; ++a) fs0[a] = fs2[a].x, fs1[a] = fs2[a].y;
       const int i0 = x + g.nx * (y + g.ny * z);
       const bool sr = Prec<P>::dev && ph.sr;
       const unsigned seed0 = sr ? sr_seed(i0, fs0[0], salt) : 0u, seed1 = sr ? sr_seed(i0 + 1, fs1[0], salt) : 0u;
@@ -684,13 +670,13 @@ __global__ void __launch_bounds__(FusedShape<P>::NT, fused_minb<P, DIAG, COLL>()
 // The single-pass step of one lattice of any size (tiles cut at its edges):
 // its source rows start on 16-byte boundaries (maps), its destination has
 // rows of px elements and dstride elements per direction (db).
-template <int P, int W, bool ODD>
-__global__ void __launch_bounds__(FusedShape<P, W>::NT, fused_minb<P, false, COLL_SRT>())
+template <int P, int COLL, int W, bool ODD>
+__global__ void __launch_bounds__(FusedShape<P, W>::NT, fused_minb<P, false, COLL>())
     ragged_kernel(const __grid_constant__ Maps maps, Geom g, Phys ph, int* flag, int ntx, int nchunks, int fz, int grp,
                   int px, long long dstride, const __grid_constant__ DirBases<typename Prec<P>::T> db) {
   const DiagOut none{0.0, 0.0, nullptr, nullptr, 0ull, 0.0f, 0.0f, 0.0f};
-  fused_body<P, false, COLL_SRT, true, W, false, false, ODD>(maps, g, ph, nullptr, flag, ntx, nchunks, fz, grp, none,
-                                                             blockIdx.x, px, dstride, &db);
+  fused_body<P, false, COLL, true, W, false, false, ODD>(maps, g, ph, nullptr, flag, ntx, nchunks, fz, grp, none,
+                                                         blockIdx.x, px, dstride, &db);
 }
 
 // One instance of the batched TMA step (device table built by the host).

@@ -62,7 +62,7 @@ cudaError_t launch_collide(int precision, int mode, int minb, bool vec, const Ge
 
 // force + collision + streaming of an A-B step into an array with rows px
 // elements apart (the first step of a run on padded rows; 4- and 2-byte
-// storage, SRT, one node per thread).
+// storage, one node per thread).
 cudaError_t launch_collide_padded(int precision, const Geom& g, const Phys& ph, const void* src, void* dst, int px,
                                   const void* psi, dim3 block, cudaStream_t s);
 
@@ -112,7 +112,7 @@ cudaError_t launch_fused(int precision, const Geom& g, const Phys& ph, const voi
 size_t fused_diag_scratch_doubles(const Geom& g, int precision, int fz);
 
 // The single-pass step for lattices that the fused step does not take (any nx
-// and ny, 4- and 2-byte storage, SRT), on tiles cut at the lattice's edges;
+// and ny, 4- and 2-byte storage), on tiles cut at the lattice's edges;
 // bitwise the two-kernel step.  TMA needs source rows that start on 16-byte
 // boundaries (src_px elements apart; src 16-byte aligned, Q px ny nz
 // elements): ragged_row is nx where the lattice's own rows do, else the pitch

@@ -165,13 +165,6 @@ __device__ __forceinline__ void store_pop(const Phys& ph, typename Prec<P>::T* p
 // arithmetic of one node
 // ---------------------------------------------------------------------------
 
-// Correctly rounded reciprocal: the bits of 1 / x (IEEE division) without
-// the division's general path.
-__device__ __forceinline__ float rcp_rn(float x) { return __frcp_rn(x); }
-
-// Lane-wise correctly rounded reciprocal of a pair.
-__device__ __forceinline__ float2 rcp_rn(float2 x) { return make_float2(__frcp_rn(x.x), __frcp_rn(x.y)); }
-
 // c_a . u for odd a, whose first nonzero velocity component is +1: sums of
 // the velocity components only (no 0 + u_x, which the compiler must keep
 // for a -0 operand).
@@ -252,19 +245,6 @@ __device__ __forceinline__ void collide_math_ls(const Phys& ph, const C f[Q], C 
   fs[0] = xfma(om1, f[0], xfma(splat<C>((S)-2), sumA, orho));
 }
 
-// 1 / x in FP64 by one third-order (Halley) iteration, y (1 + e + e^2) with e
-// = 1 - x y, on the seed of the PTX instruction rcp.approx.ftz.f64 (relative
-// error below 2^-20, so e^3 is below 2^-60): 3 FP64 instructions.  x = 0, inf
-// and NaN give NaN, where the caller's product with 1 / x is NaN or void
-// anyway (rho = 0 has zero momentum and force).
-__device__ __forceinline__ double rcp_f64(double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  double e = __fma_rn(-x, y, 1.0);
-  e = __fma_rn(e, e, e);
-  return __fma_rn(y, e, y);
-}
-
 // The FP64 form (the same equations in fewer
 // operations, since every one occupies GB300's narrow FP64 pipe for 16 clocks
 // per warp): the force enters as tau F = -(G tau / 36) psi (2 a + d), with the
@@ -325,6 +305,7 @@ __device__ __forceinline__ void collide_math(const Phys& ph, const C f[Q], C pc,
 // dy, z + dz).  The link differences of the directions with c_x = 0 are one
 // paired difference of the pair's own two values, those of the x-shifted
 // directions two scalar differences (their results pair up freely).
+template <int COLL = COLL_SRT>
 __device__ __forceinline__ void collide_pair_math(const Phys& ph, const float2 f[Q], float2 rho,
                                                   const float (&q)[3][3][4], float2 fs[Q]) {
   float2 e[Q];
@@ -341,7 +322,11 @@ __device__ __forceinline__ void collide_pair_math(const Phys& ph, const float2 f
   float2 ax, ay, az, dx, dy, dz, jx, jy, jz;
   link_combine<float2>(e, ax, ay, az, dx, dy, dz);
   mom_of<float2>(f, jx, jy, jz);
-  collide_math_ls<float2>(ph, f, rho, jx, jy, jz, make_float2(q[1][1][1], q[1][1][2]), ax, ay, az, dx, dy, dz, fs);
+  const float2 pc = make_float2(q[1][1][1], q[1][1][2]);
+  if constexpr (COLL == COLL_MRT)
+    collide_math_mrt_ls<float2>(ph, f, rho, jx, jy, jz, pc, ax, ay, az, dx, dy, dz, fs);
+  else
+    collide_math_ls<float2>(ph, f, rho, jx, jy, jz, pc, ax, ay, az, dx, dy, dz, fs);
 }
 
 // A non-positive, NaN or infinite density (the numeric flag's condition).
@@ -693,24 +678,12 @@ __device__ __forceinline__ void collide_pair(const Geom& g, const Phys& ph,
       }
     }
   C fs0[Q], fs1[Q];
-  if constexpr (COLL == COLL_MRT) {
-    C pn0[Q], pn1[Q];
-    pn0[0] = pn1[0] = 0;
+  float2 fp[Q], fs[Q];
 #pragma unroll
-    for (int a = 1; a < Q; ++a) {
-      pn0[a] = q[cy(a) + 1][cz(a) + 1][1 + cx(a)];
-      pn1[a] = q[cy(a) + 1][cz(a) + 1][2 + cx(a)];
-    }
-    collide_math_mrt<C>(ph, f0, q[1][1][1], pn0, fs0);
-    collide_math_mrt<C>(ph, f1, q[1][1][2], pn1, fs1);
-  } else {
-    float2 fp[Q], fs[Q];
+  for (int a = 0; a < Q; ++a) fp[a] = make_float2(f0[a], f1[a]);
+  collide_pair_math<COLL>(ph, fp, rho_of<float2>(fp), q, fs);
 #pragma unroll
-    for (int a = 0; a < Q; ++a) fp[a] = make_float2(f0[a], f1[a]);
-    collide_pair_math(ph, fp, rho_of<float2>(fp), q, fs);
-#pragma unroll
-    for (int a = 0; a < Q; ++a) fs0[a] = fs[a].x, fs1[a] = fs[a].y;
-  }
+  for (int a = 0; a < Q; ++a) fs0[a] = fs[a].x, fs1[a] = fs[a].y;
   const bool sr = Prec<P>::dev && ph.sr;
   const unsigned salt = sr ? salt_of(ph) : 0u;
   const unsigned seed0 = sr ? sr_seed(i0, fs0[0], salt) : 0u, seed1 = sr ? sr_seed(i0 + 1, fs1[0], salt) : 0u;

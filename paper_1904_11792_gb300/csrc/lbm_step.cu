@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(256, MINB) collide_pair_kernel(Geom g, Phys ph
 }
 
 // The one-node A-B kernel into an array with rows px elements apart.
-template <int P>
+template <int P, int COLL>
 __global__ void __launch_bounds__(256, 3) collide_padded_kernel(Geom g, Phys ph, const typename Prec<P>::T* src,
                                                                 typename Prec<P>::T* dst, int px,
                                                                 const typename Prec<P>::C* psi) {
@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(256, 3) collide_padded_kernel(Geom g, Phys ph,
   const int z = blockIdx.z * blockDim.z + threadIdx.z;
   if (x >= g.nx || y >= g.ny || z >= g.nz) return;
   advance_salt(ph);
-  collide_node<P, MODE_AB, true>(g, ph, src, dst, psi, x, y, z, px);
+  collide_node<P, MODE_AB, true, COLL>(g, ph, src, dst, psi, x, y, z, px);
 }
 
 template <int P>
@@ -109,7 +109,10 @@ cudaError_t collide_padded(const Geom& g, const Phys& ph, const void* src, void*
   using T = typename Prec<P>::T;
   using C = typename Prec<P>::C;
   const dim3 grid((g.nx + block.x - 1) / block.x, (g.ny + block.y - 1) / block.y, (g.nz + block.z - 1) / block.z);
-  collide_padded_kernel<P><<<grid, block, 0, s>>>(g, ph, (const T*)src, (T*)dst, px, (const C*)psi);
+  if (ph.coll == COLL_MRT)
+    collide_padded_kernel<P, COLL_MRT><<<grid, block, 0, s>>>(g, ph, (const T*)src, (T*)dst, px, (const C*)psi);
+  else
+    collide_padded_kernel<P, COLL_SRT><<<grid, block, 0, s>>>(g, ph, (const T*)src, (T*)dst, px, (const C*)psi);
   return cudaGetLastError();
 }
 

@@ -24,14 +24,15 @@ def L():
 SHAPES = [(251, 12, 11), (100, 13, 9), (66, 16, 9), (32, 17, 10), (129, 5, 12), (200, 9, 8), (192, 10, 7), (5, 3, 4), (8, 3, 3)]
 
 
-@pytest.mark.parametrize("precision", ["f32", "f16dev", "bf16dev"])
+@pytest.mark.parametrize("precision,mrt", [("f32", 0), ("f16dev", 0), ("bf16dev", 0), ("f32", 1), ("f16dev", 1)])
 @pytest.mark.parametrize("shape", SHAPES)
-def test_ragged_step_equals_two_kernel_step(L, shape, precision):
+def test_ragged_step_equals_two_kernel_step(L, shape, precision, mrt):
     f0 = lbm_inputs.random_populations(*shape, seed=81)
     out = []
     for fused in (2, 0):     # 2: whatever the lattice's size
         with L.Lattice(*shape, 0.9, -5.5, precision=precision, rho_ref=0.1) as lat:
             lat.set_option("fused", fused)
+            lat.set_option("collision", mrt)
             lat.set_populations(f0)
             got = []
             for n in (1, 2, 5, 23):
