@@ -179,6 +179,26 @@ int auto_minb(bool vec, int mode, int precision) {
 
 bool ragged_direct(const lbm_ctx* h);
 
+// The psi pass of a diagnostic step of the two kernels: with the diagnostics,
+// and the droplet counts where they are on.
+int enqueue_diagnostics(lbm_ctx* h, cudaStream_t s, const Geom& g, int layout, const void* src, void* dst,
+                        ReduceSide* side) {
+  const int prec = h->cfg.precision;
+  const double thr = 0.5 * (h->rho_l + h->rho_v);
+  DiagExtra x;
+  if (h->diag_ccl) x = diag_labels(prec, layout, g, src, h->psi, thr, h->d_labels, h->d_labels + g.N);
+  x.dst = dst;
+  x.side = side;
+  CK(launch_diagnostics(prec, layout, g, h->ph, src, h->rho_l, h->rho_v, h->d_scratch, h->d_ring, h->psi, h->d_flag,
+                        h->d_ring_count, lbm_ctx::kRing, s, x));
+  if (h->diag_ccl) {
+    long long* d4 = (long long*)(h->d_small + 32);
+    CK(launch_ccl(prec, layout, g, h->ph, src, thr, h->d_labels, h->d_labels + g.N, d4, s, x.labels != nullptr));
+    CK(launch_ccl_ring(d4, h->d_ring, h->d_ring_count, lbm_ctx::kRing, s));
+  }
+  return LBM_OK;
+}
+
 // Enqueues one time step on stream s.  `phase` is the step parity (AA) or
 // the index of the current array (A-B).  With timing on, each kernel is
 // bracketed by events on s.  side (captures): where the diagnostics'
@@ -259,15 +279,7 @@ int enqueue_step(lbm_ctx* h, cudaStream_t s, long long step, int cur, bool timed
     CK(cudaEventRecord(e0, s));
   }
   if (diag_step) {
-    CK(launch_diagnostics(prec, layout, g, h->ph, src, h->rho_l, h->rho_v, h->d_scratch, h->d_ring,
-                          h->psi, h->d_flag, h->d_ring_count, lbm_ctx::kRing, s,
-                          aa ? nullptr : dst, side));
-    if (h->diag_ccl) {
-      long long* d4 = (long long*)(h->d_small + 32);
-      CK(launch_ccl(prec, layout, h->g, h->ph, src, 0.5 * (h->rho_l + h->rho_v), h->d_labels,
-                    h->d_labels + h->g.N, d4, s));
-      CK(launch_ccl_ring(d4, h->d_ring, h->d_ring_count, lbm_ctx::kRing, s));
-    }
+    if (int rc = enqueue_diagnostics(h, s, g, layout, src, aa ? nullptr : dst, side)) return rc;
   } else {
     CK(launch_psi(prec, layout, h->vec, g, h->ph, src, h->psi, h->d_flag, s, aa ? nullptr : dst));
   }
@@ -340,15 +352,7 @@ int enqueue_padded_step(lbm_ctx* h, cudaStream_t s, int k, int steps, int phase,
   if (k == 0) {
     const void* src = array_ptr(h, phase);
     if (h->diag_interval > 0) {
-      if (h->diag_ccl) side = nullptr;
-      CK(launch_diagnostics(prec, LAYOUT_LOCAL, g, h->ph, src, h->rho_l, h->rho_v, h->d_scratch, h->d_ring, h->psi,
-                            h->d_flag, h->d_ring_count, lbm_ctx::kRing, s, nullptr, side));
-      if (h->diag_ccl) {
-        long long* d4 = (long long*)(h->d_small + 32);
-        CK(launch_ccl(prec, LAYOUT_LOCAL, g, h->ph, src, 0.5 * (h->rho_l + h->rho_v), h->d_labels,
-                      h->d_labels + g.N, d4, s));
-        CK(launch_ccl_ring(d4, h->d_ring, h->d_ring_count, lbm_ctx::kRing, s));
-      }
+      if (int rc = enqueue_diagnostics(h, s, g, LAYOUT_LOCAL, src, nullptr, h->diag_ccl ? nullptr : side)) return rc;
     } else {
       CK(launch_psi(prec, LAYOUT_LOCAL, h->vec, g, h->ph, src, h->psi, h->d_flag, s));
     }
@@ -521,6 +525,8 @@ void end_transfer(lbm_ctx* h) {
   h->transfer_n = 0;
 }
 
+size_t trig_bytes(const Geom& g) { return sizeof(double2) * ((size_t)g.nx + g.ny + g.nz); }
+
 struct StateHeader {
   char magic[8];
   int version, precision, pattern, nx, ny, nz, cur, pad;
@@ -607,6 +613,7 @@ void lbm_destroy(lbm_handle h) {
   dev_free(h->d_transfer, h->transfer_n * sizeof(double));
   dev_free(h->d_labels, (size_t)h->g.N * 2 * sizeof(int));
   dev_free(h->d_drop, h->drop_bytes);
+  dev_free(h->d_trig, trig_bytes(h->g));
   dev_free(h->d_ring, sizeof(double) * DIAG_STRIDE * lbm_ctx::kRing);
   dev_free(h->d_ring_count, sizeof(unsigned long long));
   if (h->own_stream) cudaStreamDestroy(h->own_stream);
@@ -1072,16 +1079,21 @@ int lbm_diagnostics(lbm_handle h, lbm_diag* out, int want_ccl) {
   if (rc) return rc;
   const int layout = cur_layout(h);
   const void* f = cur_array(h);
-  CK(launch_diagnostics(h->cfg.precision, layout, h->g, h->ph, f, h->rho_l, h->rho_v, h->d_scratch,
-                        h->d_small, nullptr, nullptr, nullptr, 0, h->stream));
-  double r[DIAG_OUT];
-  long long c4[4] = {-1, -1, -1, 0};
+  const double thr = 0.5 * (h->rho_l + h->rho_v);
+  DiagExtra x;
   if (want_ccl) {
     rc = ensure_labels(h);
     if (rc) return rc;
+    x = diag_labels(h->cfg.precision, layout, h->g, f, nullptr, thr, h->d_labels, h->d_labels + h->g.N);
+  }
+  CK(launch_diagnostics(h->cfg.precision, layout, h->g, h->ph, f, h->rho_l, h->rho_v, h->d_scratch,
+                        h->d_small, nullptr, nullptr, nullptr, 0, h->stream, x));
+  double r[DIAG_OUT];
+  long long c4[4] = {-1, -1, -1, 0};
+  if (want_ccl) {
     long long* d4 = (long long*)(h->d_small + 32);
-    CK(launch_ccl(h->cfg.precision, layout, h->g, h->ph, f, 0.5 * (h->rho_l + h->rho_v), h->d_labels,
-                  h->d_labels + h->g.N, d4, h->stream));
+    CK(launch_ccl(h->cfg.precision, layout, h->g, h->ph, f, thr, h->d_labels, h->d_labels + h->g.N, d4, h->stream,
+                  x.labels != nullptr));
     CK(cudaMemcpyAsync(c4, d4, sizeof(c4), cudaMemcpyDeviceToHost, h->stream));
   }
   CK(cudaMemcpyAsync(r, h->d_small, sizeof(r), cudaMemcpyDeviceToHost, h->stream));
@@ -1105,7 +1117,13 @@ int lbm_droplets(lbm_handle h, lbm_droplet* out, int max_droplets, int* count) {
   long long* d4 = (long long*)(h->d_small + 32);
   int* L = h->d_labels;
   int* sizes = h->d_labels + h->g.N;
-  CK(launch_ccl(h->cfg.precision, layout, h->g, h->ph, f, 0.5 * (h->rho_l + h->rho_v), L, sizes, d4, h->stream));
+  if (!h->d_trig) {
+    rc = dev_alloc((void**)&h->d_trig, trig_bytes(h->g), "angles");
+    if (rc) return rc;
+    CK(launch_trig(h->g, h->d_trig, h->stream));
+  }
+  CK(launch_ccl(h->cfg.precision, layout, h->g, h->ph, f, 0.5 * (h->rho_l + h->rho_v), L, sizes, d4, h->stream, false,
+                true));
   long long c4[4];
   CK(cudaMemcpyAsync(c4, d4, sizeof(c4), cudaMemcpyDeviceToHost, h->stream));
   CK(cudaStreamSynchronize(h->stream));
@@ -1115,7 +1133,7 @@ int lbm_droplets(lbm_handle h, lbm_droplet* out, int max_droplets, int* count) {
   if (nd == 0) return LBM_OK;
   const int words = (h->g.nx + 31) / 32;
   const size_t rec_bytes = sizeof(double) * DROP_REC * (size_t)nd;
-  const size_t need = rec_bytes + sizeof(unsigned) * ((size_t)words * nd + 1);
+  const size_t need = rec_bytes + sizeof(unsigned) * (size_t)words * nd;
   if (need > h->drop_bytes) {
     dev_free(h->d_drop, h->drop_bytes);
     h->d_drop = nullptr;
@@ -1126,17 +1144,13 @@ int lbm_droplets(lbm_handle h, lbm_droplet* out, int max_droplets, int* count) {
   }
   double* rec = h->d_drop;
   unsigned* xbits = (unsigned*)((char*)h->d_drop + rec_bytes);
-  unsigned* nslot = xbits + (size_t)words * nd;
-  CK(launch_droplets(h->cfg.precision, layout, h->g, h->ph, f, h->rho_l, h->rho_v, L, sizes, rec, xbits, nslot,
+  CK(launch_droplets(h->cfg.precision, layout, h->g, h->ph, f, h->rho_l, h->rho_v, L, sizes, h->d_trig, rec, xbits,
                      (int)nd, h->stream));
   std::vector<double> hr((size_t)DROP_REC * nd);
   std::vector<unsigned> hb((size_t)words * nd);
-  unsigned ns = 0;
   CK(cudaMemcpyAsync(hr.data(), rec, rec_bytes, cudaMemcpyDeviceToHost, h->stream));
   CK(cudaMemcpyAsync(hb.data(), xbits, sizeof(unsigned) * hb.size(), cudaMemcpyDeviceToHost, h->stream));
-  CK(cudaMemcpyAsync(&ns, nslot, sizeof(unsigned), cudaMemcpyDeviceToHost, h->stream));
   CK(cudaStreamSynchronize(h->stream));
-  if ((long long)ns != nd) return fail(LBM_ERR_STATE, "droplet roots differ from the component count");
   std::vector<lbm_droplet> d((size_t)nd);
   const double two_pi = 6.283185307179586476925286766559;
   const int dims[3] = {h->g.nx, h->g.ny, h->g.nz};

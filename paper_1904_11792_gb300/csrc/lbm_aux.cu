@@ -15,6 +15,45 @@ __device__ __forceinline__ double shift_d(int a, double rho_ref) {
   return Prec<P>::dev ? (double)storage_shift<P>(a, rho_ref) : 0.0;
 }
 
+// The shift in the arithmetic's precision (the host's FP32 form).
+template <int P>
+__device__ __forceinline__ float shift_f(int a, const Phys& ph) {
+  return Prec<P>::dev ? ph.shift_f[a == 0 ? 0 : (a <= 6 ? 1 : 2)] : 0.0f;
+}
+
+// Two stored neighbours (4- or 2-byte storage) as float2, shifted.
+template <int P>
+__device__ __forceinline__ void load_pair_nc(const typename Prec<P>::T* p, float sh, float2& v) {
+  if constexpr (P == LBM_F32) {
+    v = __ldg(reinterpret_cast<const float2*>(p));
+  } else {
+    if constexpr (P == LBM_F16DEV)
+      v = __half22float2(__ldg(reinterpret_cast<const __half2*>(p)));
+    else
+      v = __bfloat1622float2(__ldg(reinterpret_cast<const __nv_bfloat162*>(p)));
+    v.x += sh;
+    v.y += sh;
+  }
+}
+
+// DSum<float> of two lanes at once, in paired instructions.
+struct DSum2 {
+  float2 hi{0.0f, 0.0f}, lo{0.0f, 0.0f};
+  __device__ __forceinline__ void add(float2 x) {
+    float2 e;
+    hi = two_sum(hi, x, e);
+    lo = radd(lo, e);
+  }
+  __device__ __forceinline__ void add(float2 x, float2 xlo) {
+    float2 e;
+    hi = two_sum(hi, x, e);
+    lo = radd(lo, radd(e, xlo));
+  }
+  __device__ __forceinline__ double value() const {
+    return ((double)hi.x + (double)lo.x) + ((double)hi.y + (double)lo.y);
+  }
+};
+
 __device__ __forceinline__ void coords(const Geom& g, long long i, int& x, int& y, int& z) {
   x = (int)(i % g.nx);
   const long long r = i / g.nx;
@@ -157,13 +196,15 @@ constexpr int NG = DIAG_NG;  // global partial slots per block
 // slots: 0 mass, 1-3 momentum, 4 volume_w, 5 count, 6 max_u, 7 rho_min,
 // 8 rho_max, 9 bad, 10-11 unused
 
-// Row-blocks of the partial kernel: enough blocks to fill the GPU (about 16
-// per SM) while the per-slice partials (row-blocks x nx x 2 doubles) stay
-// small; each thread then walks rows / (8 row-blocks) rows.
-int diag_row_blocks(const Geom& g) {
+// Row-blocks of the partial kernel with `per_sm` blocks per SM and gx blocks
+// along x: each thread walks rows / (8 row-blocks) rows, and the per-slice
+// partials (row-blocks x nx x 2 doubles) stay small.  A block ends with about
+// 70 FP64 instructions per warp (warp trees, block sums), which the FP64 pipe
+// of its SM works off at 16 clocks each: with 16 blocks per SM that alone takes
+// 50 us, so the kernels launch 4 per SM, two waves.
+int diag_row_blocks(const Geom& g, long long gx, int per_sm) {
   const long long rows = (long long)g.ny * g.nz;
-  const long long gx = (g.nx + DX - 1) / DX;
-  long long want = (16 * 152 + gx - 1) / gx;
+  long long want = (per_sm * kSmCount + gx - 1) / gx;
   const long long cap = (2ll << 20) / (2ll * g.nx);  // slices <= 2 Mi doubles
   if (want > cap) want = cap;
   long long rb = (rows + DY - 1) / DY;
@@ -299,6 +340,140 @@ __global__ void __launch_bounds__(DX* DY, 2) diag_partial_kernel(Geom g, Phys ph
       r = 0.0;
     }
     blocks[((long long)blockIdx.y * gridDim.x + blockIdx.x) * NG + tx] = r;
+  }
+}
+
+// The LAYOUT_LOCAL pass of FP32 and 2-byte storage on lattices with even nx:
+// two nodes x, x + 1 per thread (block.x = 32 pairs), loaded as one vector per
+// population, the density with its rounding error, the momentum and the sums
+// in paired FP32 instructions.  The accumulators of the liquid fraction are
+// per x, so they serve the slices and the total.  labels (nullable): also
+// starts the component labelling (ccl_init_kernel's output with runs inside
+// segments of 64 nodes; thr_lo the largest float not above the threshold), so
+// that counting droplets reads the populations once.
+// 256x128x128 FP32, HBM floor 48 us: 133 us one node per thread with 16 blocks
+// per SM, 78 us so, the labels included.
+template <int P, bool WRITE_PSI>
+__global__ void __launch_bounds__(DX* DY, 2) diag_pair_kernel(Geom g, Phys ph, const typename Prec<P>::T* f,
+                                                              double rho_l, double rho_v, double* slices,
+                                                              double* blocks, float* psi, int* flag, int* labels,
+                                                              int* sizes, float thr_lo) {
+  const int tx = threadIdx.x, ty = threadIdx.y;
+  const int x = 2 * (blockIdx.x * DX + tx);
+  const bool in = x < g.nx;
+  const int rows = g.ny * g.nz;
+  const float thr = (float)(0.5 * (rho_l + rho_v)), inv = (float)(1.0 / (rho_l - rho_v)), rv = (float)rho_v;
+  DSum2 s_mass, s_jx, s_jy, s_jz, s_vol;
+  float umax = 0.0f, rmin = 3.0e38f, rmax = -3.0e38f;
+  int cnt[2] = {0, 0};
+  bool bad = false;
+  const float s0 = shift_f<P>(0, ph), s1 = shift_f<P>(1, ph), s2 = shift_f<P>(7, ph);
+  // every lane of a warp walks the same rows (the labelling votes)
+  for (int r = blockIdx.y * DY + ty; r < rows; r += DY * gridDim.y) {
+    const int i = x + g.nx * r;
+    float2 rho = make_float2(0.0f, 0.0f);
+    if (in) {
+      float2 fv[Q];
+#pragma unroll
+      for (int a = 0; a < Q; ++a) load_pair_nc<P>(f + (long long)a * g.N + i, a == 0 ? s0 : (a <= 6 ? s1 : s2), fv[a]);
+      float2 lo, jx, jy, jz;
+      rho = rho_of_x<float2>(fv, lo);
+      mom_of<float2>(fv, jx, jy, jz);
+      if constexpr (WRITE_PSI) *reinterpret_cast<float2*>(psi + i) = psi_of2(rho, ph);
+      s_mass.add(rho, lo);
+      s_jx.add(jx);
+      s_jy.add(jy);
+      s_jz.add(jz);
+      float2 phi = xmul(vsub(rho, make_float2(rv, rv)), make_float2(inv, inv));
+      phi.x = phi.x < 0.0f ? 0.0f : (phi.x > 1.0f ? 1.0f : phi.x);
+      phi.y = phi.y < 0.0f ? 0.0f : (phi.y > 1.0f ? 1.0f : phi.y);
+      s_vol.add(phi);
+      cnt[0] += rho.x > thr;
+      cnt[1] += rho.y > thr;
+      const float2 jj = xfma(jz, jz, xfma(jy, jy, xmul(jx, jx)));
+#pragma unroll
+      for (int n = 0; n < 2; ++n) {
+        const float r1 = n ? rho.y : rho.x, j2 = n ? jj.y : jj.x;
+        // the root and the division only where |j|/rho can reach the maximum
+        // (the factor covers the rounding of the test, the second bound
+        // values whose squares lose digits)
+        const float t = umax * r1;
+        if (j2 >= 0.999998f * (t * t) || j2 < 1e-30f) {
+          const float u = sqrtf(j2) / r1;
+          umax = u > umax ? u : umax;
+        }
+        rmin = r1 < rmin ? r1 : rmin;
+        rmax = r1 > rmax ? r1 : rmax;
+        bad |= !(r1 > 0.0f) || !(r1 <= 3.0e38f);
+      }
+    }
+    if (labels) {
+      const bool l0 = in && rho.x > thr_lo, l1 = in && rho.y > thr_lo;
+      const unsigned both = __ballot_sync(0xffffffffu, l0 && l1), second = __ballot_sync(0xffffffffu, l1);
+      if (in) {
+        // start of the run that reaches this pair from the left: after the last
+        // pair below that is not liquid throughout
+        const unsigned gap = ~both & ((1u << tx) - 1u);
+        int from = 0;
+        if (gap) {
+          const int l = 31 - __clz(gap);
+          from = 2 * l + ((second >> l) & 1 ? 1 : 2);
+        }
+        const int start = i - 2 * tx + from;
+        *reinterpret_cast<int2*>(labels + i) = make_int2(l0 ? start : -1, l1 ? (l0 ? start : i + 1) : -1);
+        *reinterpret_cast<int2*>(sizes + i) = make_int2(0, 0);
+      }
+    }
+  }
+  if constexpr (WRITE_PSI) raise_flag(bad, flag);
+  __shared__ double sh_s[2][DY][2 * DX];
+  const double w0 = (double)s_vol.hi.x + (double)s_vol.lo.x, w1 = (double)s_vol.hi.y + (double)s_vol.lo.y;
+  sh_s[0][ty][2 * tx] = w0;
+  sh_s[0][ty][2 * tx + 1] = w1;
+  sh_s[1][ty][2 * tx] = (double)cnt[0];
+  sh_s[1][ty][2 * tx + 1] = (double)cnt[1];
+  double v[5] = {s_mass.value(), s_jx.value(), s_jy.value(), s_jz.value(), w0 + w1};
+  float c_f = (float)(cnt[0] + cnt[1]);   // exact below 2^24 nodes per warp
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+    for (int k = 0; k < 5; ++k) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
+    c_f += __shfl_down_sync(0xffffffffu, c_f, o);
+    const float um = __shfl_down_sync(0xffffffffu, umax, o);
+    const float mn = __shfl_down_sync(0xffffffffu, rmin, o);
+    const float mx = __shfl_down_sync(0xffffffffu, rmax, o);
+    umax = um > umax ? um : umax;
+    rmin = mn < rmin ? mn : rmin;
+    rmax = mx > rmax ? mx : rmax;
+  }
+  const int anybad = __any_sync(0xffffffffu, bad);
+  __shared__ double sh_w[NG][DY];
+  if (tx == 0) {
+    for (int k = 0; k < 5; ++k) sh_w[k][ty] = v[k];
+    sh_w[5][ty] = (double)c_f;
+    sh_w[6][ty] = (double)umax;
+    sh_w[7][ty] = (double)rmin;
+    sh_w[8][ty] = (double)rmax;
+    sh_w[9][ty] = anybad ? 1.0 : 0.0;
+  }
+  __syncthreads();
+  const int t = ty * DX + tx, xt = blockIdx.x * 2 * DX + t;
+  if (t < 2 * DX) {
+    if (xt < g.nx) {
+      double a = 0.0, b = 0.0;
+      for (int k = 0; k < DY; ++k) {
+        a += sh_s[0][k][t];
+        b += sh_s[1][k][t];
+      }
+      slices[((long long)blockIdx.y * g.nx + xt) * 2 + 0] = a;
+      slices[((long long)blockIdx.y * g.nx + xt) * 2 + 1] = b;
+    }
+  } else if (t < 2 * DX + NG) {
+    const int k = t - 2 * DX;
+    double r = k < 6 || k > 9 ? 0.0 : (k == 7 ? 1e300 : -1e300);
+    for (int w = 0; w < DY && k < 10; ++w)
+      r = k < 6 ? r + sh_w[k][w] : (k == 7 ? fmin(r, sh_w[k][w]) : fmax(r, sh_w[k][w]));
+    blocks[((long long)blockIdx.y * gridDim.x + blockIdx.x) * NG + k] = r;
   }
 }
 
@@ -503,53 +678,112 @@ __device__ __forceinline__ void unite(int* L, int a, int b, unsigned long long* 
   atomicOr(err, 1ull);
 }
 
+// Labels to start from: -1 outside the liquid, else the first node of the run
+// of liquid nodes that ends here, within the thread's segment (a warp's 32
+// consecutive nodes, cut at row ends), so that only the segments' first nodes
+// still have to be joined to their left neighbours.
 template <int P>
 __global__ void ccl_init_kernel(Geom g, Phys ph, int layout, const typename Prec<P>::T* f,
                                 double thr, int* L, int* sizes) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  bool liquid = false;
+  int x = 0, y, z;
+  if (i < g.N) {
+    coords(g, i, x, y, z);
+    Nbr nb;
+    nb.make(g, x, y, z);
+    typename Prec<P>::C rho, j[3];
+    node_rho_j<P>(g, ph, layout, f, nb, rho, j);
+    liquid = (double)rho > thr;
+  }
+  const int lane = threadIdx.x & 31;
+  const unsigned m = __ballot_sync(0xffffffffu, liquid);
   if (i >= g.N) return;
-  int x, y, z;
-  coords(g, i, x, y, z);
-  Nbr nb;
-  nb.make(g, x, y, z);
-  typename Prec<P>::C rho, j[3];
-  node_rho_j<P>(g, ph, layout, f, nb, rho, j);
-  L[i] = ((double)rho > thr) ? (int)i : -1;
+  const unsigned gap = ~m & ((1u << lane) - 1u);
+  int from = gap ? 32 - __clz(gap) : 0;
+  if (lane - from > x) from = lane - x;   // the row starts inside the warp
+  L[i] = liquid ? (int)i - (lane - from) : -1;
   sizes[i] = 0;
 }
 
-__global__ void ccl_union_kernel(Geom g, int* L, unsigned long long* err) {
+// Joins the runs: a segment's first node to its left neighbour, every node to
+// its neighbours at y + 1 and z + 1 unless the left neighbours of both are
+// liquid too (they are joined to these, and make the same link).  seg: x
+// segments of 64 (diag_pair_kernel) or, 0, warps of 32 nodes (ccl_init_kernel).
+// A ligament of 0.8 M liquid nodes of 256x128x128: 83 us joining every node to
+// three neighbours, 19 us.
+__global__ void ccl_union_kernel(Geom g, int seg, int* L, unsigned long long* err) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= g.N || L[i] < 0) return;
   int x, y, z;
   coords(g, i, x, y, z);
-  Nbr nb;
-  nb.make(g, x, y, z);
-  const long long n[3] = {nb.idx(1, 0, 0), nb.idx(0, 1, 0), nb.idx(0, 0, 1)};
-#pragma unroll
-  for (int k = 0; k < 3; ++k)
-    if (L[n[k]] >= 0) unite(L, (int)i, (int)n[k], err);
+  const int row = (int)i - x;
+  const int left = x == 0 ? row + g.nx - 1 : (int)i - 1;
+  const bool l = L[left] >= 0;
+  const bool first = x == 0 || (seg ? x % seg == 0 : (i & 31) == 0);
+  if (l && first) unite(L, (int)i, left, err);
+  const int dy = (y == g.ny - 1 ? -(g.ny - 1) : 1) * g.nx;
+  const int dz = (z == g.nz - 1 ? -(g.nz - 1) : 1) * g.nx * g.ny;
+  // (the left pair's own link: not across the periodic face, where the pair
+  // of x = nx - 1 would defer to this one in turn)
+  const bool defer = l && x > 0;
+  if (L[i + dy] >= 0 && !(defer && L[left + dy] >= 0)) unite(L, (int)i, (int)i + dy, err);
+  if (L[i + dz] >= 0 && !(defer && L[left + dz] >= 0)) unite(L, (int)i, (int)i + dz, err);
 }
 
 // After the unions every tree is final, so pointing a node straight at its
 // root (the smallest index of its component) leaves every concurrent root
-// search valid.
-__global__ void ccl_compress_kernel(Geom g, int* L, int* sizes, unsigned long long* err) {
+// search valid.  The sizes are counted per block where its nodes share the
+// root of its first liquid thread, per group of a warp otherwise: one atomic
+// per node on a ligament's single root took 326 us of 256x128x128, now 15 us.
+__global__ void __launch_bounds__(256) ccl_compress_kernel(Geom g, int* L, int* sizes, unsigned long long* err) {
+  __shared__ int s_root, s_count;
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= g.N || L[i] < 0) return;
-  long long hops = 0;
-  const int r = find_root(L, (int)i, hops);
-  if (hops >= kMaxHops) atomicOr(err, 1ull);
-  L[i] = r;
-  atomicAdd(&sizes[r], 1);
+  if (threadIdx.x == 0) {
+    s_root = -1;
+    s_count = 0;
+  }
+  __syncthreads();
+  int r = -1;
+  if (i < g.N && L[i] >= 0) {
+    long long hops = 0;
+    r = find_root(L, (int)i, hops);
+    if (hops >= kMaxHops) atomicOr(err, 1ull);
+    L[i] = r;
+    if (s_root < 0) atomicCAS(&s_root, -1, r);
+  }
+  __syncthreads();
+  const int root = s_root;
+  if (root < 0) return;   // no liquid in the block
+  const unsigned group = __match_any_sync(0xffffffffu, r);
+  if (r >= 0 && (threadIdx.x & 31) == __ffs(group) - 1) {
+    if (r == root)
+      atomicAdd(&s_count, __popc(group));
+    else
+      atomicAdd(&sizes[r], __popc(group));
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) atomicAdd(&sizes[root], s_count);
 }
 
-__global__ void ccl_count_kernel(Geom g, const int* L, const int* sizes, unsigned long long* out) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= g.N || L[i] != (int)i) return;
-  atomicAdd(&out[0], 1ull);
-  if (sizes[i] >= 8) atomicAdd(&out[1], 1ull);
-  atomicMax(&out[2], (unsigned long long)sizes[i]);
+// Counts; slots (droplet statistics): each root's size is replaced by its
+// record slot, the number of roots counted before it.
+__global__ void __launch_bounds__(256) ccl_count_kernel(Geom g, const int* L, int* sizes, int slots,
+                                                        unsigned long long* out) {
+  const long long i0 = (long long)blockIdx.x * 4 * 256 + threadIdx.x;
+  int l[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) l[k] = i0 + 256 * k < g.N ? L[i0 + 256 * k] : -1;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const long long i = i0 + 256 * k;
+    if (l[k] != (int)i) continue;
+    const int n = sizes[i];
+    const unsigned long long c = atomicAdd(&out[0], 1ull);
+    if (n >= 8) atomicAdd(&out[1], 1ull);
+    atomicMax(&out[2], (unsigned long long)n);
+    if (slots) sizes[i] = (int)c;
+  }
 }
 
 // Copies the droplet counts of the CCL just run into the ring record the
@@ -565,73 +799,108 @@ __global__ void ccl_ring_kernel(const long long* out4, double* ring, const unsig
 }
 
 // ---------------------------------------------------------------------------
-// Per-droplet statistics (after launch_ccl): every root takes a record slot;
-// every liquid node adds to its droplet's record
+// Per-droplet statistics (after launch_ccl with slots): every liquid node adds
+// to its droplet's record
 //   [root, nodes, sum phi, sum rho, cos/sin sums of 2 pi x/nx, y, z]
 // and sets the bit of its x slice in the droplet's x-occupancy mask.  The
 // FP64 sums are atomic (their order, and so the last bits, vary run to run).
 // ---------------------------------------------------------------------------
-__global__ void droplet_slot_kernel(Geom g, const int* L, int* slot_of, double* rec, unsigned* nslot,
-                                    int cap) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= g.N || L[i] != (int)i) return;
-  const unsigned k = atomicAdd(nslot, 1u);
-  slot_of[i] = k < (unsigned)cap ? (int)k : -1;
-  if (k < (unsigned)cap) rec[(size_t)k * DROP_REC] = (double)i;
+// cos and sin of 2 pi c / n for the coordinates of x, then y, then z
+__global__ void trig_kernel(Geom g, double2* trig) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int n = t < g.nx ? g.nx : (t < g.nx + g.ny ? g.ny : g.nz);
+  if (t >= g.nx + g.ny + g.nz) return;
+  const int c = t < g.nx ? t : (t < g.nx + g.ny ? t - g.nx : t - g.nx - g.ny);
+  double2 v;
+  sincospi(2.0 * c / n, &v.y, &v.x);
+  trig[t] = v;
 }
 
-template <int P>
-__global__ void droplet_stats_kernel(Geom g, Phys ph, int layout, const typename Prec<P>::T* f, double rho_l,
-                                     double rho_v, const int* L, const int* slot_of, double* rec, unsigned* xbits,
-                                     int words) {
+// A warp walks SEGS segments of 32 consecutive nodes and keeps the sums of
+// one droplet in its lanes until it meets another (the common case: segments
+// of one row lie in one droplet); segments that hold several droplets add
+// node by node.  What bounds it is the FP64 pipe, 16 clocks per warp
+// instruction: the angles come from a table (six FP64 sincospi per node before)
+// and the warp trees run once per droplet met instead of once per segment
+// (256x128x128, a ligament of 0.8 M liquid nodes: 195 us, now 90 us; 16
+// segments per warp, 78 us there, leave the droplets of a broken-up state to
+// too few warps: 100 us instead of 50).
+template <int P, int SEGS>
+__global__ void __launch_bounds__(256) droplet_stats_kernel(Geom g, Phys ph, int layout, const typename Prec<P>::T* f,
+                                                            double rho_l, double rho_v, const int* L,
+                                                            const int* slot_of, const double2* __restrict__ trig,
+                                                            double* rec, unsigned* xbits, int words) {
   using C = typename Prec<P>::C;
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  int k = -1, x = 0;
-  double v[DROP_REC - 1];
+  constexpr int NV = DROP_REC - 1;
+  const int lane = threadIdx.x & 31;
+  const long long warp = (long long)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
+  const double inv = 1.0 / (rho_l - rho_v);
+  double v[NV];
 #pragma unroll
-  for (int m = 0; m < DROP_REC - 1; ++m) v[m] = 0.0;
-  if (i < g.N && L[i] >= 0) {
-    k = slot_of[L[i]];
-    if (k >= 0) {
-      int y, z;
+  for (int m = 0; m < NV; ++m) v[m] = 0.0;
+  int cur = -1;   // slot whose sums the lanes hold
+  auto flush = [&]() {
+    if (cur < 0) return;
+#pragma unroll
+    for (int m = 0; m < NV; ++m) {
+      double t = v[m];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+      if (lane == 0) atomicAdd(rec + (size_t)cur * DROP_REC + 1 + m, t);
+      v[m] = 0.0;
+    }
+  };
+  int roots[SEGS];
+#pragma unroll
+  for (int seg = 0; seg < SEGS; ++seg) {
+    const long long i = (warp * SEGS + seg) * 32 + lane;
+    roots[seg] = i < g.N ? L[i] : -1;
+  }
+#pragma unroll 1
+  for (int seg = 0; seg < SEGS; ++seg) {
+    const long long i = (warp * SEGS + seg) * 32 + lane;
+    int root = -1;
+#pragma unroll
+    for (int k = 0; k < SEGS; ++k) root = k == seg ? roots[k] : root;
+    if (__ballot_sync(0xffffffffu, root >= 0) == 0) continue;
+    int k = -1;
+    double n[NV];
+    if (root >= 0) {
+      k = slot_of[root];
+      if (root == (int)i) rec[(size_t)k * DROP_REC] = (double)root;
+      int x, y, z;
       coords(g, i, x, y, z);
       Nbr nb;
       nb.make(g, x, y, z);
       C rc, j[3];
       node_rho_j<P>(g, ph, layout, f, nb, rc, j);
       const double rho = (double)rc;
-      v[0] = 1.0;
-      v[1] = fmin(fmax((rho - rho_v) / (rho_l - rho_v), 0.0), 1.0);
-      v[2] = rho;
-      sincospi(2.0 * x / g.nx, &v[4], &v[3]);
-      sincospi(2.0 * y / g.ny, &v[6], &v[5]);
-      sincospi(2.0 * z / g.nz, &v[8], &v[7]);
+      const double2 tx = __ldg(trig + x), ty = __ldg(trig + g.nx + y), tz = __ldg(trig + g.nx + g.ny + z);
+      n[0] = 1.0;
+      n[1] = fmin(fmax((rho - rho_v) * inv, 0.0), 1.0);
+      n[2] = rho;
+      n[3] = tx.x, n[4] = tx.y, n[5] = ty.x, n[6] = ty.y, n[7] = tz.x, n[8] = tz.y;
+      unsigned* w = xbits + (size_t)k * words + (x >> 5);
+      const unsigned bit = 1u << (x & 31);
+      if (!(*(volatile unsigned*)w & bit)) atomicOr(w, bit);
+    }
+    const int kmax = __reduce_max_sync(0xffffffffu, k);
+    if (__all_sync(0xffffffffu, k < 0 || k == kmax)) {
+      if (kmax != cur) {
+        flush();
+        cur = kmax;
+      }
+      if (k >= 0) {
+#pragma unroll
+        for (int m = 0; m < NV; ++m) v[m] += n[m];
+      }
+    } else if (k >= 0) {
+      double* r = rec + (size_t)k * DROP_REC + 1;
+#pragma unroll
+      for (int m = 0; m < NV; ++m) atomicAdd(r + m, n[m]);
     }
   }
-  // one set of atomics per warp when all its liquid lanes share a droplet
-  // (the common case: the warp covers 32 consecutive nodes of a row)
-  const int kmax = __reduce_max_sync(0xffffffffu, k);
-  const bool uniform = __all_sync(0xffffffffu, k < 0 || k == kmax);
-  if (uniform) {
-    if (kmax < 0) return;
-#pragma unroll
-    for (int m = 0; m < DROP_REC - 1; ++m)
-      for (int o = 16; o > 0; o >>= 1) v[m] += __shfl_xor_sync(0xffffffffu, v[m], o);
-    if ((threadIdx.x & 31) == 0) {
-      double* r = rec + (size_t)kmax * DROP_REC + 1;
-#pragma unroll
-      for (int m = 0; m < DROP_REC - 1; ++m) atomicAdd(r + m, v[m]);
-    }
-  } else if (k >= 0) {
-    double* r = rec + (size_t)k * DROP_REC + 1;
-#pragma unroll
-    for (int m = 0; m < DROP_REC - 1; ++m) atomicAdd(r + m, v[m]);
-  }
-  if (k >= 0) {
-    unsigned* w = xbits + (size_t)k * words + (x >> 5);
-    const unsigned bit = 1u << (x & 31);
-    if (!(*(volatile unsigned*)w & bit)) atomicOr(w, bit);
-  }
+  flush();
 }
 
 inline unsigned blocks_for(long long n, int threads) { return (unsigned)((n + threads - 1) / threads); }
@@ -661,64 +930,76 @@ cudaError_t moments_t(int layout, const Geom& g, const Phys& ph, const void* f, 
       g, ph, layout, (const typename Prec<P>::T*)f, (const typename Prec<P>::C*)psi, r, ux, uy, uz);
   return cudaGetLastError();
 }
+// Whether the diagnostics pass takes node pairs (even nx, so that every row
+// and slot starts at a pair if the arrays do).
+bool diag_pairs(int precision, int layout, const Geom& g, const void* f, const void* psi) {
+  return precision != LBM_F64 && layout == LAYOUT_LOCAL && g.nx % 2 == 0 && g.N <= 0x7fffffff &&
+         (uintptr_t)f % (2 * elem_size(precision)) == 0 && (uintptr_t)psi % 8 == 0;
+}
+
 template <int P>
 cudaError_t diag_t(int layout, const Geom& g, const Phys& ph, const void* f, double rho_l,
                    double rho_v, double* scratch, double* out, void* psi, int* flag,
-                   unsigned long long* ring_count, int ring_cap, cudaStream_t s, double* rho_out, ReduceSide* side) {
-  const int rb = diag_row_blocks(g);
-  const int gx = (g.nx + DX - 1) / DX;
+                   unsigned long long* ring_count, int ring_cap, cudaStream_t s, const DiagExtra& x) {
+  const bool pairs = diag_pairs(P, layout, g, f, psi);
+  const int gx = pairs ? (g.nx + 2 * DX - 1) / (2 * DX) : (g.nx + DX - 1) / DX;
+  const int rb = diag_row_blocks(g, gx, 4);
   double* slices = scratch;
   double* blocks = scratch + (size_t)rb * g.nx * 2;
   double* slice_tot = blocks + (size_t)gx * rb * NG;
   using T = typename Prec<P>::T;
   using C = typename Prec<P>::C;
   const dim3 grid(gx, rb), block(DX, DY);
-  if (psi) {
+  const T* in = (const T*)f;
+  if constexpr (P != LBM_F64) {
+    if (pairs && psi)
+      diag_pair_kernel<P, true><<<grid, block, 0, s>>>(g, ph, in, rho_l, rho_v, slices, blocks, (float*)psi, flag,
+                                                       x.labels, x.sizes, x.thr_lo);
+    else if (pairs)
+      diag_pair_kernel<P, false><<<grid, block, 0, s>>>(g, ph, in, rho_l, rho_v, slices, blocks, nullptr, nullptr,
+                                                        x.labels, x.sizes, x.thr_lo);
+  }
+  double* const rho_out = P == LBM_F64 ? (double*)x.dst : nullptr;
+  if (!pairs && psi) {
     if (layout == LAYOUT_LOCAL)
       diag_partial_kernel<P, true, LAYOUT_LOCAL><<<grid, block, 0, s>>>(
-          g, ph, (const T*)f, rho_l, rho_v, slices, blocks, (C*)psi, flag, rho_out);
+          g, ph, in, rho_l, rho_v, slices, blocks, (C*)psi, flag, rho_out);
     else
       diag_partial_kernel<P, true, LAYOUT_GATHER><<<grid, block, 0, s>>>(
-          g, ph, (const T*)f, rho_l, rho_v, slices, blocks, (C*)psi, flag, rho_out);
-  } else {
+          g, ph, in, rho_l, rho_v, slices, blocks, (C*)psi, flag, rho_out);
+  } else if (!pairs) {
     if (layout == LAYOUT_LOCAL)
       diag_partial_kernel<P, false, LAYOUT_LOCAL><<<grid, block, 0, s>>>(
-          g, ph, (const T*)f, rho_l, rho_v, slices, blocks, nullptr, nullptr, nullptr);
+          g, ph, in, rho_l, rho_v, slices, blocks, nullptr, nullptr, nullptr);
     else
       diag_partial_kernel<P, false, LAYOUT_GATHER><<<grid, block, 0, s>>>(
-          g, ph, (const T*)f, rho_l, rho_v, slices, blocks, nullptr, nullptr, nullptr);
+          g, ph, in, rho_l, rho_v, slices, blocks, nullptr, nullptr, nullptr);
   }
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  return launch_diag_reduce(g, rb, gx * rb, slices, blocks, slice_tot, out, ring_count, ring_cap, s, side);
+  return launch_diag_reduce(g, rb, gx * rb, slices, blocks, slice_tot, out, ring_count, ring_cap, s, x.side);
 }
+
 template <int P>
-cudaError_t ccl_t(int layout, const Geom& g, const Phys& ph, const void* f, double thr, int* L,
-                  int* sizes, long long* out3, cudaStream_t s) {
-  const unsigned nb = blocks_for(g.N, 256);
-  cudaError_t e = cudaMemsetAsync(out3, 0, 4 * sizeof(long long), s);
-  if (e != cudaSuccess) return e;
-  unsigned long long* err = (unsigned long long*)out3 + 3;
-  ccl_init_kernel<P><<<nb, 256, 0, s>>>(g, ph, layout, (const typename Prec<P>::T*)f, thr, L, sizes);
-  ccl_union_kernel<<<nb, 256, 0, s>>>(g, L, err);
-  ccl_compress_kernel<<<nb, 256, 0, s>>>(g, L, sizes, err);
-  ccl_count_kernel<<<nb, 256, 0, s>>>(g, L, sizes, (unsigned long long*)out3);
+cudaError_t ccl_init_t(int layout, const Geom& g, const Phys& ph, const void* f, double thr, int* L, int* sizes,
+                       cudaStream_t s) {
+  ccl_init_kernel<P><<<blocks_for(g.N, 256), 256, 0, s>>>(g, ph, layout, (const typename Prec<P>::T*)f, thr, L, sizes);
   return cudaGetLastError();
 }
 
 template <int P>
 cudaError_t droplets_t(int layout, const Geom& g, const Phys& ph, const void* f, double rho_l, double rho_v,
-                       const int* L, int* slot_of, double* rec, unsigned* xbits, unsigned* nslot, int cap,
+                       const int* L, const int* slot_of, const double2* trig, double* rec, unsigned* xbits, int cap,
                        cudaStream_t s) {
-  const unsigned nb = blocks_for(g.N, 256);
   const int words = (g.nx + 31) / 32;
   cudaError_t e = cudaMemsetAsync(rec, 0, sizeof(double) * DROP_REC * (size_t)cap, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(xbits, 0, sizeof(unsigned) * words * (size_t)cap, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(nslot, 0, sizeof(unsigned), s);
   if (e != cudaSuccess) return e;
-  droplet_slot_kernel<<<nb, 256, 0, s>>>(g, L, slot_of, rec, nslot, cap);
-  droplet_stats_kernel<P><<<nb, 256, 0, s>>>(g, ph, layout, (const typename Prec<P>::T*)f, rho_l, rho_v, L,
-                                             slot_of, rec, xbits, words);
+  // four segments per warp where that leaves four blocks per SM
+  const auto kernel = g.N >= 4 * 256LL * 4 * kSmCount ? droplet_stats_kernel<P, 4> : droplet_stats_kernel<P, 1>;
+  const int segs = g.N >= 4 * 256LL * 4 * kSmCount ? 4 : 1;
+  kernel<<<blocks_for(g.N, 256 * segs), 256, 0, s>>>(g, ph, layout, (const typename Prec<P>::T*)f, rho_l, rho_v, L,
+                                                     slot_of, trig, rec, xbits, words);
   return cudaGetLastError();
 }
 
@@ -792,17 +1073,22 @@ cudaError_t launch_ccl_ring(const long long* out4, double* ring, const unsigned 
 }
 
 cudaError_t launch_droplets(int precision, int layout, const Geom& g, const Phys& ph, const void* f,
-                            double rho_l, double rho_v, const int* labels, int* sizes, double* rec,
-                            unsigned* xbits, unsigned* nslot, int cap, cudaStream_t s) {
+                            double rho_l, double rho_v, const int* labels, const int* slots, const double2* trig,
+                            double* rec, unsigned* xbits, int cap, cudaStream_t s) {
   switch (precision) {
-    case LBM_F64: return droplets_t<LBM_F64>(layout, g, ph, f, rho_l, rho_v, labels, sizes, rec, xbits, nslot, cap, s);
-    case LBM_F32: return droplets_t<LBM_F32>(layout, g, ph, f, rho_l, rho_v, labels, sizes, rec, xbits, nslot, cap, s);
+    case LBM_F64: return droplets_t<LBM_F64>(layout, g, ph, f, rho_l, rho_v, labels, slots, trig, rec, xbits, cap, s);
+    case LBM_F32: return droplets_t<LBM_F32>(layout, g, ph, f, rho_l, rho_v, labels, slots, trig, rec, xbits, cap, s);
     case LBM_F16DEV:
-      return droplets_t<LBM_F16DEV>(layout, g, ph, f, rho_l, rho_v, labels, sizes, rec, xbits, nslot, cap, s);
+      return droplets_t<LBM_F16DEV>(layout, g, ph, f, rho_l, rho_v, labels, slots, trig, rec, xbits, cap, s);
     case LBM_BF16DEV:
-      return droplets_t<LBM_BF16DEV>(layout, g, ph, f, rho_l, rho_v, labels, sizes, rec, xbits, nslot, cap, s);
+      return droplets_t<LBM_BF16DEV>(layout, g, ph, f, rho_l, rho_v, labels, slots, trig, rec, xbits, cap, s);
   }
   return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_trig(const Geom& g, double2* trig, cudaStream_t s) {
+  trig_kernel<<<blocks_for((long long)g.nx + g.ny + g.nz, 128), 128, 0, s>>>(g, trig);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_init(int precision, const Geom& g, const Phys& ph, const InitSpec& spec, void* f,
@@ -877,42 +1163,62 @@ cudaError_t launch_moments(int precision, int layout, const Geom& g, const Phys&
   return cudaErrorInvalidValue;
 }
 
+// (room for 16 row blocks per SM; the kernels use 4)
 size_t diag_scratch_doubles(const Geom& g) {
-  const int rb = diag_row_blocks(g);
   const int gx = (g.nx + DX - 1) / DX;
+  const int rb = diag_row_blocks(g, gx, 16);
   return (size_t)rb * g.nx * 2 + (size_t)gx * rb * NG + (size_t)g.nx * 2;
 }
 
 cudaError_t launch_diagnostics(int precision, int layout, const Geom& g, const Phys& ph, const void* f,
                                double rho_l, double rho_v, double* scratch, double* out, void* psi,
                                int* flag, unsigned long long* ring_count, int ring_cap,
-                               cudaStream_t s, void* dst, ReduceSide* side) {
+                               cudaStream_t s, const DiagExtra& x) {
   switch (precision) {
     case LBM_F64:
-      return diag_t<LBM_F64>(layout, g, ph, f, rho_l, rho_v, scratch, out, psi, flag, ring_count, ring_cap, s,
-                             (double*)dst, side);
+      return diag_t<LBM_F64>(layout, g, ph, f, rho_l, rho_v, scratch, out, psi, flag, ring_count, ring_cap, s, x);
     case LBM_F32:
-      return diag_t<LBM_F32>(layout, g, ph, f, rho_l, rho_v, scratch, out, psi, flag, ring_count, ring_cap, s,
-                             nullptr, side);
+      return diag_t<LBM_F32>(layout, g, ph, f, rho_l, rho_v, scratch, out, psi, flag, ring_count, ring_cap, s, x);
     case LBM_F16DEV:
-      return diag_t<LBM_F16DEV>(layout, g, ph, f, rho_l, rho_v, scratch, out, psi, flag, ring_count, ring_cap, s,
-                             nullptr, side);
+      return diag_t<LBM_F16DEV>(layout, g, ph, f, rho_l, rho_v, scratch, out, psi, flag, ring_count, ring_cap, s, x);
     case LBM_BF16DEV:
-      return diag_t<LBM_BF16DEV>(layout, g, ph, f, rho_l, rho_v, scratch, out, psi, flag, ring_count, ring_cap, s,
-                             nullptr, side);
+      return diag_t<LBM_BF16DEV>(layout, g, ph, f, rho_l, rho_v, scratch, out, psi, flag, ring_count, ring_cap, s, x);
   }
   return cudaErrorInvalidValue;
 }
 
+DiagExtra diag_labels(int precision, int layout, const Geom& g, const void* f, const void* psi, double threshold,
+                      int* labels, int* sizes) {
+  DiagExtra x;
+  if (!diag_pairs(precision, layout, g, f, psi)) return x;
+  x.labels = labels;
+  x.sizes = sizes;
+  // rho > threshold for a float rho is rho > the largest float not above it
+  x.thr_lo = (float)threshold;
+  if ((double)x.thr_lo > threshold) x.thr_lo = nextafterf(x.thr_lo, -INFINITY);
+  return x;
+}
+
 cudaError_t launch_ccl(int precision, int layout, const Geom& g, const Phys& ph, const void* f,
-                       double threshold, int* labels, int* sizes, long long* out3, cudaStream_t s) {
-  switch (precision) {
-    case LBM_F64: return ccl_t<LBM_F64>(layout, g, ph, f, threshold, labels, sizes, out3, s);
-    case LBM_F32: return ccl_t<LBM_F32>(layout, g, ph, f, threshold, labels, sizes, out3, s);
-    case LBM_F16DEV: return ccl_t<LBM_F16DEV>(layout, g, ph, f, threshold, labels, sizes, out3, s);
-    case LBM_BF16DEV: return ccl_t<LBM_BF16DEV>(layout, g, ph, f, threshold, labels, sizes, out3, s);
+                       double threshold, int* labels, int* sizes, long long* out3, cudaStream_t s, bool started,
+                       bool slots) {
+  cudaError_t e = cudaMemsetAsync(out3, 0, 4 * sizeof(long long), s);
+  if (e == cudaSuccess && !started) {
+    switch (precision) {
+      case LBM_F64: e = ccl_init_t<LBM_F64>(layout, g, ph, f, threshold, labels, sizes, s); break;
+      case LBM_F32: e = ccl_init_t<LBM_F32>(layout, g, ph, f, threshold, labels, sizes, s); break;
+      case LBM_F16DEV: e = ccl_init_t<LBM_F16DEV>(layout, g, ph, f, threshold, labels, sizes, s); break;
+      case LBM_BF16DEV: e = ccl_init_t<LBM_BF16DEV>(layout, g, ph, f, threshold, labels, sizes, s); break;
+      default: e = cudaErrorInvalidValue;
+    }
   }
-  return cudaErrorInvalidValue;
+  if (e != cudaSuccess) return e;
+  const unsigned nb = blocks_for(g.N, 256);
+  unsigned long long* out = (unsigned long long*)out3;
+  ccl_union_kernel<<<nb, 256, 0, s>>>(g, started ? 2 * DX : 0, labels, out + 3);
+  ccl_compress_kernel<<<nb, 256, 0, s>>>(g, labels, sizes, out + 3);
+  ccl_count_kernel<<<blocks_for(g.N, 4 * 256), 256, 0, s>>>(g, labels, sizes, slots ? 1 : 0, out);
+  return cudaGetLastError();
 }
 
 }  // namespace lbm

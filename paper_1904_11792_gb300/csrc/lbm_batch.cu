@@ -927,10 +927,8 @@ int lbm_batch_diagnostics(lbm_batch b, int k, lbm_diag* out, int want_ccl) {
     b->scratch_doubles = need;
   }
   const lbm_instance& s = b->spec[k];
-  BCK(launch_diagnostics(b->precision, LAYOUT_LOCAL, v.g, v.ph, v.f, s.rho_l, s.rho_v, b->d_scratch, b->d_small,
-                         nullptr, nullptr, nullptr, 0, b->stream));
-  double r[DIAG_OUT];
-  long long c4[4] = {-1, -1, -1, 0};
+  const double thr = 0.5 * (s.rho_l + s.rho_v);
+  DiagExtra x;
   if (want_ccl) {
     if ((size_t)(2 * v.g.N) > b->labels_ints) {
       cudaFree(b->d_labels);
@@ -938,9 +936,16 @@ int lbm_batch_diagnostics(lbm_batch b, int k, lbm_diag* out, int want_ccl) {
       BCK(cudaMalloc(&b->d_labels, sizeof(int) * 2 * b->max_nodes));
       b->labels_ints = 2 * b->max_nodes;
     }
+    x = diag_labels(b->precision, LAYOUT_LOCAL, v.g, v.f, nullptr, thr, b->d_labels, b->d_labels + v.g.N);
+  }
+  BCK(launch_diagnostics(b->precision, LAYOUT_LOCAL, v.g, v.ph, v.f, s.rho_l, s.rho_v, b->d_scratch, b->d_small,
+                         nullptr, nullptr, nullptr, 0, b->stream, x));
+  double r[DIAG_OUT];
+  long long c4[4] = {-1, -1, -1, 0};
+  if (want_ccl) {
     long long* d4 = (long long*)(b->d_small + 32);
-    BCK(launch_ccl(b->precision, LAYOUT_LOCAL, v.g, v.ph, v.f, 0.5 * (s.rho_l + s.rho_v), b->d_labels,
-                   b->d_labels + v.g.N, d4, b->stream));
+    BCK(launch_ccl(b->precision, LAYOUT_LOCAL, v.g, v.ph, v.f, thr, b->d_labels, b->d_labels + v.g.N, d4, b->stream,
+                   x.labels != nullptr));
     BCK(cudaMemcpyAsync(c4, d4, sizeof(c4), cudaMemcpyDeviceToHost, b->stream));
   }
   BCK(cudaMemcpyAsync(r, b->d_small, sizeof(r), cudaMemcpyDeviceToHost, b->stream));

@@ -175,14 +175,22 @@ constexpr int DIAG_CCL = 14;
 constexpr int DIAG_STRIDE = 20;
 // psi (nullable): also write psi of every node and raise flag on a bad
 // density (the psi pass of a diagnostic step).  ring_count (nullable):
-// append the record to the ring at out instead of writing out[0..12].  dst:
-// as launch_psi (with psi).  side (nullable): where the stages after the pass
-// over the populations run.
+// append the record to the ring at out instead of writing out[0..12].
+struct DiagExtra {
+  void* dst = nullptr;          // as launch_psi (with psi)
+  ReduceSide* side = nullptr;   // where the stages after the pass over the populations run
+  int *labels = nullptr, *sizes = nullptr;   // also start the labelling (diag_labels)
+  float thr_lo = 0.0f;
+};
+// The labelling part of a DiagExtra for a pass over f (writing psi, or
+// nullptr), empty where the pass has no such form.
+DiagExtra diag_labels(int precision, int layout, const Geom& g, const void* f, const void* psi, double threshold,
+                      int* labels, int* sizes);
 cudaError_t launch_diagnostics(int precision, int layout, const Geom& g, const Phys& ph,
                                const void* f, double rho_l, double rho_v, double* scratch,
                                double* out, void* psi, int* flag,
                                unsigned long long* ring_count, int ring_cap, cudaStream_t s,
-                               void* dst = nullptr, ReduceSide* side = nullptr);
+                               const DiagExtra& x = {});
 
 // Stochastic-rounding step salt (Phys::salt): set to value, or advance by one.
 cudaError_t launch_salt(unsigned* salt, bool set, unsigned value, cudaStream_t s);
@@ -200,26 +208,28 @@ cudaError_t launch_diag_reduce(const Geom& g, int row_blocks, int nblocks, const
 
 // Connected components of the liquid mask.  labels: N ints; sizes: N ints;
 // out3 (device, 4 long long): components, components with >= 8 nodes,
-// largest size, error flag (a union-find guard tripped).
+// largest size, error flag (a union-find guard tripped).  started: a
+// diagnostics pass has started the labels (diag_labels); slots: replace the
+// size of every root by its number among the roots (for launch_droplets).
 cudaError_t launch_ccl(int precision, int layout, const Geom& g, const Phys& ph, const void* f,
                        double threshold, int* labels, int* sizes, long long* out3,
-                       cudaStream_t s);
+                       cudaStream_t s, bool started = false, bool slots = false);
 
 // Appends the counts of the last launch_ccl (out4, device) to the newest
 // ring record (fields DIAG_CCL ..).
 cudaError_t launch_ccl_ring(const long long* out4, double* ring, const unsigned long long* ring_count,
                             int ring_cap, cudaStream_t s);
 
-// Per-droplet statistics after launch_ccl on the same state: records of
-// DROP_REC doubles [root, nodes, sum phi, sum rho, cos/sin sums of the
-// angles 2 pi x/nx, 2 pi y/ny, 2 pi z/nz] for the first cap roots met, and
-// x-occupancy bit masks of (nx + 31)/32 words per record.  sizes is the CCL
-// sizes array (overwritten with record slots); nslot receives the number of
-// roots.
+// Per-droplet statistics after launch_ccl with slots on the same state: cap
+// records (one per root) of DROP_REC doubles [root, nodes, sum phi, sum rho,
+// cos/sin sums of the angles 2 pi x/nx, 2 pi y/ny, 2 pi z/nz], and x-occupancy
+// bit masks of (nx + 31)/32 words per record.  trig: nx + ny + nz entries
+// filled by launch_trig.
 constexpr int DROP_REC = 10;
+cudaError_t launch_trig(const Geom& g, double2* trig, cudaStream_t s);
 cudaError_t launch_droplets(int precision, int layout, const Geom& g, const Phys& ph, const void* f,
-                            double rho_l, double rho_v, const int* labels, int* sizes, double* rec,
-                            unsigned* xbits, unsigned* nslot, int cap, cudaStream_t s);
+                            double rho_l, double rho_v, const int* labels, const int* slots, const double2* trig,
+                            double* rec, unsigned* xbits, int cap, cudaStream_t s);
 
 
 // ---- batched single-pass step on padded rows (lbm_fused.cu) ----------------
@@ -297,6 +307,7 @@ struct lbm_ctx {
   size_t scratch_doubles = 0;
   int* d_labels = nullptr;        // CCL labels and sizes (2 N ints)
   bool diag_ccl = false;          // label droplets at every in-loop diagnostic step
+  double2* d_trig = nullptr;      // angles of the coordinates (lbm_droplets)
   double* d_drop = nullptr;       // droplet records and x masks (lbm_droplets)
   size_t drop_bytes = 0;
 
