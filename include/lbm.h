@@ -165,6 +165,8 @@ int lbm_set_stream(lbm_handle h, void *stream);
  * in-loop diagnostics on diagnostic steps; applies to FP32,
  * FP16-dev and BF16-dev storage when nx % 64 == 0 and ny % 4 == 0 (FP32) or
  * ny % 8 == 0 (2-byte storage); lbm_get_option answers whether it applies.
+ * Until the option (or "fused_fz" or "fused_group") is set, lattices of at most
+ * 2^18 nodes take the two-kernel step all the same, which is faster there.
  * Of the other lattices of these storage forms, larger ones (more than 1 M
  * nodes in FP32, 2.6 M in 2-byte storage, nx >= 32; with the value 2 all of
  * them) run plain steps as a single pass on tiles cut at their edges: every

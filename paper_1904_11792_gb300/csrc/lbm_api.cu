@@ -179,6 +179,13 @@ int auto_minb(bool vec, int mode, int precision) {
 
 bool ragged_direct(const lbm_ctx* h);
 
+// Whether steps run as the fused single pass: small lattices only when asked
+// for (option "fused", or one of its launch shape or test hook).
+bool fused_form(const lbm_ctx* h) {
+  return h->fused && h->cfg.pattern == LBM_AB && fused_applicable(h->g, h->cfg.precision) &&
+         (h->fused > 0 || h->g.N > kFusedNodes || h->fused_fz || h->fused_group || h->fused_stall_test_ns);
+}
+
 // The psi pass of a diagnostic step of the two kernels: with the diagnostics,
 // and the droplet counts where they are on.
 int enqueue_diagnostics(lbm_ctx* h, cudaStream_t s, const Geom& g, int layout, const void* src, void* dst,
@@ -212,7 +219,7 @@ int enqueue_step(lbm_ctx* h, cudaStream_t s, long long step, int cur, bool timed
   const int mode = aa ? ((step & 1) ? MODE_AA_ODD : MODE_AA_EVEN) : MODE_AB;
   cudaEvent_t e0 = nullptr, e1 = nullptr, e2 = nullptr;
   const bool diag_step = h->diag_interval > 0 && step % h->diag_interval == 0;
-  const bool fused = h->fused && !aa && fused_applicable(h->g, prec);
+  const bool fused = fused_form(h);
   Geom g = h->g;
   if (h->diag_ccl) side = nullptr;   // the labelling appends to the record of its own step
   if (side && side->open && diag_step) {

@@ -66,6 +66,14 @@ cudaError_t launch_collide(int precision, int mode, int minb, bool vec, const Ge
 cudaError_t launch_collide_padded(int precision, const Geom& g, const Phys& ph, const void* src, void* dst, int px,
                                   const void* psi, dim3 block, cudaStream_t s);
 
+// Lattices up to this many nodes run the two kernels by default where the
+// fused step applies: their populations stay in L2, and two short passes over
+// all nodes at once beat a march through planes by few blocks (chained,
+// plain steps: 64x32x32 FP32 5.57 against 7.76 us, FP16 4.96 / 10.44;
+// 128x32x32 6.52 / 8.01, 6.23 / 10.57; 64x64x64 9.16 / 12.91, 9.29 / 10.59;
+// but 128x48x48 9.91 / 13.28, FP16 11.47 / 10.83; 192x48x48 14.17 / 13.55,
+// 14.99 / 14.94).
+constexpr long long kFusedNodes = 1 << 18;
 // Lattices up to this many nodes launch their steps chained (lbm_launch.cuh)
 // and replay longer graphs: their kernels take a few microseconds each.
 constexpr long long kChainNodes = 1 << 20;
@@ -320,7 +328,10 @@ struct lbm_ctx {
   bool block_asked = false;       // block was given (else auto_block is launched)
   int minb = 0;                   // collide kernel register budget variant (0 = auto)
   bool vec = true;                // two nodes per thread (when nx is even)
-  int fused = 1;                  // single-pass A-B steps: 0 never, 1 where they apply and pay, 2 where they apply
+  // single-pass A-B steps: -1 (until the option is set) where they apply and
+  // pay, 0 never, 1 the 64-wide tiles where they apply and cut tiles where
+  // they pay, 2 both where they apply
+  int fused = -1;
   int fused_fz = 0;               // z planes per block of the fused step (0 = automatic)
   int fused_group = 0;            // z runs per group of its block order (0 = automatic)
   unsigned long long fused_stall_test_ns = 0;   // test hook of the fused step's timeout path

@@ -134,3 +134,21 @@ def test_diag_history_across_the_ring_end(L):
         d = lat.diagnostics()
     assert [r["step"] for r in a + b] == list(range(1100)) and [r["step"] for r in c] == list(range(1123, 1130))
     assert all(abs(r["mass"] / d["mass"] - 1) < 1e-11 for r in a + b + c)
+
+
+@pytest.mark.parametrize("precision", ["f32", "f16dev"])
+def test_small_lattices_take_the_two_kernels_until_asked(L, precision):
+    shape, f0 = (64, 8, 12), lbm_inputs.random_populations(64, 8, 12, seed=75)
+    out = []
+    for option in (None, ("fused", 1), ("fused_fz", 4), ("fused_group", 1)):
+        with L.Lattice(*shape, 0.9, -5.5, precision=precision, rho_ref=0.1) as lat:
+            assert lat.get_option("fused") == 1
+            if option:
+                lat.set_option(*option)
+            lat.set_option("kernel_timing", 1)
+            lat.set_populations(f0)
+            lat.step(3)
+            assert [L.lbm_kernel_time(lat.h, k)[0] for k in range(3)] == ([0, 0, 3] if option else [3, 3, 0])
+            out.append(lat.populations())
+    for f in out[1:]:
+        np.testing.assert_array_equal(out[0], f)
