@@ -168,13 +168,15 @@ int salt_word(const lbm_ctx* h, long long step, int cur) {
 // and stores: no spills at 80 registers); for the AA odd step's two-node
 // kernel 3 with 2-byte storage (6.93 ms per FP16 AA step against 7.65 with
 // 2, although it spills a little at 80 registers) and 2 otherwise (FP32:
-// 9.11 ms against 9.84); 2 for the A-B step's two-node kernel (no spills at
-// <= 128 registers).
-int auto_minb(bool vec, int mode, int precision) {
+// 9.11 ms against 9.84); for the A-B step's two-node kernel 3 with 2-byte
+// storage (512x256x256 FP16: 780 us per step against 885 with 2) but on
+// lattices of a few thousand warps (64x64x64: 9.9 against 9.0 us), and 2
+// otherwise (no spills at <= 128 registers).
+int auto_minb(bool vec, int mode, int precision, long long N) {
   if (precision == LBM_F64) return 2;   // 988 us per launch on 256x128x128 against 1013 with 3 (spills)
   if (!vec || mode == MODE_AA_EVEN) return 3;
-  if (mode == MODE_AA_ODD && (precision == LBM_F16DEV || precision == LBM_BF16DEV)) return 3;
-  return 2;
+  if (precision != LBM_F16DEV && precision != LBM_BF16DEV) return 2;
+  return mode == MODE_AA_ODD || N > kFusedNodes ? 3 : 2;
 }
 
 bool ragged_direct(const lbm_ctx* h);
@@ -292,7 +294,7 @@ int enqueue_step(lbm_ctx* h, cudaStream_t s, long long step, int cur, bool timed
   }
   if (timed) CK(cudaEventRecord(e1, s));
   const bool vec = node_pairs(prec, h->vec, h->g);
-  const int minb = h->minb ? h->minb : auto_minb(vec, mode, prec);
+  const int minb = h->minb ? h->minb : auto_minb(vec, mode, prec, h->g.N);
   const dim3 block = h->block_asked ? h->block : auto_block(h->g, vec);
   if (h->ph.coll == COLL_MRT)
     CK(launch_collide_mrt(prec, mode, vec, g, ph, src, dst, h->psi, block, s));
@@ -867,7 +869,7 @@ int lbm_get_option(lbm_handle h, const char* key, double* v) {
   else if (k == "occupancy")
     *v = h->minb ? h->minb
                  : auto_minb(node_pairs(h->cfg.precision, h->vec, h->g), h->cfg.pattern == LBM_AA ? MODE_AA_ODD : MODE_AB,
-                             h->cfg.precision);
+                             h->cfg.precision, h->g.N);
   else if (k == "vector") *v = h->vec && (h->g.nx % 2 == 0);
   else if (k == "stochastic_rounding") *v = h->ph.sr;
   else if (k == "fused")

@@ -60,12 +60,13 @@ __device__ __forceinline__ unsigned mix32(unsigned h) {
 // (a per-step counter; without it a node whose state no longer changes would
 // round the same way every step and its rounding error would grow linearly
 // in time instead of averaging out).
-__device__ __forceinline__ unsigned sr_seed(long long node, float rest, unsigned salt) {
-  return mix32((unsigned)node * 0x9E3779B9u ^ (unsigned)(node >> 32) ^ __float_as_uint(rest) ^
-               mix32(salt + 0x6A09E667u));
+// sr_salt: the salt's part, the same for every node.
+__device__ __forceinline__ unsigned sr_salt(unsigned salt) { return mix32(salt + 0x6A09E667u); }
+__device__ __forceinline__ unsigned sr_seed(int node, float rest, unsigned mixed_salt) {
+  return mix32((unsigned)node * 0x9E3779B9u ^ __float_as_uint(rest) ^ mixed_salt);
 }
-__device__ __forceinline__ unsigned sr_seed(long long node, double rest, unsigned salt) {
-  return sr_seed(node, (float)rest, salt);
+__device__ __forceinline__ unsigned sr_seed(int node, double rest, unsigned mixed_salt) {
+  return sr_seed(node, (float)rest, mixed_salt);
 }
 // 32 random bits shared by the opposite directions 2j - 1 and 2j of a node
 // with (well mixed) seed s (j = 1..9; j = 0: the rest population).  The
@@ -84,6 +85,22 @@ __device__ __forceinline__ unsigned sr_word(unsigned s, int j) {
 __device__ __forceinline__ unsigned sr_bits(unsigned s, int a) {
   const unsigned w = sr_word(s, (a + 1) >> 1);
   return (a == 0 || (a & 1)) ? w >> 16 : w & 0xFFFFu;
+}
+// The bits of pair j for the neighbours x and x + 1 (seeds s0 and s1) at once,
+// as a conversion of both nodes takes them (low half node x, high half x + 1):
+// odd for direction 2j - 1 (or the rest population), even for 2j.  The high
+// halves of both products in one byte permutation, the low halves in another,
+// xored with the first: five instructions for four values.
+struct SrPair {
+  unsigned odd, even;
+};
+__device__ __forceinline__ SrPair sr_pair(unsigned s0, unsigned s1, int j) {
+  const unsigned k = 0x9E3779B1u + 0x6A09E668u * (unsigned)j;
+  const unsigned w0 = s0 * k, w1 = s1 * k;
+  SrPair r;
+  r.odd = __byte_perm(w0, w1, 0x7632);
+  r.even = __byte_perm(w0, w1, 0x5410) ^ r.odd;
+  return r;
 }
 // Stochastic rounding by the conversion instruction (cvt.rs, sm_100 and
 // later): two FP32 values to a packed FP16 / BF16 pair, each rounded up with

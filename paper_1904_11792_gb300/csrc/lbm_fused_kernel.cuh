@@ -351,7 +351,7 @@ __device__ __forceinline__ void fused_body(const Maps& maps, const Geom& g, cons
 
   // the step's stochastic-rounding salt (SALT_GIVEN: by the caller, which
   // runs several steps in one launch)
-  const unsigned salt = (Prec<P>::dev && ph.sr) ? (SALT_GIVEN ? salt_given : salt_of(ph)) : 0u;
+  const unsigned salt = (Prec<P>::dev && ph.sr) ? sr_salt(SALT_GIVEN ? salt_given : salt_of(ph)) : 0u;
   // a non-positive or non-finite density met by this thread's psi
   // evaluations (raised on the flag once, after the run: the host reads the
   // flag only after the kernel)
@@ -517,48 +517,36 @@ __device__ __forceinline__ void fused_body(const Maps& maps, const Geom& g, cons
       const int i0 = x + g.nx * (y + g.ny * z);
       const bool sr = Prec<P>::dev && ph.sr;
       const unsigned seed0 = sr ? sr_seed(i0, fs0[0], salt) : 0u, seed1 = sr ? sr_seed(i0 + 1, fs1[0], salt) : 0u;
+      SrPair r{0u, 0u};
 #pragma unroll
       for (int a = 0; a < Q; ++a) {
         const C sh = a == 0 ? s0 : (a <= 6 ? s1 : s2);
         const int row = rowp * (yv[1 + cy(a)] + g.ny * zv[1 + cz(a)]);
         if constexpr (Prec<P>::dev) {
           T* const base = TABLE ? s_dir[a] : db->p[a];
-          // the shift comes off both nodes in one paired difference
-          const float2 sh2 = splat<float2>(sh);
+          if (sr && (a == 0 || (a & 1))) r = sr_pair(seed0, seed1, (a + 1) >> 1);
           if (cx(a) == 0) {
             if (ODD || (BATCH && !act1)) {
               store_pop<P>(ph, base + (row + x), fs0[a], sh, seed0, a);   // alone: its bits as in the pair
               if (ODD && act1) store_pop<P>(ph, base + (row + x + 1), fs1[a], sh, seed1, a);
             } else if (sr) {
-              const float2 d = vsub(make_float2(fs0[a], fs1[a]), sh2);   // node x low, x + 1 high
               *reinterpret_cast<unsigned*>(base + (row + x)) =
-                  cvt_pair_sr<P>(d.y, d.x, (sr_bits(seed1, a) << 16) | (sr_bits(seed0, a) & 0xFFFFu));
+                  round_pair_sr<P>(make_float2(fs0[a], fs1[a]), sh, a == 0 || (a & 1) ? r.odd : r.even);
             } else {
               store_pair<P>(base + (row + x), fs0[a], fs1[a], sh);
             }
           } else if (!sr) {
             store_pop<P>(ph, base + (row + (cx(a) > 0 ? xr0 : xm)), fs0[a], sh, seed0, a);
             if (act1) store_pop<P>(ph, base + (row + (cx(a) > 0 ? xp : x)), fs1[a], sh, seed1, a);
-          } else if (a & 1) {
-            // a and its opposite a + 1 (c_x != 0, the same weight and shift):
-            // one conversion per node rounds both with the bits sr_bits gives
-            // them (the high half a, the low half a + 1), so the stored values
-            // equal those of the one-value conversions of the two-kernel step
-            T* const base_b = TABLE ? s_dir[a + 1] : db->p[a + 1];
-            const int row_b = rowp * (yv[1 + cy(a + 1)] + g.ny * zv[1 + cz(a + 1)]);
-            const unsigned j = (unsigned)(a + 1) >> 1;
-            const float2 da = vsub(make_float2(fs0[a], fs1[a]), sh2);
-            const float2 db = vsub(make_float2(fs0[a + 1], fs1[a + 1]), sh2);
-            const unsigned d0 = cvt_pair_sr<P>(da.x, db.x, sr_word(seed0, j));
-            const unsigned d1 = cvt_pair_sr<P>(da.y, db.y, sr_word(seed1, j));
+          } else {
+            // one conversion rounds both nodes (the bits of the one-value
+            // conversions of the two-kernel step), stored one by one
+            const unsigned d =
+                round_pair_sr<P>(make_float2(fs0[a], fs1[a]), sh, (a & 1) ? r.odd : r.even);
             unsigned short* const pa = reinterpret_cast<unsigned short*>(base + row);
-            unsigned short* const pb = reinterpret_cast<unsigned short*>(base_b + row_b);
-            pa[cx(a) > 0 ? xr0 : xm] = (unsigned short)(d0 >> 16);
-            if (act1) pa[cx(a) > 0 ? xp : x] = (unsigned short)(d1 >> 16);
-            pb[cx(a + 1) > 0 ? xr0 : xm] = (unsigned short)d0;
-            if (act1) pb[cx(a + 1) > 0 ? xp : x] = (unsigned short)d1;
+            pa[cx(a) > 0 ? xr0 : xm] = (unsigned short)d;
+            if (act1) pa[cx(a) > 0 ? xp : x] = (unsigned short)(d >> 16);
           }
-          // even a with c_x != 0 under stochastic rounding: stored with a - 1
         } else {
           T* base = (TABLE ? dst + (long long)a * N : db->p[a]) + row;
           if (cx(a) == 0) {

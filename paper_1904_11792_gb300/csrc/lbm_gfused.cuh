@@ -243,7 +243,7 @@ __device__ __forceinline__ void gfused_item(const GInst* __restrict__ inst, int 
         collide_math_r<C>(ph, fp, prho, pc, pn, fs);
       }
       const int i = x + g.nx * (y + g.ny * z);
-      const unsigned seed = (Prec<P>::dev && ph.sr) ? sr_seed(i, fs[0], salt) : 0u;
+      const unsigned seed = (Prec<P>::dev && ph.sr) ? sr_seed(i, fs[0], sr_salt(salt)) : 0u;
       // destination offsets: x + row of y + plane of z, and a N
       const int pz[3] = {plane_n * zv[0], plane_n * zv[1], plane_n * zv[2]};
 #pragma unroll

@@ -40,7 +40,6 @@ template <> struct Pair<LBM_F32> {
   using V = float2;
   __device__ static __forceinline__ void unpack(V v, float& a, float& b) { a = v.x; b = v.y; }
   __device__ static __forceinline__ V pack(float a, float b) { return make_float2(a, b); }
-  __device__ static __forceinline__ V pack_sr(float a, float b, unsigned, unsigned) { return make_float2(a, b); }
 };
 template <> struct Pair<LBM_F16DEV> {
   using V = __half2;
@@ -51,12 +50,6 @@ template <> struct Pair<LBM_F16DEV> {
   __device__ static __forceinline__ V pack(float a, float b) {
     return __halves2half2(__float2half_rn(a), __float2half_rn(b));
   }
-  __device__ static __forceinline__ V pack_sr(float a, float b, unsigned ra, unsigned rb) {
-    const unsigned d = cvt_rs_f16x2(b, a, (rb << 16) | (ra & 0xFFFFu));   // x + 1 high, x low
-    V v;
-    memcpy(&v, &d, 4);
-    return v;
-  }
 };
 template <> struct Pair<LBM_BF16DEV> {
   using V = __nv_bfloat162;
@@ -66,12 +59,6 @@ template <> struct Pair<LBM_BF16DEV> {
   }
   __device__ static __forceinline__ V pack(float a, float b) {
     return __halves2bfloat162(__float2bfloat16_rn(a), __float2bfloat16_rn(b));
-  }
-  __device__ static __forceinline__ V pack_sr(float a, float b, unsigned ra, unsigned rb) {
-    const unsigned d = cvt_rs_bf16x2(b, a, (rb << 16) | (ra & 0xFFFFu));
-    V v;
-    memcpy(&v, &d, 4);
-    return v;
   }
 };
 
@@ -141,12 +128,12 @@ __device__ __forceinline__ void store_pair(typename Prec<P>::T* p, typename Prec
   *reinterpret_cast<V*>(p) = Pair<P>::pack(a - sh, b - sh);
 }
 
+// A pair of nodes rounded stochastically with the bits of SrPair: the packed
+// 2-byte values, node x in the low half.
 template <int P>
-__device__ __forceinline__ void store_pair_sr(typename Prec<P>::T* p, typename Prec<P>::C a,
-                                              typename Prec<P>::C b, typename Prec<P>::C sh,
-                                              unsigned ra, unsigned rb) {
-  using V = typename Pair<P>::V;
-  *reinterpret_cast<V*>(p) = Pair<P>::pack_sr(a - sh, b - sh, ra, rb);
+__device__ __forceinline__ unsigned round_pair_sr(float2 v, float sh, unsigned bits) {
+  const float2 d = vsub(v, splat<float2>(sh));
+  return cvt_pair_sr<P>(d.y, d.x, bits);
 }
 
 // Store of population a of a node with seed s: nearest, or stochastic when
@@ -587,7 +574,7 @@ __device__ __forceinline__ void collide_node(const Geom& g, const Phys& ph,
     collide_math_r<C>(ph, f, dst[i], ld<NC>(psi + i), pn, fs);
   else
     collide_math<C>(ph, f, ld<NC>(psi + i), pn, fs);
-  const unsigned seed = (Prec<P>::dev && ph.sr) ? sr_seed(i, fs[0], salt_of(ph)) : 0u;
+  const unsigned seed = (Prec<P>::dev && ph.sr) ? sr_seed(i, fs[0], sr_salt(salt_of(ph))) : 0u;
   Nbr nd = nb;
   long long Nd = N;
   if (MODE == MODE_AB && px > 0) {
@@ -677,37 +664,68 @@ __device__ __forceinline__ void collide_pair(const Geom& g, const Phys& ph,
         q[dy + 1][dz + 1][3] = 0;
       }
     }
-  C fs0[Q], fs1[Q];
   float2 fp[Q], fs[Q];
 #pragma unroll
   for (int a = 0; a < Q; ++a) fp[a] = make_float2(f0[a], f1[a]);
   collide_pair_math<COLL>(ph, fp, rho_of<float2>(fp), q, fs);
+  C fs0[Q], fs1[Q];
 #pragma unroll
   for (int a = 0; a < Q; ++a) fs0[a] = fs[a].x, fs1[a] = fs[a].y;
   const bool sr = Prec<P>::dev && ph.sr;
-  const unsigned salt = sr ? salt_of(ph) : 0u;
-  const unsigned seed0 = sr ? sr_seed(i0, fs0[0], salt) : 0u, seed1 = sr ? sr_seed(i0 + 1, fs1[0], salt) : 0u;
+  const unsigned salt = sr ? sr_salt(salt_of(ph)) : 0u;
+  const unsigned seed0 = sr ? sr_seed(i0, fs[0].x, salt) : 0u, seed1 = sr ? sr_seed(i0 + 1, fs[0].y, salt) : 0u;
 
+  auto slot = [&](int a) -> typename Prec<P>::T* {   // population a of the row it streams to
+    return MODE == MODE_AA_EVEN ? dst + (long long)opp(a) * N + rows[1][1]
+                                : dst + (long long)a * N + rows[1 + cy(a)][1 + cz(a)];
+  };
+  if constexpr (Prec<P>::dev && MODE == MODE_AA_ODD) {
+    // its x-shifted values one by one, the choice of rounding made at every
+    // store: in this form its register budget of 80 spills 88 bytes, with
+    // paired conversions 168 (512x256x256 FP16: 836 against 857 us per AA step)
+#pragma unroll
+    for (int a = 0; a < Q; ++a) {
+      const C sh = a == 0 ? s0 : (a <= 6 ? s1 : s2);
+      typename Prec<P>::T* const b = slot(a);
+      if (cx(a) != 0) {
+        store_pop<P>(ph, b + xof(0, cx(a)), fs0[a], sh, seed0, a);
+        store_pop<P>(ph, b + xof(1, cx(a)), fs1[a], sh, seed1, a);
+      } else if (sr) {
+        *reinterpret_cast<unsigned*>(b + x0) = cvt_pair_sr<P>(
+            fs1[a] - sh, fs0[a] - sh, (sr_bits(seed1, a) << 16) | (sr_bits(seed0, a) & 0xFFFFu));
+      } else {
+        store_pair<P>(b + x0, fs0[a], fs1[a], sh);
+      }
+    }
+    return;
+  } else if constexpr (Prec<P>::dev) {
+    if (sr) {
+      SrPair r{0u, 0u};
+#pragma unroll
+      for (int a = 0; a < Q; ++a) {
+        const C sh = a == 0 ? s0 : (a <= 6 ? s1 : s2);
+        if (a == 0 || (a & 1)) r = sr_pair(seed0, seed1, (a + 1) >> 1);
+        const unsigned d = round_pair_sr<P>(fs[a], sh, a == 0 || (a & 1) ? r.odd : r.even);
+        unsigned short* const b = reinterpret_cast<unsigned short*>(slot(a));
+        if (MODE == MODE_AA_EVEN || cx(a) == 0) {
+          *reinterpret_cast<unsigned*>(b + x0) = d;
+        } else {
+          b[xof(0, cx(a))] = (unsigned short)d;
+          b[xof(1, cx(a))] = (unsigned short)(d >> 16);
+        }
+      }
+      return;
+    }
+  }
 #pragma unroll
   for (int a = 0; a < Q; ++a) {
     const C sh = a == 0 ? s0 : (a <= 6 ? s1 : s2);
-    if constexpr (MODE == MODE_AA_EVEN) {
-      if (sr)
-        store_pair_sr<P>(dst + (long long)opp(a) * N + i0, fs0[a], fs1[a], sh, sr_bits(seed0, a),
-                         sr_bits(seed1, a));
-      else
-        store_pair<P>(dst + (long long)opp(a) * N + i0, fs0[a], fs1[a], sh);
+    typename Prec<P>::T* const b = slot(a);
+    if (MODE == MODE_AA_EVEN || cx(a) == 0) {
+      store_pair<P>(b + x0, fs[a].x, fs[a].y, sh);
     } else {
-      typename Prec<P>::T* base = dst + (long long)a * N + rows[1 + cy(a)][1 + cz(a)];
-      if (cx(a) == 0) {
-        if (sr)
-          store_pair_sr<P>(base + x0, fs0[a], fs1[a], sh, sr_bits(seed0, a), sr_bits(seed1, a));
-        else
-          store_pair<P>(base + x0, fs0[a], fs1[a], sh);
-      } else {
-        store_pop<P>(ph, base + xof(0, cx(a)), fs0[a], sh, seed0, a);
-        store_pop<P>(ph, base + xof(1, cx(a)), fs1[a], sh, seed1, a);
-      }
+      Prec<P>::store(b + xof(0, cx(a)), fs[a].x, sh);
+      Prec<P>::store(b + xof(1, cx(a)), fs[a].y, sh);
     }
   }
 }
