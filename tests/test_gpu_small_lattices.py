@@ -152,3 +152,25 @@ def test_small_lattices_take_the_two_kernels_until_asked(L, precision):
             out.append(lat.populations())
     for f in out[1:]:
         np.testing.assert_array_equal(out[0], f)
+
+
+@pytest.mark.parametrize("precision", ["f16dev", "bf16dev"])
+@pytest.mark.parametrize("rounding", [0, 1])
+@pytest.mark.parametrize("shape,blocks", [((64, 64, 64), 2), ((66, 64, 64), 3), ((64, 72, 58), 3)])
+def test_two_byte_pairs_round_as_single_nodes(L, shape, blocks, rounding, precision):
+    """The rounding bits of two nodes taken at once, and the two-kernel step's
+    blocks per SM either side of 2^18 nodes: bitwise the one-node kernels."""
+    f0 = lbm_inputs.random_populations(*shape, seed=72)
+    out = []
+    for vector, fused in ((1, 0), (0, 0), (1, 1)):
+        with L.Lattice(*shape, 0.9, -5.5, precision=precision, rho_ref=0.1) as lat:
+            lat.set_option("fused", fused if shape[0] % 64 == 0 else 0)
+            lat.set_option("vector", vector)
+            lat.set_option("stochastic_rounding", rounding)
+            if vector and not fused:
+                assert lat.get_option("occupancy") == blocks
+            lat.set_populations(f0)
+            lat.step(5)
+            out.append(lat.populations())
+    np.testing.assert_array_equal(out[0], out[1])
+    np.testing.assert_array_equal(out[0], out[2])
