@@ -353,7 +353,8 @@ int lbm_batch_set_stream(lbm_batch b, void *stream);
  * reports LBM_ERR_TIMEOUT with the state void), "persistent_stall_test" (a
  * test hook of that failure path, in ms, 0..10: one block skips the first
  * barrier and the others give up after this long), "fused_fz" (z planes
- * per block of the single-pass step, default 16), "fused_group" (form 2:
+ * per block of the single-pass step; default: chosen from the batch for form
+ * 2, 16 for form 1), "fused_group" (form 2:
  * z runs per block-order group, as lbm_set_option's; 0, the default: all
  * runs of a tile one after another), "tile_width" (form 2: 64 - tiles of
  * 64 x 4 (FP32) or 64 x 8 (2-byte) nodes -, 32 - tiles of 32 x 8 or 32 x

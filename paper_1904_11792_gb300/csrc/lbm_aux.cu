@@ -1016,20 +1016,18 @@ cudaError_t psi_table_launch(double2* tab, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// Stochastic-rounding step salt: set it (mode 1), advance it by one (mode
-// 0, after each time step's collision) or by `value` (mode 2, after a launch
-// that ran `value` steps).
-__global__ void salt_kernel(unsigned* salt, int mode, unsigned value) {
-  *salt = mode == 1 ? value : *salt + (mode == 2 ? value : 1u);
-}
+// Stochastic-rounding step salt: set it, or write another word's value plus n.
+__global__ void salt_set_kernel(unsigned* salt, unsigned value) { *salt = value; }
+__global__ void salt_add_kernel(const unsigned* from, unsigned* to, unsigned n) { *to = *from + n; }
 
 cudaError_t launch_salt(unsigned* salt, bool set, unsigned value, cudaStream_t s) {
-  salt_kernel<<<1, 1, 0, s>>>(salt, set ? 1 : 0, value);
+  if (!set) return launch_salt_add(salt, salt, 1u, s);
+  salt_set_kernel<<<1, 1, 0, s>>>(salt, value);
   return cudaGetLastError();
 }
 
-cudaError_t launch_salt_add(unsigned* salt, unsigned n, cudaStream_t s) {
-  salt_kernel<<<1, 1, 0, s>>>(salt, 2, n);
+cudaError_t launch_salt_add(const unsigned* from, unsigned* to, unsigned n, cudaStream_t s) {
+  salt_add_kernel<<<1, 1, 0, s>>>(from, to, n);
   return cudaGetLastError();
 }
 

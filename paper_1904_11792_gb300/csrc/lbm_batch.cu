@@ -251,7 +251,7 @@ struct lbm_batch_ctx {
   GInst* d_ginst = nullptr;        // single-pass step: per-instance tile table
   int gblocks = 0;
   bool fused = true;               // option "fused": the single-pass step
-  int gfz = 16;                    // its z run length (option "fused_fz")
+  int gfz = 0;                     // its z run length (option "fused_fz"; 0: chosen, 16 for the per-element form)
   int ggrp = 0;                    // runs per block-order group of the padded form (option "fused_group")
   int tma_w = 0;                   // tile width of the padded form, 32 or 64, 0: by storage (option "tile_width")
   bool tma = true;                 // option "fused" = 2 (the default): the single pass on padded rows (TMA)
@@ -290,7 +290,7 @@ struct lbm_batch_ctx {
   long long step = 0;
   bool initialized = false;
   bool use_graph = true;
-  cudaGraphExec_t graph[2] = {nullptr, nullptr};
+  cudaGraphExec_t graph[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};   // [array][2 or kLongSteps steps]
   // the persistent form's graphs: one cooperative launch of m steps from
   // array `cur`, with its counter resets and the salt advance
   struct PersistGraph {
@@ -307,6 +307,7 @@ thread_local std::string b_err;
 
 int bfail(int status, const std::string& m);
 int bcuda(cudaError_t e, const char* where);
+int bresult(cudaError_t e, const char* where) { return e == cudaSuccess ? LBM_OK : bcuda(e, where); }
 
 #define BCK(call)                                    \
   do {                                               \
@@ -315,11 +316,12 @@ int bcuda(cudaError_t e, const char* where);
   } while (0)
 
 void drop_graphs(lbm_batch_ctx* b) {
-  for (auto& g : b->graph)
-    if (g) {
-      cudaGraphExecDestroy(g);
-      g = nullptr;
-    }
+  for (auto& pair : b->graph)
+    for (auto& g : pair)
+      if (g) {
+        cudaGraphExecDestroy(g);
+        g = nullptr;
+      }
   for (auto& pg : b->pgraphs) cudaGraphExecDestroy(pg.exec);
   b->pgraphs.clear();
 }
@@ -351,7 +353,7 @@ int layout_tiles(lbm_batch_ctx* b) {
     G.off_f = I.off_f;
     G.ntx = (I.g.nx + GX - 1) / GX;
     G.nty = (I.g.ny + GY - 1) / GY;
-    G.fz = std::min(b->gfz, I.g.nz);
+    G.fz = std::min(b->gfz ? b->gfz : 16, I.g.nz);
     G.nchunks = (I.g.nz + G.fz - 1) / G.fz;
     G.block0 = (int)gblocks;
     gblocks += (long long)G.ntx * G.nty * G.nchunks;
@@ -404,12 +406,17 @@ int ensure_contig_instance(lbm_batch_ctx* b, int k) {
   return LBM_OK;
 }
 
+bool two_byte(const lbm_batch_ctx* b) { return b->precision == LBM_F16DEV || b->precision == LBM_BF16DEV; }
+bool batch_sr(const lbm_batch_ctx* b) { return two_byte(b) && !b->inst.empty() && b->inst[0].ph.sr; }
+
 // The state back in the unpadded pool (every step form but the padded
 // single pass).
 int ensure_contig(lbm_batch_ctx* b) {
   if (!b->padded) return LBM_OK;
   for (int k = 0; k < b->count; ++k)
     if (int rc = ensure_contig_instance(b, k)) return rc;
+  if (two_byte(b) && b->cur)
+    BCK(launch_salt_add((unsigned*)(b->d_flag + 3), (unsigned*)(b->d_flag + 2), 0u, b->stream));
   b->padded = false;
   return LBM_OK;
 }
@@ -459,14 +466,14 @@ int ensure_padded(lbm_batch_ctx* b) {
   if (!b->padded) {
     for (int k = 0; k < b->count; ++k)
       if (int rc = copy_instance(b, k, true)) return rc;
+    // the padded form's salt words follow the array (word cur is the next
+    // step's), the other forms use the first one
+    if (two_byte(b) && b->cur)
+      BCK(launch_salt_add((unsigned*)(b->d_flag + 2), (unsigned*)(b->d_flag + 3), 0u, b->stream));
     b->padded = true;
     b->contig_ok.assign(b->count, 1);   // both copies current until the next step
   }
   return LBM_OK;
-}
-
-bool batch_sr(const lbm_batch_ctx* b) {
-  return (b->precision == LBM_F16DEV || b->precision == LBM_BF16DEV) && !b->inst.empty() && b->inst[0].ph.sr;
 }
 
 int enqueue_batch_step(lbm_batch_ctx* b, cudaStream_t s, int cur) {
@@ -474,9 +481,11 @@ int enqueue_batch_step(lbm_batch_ctx* b, cudaStream_t s, int cur) {
   // offsets: instances of 113 M nodes or more take the two kernels
   const bool fused_fits = 19LL * b->max_nodes <= 0x7fffffffLL;
   if (tma_form(b))
-    BCK(batch_tma_launch(b->precision, b->d_ttable, b->tplan, b->pool_p, cur, b->d_flag, s));
-  // (the caller marks the unpadded copies stale: lbm_batch_step)
-  else if (b->fused && fused_fits)
+    // (it advances the salt itself; the caller marks the unpadded copies
+    // stale: lbm_batch_step)
+    return bresult(batch_tma_launch(b->precision, b->d_ttable, b->tplan, b->pool_p, cur, b->d_flag,
+                                    (unsigned*)(b->d_flag + 2), s), "batched step");
+  if (b->fused && fused_fits)
     BCK(batch_fused_launch(b->precision, b->d_ginst, b->count, b->gblocks, b->pool_f, cur, b->d_flag,
                            b->inst[0].g.chain, s));
   else
@@ -486,15 +495,20 @@ int enqueue_batch_step(lbm_batch_ctx* b, cudaStream_t s, int cur) {
   return LBM_OK;
 }
 
-int capture_pair(lbm_batch_ctx* b, int phase) {
+// Steps of the longer graph, replayed while as many are left: the gap between
+// two graph replays (about 2.7 us) is 2 % of two steps of an 8-ligament sweep
+// and 10 % of two steps of three small ligaments.  Capturing it pays from
+// kLongFrom steps in one call.
+constexpr int kLongSteps = 16, kLongFrom = 64;
+
+int capture_steps(lbm_batch_ctx* b, int phase, int steps, cudaGraphExec_t* exec) {
   cudaStream_t cs;
   BCK(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
   cudaGraph_t g = nullptr;
   cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
   int rc = LBM_OK;
   if (e == cudaSuccess) {
-    rc = enqueue_batch_step(b, cs, phase);
-    if (rc == LBM_OK) rc = enqueue_batch_step(b, cs, phase ^ 1);
+    for (int k = 0; k < steps && rc == LBM_OK; ++k) rc = enqueue_batch_step(b, cs, phase ^ (k & 1));
     e = cudaStreamEndCapture(cs, &g);
   }
   cudaStreamDestroy(cs);
@@ -503,10 +517,10 @@ int capture_pair(lbm_batch_ctx* b, int phase) {
     return rc;
   }
   if (e != cudaSuccess) return bcuda(e, "batch graph capture");
-  e = cudaGraphInstantiate(&b->graph[phase], g, 0);
+  e = cudaGraphInstantiate(exec, g, 0);
   cudaGraphDestroy(g);
   if (e != cudaSuccess) {
-    b->graph[phase] = nullptr;
+    *exec = nullptr;
     return bcuda(e, "cudaGraphInstantiate");
   }
   return LBM_OK;
@@ -552,11 +566,17 @@ int enqueue_persist(lbm_batch_ctx* b, cudaStream_t s, int cur, int m) {
   const unsigned long long stall_ns = (unsigned long long)(b->persist_stall_ms * 1e6);
   if (tma_form(b))
     BCK(batch_tma_persist_launch(b->precision, b->d_ttable, b->tplan, b->pool_p, cur, m,
-                                 (unsigned*)(b->d_flag + 4), b->d_tickets, b->d_flag, stall_ns, s));
+                                 (unsigned*)(b->d_flag + 4), b->d_tickets, b->d_flag, (unsigned*)(b->d_flag + 2),
+                                 stall_ns, s));
   else
     BCK(batch_persist_launch(b->precision, b->d_ginst, b->count, b->gblocks, b->pool_f, cur, m,
                              (unsigned*)(b->d_flag + 4), b->d_tickets, b->d_flag, stall_ns, s));
-  if (batch_sr(b)) BCK(launch_salt_add((unsigned*)(b->d_flag + 2), (unsigned)m, s));
+  if (tma_form(b)) {   // into the word the next launch reads
+    if (two_byte(b))
+      BCK(launch_salt_add((unsigned*)(b->d_flag + 2 + cur), (unsigned*)(b->d_flag + 2 + (cur ^ (m & 1))),
+                          batch_sr(b) ? (unsigned)m : 0u, s));
+  } else if (batch_sr(b))
+    BCK(launch_salt_add((unsigned*)(b->d_flag + 2), (unsigned*)(b->d_flag + 2), (unsigned)m, s));
   return LBM_OK;
 }
 
@@ -688,7 +708,7 @@ lbm_batch lbm_batch_create(const lbm_instance* inst, int count, int precision, i
   if (err == cudaSuccess) err = cudaMalloc(&b->d_flag, sizeof(int) * 8);
   if (err == cudaSuccess) err = cudaMalloc(&b->d_small, sizeof(double) * 64);
   if (err == cudaSuccess) err = cudaMemsetAsync(b->d_flag, 0, sizeof(int) * 8, b->stream);
-  // d_flag[2] is the stochastic-rounding step salt of every instance
+  // d_flag[2] (and [3]: the padded form's pair) is the stochastic-rounding step salt of every instance
   if (err == cudaSuccess)
     for (auto& I : b->inst) I.ph.salt = (const unsigned*)(b->d_flag + 2);
   if (err == cudaSuccess && precision == LBM_F64) {
@@ -851,13 +871,16 @@ int lbm_batch_step(lbm_batch b, int n) {
   }
   while (n > 0) {
     if (b->use_graph && n >= 2) {
-      if (!b->graph[b->cur]) {
-        int rc = capture_pair(b, b->cur);
+      const bool longer = n >= kLongFrom || (n >= kLongSteps && b->graph[b->cur][1]);
+      const int steps = longer ? kLongSteps : 2;
+      cudaGraphExec_t& ge = b->graph[b->cur][longer];
+      if (!ge) {
+        int rc = capture_steps(b, b->cur, steps, &ge);
         if (rc) return rc;
       }
-      BCK(cudaGraphLaunch(b->graph[b->cur], b->stream));
-      n -= 2;
-      b->step += 2;
+      BCK(cudaGraphLaunch(ge, b->stream));
+      n -= steps;
+      b->step += steps;
     } else {
       int rc = enqueue_batch_step(b, b->stream, b->cur);
       if (rc) return rc;

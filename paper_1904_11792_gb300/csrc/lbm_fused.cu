@@ -392,6 +392,43 @@ cudaError_t launch_fused(int precision, const Geom& g, const Phys& ph, const voi
 
 namespace {
 
+// z planes per block of a batch's tiles, one length for all instances: whole
+// waves of blocks take their mean cost (the two planes a run does not collide
+// count `halo` each half), the last wave what its blocks cost at full rate but
+// at least `lat` of its planes' latency; times 1 + fz / k.  Fitted to the times
+// of these run lengths on five sweeps of 3 to 48 ligaments (0.2 to 35 M nodes): it
+// picks the best of them in FP32 and within 0.5 % in FP16.  The fixed 16 planes
+// before cost 0 to 8 % (FP32) and 0 to 26 % (FP16) on the sweeps of 6 to 48 and
+// twice (FP32, 28.0 / 14.4 us) to three times (FP16, 55.4 / 18.5 us) on three
+// small ones.
+template <int P, int W>
+int choose_batch_fz(const BatchTmaInst* in, int count, long long slots) {
+  constexpr bool dev = Prec<P>::dev;
+  const double halo = dev ? 1.0 : 2.0, lat = dev ? 0.75 : 0.9, k = dev ? 400.0 : 160.0;
+  int best = 16;
+  double best_cost = -1.0;
+  for (int fz : {2, 3, 4, 5, 6, 8, 10, 12, 16, 20, 24, 32, 48, 64}) {
+    long long blocks = 0, planes = 0;
+    for (int i = 0; i < count; ++i) {
+      const Geom& g = in[i].g;
+      const long long tiles =
+          (long long)((g.nx + W - 1) / W) * ((g.ny + FusedShape<P, W>::TY - 1) / FusedShape<P, W>::TY);
+      blocks += tiles * ((g.nz + fz - 1) / fz);
+      planes += tiles * g.nz;
+    }
+    const long long waves = blocks / slots, last = blocks - waves * slots;
+    const double mean = (double)planes / blocks + halo;
+    double cost = waves * mean;
+    if (last) cost += std::max(mean * last / slots, lat * (fz + 2));
+    cost *= 1.0 + fz / k;
+    if (best_cost < 0.0 || cost < best_cost) {
+      best_cost = cost;
+      best = fz;
+    }
+  }
+  return best;
+}
+
 template <int P, int W>
 cudaError_t batch_tma_build_t(const BatchTmaInst* in, int count, int fz_req, int grp_req, const void* pool,
                               void* d_table, BatchTmaPlan* plan, cudaStream_t s) {
@@ -406,6 +443,7 @@ cudaError_t batch_tma_build_t(const BatchTmaInst* in, int count, int fz_req, int
   Maps* tm = reinterpret_cast<Maps*>(host.data() + inst_bytes);
   const Maps* d_maps = reinterpret_cast<const Maps*>((const unsigned char*)d_table + inst_bytes);
   const int cw = 16 / (int)es;
+  if (fz_req <= 0) fz_req = choose_batch_fz<P, W>(in, count, (long long)slots_per_sm * sms);
   long long blocks = 0;
   for (int k = 0; k < count; ++k) {
     const BatchTmaInst& b = in[k];
@@ -421,7 +459,7 @@ cudaError_t batch_tma_build_t(const BatchTmaInst* in, int count, int fz_req, int
     t.maps = d_maps + 2 * k;
     t.ntx = (b.g.nx + W - 1) / W;
     const int nty = (b.g.ny + S::TY - 1) / S::TY;
-    t.fz = std::min(fz_req > 0 ? fz_req : 16, b.g.nz);
+    t.fz = std::min(fz_req, b.g.nz);
     t.nchunks = (b.g.nz + t.fz - 1) / t.fz;
     // runs per block-order group (0: a tile's z runs one after another)
     t.grp = grp_req > 0 ? std::min(grp_req, t.nchunks) : t.nchunks;
@@ -456,23 +494,24 @@ cudaError_t batch_tma_build_w(int tile_w, const BatchTmaInst* insts, int count, 
 
 template <int P, int W>
 cudaError_t batch_tma_launch_t(const void* d_table, const BatchTmaPlan& plan, void* pool, int cur, int* flag,
-                               cudaStream_t s) {
+                               unsigned* salt, cudaStream_t s) {
   using S = FusedShape<P, W>;
   return chain_launch(plan.chain, bfused_kernel<P, W>, plan.blocks, S::NT, S::smem, s, reinterpret_cast<const BTInst*>(d_table),
-                      plan.count, (typename Prec<P>::T*)pool, cur, flag);
+                      plan.count, (typename Prec<P>::T*)pool, cur, flag, salt);
 }
 
 template <int P>
 cudaError_t batch_tma_launch_w(const void* d_table, const BatchTmaPlan& plan, void* pool, int cur, int* flag,
-                               cudaStream_t s) {
-  if (plan.width == 32) return batch_tma_launch_t<P, 32>(d_table, plan, pool, cur, flag, s);
-  if (plan.width == TX) return batch_tma_launch_t<P, TX>(d_table, plan, pool, cur, flag, s);
+                               unsigned* salt, cudaStream_t s) {
+  if (plan.width == 32) return batch_tma_launch_t<P, 32>(d_table, plan, pool, cur, flag, salt, s);
+  if (plan.width == TX) return batch_tma_launch_t<P, TX>(d_table, plan, pool, cur, flag, salt, s);
   return cudaErrorInvalidValue;
 }
 
 template <int P, int W>
 cudaError_t batch_tma_persist_t(const void* d_table, const BatchTmaPlan& plan, void* pool, int cur, int nsteps,
-                                unsigned* bar, unsigned* tickets, int* flag, unsigned long long stall_ns,
+                                unsigned* bar, unsigned* tickets, int* flag, const unsigned* salt,
+                                unsigned long long stall_ns,
                                 cudaStream_t s) {
   using S = FusedShape<P, W>;
   using T = typename Prec<P>::T;
@@ -490,18 +529,19 @@ cudaError_t batch_tma_persist_t(const void* d_table, const BatchTmaPlan& plan, v
   const BTInst* t = reinterpret_cast<const BTInst*>(d_table);
   T* pf = (T*)pool;
   void* args[] = {(void*)&t, (void*)&count, (void*)&pf, (void*)&cur, (void*)&nsteps,
-                  (void*)&items, (void*)&bar, (void*)&tickets, (void*)&flag, (void*)&stall_ns};
+                  (void*)&items, (void*)&bar, (void*)&tickets, (void*)&flag, (void*)&salt, (void*)&stall_ns};
   return cudaLaunchCooperativeKernel((const void*)bpersist_kernel<P, W>, dim3(grid), dim3(S::NT), args, S::smem, s);
 }
 
 template <int P>
 cudaError_t batch_tma_persist_w(const void* d_table, const BatchTmaPlan& plan, void* pool, int cur, int nsteps,
-                                unsigned* bar, unsigned* tickets, int* flag, unsigned long long stall_ns,
+                                unsigned* bar, unsigned* tickets, int* flag, const unsigned* salt,
+                                unsigned long long stall_ns,
                                 cudaStream_t s) {
   if (plan.width == 32)
-    return batch_tma_persist_t<P, 32>(d_table, plan, pool, cur, nsteps, bar, tickets, flag, stall_ns, s);
+    return batch_tma_persist_t<P, 32>(d_table, plan, pool, cur, nsteps, bar, tickets, flag, salt, stall_ns, s);
   if (plan.width == TX)
-    return batch_tma_persist_t<P, TX>(d_table, plan, pool, cur, nsteps, bar, tickets, flag, stall_ns, s);
+    return batch_tma_persist_t<P, TX>(d_table, plan, pool, cur, nsteps, bar, tickets, flag, salt, stall_ns, s);
   return cudaErrorInvalidValue;
 }
 
@@ -524,25 +564,25 @@ cudaError_t batch_tma_build(int precision, int tile_w, const BatchTmaInst* insts
 }
 
 cudaError_t batch_tma_launch(int precision, const void* d_table, const BatchTmaPlan& plan, void* pool, int cur,
-                             int* flag, cudaStream_t s) {
+                             int* flag, unsigned* salt, cudaStream_t s) {
   switch (precision) {
-    case LBM_F32: return batch_tma_launch_w<LBM_F32>(d_table, plan, pool, cur, flag, s);
-    case LBM_F16DEV: return batch_tma_launch_w<LBM_F16DEV>(d_table, plan, pool, cur, flag, s);
-    case LBM_BF16DEV: return batch_tma_launch_w<LBM_BF16DEV>(d_table, plan, pool, cur, flag, s);
+    case LBM_F32: return batch_tma_launch_w<LBM_F32>(d_table, plan, pool, cur, flag, salt, s);
+    case LBM_F16DEV: return batch_tma_launch_w<LBM_F16DEV>(d_table, plan, pool, cur, flag, salt, s);
+    case LBM_BF16DEV: return batch_tma_launch_w<LBM_BF16DEV>(d_table, plan, pool, cur, flag, salt, s);
   }
   return cudaErrorInvalidValue;
 }
 
 cudaError_t batch_tma_persist_launch(int precision, const void* d_table, const BatchTmaPlan& plan, void* pool,
                                      int cur, int nsteps, unsigned* bar, unsigned* tickets, int* flag,
-                                     unsigned long long stall_ns, cudaStream_t s) {
+                                     const unsigned* salt, unsigned long long stall_ns, cudaStream_t s) {
   switch (precision) {
     case LBM_F32:
-      return batch_tma_persist_w<LBM_F32>(d_table, plan, pool, cur, nsteps, bar, tickets, flag, stall_ns, s);
+      return batch_tma_persist_w<LBM_F32>(d_table, plan, pool, cur, nsteps, bar, tickets, flag, salt, stall_ns, s);
     case LBM_F16DEV:
-      return batch_tma_persist_w<LBM_F16DEV>(d_table, plan, pool, cur, nsteps, bar, tickets, flag, stall_ns, s);
+      return batch_tma_persist_w<LBM_F16DEV>(d_table, plan, pool, cur, nsteps, bar, tickets, flag, salt, stall_ns, s);
     case LBM_BF16DEV:
-      return batch_tma_persist_w<LBM_BF16DEV>(d_table, plan, pool, cur, nsteps, bar, tickets, flag, stall_ns, s);
+      return batch_tma_persist_w<LBM_BF16DEV>(d_table, plan, pool, cur, nsteps, bar, tickets, flag, salt, stall_ns, s);
   }
   return cudaErrorInvalidValue;
 }

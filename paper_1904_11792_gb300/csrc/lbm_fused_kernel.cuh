@@ -713,12 +713,23 @@ __device__ __forceinline__ void batch_item(const BTInst& I, int u, typename Prec
 // padded to 16-byte multiples: one launch, each block finds its instance
 // and runs fused_body on its work item with that instance's tensor maps,
 // which live in global memory (ordered before their use by the tensor-map
-// proxy fence).  W: the tile width the table was built for.
+// proxy fence).  W: the tile width the table was built for.  salt: the pair of
+// stochastic-rounding salt words; the step from array cur reads word cur and
+// writes the next step's salt into the other one, which nothing of it reads
+// (instead of a one-thread kernel between the steps).  Rounding to nearest
+// carries the salt over unchanged.
 template <int P, int W>
 __global__ void __launch_bounds__(FusedShape<P, W>::NT, fused_minb<P, false, COLL_SRT>())
-    bfused_kernel(const BTInst* __restrict__ inst, int count, typename Prec<P>::T* pool, int cur, int* flag) {
+    bfused_kernel(const BTInst* __restrict__ inst, int count, typename Prec<P>::T* pool, int cur, int* flag,
+                  unsigned* salt) {
   const BTInst& I = find_inst(inst, count, (int)blockIdx.x);
-  batch_item<P, W, false>(I, (int)blockIdx.x - I.block0, pool, cur, flag, 0u);
+  unsigned now = 0u;
+  if constexpr (Prec<P>::dev) {
+    if (I.g.chain) chain_wait();
+    now = salt[cur];
+    if (blockIdx.x == 0 && threadIdx.x == 0) salt[cur ^ 1] = now + (I.ph.sr ? 1u : 0u);
+  }
+  batch_item<P, W, true>(I, (int)blockIdx.x - I.block0, pool, cur, flag, now);
 }
 
 // nsteps steps of the batched TMA step in one cooperative launch of
@@ -736,14 +747,14 @@ __global__ void __launch_bounds__(FusedShape<P, W>::NT, fused_minb<P, false, COL
 template <int P, int W>
 __global__ void __launch_bounds__(FusedShape<P, W>::NT, fused_minb<P, false, COLL_SRT>())
     bpersist_kernel(const BTInst* __restrict__ inst, int count, typename Prec<P>::T* pool, int cur0, int nsteps,
-                    int items, unsigned* bar, unsigned* tickets, int* flag, unsigned long long stall_test_ns) {
+                    int items, unsigned* bar, unsigned* tickets, int* flag, const unsigned* salt,
+                    unsigned long long stall_test_ns) {
   using S = FusedShape<P, W>;
   extern __shared__ __align__(128) unsigned char smem[];
   unsigned long long* full = reinterpret_cast<unsigned long long*>(smem + S::off_bar);
   __shared__ int s_item;
-  const Phys& ph0 = inst[0].ph;   // every instance shares the salt word
   unsigned salt0 = 0u;
-  if (Prec<P>::dev && ph0.sr) salt0 = *(const volatile unsigned*)ph0.salt;
+  if (Prec<P>::dev) salt0 = salt[cur0];   // (word cur0 is this launch's, see bfused_kernel)
   const unsigned long long limit = stall_test_ns ? stall_test_ns : kGridWaitNs;
   for (int s = 0; s < nsteps; ++s) {
     // one read of the flag for the whole block: every thread returns or none

@@ -202,8 +202,9 @@ cudaError_t launch_diagnostics(int precision, int layout, const Geom& g, const P
 
 // Stochastic-rounding step salt (Phys::salt): set to value, or advance by one.
 cudaError_t launch_salt(unsigned* salt, bool set, unsigned value, cudaStream_t s);
-// Advances the salt word by n (after a launch that ran n steps).
-cudaError_t launch_salt_add(unsigned* salt, unsigned n, cudaStream_t s);
+// The salt after n steps from the word `from` into the word `to` (the same or
+// another one), after a launch that ran them.
+cudaError_t launch_salt_add(const unsigned* from, unsigned* to, unsigned n, cudaStream_t s);
 
 // Second and third stage of the diagnostics reduction from partials
 // slices[row_blocks][nx][2] and blocks[nblocks][DIAG_NG] (slice_tot: 2 nx
@@ -259,20 +260,23 @@ struct BatchTmaPlan {
 // Bytes of the device table (instance records and their tensor maps).
 size_t batch_tma_table_bytes(int count);
 // Encodes the tensor maps, builds the block table for tiles tile_w (32 or
-// 64) nodes wide and z runs of fz planes in groups of grp runs (0: all runs
+// 64) nodes wide and z runs of fz planes (0: chosen) in groups of grp runs (0: all runs
 // of a tile one after another), and copies it to d_table (device,
 // batch_tma_table_bytes).  FP32, FP16-dev, BF16-dev.  Synchronises s.
 cudaError_t batch_tma_build(int precision, int tile_w, const BatchTmaInst* insts, int count, int fz, int grp,
                             const void* pool, void* d_table, BatchTmaPlan* plan, cudaStream_t s);
-// One step of every instance: padded pool arrays cur -> cur ^ 1.
+// One step of every instance: padded pool arrays cur -> cur ^ 1.  salt: two
+// words, of which the step reads word cur (its step number) and writes the
+// other.
 cudaError_t batch_tma_launch(int precision, const void* d_table, const BatchTmaPlan& plan, void* pool, int cur,
-                             int* flag, cudaStream_t s);
+                             int* flag, unsigned* salt, cudaStream_t s);
 // nsteps such steps in one cooperative launch of persistent blocks: grid
 // barriers on *bar (zeroed here), per-step work tickets tickets[nsteps]
-// (zeroed here); stall_ns > 0 is the barrier-timeout test hook.
+// (zeroed here); salt as batch_tma_launch (read only: the caller sets the word
+// of the next launch); stall_ns > 0 is the barrier-timeout test hook.
 cudaError_t batch_tma_persist_launch(int precision, const void* d_table, const BatchTmaPlan& plan, void* pool,
                                      int cur, int nsteps, unsigned* bar, unsigned* tickets, int* flag,
-                                     unsigned long long stall_ns, cudaStream_t s);
+                                     const unsigned* salt, unsigned long long stall_ns, cudaStream_t s);
 
 // True if LBM_ALLOC_CAP_BYTES is set and a device allocation of `bytes`
 // exceeds it (out-of-memory handling without exhausting a GPU).

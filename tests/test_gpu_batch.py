@@ -275,3 +275,29 @@ def test_batch_alloc_cap_gives_oom(L, monkeypatch):
         b.sync()
         assert b.diagnostics(0)["numeric_ok"] == 1
     monkeypatch.delenv("LBM_ALLOC_CAP_BYTES")
+
+
+# The run length the padded form chooses by itself (a small batch: short runs;
+# one with a large instance: longer ones), its longer graphs (64 steps and
+# more in a call) and its pair of salt words, against the two-kernel batch,
+# bitwise: the rounding switched in the middle, form and persistence too.
+@pytest.mark.parametrize("precision", ["f32", "f16dev", "bf16dev"])
+@pytest.mark.parametrize("big", [False, True])
+def test_padded_batch_of_chosen_run_length(L, precision, big):
+    insts = [dict(nx=nx, ny=ny, nz=nz, tau=0.9, G=-5.5, R0=max(1.0, min(ny, nz) / 4.0), lam=float(nx), eps=0.1,
+                  phase=0.2, rho_l=2.5, rho_v=0.15, width=2.0)
+             for nx, ny, nz in SHAPES + (((130, 64, 96),) if big else ())]
+    res = []
+    for plan in (((0, 0),) * 6, ((2, 0),) * 6, ((2, 0), (0, 0), (2, 1), (2, 0), (1, 0), (2, 1))):
+        with L.Batch(insts, precision=precision) as b:
+            b.init()
+            for (form, persistent), n, sr in zip(plan, (65, 3, 18, 7, 1, 33), (1, 1, 0, 0, 1, 1)):
+                b.set_option("fused", form)
+                b.set_option("persistent", persistent)
+                b.set_option("stochastic_rounding", sr)
+                b.step(n)
+            b.sync()
+            res.append([b.populations(k) for k in range(len(insts))])
+    for r in res[1:]:
+        for k in range(len(insts)):
+            np.testing.assert_array_equal(r[k], res[0][k])
