@@ -154,8 +154,8 @@ int lbm_set_stream(lbm_handle h, void *stream);
  * shape, at most 256 threads), "occupancy" (2, 3 or 4: 256-thread blocks
  * per SM the collide-stream kernel's register budget allows; 0 = auto,
  * the default: 3 for the one-node kernel and the AA even step's two-node
- * kernel, for the AA odd step's and, above 2^18 nodes, the A-B step's with
- * 2-byte storage, 2 otherwise and in FP64; get answers the odd step's (AA) or
+ * kernel and, above 2^21 nodes, for the A-B step's with 2-byte storage, 2
+ * otherwise and in FP64; get answers the odd step's (AA) or
  * the A-B step's value),
  * "vector" (0/1, default 1: when nx is even each thread updates two
  * neighbouring nodes with 2-element vector loads and stores; block_x then
@@ -166,10 +166,11 @@ int lbm_set_stream(lbm_handle h, void *stream);
  * FP16-dev and BF16-dev storage when nx % 64 == 0 and ny % 4 == 0 (FP32) or
  * ny % 8 == 0 (2-byte storage); lbm_get_option answers whether it applies.
  * Until the option (or "fused_fz" or "fused_group") is set, lattices of at most
- * 2^18 nodes take the two-kernel step all the same, which is faster there.
+ * 640 Ki nodes (1 Mi with 2-byte storage or the MRT collision) take the
+ * two-kernel step all the same, which is faster there.
  * Of the other lattices of these storage forms, larger ones (more than 1 M
- * nodes in FP32, 2.6 M in 2-byte storage, nx >= 32; with the value 2 all of
- * them) run plain steps as a single pass on tiles cut at their edges: every
+ * nodes in FP32, 2.6 M and odd nx in 2-byte storage, nx >= 32; with the value
+ * 2 all of them) run plain steps as a single pass on tiles cut at their edges: every
  * step where rows are a multiple of 16 bytes; otherwise the steps inside a
  * replayed graph but its first one, on two private arrays with padded rows
  * (allocated on the first such call if they take at most a quarter of the

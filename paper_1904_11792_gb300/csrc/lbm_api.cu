@@ -26,19 +26,26 @@ dim3 default_block(const Geom& g) {
 }
 
 // The block a collide-stream kernel launches with where no shape was asked
-// for: the default, but rows shorter than a warp are not padded to one - the
-// block takes whole rows of several y and z, so a warp's lanes all hold nodes -
-// and lattices too small to give every SM two blocks take smaller blocks,
-// down to one warp.  (4x49x49 FP64, whose pipe a warp instruction occupies
-// for 16 clocks whatever its live lanes: 68 us per step in 32 x 8 blocks, 2 of
-// 32 lanes live, 10.3 us in 4 x 8 x 1.)
-dim3 auto_block(const Geom& g, bool pairs) {
+// for: two warps.  These kernels hold 80 to 100 registers, so an SM takes few
+// warps, and a block's place is free for the next one only when its last warp
+// is done: small blocks keep more warps in flight (per collide kernel, 256 ->
+// 64 threads: 512x256x256 FP16 A-B 580 -> 565 us, AA odd 707 -> 633 us with
+// its larger register budget, auto_minb; 256x128x128 FP64 988 -> 981 us; per
+// step: 150x80x80 FP32 37.8 -> 33.7 us, FP16 30.4 -> 25.6 us).  64 along x, 32
+// where that pads the row less (150x80x80 FP32 in 64 x 1: 36.1 us), and for
+// FP32 rows of whole 128s four warps (512x256x256 A-B: 767 us, 64 x 1 775).
+// Lattices too small to give every SM two such blocks take one warp, and rows
+// shorter than a warp are not padded to one: the block takes whole rows of
+// several y and z, so a warp's lanes all hold nodes (4x49x49 FP64, whose pipe a
+// warp instruction occupies for 16 clocks whatever its live lanes: 68 us per
+// step in 32 x 8 blocks, 2 of 32 lanes live, 10.3 us in 4 x 8 x 1).
+dim3 auto_block(const Geom& g, bool pairs, int precision) {
   const unsigned ux = pairs ? g.nx / 2 : g.nx;
   const long long units = (long long)ux * g.ny * g.nz;
-  unsigned threads = 256;
-  while (threads > 32 && units < (long long)threads * 2 * kSmCount) threads /= 2;
+  const unsigned threads = units < 64LL * 2 * kSmCount ? 32 : 64;
   if (ux >= 32) {
-    const unsigned bx = std::min(threads, default_block(g).x);
+    if (threads == 64 && precision == LBM_F32 && ux % 128 == 0) return dim3(128, 1, 1);
+    const unsigned bx = threads == 64 && (ux - 1) % 64 >= 32 ? 64 : 32;
     return dim3(bx, threads / bx, 1);
   }
   const unsigned by = std::min<unsigned>(g.ny, std::max(1u, threads / ux));
@@ -162,21 +169,18 @@ int salt_word(const lbm_ctx* h, long long step, int cur) {
   return h->cfg.pattern == LBM_AA ? (int)(step & 1) : (cur & 1);
 }
 
-// Default register budget of the collide-stream kernel (blocks of 256
-// threads per SM), as measured on the 1024x512x512 lattice: 3 for the
-// one-node kernel and for the AA even step's two-node kernel (local loads
-// and stores: no spills at 80 registers); for the AA odd step's two-node
-// kernel 3 with 2-byte storage (6.93 ms per FP16 AA step against 7.65 with
-// 2, although it spills a little at 80 registers) and 2 otherwise (FP32:
-// 9.11 ms against 9.84); for the A-B step's two-node kernel 3 with 2-byte
-// storage (512x256x256 FP16: 780 us per step against 885 with 2) but on
-// lattices of a few thousand warps (64x64x64: 9.9 against 9.0 us), and 2
-// otherwise (no spills at <= 128 registers).
+// Default register budget of the collide-stream kernel (as blocks of 256
+// threads per SM), measured in the blocks of auto_block: 3 for the one-node
+// kernel and for the AA even step's two-node kernel (local loads and stores: no
+// spills at 80 registers); for the A-B step's two-node kernel 3 with 2-byte
+// storage above 2^21 nodes (512x256x256 FP16: 565 us per launch against 584
+// with 2; 150x80x80: 26.5 us per step against 25.6); 2 otherwise, with which
+// nothing spills (AA odd step of 512x256x256, FP16: 633 us per launch, with 3
+// 666; FP32: 783 against 930).
 int auto_minb(bool vec, int mode, int precision, long long N) {
-  if (precision == LBM_F64) return 2;   // 988 us per launch on 256x128x128 against 1013 with 3 (spills)
+  if (precision == LBM_F64) return 2;   // 981 us per launch on 256x128x128 against 1009 with 3 (spills)
   if (!vec || mode == MODE_AA_EVEN) return 3;
-  if (precision != LBM_F16DEV && precision != LBM_BF16DEV) return 2;
-  return mode == MODE_AA_ODD || N > kFusedNodes ? 3 : 2;
+  return mode == MODE_AB && precision != LBM_F32 && N > 2LL << 20 ? 3 : 2;
 }
 
 bool ragged_direct(const lbm_ctx* h);
@@ -184,8 +188,9 @@ bool ragged_direct(const lbm_ctx* h);
 // Whether steps run as the fused single pass: small lattices only when asked
 // for (option "fused", or one of its launch shape or test hook).
 bool fused_form(const lbm_ctx* h) {
+  const long long least = h->cfg.precision == LBM_F32 && h->ph.coll == COLL_SRT ? kFusedNodes : kFusedNodesLate;
   return h->fused && h->cfg.pattern == LBM_AB && fused_applicable(h->g, h->cfg.precision) &&
-         (h->fused > 0 || h->g.N > kFusedNodes || h->fused_fz || h->fused_group || h->fused_stall_test_ns);
+         (h->fused > 0 || h->g.N > least || h->fused_fz || h->fused_group || h->fused_stall_test_ns);
 }
 
 // The psi pass of a diagnostic step of the two kernels: with the diagnostics,
@@ -295,7 +300,7 @@ int enqueue_step(lbm_ctx* h, cudaStream_t s, long long step, int cur, bool timed
   if (timed) CK(cudaEventRecord(e1, s));
   const bool vec = node_pairs(prec, h->vec, h->g);
   const int minb = h->minb ? h->minb : auto_minb(vec, mode, prec, h->g.N);
-  const dim3 block = h->block_asked ? h->block : auto_block(h->g, vec);
+  const dim3 block = h->block_asked ? h->block : auto_block(h->g, vec, prec);
   if (h->ph.coll == COLL_MRT)
     CK(launch_collide_mrt(prec, mode, vec, g, ph, src, dst, h->psi, block, s));
   else
@@ -312,8 +317,8 @@ int enqueue_step(lbm_ctx* h, cudaStream_t s, long long step, int cur, bool timed
 // arrays (its rows are 16-byte multiples), and whether the steps inside a
 // captured chunk run on padded copies (they are not, and there is room).
 bool ragged_form(const lbm_ctx* h) {
-  const long long least = Prec_dev(h->cfg.precision) ? kRaggedNodesDev : kRaggedNodes;
-  return h->fused && (h->fused == 2 || (h->g.N > least && h->g.nx >= kRaggedMinNx)) &&
+  const bool pays = Prec_dev(h->cfg.precision) ? h->g.N > kRaggedNodesDev && h->g.nx % 2 : h->g.N > kRaggedNodes;
+  return h->fused && (h->fused == 2 || (pays && h->g.nx >= kRaggedMinNx)) &&
          h->cfg.pattern == LBM_AB && ragged_applicable(h->g, h->cfg.precision);
 }
 bool ragged_direct(const lbm_ctx* h) {
@@ -365,7 +370,7 @@ int enqueue_padded_step(lbm_ctx* h, cudaStream_t s, int k, int steps, int phase,
     } else {
       CK(launch_psi(prec, LAYOUT_LOCAL, h->vec, g, h->ph, src, h->psi, h->d_flag, s));
     }
-    CK(launch_collide_padded(prec, g, ph, src, h->pad[0], px, h->psi, auto_block(g, false), s));
+    CK(launch_collide_padded(prec, g, ph, src, h->pad[0], px, h->psi, auto_block(g, false, prec), s));
     return LBM_OK;
   }
   const bool last = k == steps - 1;

@@ -68,12 +68,13 @@ cudaError_t launch_collide_padded(int precision, const Geom& g, const Phys& ph, 
 
 // Lattices up to this many nodes run the two kernels by default where the
 // fused step applies: their populations stay in L2, and two short passes over
-// all nodes at once beat a march through planes by few blocks (chained,
-// plain steps: 64x32x32 FP32 5.57 against 7.76 us, FP16 4.96 / 10.44;
-// 128x32x32 6.52 / 8.01, 6.23 / 10.57; 64x64x64 9.16 / 12.91, 9.29 / 10.59;
-// but 128x48x48 9.91 / 13.28, FP16 11.47 / 10.83; 192x48x48 14.17 / 13.55,
-// 14.99 / 14.94).
-constexpr long long kFusedNodes = 1 << 18;
+// all nodes at once beat a march through planes by few blocks (plain steps,
+// two kernels against single pass: 64x32x32 FP32 5.57 / 7.76 us, FP16 4.85 /
+// 10.6; 64x96x96 14.9 / 17.1, 14.2 / 14.8; 128x80x80 24.0 / 22.8, 18.3 / 20.2;
+// 256x64x64 32.7 / 31.9, 22.8 / 22.8; 128x96x96 38.3 / 36.1, 27.6 / 26.7; MRT:
+// 128x80x80 27.4 / 28.8, 256x64x64 36.6 / 38.3, 192x96x96 69.8 / 57.8).
+// kFusedNodes: FP32 and the paper's collision; kFusedNodesLate: the others.
+constexpr long long kFusedNodes = 5 << 17, kFusedNodesLate = 1 << 20;
 // Lattices up to this many nodes launch their steps chained (lbm_launch.cuh)
 // and replay longer graphs: their kernels take a few microseconds each.
 constexpr long long kChainNodes = 1 << 20;
@@ -84,7 +85,7 @@ constexpr int kSmCount = 152;
 // options start from, and the shape launched where none was asked for
 // (lbm_api.cu).
 dim3 default_block(const Geom& g);
-dim3 auto_block(const Geom& g, bool pairs);
+dim3 auto_block(const Geom& g, bool pairs, int precision);
 
 // force + collision + streaming with the MRT collision (lbm_mrt.cu); the
 // same modes and layouts as launch_collide
@@ -127,11 +128,13 @@ size_t fused_diag_scratch_doubles(const Geom& g, int precision, int fz);
 // of a padded copy.  dst_px: row pitch of the destination, any.  fz, grp: as
 // launch_fused.
 // Smaller lattices keep the two kernels by default: they live in L2, where the
-// two short passes are as fast or faster (plain steps, two-kernel against
-// single pass: FP32 181x56x56 20.8 / 20.4 us, 172x80x80 42.2 / 37.5, 201x100x100
-// 90.5 / 71.3, 303x150x150 295 / 199; FP16 201x100x100 78 / 70, 200x100x100 68 /
-// 71, 251x112x112 111 / 101, 303x150x150 264 / 194); so do rows of less than
-// half a tile.
+// two short passes are as fast or faster (plain steps, two kernels against
+// single pass: FP32 150x80x80 33.7 / 36.2 us, 101x100x100 42.2 / 39.7, 180x90x90
+// 53.6 / 48.9, 251x128x128 170 / 130; FP16 199x100x100 72 / 76, 251x100x100 87 /
+// 87, 251x128x128 136 / 126, 503x200x200 624 / 553); so do rows of less than
+// half a tile, and 2-byte storage with even nx, whose two kernels take node
+// pairs (FP16 198x120x119 84 / 97, 502x112x112 157 / 173, 504x200x200 468 / 533;
+// MRT 502x112x112 197 / 203, 456x256x256 949 / 915).
 constexpr long long kRaggedNodes = 1 << 20, kRaggedNodesDev = 5 << 19;
 constexpr int kRaggedMinNx = 32;
 bool ragged_applicable(const Geom& g, int precision);

@@ -116,10 +116,11 @@ cudaError_t collide_padded(const Geom& g, const Phys& ph, const void* src, void*
   return cudaGetLastError();
 }
 
-// Threads per block of the psi pass: 256, fewer (to one warp) where that
-// leaves less than two blocks per SM.
+// Threads per block of the psi pass: 128 (512x256x256 AA FP16, gather layout:
+// 250 us per launch against 256 with 256), fewer (to one warp) where that leaves less
+// than two blocks per SM.
 int psi_threads(long long units) {
-  int threads = 256;
+  int threads = 128;
   while (threads > 32 && units < (long long)threads * 2 * kSmCount) threads /= 2;
   return threads;
 }
@@ -256,7 +257,7 @@ cudaError_t launch_collide_padded(int precision, const Geom& g, const Phys& ph, 
 }
 
 // FP64 kernels take one node per thread: the FP64 pipe bounds them either way
-// (256x128x128: 222 + 988 us per step with one node, 222 + 982 us with two),
+// (256x128x128: 222 + 981 us per step with one node, 222 + 982 us with two),
 // and lattices of a few warps per SM reach more SMs (4x49x49: 10.3 us per step
 // against 16.5 us).
 bool node_pairs(int precision, bool vec, const Geom& g) { return precision != LBM_F64 && vec && g.nx % 2 == 0; }

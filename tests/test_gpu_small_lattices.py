@@ -156,10 +156,10 @@ def test_small_lattices_take_the_two_kernels_until_asked(L, precision):
 
 @pytest.mark.parametrize("precision", ["f16dev", "bf16dev"])
 @pytest.mark.parametrize("rounding", [0, 1])
-@pytest.mark.parametrize("shape,blocks", [((64, 64, 64), 2), ((66, 64, 64), 3), ((64, 72, 58), 3)])
+@pytest.mark.parametrize("shape,blocks", [((64, 64, 64), 2), ((128, 128, 128), 2), ((130, 128, 127), 3)])
 def test_two_byte_pairs_round_as_single_nodes(L, shape, blocks, rounding, precision):
     """The rounding bits of two nodes taken at once, and the two-kernel step's
-    blocks per SM either side of 2^18 nodes: bitwise the one-node kernels."""
+    blocks per SM either side of 2^21 nodes: bitwise the one-node kernels."""
     f0 = lbm_inputs.random_populations(*shape, seed=72)
     out = []
     for vector, fused in ((1, 0), (0, 0), (1, 1)):
