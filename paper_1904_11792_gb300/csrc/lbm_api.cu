@@ -418,7 +418,11 @@ int chunk_len(const lbm_ctx* h) {
 // the multiple of chunk_len() from 16 on.  A graph launch costs about
 // 2.7 us between two replays (64x32x32 FP32 and 4x49x49 FP64, 2-step against
 // 50- and 100-step graphs), as much as a kernel of such a step; larger
-// lattices do not feel it and keep the shorter capture.
+// lattices do not feel it and keep the shorter capture.  On small lattices it
+// is captured once the replays it saves in a call, and those done before, come
+// to twice its steps: capturing takes about 5 us a step, as much as two replays
+// (a first call of 100 steps with a diagnostic step in ten took 550 us with
+// the 20-step graph captured at once, 480 with the 10-step one).
 int long_chunk_len(const lbm_ctx* h) {
   const int c = chunk_len(h);
   const bool longer = padded_form(h) ? h->diag_interval == 0 : h->g.chain != 0;
@@ -977,7 +981,11 @@ int lbm_step(lbm_handle h, int n) {
   while (n > 0) {
     if (h->use_graph && !h->kernel_timing && n >= base && h->step % base == 0) {
       const int phase = aa ? 0 : h->cur;
-      const int C = n >= longer ? longer : base;
+      const int C = n >= longer && (h->graph[phase][1] || padded_form(h) ||
+                                    h->replays + n / base - n / longer >= 2 * longer)
+                        ? longer
+                        : base;
+      h->replays += C == base;
       cudaGraphExec_t& ge = h->graph[phase][C != base];
       if (!ge) {
         int rc = capture_chunk(h, phase, C, &ge);

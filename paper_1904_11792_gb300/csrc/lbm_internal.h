@@ -330,6 +330,7 @@ struct lbm_ctx {
   // (AA chunks always start on an even step)
   cudaGraphExec_t graph[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};   // [phase][longer chunk]
   int graph_chunk = 0;            // steps per captured chunk (the shorter one)
+  long long replays = 0;          // of the shorter chunk's graphs
   bool use_graph = true;
   dim3 block{0, 0, 0};
   bool block_asked = false;       // block was given (else auto_block is launched)
