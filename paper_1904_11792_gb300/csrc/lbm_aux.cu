@@ -196,6 +196,24 @@ constexpr int NG = DIAG_NG;  // global partial slots per block
 // slots: 0 mass, 1-3 momentum, 4 volume_w, 5 count, 6 max_u, 7 rho_min,
 // 8 rho_max, 9 bad, 10-11 unused
 
+// The warp's sums of eight values at once: halves of the lanes exchange halves
+// of the values until each lane holds one, 9 FP64 additions instead of 40.
+// Lane l returns the sum of v[l / 4].
+__device__ __forceinline__ double warp_sum8(double v[8], int lane) {
+#pragma unroll
+  for (int o = 16, n = 4; n >= 1; o >>= 1, n >>= 1) {
+    const bool hi = lane & o;
+#pragma unroll
+    for (int m = 0; m < n; ++m) {
+      const double give = hi ? v[m] : v[m + n], keep = hi ? v[m + n] : v[m];
+      v[m] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+    }
+  }
+  double t = v[0];
+  t += __shfl_xor_sync(0xffffffffu, t, 2);
+  return t + __shfl_xor_sync(0xffffffffu, t, 1);
+}
+
 // Row-blocks of the partial kernel with `per_sm` blocks per SM and gx blocks
 // along x: each thread walks rows / (8 row-blocks) rows, and the per-slice
 // partials (row-blocks x nx x 2 doubles) stay small.  A block ends with about
@@ -273,8 +291,14 @@ __global__ void __launch_bounds__(DX* DY, 2) diag_partial_kernel(Geom g, Phys ph
       phi = phi < (C)0 ? (C)0 : (phi > (C)1 ? (C)1 : phi);
       s_vol.add(phi);
       cnt += rho > thr;
-      const C u = sqrt(xfma(jz, jz, xfma(jy, jy, xmul(jx, jx)))) / rho;
-      umax = u > umax ? u : umax;
+      // the root and the division only where |j|/rho can reach the maximum, as
+      // in diag_pair_kernel (FP64 256x128x128, in the loop: 433 -> 369 us per
+      // record beyond the psi pass)
+      const C j2 = xfma(jz, jz, xfma(jy, jy, xmul(jx, jx))), t = umax * rho;
+      if (j2 >= (C)0.999998 * (t * t) || j2 < (C)1e-30) {
+        const C u = sqrt(j2) / rho;
+        umax = u > umax ? u : umax;
+      }
       rmin = rho < rmin ? rho : rmin;
       rmax = rho > rmax ? rho : rmax;
       bad |= !(rho > (C)0) || !(rho <= (C)3.0e38);
@@ -285,15 +309,12 @@ __global__ void __launch_bounds__(DX* DY, 2) diag_partial_kernel(Geom g, Phys ph
   __shared__ double sh_s[2][DY][DX];
   sh_s[0][ty][tx] = s_vol.value();
   sh_s[1][ty][tx] = (double)cnt;
-  // block totals: a fixed FP64 shuffle tree within each warp, then the 8
+  // block totals: FP64 sums within each warp in a fixed order, then the 8
   // warp results in FP64 in warp order
-  double v[5] = {s_mass.value(), s_jx.value(), s_jy.value(), s_jz.value(), s_vol.value()};
-  float c_f = (float)cnt;  // exact below 2^24 nodes per warp
+  double v[8] = {s_mass.value(), s_jx.value(), s_jy.value(), s_jz.value(), s_vol.value(), (double)cnt, 0.0, 0.0};
+  const double sum = warp_sum8(v, tx);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-    for (int k = 0; k < 5; ++k) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
-    c_f += __shfl_down_sync(0xffffffffu, c_f, o);
     const C um = __shfl_down_sync(0xffffffffu, umax, o);
     const C mn = __shfl_down_sync(0xffffffffu, rmin, o);
     const C mx = __shfl_down_sync(0xffffffffu, rmax, o);
@@ -303,13 +324,8 @@ __global__ void __launch_bounds__(DX* DY, 2) diag_partial_kernel(Geom g, Phys ph
   }
   const int anybad = __any_sync(0xffffffffu, bad);
   __shared__ double sh_w[NG][DY];
+  if (tx % 4 == 0 && tx < 24) sh_w[tx / 4][ty] = sum;
   if (tx == 0) {
-    sh_w[0][ty] = v[0];
-    sh_w[1][ty] = v[1];
-    sh_w[2][ty] = v[2];
-    sh_w[3][ty] = v[3];
-    sh_w[4][ty] = v[4];
-    sh_w[5][ty] = (double)c_f;
     sh_w[6][ty] = (double)umax;
     sh_w[7][ty] = (double)rmin;
     sh_w[8][ty] = (double)rmax;
@@ -432,13 +448,10 @@ __global__ void __launch_bounds__(DX* DY, 2) diag_pair_kernel(Geom g, Phys ph, c
   sh_s[0][ty][2 * tx + 1] = w1;
   sh_s[1][ty][2 * tx] = (double)cnt[0];
   sh_s[1][ty][2 * tx + 1] = (double)cnt[1];
-  double v[5] = {s_mass.value(), s_jx.value(), s_jy.value(), s_jz.value(), w0 + w1};
-  float c_f = (float)(cnt[0] + cnt[1]);   // exact below 2^24 nodes per warp
+  double v[8] = {s_mass.value(), s_jx.value(), s_jy.value(), s_jz.value(), w0 + w1, (double)(cnt[0] + cnt[1]), 0.0, 0.0};
+  const double sum = warp_sum8(v, tx);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-    for (int k = 0; k < 5; ++k) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
-    c_f += __shfl_down_sync(0xffffffffu, c_f, o);
     const float um = __shfl_down_sync(0xffffffffu, umax, o);
     const float mn = __shfl_down_sync(0xffffffffu, rmin, o);
     const float mx = __shfl_down_sync(0xffffffffu, rmax, o);
@@ -448,9 +461,8 @@ __global__ void __launch_bounds__(DX* DY, 2) diag_pair_kernel(Geom g, Phys ph, c
   }
   const int anybad = __any_sync(0xffffffffu, bad);
   __shared__ double sh_w[NG][DY];
+  if (tx % 4 == 0 && tx < 24) sh_w[tx / 4][ty] = sum;
   if (tx == 0) {
-    for (int k = 0; k < 5; ++k) sh_w[k][ty] = v[k];
-    sh_w[5][ty] = (double)c_f;
     sh_w[6][ty] = (double)umax;
     sh_w[7][ty] = (double)rmin;
     sh_w[8][ty] = (double)rmax;
@@ -814,24 +826,6 @@ __global__ void trig_kernel(Geom g, double2* trig) {
   double2 v;
   sincospi(2.0 * c / n, &v.y, &v.x);
   trig[t] = v;
-}
-
-// The warp's sums of eight values at once: halves of the lanes exchange halves
-// of the values until each lane holds one, 9 FP64 additions instead of 40.
-// Lane l returns the sum of v[l / 4].
-__device__ __forceinline__ double warp_sum8(double v[8], int lane) {
-#pragma unroll
-  for (int o = 16, n = 4; n >= 1; o >>= 1, n >>= 1) {
-    const bool hi = lane & o;
-#pragma unroll
-    for (int m = 0; m < n; ++m) {
-      const double give = hi ? v[m] : v[m + n], keep = hi ? v[m + n] : v[m];
-      v[m] = keep + __shfl_xor_sync(0xffffffffu, give, o);
-    }
-  }
-  double t = v[0];
-  t += __shfl_xor_sync(0xffffffffu, t, 2);
-  return t + __shfl_xor_sync(0xffffffffu, t, 1);
 }
 
 // A warp walks SEGS segments of 32 consecutive nodes and keeps the sums of

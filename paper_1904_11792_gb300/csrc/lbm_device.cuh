@@ -277,7 +277,7 @@ template <> struct DSum<float> {
 template <> struct DSum<double> {
   double v = 0.0;
   __device__ __forceinline__ void add(double x) { v += x; }
-  __device__ __forceinline__ void add(double x, double xlo) { v += x + xlo; }
+  __device__ __forceinline__ void add(double x, double) { v += x; }   // (rho_of_x: no correction)
   __device__ __forceinline__ double value() const { return v; }
 };
 
