@@ -225,18 +225,18 @@ def measure_lattice(torch, L, autotune, w, precision, patterns, args, rho_l, rho
     import torch.distributed as dist
     dev = precision.endswith("dev")
     if args.no_tune:
-        choice = dict(pattern=patterns[-1], block=(128, 2, 1), occupancy=0, fused=int(args.fused),
+        choice = dict(pattern=patterns[-1], block=(64, 1, 1), occupancy=0, fused=int(args.fused),
                       fused_fz=args.fused_fz, fused_group=args.fused_group)
     elif full_tune:
         choice = autotune.tune_lattice(w.nx, w.ny, w.nz, precision=precision, patterns=patterns,
-                                       blocks=((128, 2, 1), (64, 4, 1), (32, 8, 1)), occupancies=(2, 3),
+                                       blocks=((64, 1, 1), (128, 1, 1), (128, 2, 1)), occupancies=(2, 3),
                                        tau=w.tau, G=w.G, steps=10, use_cache=False)
     else:
         # variants: the fused step's launch shapes where it applies (A-B),
         # two block shapes of the two-kernel step otherwise
         choice = autotune.tune_lattice(w.nx, w.ny, w.nz, precision=precision, patterns=patterns,
-                                       blocks=((128, 2, 1), (64, 4, 1)) if patterns == ("aa",) else
-                                       ((128, 2, 1),),
+                                       blocks=((64, 1, 1), (128, 1, 1)) if patterns == ("aa",) else
+                                       ((64, 1, 1),),
                                        occupancies=(2, 3), tau=w.tau, G=w.G, steps=10, use_cache=False,
                                        fused_runs=(8, 12, 16, 32), fused_groups=(1, 4), reps=2)
     pattern = choice["pattern"]

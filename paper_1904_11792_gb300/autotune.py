@@ -16,8 +16,8 @@ import time
 
 from . import lbm as L
 
-DEFAULT_BLOCKS = ((256, 1, 1), (128, 2, 1), (64, 4, 1), (32, 8, 1), (64, 2, 2), (32, 4, 2),
-                  (128, 1, 2), (32, 2, 4))
+DEFAULT_BLOCKS = ((64, 1, 1), (32, 2, 1), (128, 1, 1), (32, 4, 1), (256, 1, 1), (128, 2, 1), (64, 4, 1),
+                  (32, 8, 1))
 DEFAULT_OCC = (2, 3, 4)
 
 
