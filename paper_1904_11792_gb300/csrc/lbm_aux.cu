@@ -217,9 +217,9 @@ __device__ __forceinline__ double warp_sum8(double v[8], int lane) {
 // Row-blocks of the partial kernel with `per_sm` blocks per SM and gx blocks
 // along x: each thread walks rows / (8 row-blocks) rows, and the per-slice
 // partials (row-blocks x nx x 2 doubles) stay small.  A block ends with about
-// 70 FP64 instructions per warp (warp trees, block sums), which the FP64 pipe
-// of its SM works off at 16 clocks each: with 16 blocks per SM that alone takes
-// 50 us, so the kernels launch 4 per SM, two waves.
+// 50 FP64 instructions per warp (warp and block sums; 70 with a tree per sum),
+// which the FP64 pipe of its SM works off at 16 clocks each: with 16 blocks per
+// SM that alone took 50 us, so the kernels launch 4 per SM, two waves.
 int diag_row_blocks(const Geom& g, long long gx, int per_sm) {
   const long long rows = (long long)g.ny * g.nz;
   long long want = (per_sm * kSmCount + gx - 1) / gx;
