@@ -888,7 +888,7 @@ int lbm_get_option(lbm_handle h, const char* key, double* v) {
   else if (k == "fused_fz_used" || k == "fused_group_used") {
     int fz = 0, grp = 0;
     if (fused_applicable(h->g, h->cfg.precision)) {
-      const cudaError_t e = fused_launch_shape(h->cfg.precision, h->g, h->fused_fz, h->fused_group, &fz, &grp);
+      const cudaError_t e = fused_launch_shape(h->cfg.precision, h->g, h->ph.coll, h->fused_fz, h->fused_group, &fz, &grp);
       if (e != cudaSuccess) return cuda_fail(e, "fused launch shape");
     }
     *v = k == "fused_fz_used" ? fz : grp;

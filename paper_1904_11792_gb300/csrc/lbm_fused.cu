@@ -111,15 +111,18 @@ double run_cost_f32(long long tiles, long long slots, int nz, int fz) {
   return cost * (1.0 + fz / 80.0);
 }
 
-// 2-byte storage (bound by instruction issue): a small simulation of how the
-// blocks run.  They start in launch order (the short last runs last) as slots
-// come free, and all resident blocks progress at the same rate, a plane taking
-// max(R, 0.9 slots) / slots while R blocks are resident; the two planes a run
-// does not collide count 0.8 each; times 1 + fz / 300.  The chosen length is
-// 0.8 % slower than the best one on average, at most 3 %; the rule before 2.6 %,
-// at most 6 % (256x128x128 FP16: 15 planes 88.3 us, 29 planes 84.1 us).
-double run_cost_dev(long long tiles, long long slots, int nz, int fz) {
-  constexpr double h = 0.8;
+// 2-byte storage and the MRT collision (bound by instruction issue): a small
+// simulation of how the blocks run.  They start in launch order (the short last
+// runs last) as slots come free, and all resident blocks progress at the same
+// rate, a plane taking max(R, 0.9 slots) / slots while R blocks are resident;
+// the two planes a run does not collide count h each; times 1 + fz / k.
+// 2-byte storage, h = 0.8, k = 300: the chosen length is 0.8 % slower than the
+// best one on average, at most 3 %; the rule before 2.6 %, at most 6 %
+// (256x128x128 FP16: 15 planes 88.3 us, 29 planes 84.1 us).  FP32 with the MRT
+// collision, h = 1.2, k = 100: 1.3 %, at most 3 % on ten lattices of 0.7 to 10 M
+// nodes; by run_cost_f32 4.2 %, at most 12 % (576x80x83: 9 planes 121 us, 17
+// planes 111 us; 256x128x128: 13 planes 119 us, 19 planes 116 us).
+double run_cost_issue(long long tiles, long long slots, int nz, int fz, double h, double k) {
   struct Group {
     double left;
     long long count;
@@ -151,7 +154,7 @@ double run_cost_dev(long long tiles, long long slots, int nz, int fz) {
     }
     run.resize(keep);
   }
-  return t / slots * (1.0 + fz / 300.0);
+  return t / slots * (1.0 + fz / k);
 }
 
 // z planes per block.  Lattices with more than twice as many tiles as slots
@@ -162,13 +165,14 @@ double run_cost_dev(long long tiles, long long slots, int nz, int fz) {
 // and 4.700 ms).  Others take the run length of the least predicted time, kept
 // per shape (a pure function of its arguments).
 template <int P>
-int choose_fz(const Geom& g, long long tiles, long long slots) {
+int choose_fz(const Geom& g, int coll, long long tiles, long long slots) {
   constexpr bool dev = Prec<P>::dev;
+  const bool mrt32 = !dev && coll == COLL_MRT;
   const bool many = tiles > 2 * slots;
   if (!dev && many) return std::min(g.nz, 8);
   static std::mutex mu;
-  static std::map<std::tuple<long long, long long, int>, int> kept;
-  const auto key = std::make_tuple(tiles, slots, g.nz);
+  static std::map<std::tuple<long long, long long, int, bool>, int> kept;
+  const auto key = std::make_tuple(tiles, slots, g.nz, mrt32);
   std::lock_guard<std::mutex> lock(mu);
   const auto it = kept.find(key);
   if (it != kept.end()) return it->second;
@@ -177,7 +181,9 @@ int choose_fz(const Geom& g, long long tiles, long long slots) {
   for (int fz = best; fz <= (many ? g.nz : std::min(g.nz, 64)); ++fz) {
     const long long waves = (tiles * ((g.nz + fz - 1) / fz) + slots - 1) / slots;
     const double cost = many ? (double)waves * (fz + 2) * (1.0 + fz / 2048.0)
-                             : (dev ? run_cost_dev : run_cost_f32)(tiles, slots, g.nz, fz);
+                        : dev   ? run_cost_issue(tiles, slots, g.nz, fz, 0.8, 300.0)
+                        : mrt32 ? run_cost_issue(tiles, slots, g.nz, fz, 1.2, 100.0)
+                                : run_cost_f32(tiles, slots, g.nz, fz);
     if (best_cost < 0.0 || cost < best_cost) {
       best_cost = cost;
       best = fz;
@@ -246,13 +252,13 @@ cudaError_t fused_device_info(int* slots_per_sm, int* sms) {
 
 // Grid of the fused step: z run length, runs per tile column, blocks.
 template <int P>
-cudaError_t fused_grid(const Geom& g, int fz_req, int grp_req, int* fz, int* nchunks, int* grp,
+cudaError_t fused_grid(const Geom& g, int coll, int fz_req, int grp_req, int* fz, int* nchunks, int* grp,
                        long long* blocks) {
   int slots_per_sm = 0, sms = 0;
   cudaError_t e = fused_device_info<P>(&slots_per_sm, &sms);
   if (e != cudaSuccess) return e;
   const long long tiles = (long long)(g.nx / TX) * (g.ny / FusedShape<P>::TY);
-  *fz = fz_req > 0 ? std::min(fz_req, g.nz) : choose_fz<P>(g, tiles, (long long)slots_per_sm * sms);
+  *fz = fz_req > 0 ? std::min(fz_req, g.nz) : choose_fz<P>(g, coll, tiles, (long long)slots_per_sm * sms);
   *nchunks = (g.nz + *fz - 1) / *fz;
   *blocks = tiles * *nchunks;
   *grp = std::min(grp_req > 0 ? grp_req : choose_grp<P>(g.nx / TX), *nchunks);
@@ -266,7 +272,7 @@ cudaError_t fused_t(const Geom& g, const Phys& ph, const void* src, void* dst, i
   using S = FusedShape<P>;
   int fz = 0, nchunks = 0, grp = 0;
   long long blocks = 0;
-  cudaError_t e = fused_grid<P>(g, fz_req, grp_req, &fz, &nchunks, &grp, &blocks);
+  cudaError_t e = fused_grid<P>(g, ph.coll, fz_req, grp_req, &fz, &nchunks, &grp, &blocks);
   if (e != cudaSuccess) return e;
   Maps m;
   e = maps_for(P, g, src, &m);
@@ -298,8 +304,13 @@ template <int P>
 size_t fused_scratch_t(const Geom& g, int fz_req) {
   int fz = 0, nchunks = 0, grp = 0;
   long long blocks = 0;
-  if (fused_grid<P>(g, fz_req, 0, &fz, &nchunks, &grp, &blocks) != cudaSuccess) return 0;
-  return (size_t)(g.ny / FusedShape<P>::TY) * nchunks * g.nx * 2 + (size_t)blocks * DIAG_NG + (size_t)g.nx * 2;
+  size_t need = 0;   // of either collision's run length
+  for (int coll : {COLL_SRT, COLL_MRT}) {
+    if (fused_grid<P>(g, coll, fz_req, 0, &fz, &nchunks, &grp, &blocks) != cudaSuccess) return 0;
+    need = std::max(need, (size_t)(g.ny / FusedShape<P>::TY) * nchunks * g.nx * 2 + (size_t)blocks * DIAG_NG +
+                              (size_t)g.nx * 2);
+  }
+  return need;
 }
 
 template <int P>
@@ -321,7 +332,7 @@ cudaError_t ragged_t(const Geom& g, const Phys& ph, const void* src, int src_px,
   const int ntx = (g.nx + W - 1) / W;
   const long long tiles = (long long)ntx * ((g.ny + S::TY - 1) / S::TY);
   const int fz =
-      fz_req > 0 ? std::min(fz_req, g.nz) : choose_fz<P>(g, tiles, (long long)slots_per_sm * sms);
+      fz_req > 0 ? std::min(fz_req, g.nz) : choose_fz<P>(g, ph.coll, tiles, (long long)slots_per_sm * sms);
   const int nchunks = (g.nz + fz - 1) / fz;
   if (tiles * nchunks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
   const int grp = std::min(grp_req > 0 ? grp_req : choose_grp<P>(ntx), nchunks);
@@ -361,13 +372,13 @@ cudaError_t launch_ragged(int precision, const Geom& g, const Phys& ph, const vo
   return cudaErrorInvalidValue;
 }
 
-cudaError_t fused_launch_shape(int precision, const Geom& g, int fz_req, int grp_req, int* fz, int* grp) {
+cudaError_t fused_launch_shape(int precision, const Geom& g, int coll, int fz_req, int grp_req, int* fz, int* grp) {
   int nchunks = 0;
   long long blocks = 0;
   switch (precision) {
-    case LBM_F32: return fused_grid<LBM_F32>(g, fz_req, grp_req, fz, &nchunks, grp, &blocks);
-    case LBM_F16DEV: return fused_grid<LBM_F16DEV>(g, fz_req, grp_req, fz, &nchunks, grp, &blocks);
-    case LBM_BF16DEV: return fused_grid<LBM_BF16DEV>(g, fz_req, grp_req, fz, &nchunks, grp, &blocks);
+    case LBM_F32: return fused_grid<LBM_F32>(g, coll, fz_req, grp_req, fz, &nchunks, grp, &blocks);
+    case LBM_F16DEV: return fused_grid<LBM_F16DEV>(g, coll, fz_req, grp_req, fz, &nchunks, grp, &blocks);
+    case LBM_BF16DEV: return fused_grid<LBM_BF16DEV>(g, coll, fz_req, grp_req, fz, &nchunks, grp, &blocks);
   }
   return cudaErrorInvalidValue;
 }

@@ -76,3 +76,23 @@ def test_ragged_step_is_the_default_on_larger_lattices(L):
             lat.set_option("kernel_timing", 1)
             lat.step(4)
             assert L.lbm_kernel_time(lat.h, 2)[0] == want
+
+
+@pytest.mark.parametrize("shape,srt,mrt", [((576, 80, 83), 9, 17), ((128, 96, 101), 12, 11), ((64, 8, 5), 4, 4)])
+def test_run_length_follows_the_collision(L, shape, srt, mrt):
+    """The single pass chooses its run length by the collision; its bits, the
+    diagnostics' scratch and the switch between them do not depend on it."""
+    out = []
+    for fused in (1, 0):
+        with L.Lattice(*shape, 0.95, -5.3, precision="f32") as lat:
+            lat.init_ligament(min(shape[1:]) / 4.0, float(shape[0]), 0.1, 0.3, 2.1085, 0.0778, 2.0)
+            lat.set_option("fused", fused)
+            lat.set_option("diag_interval", 3)
+            for collision, fz in ((1, mrt), (0, srt), (1, mrt)):
+                lat.set_option("collision", collision)
+                assert lat.get_option("fused_fz_used") == fz
+                lat.step(4)
+            lat.sync()
+            out.append((lat.populations(), [d["mass"] for d in lat.diag_history()]))
+    np.testing.assert_array_equal(out[0][0], out[1][0])
+    np.testing.assert_allclose(out[0][1], out[1][1], rtol=1e-13)   # FP64 sums of N < 2^22 terms
