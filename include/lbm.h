@@ -177,7 +177,7 @@ int lbm_set_stream(lbm_handle h, void *stream);
  * free device memory, else not at all).  Everything else is the two-kernel
  * step; results equal it bitwise), "fused_fz" (z planes
  * each block of the fused step marches through; 0 = chosen from the lattice
- * size and the GPU, the default), "fused_group" (the fused step launches
+ * size, the collision and the GPU, the default), "fused_group" (the fused step launches
  * its blocks in groups of this many consecutive z runs, the run varying
  * fastest inside a group, then the tile x, then the tile y; 0 = one run
  * per 4 tile columns of 64 nodes (FP32; one run for 2-byte storage), at
