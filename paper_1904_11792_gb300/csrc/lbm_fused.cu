@@ -93,22 +93,23 @@ template <int P> constexpr int kRaggedW = Prec<P>::dev ? 32 : TX;
 
 // Predicted time of a launch with z runs of fz planes on `tiles` tiles.  Unit:
 // a plane collided by one block while every slot is taken.  Both forms were
-// fitted to the times of 38 run lengths on 14 lattices of 0.5 to 34 M nodes.
+// fitted to the times of 15 to 38 run lengths on 30 (FP32) and 14 lattices of
+// 0.7 to 34 M nodes.
 //
 // FP32 (bound by HBM): whole waves take their blocks' mean cost, where the two
-// planes a run loads but does not collide count 0.6 each; the last wave what
-// its blocks cost at full bandwidth, but at least 0.75 of its planes' latency;
-// times 1 + fz / 80, because the longer a run, the further apart in time
-// neighbouring tiles read the rows they share.  The chosen length is 3.1 %
+// planes a run loads but does not collide count one each; the last wave what
+// its blocks cost at full bandwidth, but at least 0.85 of its planes' latency;
+// times 1 + fz / 50, because the longer a run, the further apart in time
+// neighbouring tiles read the rows they share.  The chosen length is 2.1 %
 // slower than the best one on average, at most 11 %; whole waves x (fz + 2) x
-// (1 + fz / 256), the rule before, 6.6 %, at most 20 % (256x110x112: 28 planes
-// 104.7 us, 10 planes 87.1 us).
+// (1 + fz / 256), the rule before, 6.5 %, at most 20 % (256x110x112: 28 planes
+// 104.7 us, 10 planes 87.1 us), and on none of them more than 1.6 % faster.
 double run_cost_f32(long long tiles, long long slots, int nz, int fz) {
   const long long blocks = tiles * ((nz + fz - 1) / fz), waves = blocks / slots, last = blocks - waves * slots;
-  const double mean = (double)tiles * nz / blocks + 1.2;
+  const double mean = (double)tiles * nz / blocks + 2.0;
   double cost = waves * mean;
-  if (last) cost += std::max(mean * last / slots, 0.75 * (fz + 2));
-  return cost * (1.0 + fz / 80.0);
+  if (last) cost += std::max(mean * last / slots, 0.85 * (fz + 2));
+  return cost * (1.0 + fz / 50.0);
 }
 
 // 2-byte storage and the MRT collision (bound by instruction issue): a small
@@ -265,6 +266,13 @@ cudaError_t fused_grid(const Geom& g, int coll, int fz_req, int grp_req, int* fz
   return *blocks > 0x7fffffffLL ? cudaErrorInvalidConfiguration : cudaSuccess;
 }
 
+// The steps are launched chained (Geom::chain) only where the blocks of two of
+// them are resident at once.  Else the next step's first blocks take the places
+// this one leaves, wherever they are, the rest comes as places fall free, and
+// the SMs are unevenly loaded (192x80x68 FP32, 300 blocks on 456 places: 34.3 us
+// per step chained, 30.0 plainly; 256x64x64, 448 blocks: 31.1 / 29.3).
+inline int chain_steps(const Geom& g, long long blocks, long long slots) { return g.chain && 2 * blocks <= slots; }
+
 template <int P>
 cudaError_t fused_t(const Geom& g, const Phys& ph, const void* src, void* dst, int* flag, int fz_req,
                     int grp_req, const FusedDiag* diag, unsigned long long stall_ns, cudaStream_t s,
@@ -273,7 +281,10 @@ cudaError_t fused_t(const Geom& g, const Phys& ph, const void* src, void* dst, i
   int fz = 0, nchunks = 0, grp = 0;
   long long blocks = 0;
   cudaError_t e = fused_grid<P>(g, ph.coll, fz_req, grp_req, &fz, &nchunks, &grp, &blocks);
+  int slots_per_sm = 0, sms = 0;
+  if (e == cudaSuccess) e = fused_device_info<P>(&slots_per_sm, &sms);
   if (e != cudaSuccess) return e;
+  const int chain = chain_steps(g, blocks, (long long)slots_per_sm * sms);
   Maps m;
   e = maps_for(P, g, src, &m);
   if (e != cudaSuccess) return e;
@@ -283,7 +294,7 @@ cudaError_t fused_t(const Geom& g, const Phys& ph, const void* src, void* dst, i
   for (int a = 0; a < Q; ++a) db.p[a] = (T*)dst + (long long)a * g.N;
   if (!diag) {
     const DiagOut none = diag_out(0.0, 0.0, nullptr, nullptr, stall_ns);
-    return chain_launch(g.chain, ph.coll == COLL_MRT ? fused_kernel<P, false, COLL_MRT> : fused_kernel<P, false, COLL_SRT>,
+    return chain_launch(chain, ph.coll == COLL_MRT ? fused_kernel<P, false, COLL_MRT> : fused_kernel<P, false, COLL_SRT>,
                         (unsigned)blocks, S::NT, S::smem, s, m, g, ph, (T*)dst, flag, ntx, nchunks, fz, grp, none, db);
   }
   const long long row_blocks = (long long)(g.ny / S::TY) * nchunks;
@@ -293,7 +304,7 @@ cudaError_t fused_t(const Geom& g, const Phys& ph, const void* src, void* dst, i
   double* bl = slices + (size_t)row_blocks * g.nx * 2;
   double* slice_tot = bl + (size_t)blocks * DIAG_NG;
   const DiagOut dg = diag_out(diag->rho_l, diag->rho_v, slices, bl, stall_ns);
-  e = chain_launch(g.chain, ph.coll == COLL_MRT ? fused_kernel<P, true, COLL_MRT> : fused_kernel<P, true, COLL_SRT>,
+  e = chain_launch(chain, ph.coll == COLL_MRT ? fused_kernel<P, true, COLL_MRT> : fused_kernel<P, true, COLL_SRT>,
                    (unsigned)blocks, S::NT, S::smem, s, m, g, ph, (T*)dst, flag, ntx, nchunks, fz, grp, dg, db);
   if (e != cudaSuccess) return e;
   return launch_diag_reduce(g, (int)row_blocks, (int)blocks, slices, bl, slice_tot, diag->out, diag->ring_count,
@@ -345,7 +356,8 @@ cudaError_t ragged_t(const Geom& g, const Phys& ph, const void* src, int src_px,
   const auto kernel = ph.coll == COLL_MRT
                           ? (odd ? ragged_kernel<P, COLL_MRT, W, true> : ragged_kernel<P, COLL_MRT, W, false>)
                           : (odd ? ragged_kernel<P, COLL_SRT, W, true> : ragged_kernel<P, COLL_SRT, W, false>);
-  return chain_launch(g.chain, kernel, (unsigned)(tiles * nchunks), S::NT, S::smem, s, m, g, ph, flag, ntx, nchunks, fz,
+  const int chain = chain_steps(g, tiles * nchunks, (long long)slots_per_sm * sms);
+  return chain_launch(chain, kernel, (unsigned)(tiles * nchunks), S::NT, S::smem, s, m, g, ph, flag, ntx, nchunks, fz,
                       grp, dst_px, dstride, db);
 }
 
