@@ -38,8 +38,10 @@ dim3 default_block(const Geom& g) {
 // shorter than a warp are not padded to one: the block takes whole rows of
 // several y and z, so a warp's lanes all hold nodes (4x49x49 FP64, whose pipe a
 // warp instruction occupies for 16 clocks whatever its live lanes: 68 us per
-// step in 32 x 8 blocks, 2 of 32 lanes live, 10.3 us in 4 x 8 x 1).
-dim3 auto_block(const Geom& g, bool pairs, int precision) {
+// step in 32 x 8 blocks, 2 of 32 lanes live, 10.3 us in 4 x 8 x 1).  More rows
+// than 65535 such blocks take (the limit of a grid along y) go in the default
+// shape, whose blocks hold up to 8.
+static dim3 small_block(const Geom& g, bool pairs, int precision) {
   const unsigned ux = pairs ? g.nx / 2 : g.nx;
   const long long units = (long long)ux * g.ny * g.nz;
   const unsigned threads = units < 64LL * 2 * kSmCount ? 32 : 64;
@@ -51,6 +53,10 @@ dim3 auto_block(const Geom& g, bool pairs, int precision) {
   const unsigned by = std::min<unsigned>(g.ny, std::max(1u, threads / ux));
   const unsigned bz = std::min<unsigned>(std::min(g.nz, 64), std::max(1u, threads / (ux * by)));
   return dim3(ux, by, bz);
+}
+dim3 auto_block(const Geom& g, bool pairs, int precision) {
+  const dim3 b = small_block(g, pairs, precision);
+  return (g.ny + b.y - 1) / b.y > 65535 ? default_block(g) : b;
 }
 }  // namespace lbm
 

@@ -1,0 +1,43 @@
+"""Lattices at the limits of launches and memory, and calls after one that
+failed: what is accepted there, and that nothing of a failed call stays."""
+import gc
+
+import numpy as np
+import pytest
+
+import lbm_inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def L():
+    from paper_1904_11792_gb300 import build, lbm
+    build.build()
+    lbm.load()
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    return lbm
+
+
+# More rows than a grid has blocks along y (65535): rows of several warps, which
+# the automatic blocks of two warps would take one at a time.  Even nx in pairs
+# and odd in single nodes, both collisions, and the step into padded rows (251
+# nodes, from the second step of a replayed graph on).
+@pytest.mark.parametrize("shape,precision,pattern,mrt", [
+    ((64, 70000, 3), "f64", "ab", 0), ((64, 70000, 3), "f64", "aa", 1), ((128, 70000, 3), "f32", "aa", 0),
+    ((256, 65536, 3), "f32", "ab", 0), ((128, 70000, 3), "f16dev", "aa", 1), ((251, 65537, 3), "f32", "ab", 0)])
+def test_more_rows_than_a_grid_takes(L, shape, precision, pattern, mrt):
+    import torch
+    out = []
+    for block in (None, (32, 8, 1)):
+        with L.Lattice(*shape, 0.9, -5.5, precision=precision, pattern=pattern, block=block, rho_ref=0.1) as lat:
+            lat.set_option("collision", mrt)
+            if block or shape[0] % 64 == 0:
+                lat.set_option("fused", 0)
+            lat.init_ligament(5000.0, float(shape[0]), 0.01, 0.3, 2.1, 0.1, 20.0)
+            lat.step(4)
+            lat.sync()
+            n = 19 * shape[0] * shape[1] * shape[2]     # the first array holds the state
+            out.append(lat._buffers[0].view({"f64": torch.float64, "f32": torch.float32}.get(precision, torch.float16))[:n].clone())
+    assert torch.equal(out[0], out[1])
