@@ -69,7 +69,11 @@ int fail(int status, const std::string& msg) {
   return status;
 }
 
+// The error is reported by this call alone: the runtime keeps the last one
+// until it is read, and a later check of a launch (here or in the caller's
+// program) would take it for its own.
 int cuda_fail(cudaError_t e, const char* where) {
+  (void)cudaGetLastError();
   g_last_error = std::string(where) + ": " + cudaGetErrorString(e);
   return e == cudaErrorMemoryAllocation ? LBM_ERR_OOM : LBM_ERR_CUDA;
 }
@@ -468,6 +472,7 @@ int capture_chunk(lbm_ctx* h, int phase, int steps, cudaGraphExec_t* exec) {
   if (cs) cudaStreamDestroy(cs);
   if (rc != LBM_OK || e != cudaSuccess) {
     if (graph) cudaGraphDestroy(graph);
+    (void)cudaGetLastError();   // of ending a capture that a failed launch had spoilt
     return rc != LBM_OK ? rc : cuda_fail(e, "graph capture of the steps");
   }
   e = cudaGraphInstantiate(exec, graph, 0);

@@ -514,6 +514,7 @@ int capture_steps(lbm_batch_ctx* b, int phase, int steps, cudaGraphExec_t* exec)
   cudaStreamDestroy(cs);
   if (rc != LBM_OK) {
     if (g) cudaGraphDestroy(g);
+    (void)cudaGetLastError();   // of ending a capture that a failed launch had spoilt
     return rc;
   }
   if (e != cudaSuccess) return bcuda(e, "batch graph capture");
@@ -553,6 +554,7 @@ int bfail(int status, const std::string& m) {
 }
 
 int bcuda(cudaError_t e, const char* where) {
+  (void)cudaGetLastError();   // reported here, not by the next check of a launch
   b_err = std::string(where) + ": " + cudaGetErrorString(e);
   return e == cudaErrorMemoryAllocation ? LBM_ERR_OOM : LBM_ERR_CUDA;
 }

@@ -29,6 +29,7 @@ double* g_scratch_ptr[kMaxDevices] = {};
 thread_local std::string g_err;
 
 int nfail(int status, const std::string& m) {
+  if (status == LBM_ERR_CUDA) (void)cudaGetLastError();   // reported here, not by the next check of a launch
   g_err = m;
   return status;
 }

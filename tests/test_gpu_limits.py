@@ -41,3 +41,21 @@ def test_more_rows_than_a_grid_takes(L, shape, precision, pattern, mrt):
             n = 19 * shape[0] * shape[1] * shape[2]     # the first array holds the state
             out.append(lat._buffers[0].view({"f64": torch.float64, "f32": torch.float32}.get(precision, torch.float16))[:n].clone())
     assert torch.equal(out[0], out[1])
+
+
+# A launch that the device refuses (blocks of one node, more rows than a grid
+# takes) fails the call, and only that one.
+def test_a_refused_launch_fails_one_call(L):
+    import torch
+    with L.Lattice(4, 70000, 3, 0.9, -5.5, precision="f64", block=(1, 1, 1)) as lat:
+        lat.init_ligament(5000.0, 4.0, 0.01, 0.3, 2.1, 0.1, 20.0)
+        lat.set_option("graph", 0)
+        with pytest.raises(L.LbmError) as ei:
+            lat.step(1)
+        assert ei.value.status == L.LBM_ERR_CUDA
+        torch.zeros(3, device="cuda").add_(1)       # torch checks the last CUDA error
+        rho = lat.rho()
+        lat.set_option("block_y", 8)
+        lat.step(1)
+        lat.sync()
+        assert abs(lat.rho().sum() / rho.sum() - 1) < 1e-12
