@@ -1284,6 +1284,8 @@ int lbm_load_state(lbm_handle h, const void* host, size_t bytes) {
   h->cur = 0;
   h->step = hd.step;
   CK(launch_salt((unsigned*)(h->d_flag + 2 + salt_word(h, h->step, h->cur)), true, (unsigned)hd.step, h->stream));
+  // the in-loop diagnostics capture the densities
+  if (hd.rho_l != h->rho_l || hd.rho_v != h->rho_v) drop_graphs(h);
   h->rho_l = hd.rho_l;
   h->rho_v = hd.rho_v;
   CK(cudaMemcpyAsync(array_ptr(h, 0), (const char*)host + sizeof(hd), need - sizeof(hd),

@@ -59,3 +59,25 @@ def test_a_refused_launch_fails_one_call(L):
         lat.step(1)
         lat.sync()
         assert abs(lat.rho().sum() / rho.sum() - 1) < 1e-12
+
+
+# A state brings the densities that tell liquid from vapour: steps recorded
+# after loading it use them, replayed or not.
+@pytest.mark.parametrize("shape,fused", [((64, 16, 12), 1), ((40, 12, 10), 0)])
+@pytest.mark.parametrize("ccl", [0, 1])
+def test_loaded_densities_reach_replayed_diagnostics(L, shape, fused, ccl):
+    with L.Lattice(*shape, 1.0, -5.3) as lat:
+        lat.init_ligament(3.0, float(shape[0]), 0.1, 0.3, 2.1085, 0.0778, 2.0)
+        saved = lat.save_state()
+    out = []
+    for graph in (1, 0):
+        with L.Lattice(*shape, 1.0, -5.3) as lat:
+            for k, v in (("fused", fused), ("graph", graph), ("diag_ccl", ccl), ("diag_interval", 2)):
+                lat.set_option(k, v)
+            lat.init_ligament(3.0, float(shape[0]), 0.1, 0.3, 0.3, 0.2, 2.0)
+            lat.step(4)
+            lat.load_state(saved)
+            lat.step(4)
+            out.append(lat.diag_history())
+    assert out[0] == out[1]
+    assert out[0][0]["liquid_volume_w"] != out[0][2]["liquid_volume_w"]
