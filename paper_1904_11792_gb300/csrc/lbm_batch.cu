@@ -527,6 +527,19 @@ int capture_steps(lbm_batch_ctx* b, int phase, int steps, cudaGraphExec_t* exec)
   return LBM_OK;
 }
 
+// Room for n elements in place of the *count at *p; nothing (and a count of
+// zero) where the allocation fails.
+template <typename T>
+cudaError_t grow(T** p, size_t* count, size_t n) {
+  cudaFree(*p);
+  *p = nullptr;
+  *count = 0;
+  if (alloc_over_cap(sizeof(T) * n)) return cudaErrorMemoryAllocation;
+  const cudaError_t e = cudaMalloc(p, sizeof(T) * n);
+  if (e == cudaSuccess) *count = n;
+  return e;
+}
+
 // A single-lattice view (geometry, physics, current array) of instance k.
 struct View {
   Geom g;
@@ -946,20 +959,14 @@ int lbm_batch_diagnostics(lbm_batch b, int k, lbm_diag* out, int want_ccl) {
   View v = view_of(b, k);
   const size_t need = diag_scratch_doubles(v.g);
   if (need > b->scratch_doubles) {
-    cudaFree(b->d_scratch);
-    b->d_scratch = nullptr;
-    BCK(cudaMalloc(&b->d_scratch, sizeof(double) * need));
-    b->scratch_doubles = need;
+    BCK(grow(&b->d_scratch, &b->scratch_doubles, need));
   }
   const lbm_instance& s = b->spec[k];
   const double thr = 0.5 * (s.rho_l + s.rho_v);
   DiagExtra x;
   if (want_ccl) {
     if ((size_t)(2 * v.g.N) > b->labels_ints) {
-      cudaFree(b->d_labels);
-      b->d_labels = nullptr;
-      BCK(cudaMalloc(&b->d_labels, sizeof(int) * 2 * b->max_nodes));
-      b->labels_ints = 2 * b->max_nodes;
+      BCK(grow(&b->d_labels, &b->labels_ints, 2 * (size_t)b->max_nodes));
     }
     x = diag_labels(b->precision, LAYOUT_LOCAL, v.g, v.f, nullptr, thr, b->d_labels, b->d_labels + v.g.N);
   }

@@ -81,3 +81,27 @@ def test_loaded_densities_reach_replayed_diagnostics(L, shape, fused, ccl):
             out.append(lat.diag_history())
     assert out[0] == out[1]
     assert out[0][0]["liquid_volume_w"] != out[0][2]["liquid_volume_w"]
+
+
+# A growth of the diagnostics' scratch or labels that fails leaves the batch
+# without them, not with the size they had: smaller instances get their own.
+def test_batch_diagnostics_after_a_failed_growth(L, monkeypatch):
+    insts = [dict(nx=nx, ny=n, nz=n, tau=0.9, G=-5.5, R0=n / 4.0, lam=float(nx), eps=0.1, phase=0.0, rho_l=2.5,
+                  rho_v=0.15, width=2.0) for nx, n in ((8, 8), (64, 32))]
+    with L.Batch(insts) as b:
+        b.init()
+        want = [b.diagnostics(0), b.diagnostics(0, True)]
+    with L.Batch(insts) as b:
+        b.init()
+        assert b.diagnostics(0) == want[0]
+        monkeypatch.setenv("LBM_ALLOC_CAP_BYTES", str(1 << 16))    # 2 KB of scratch fit, 157 KB do not
+        for ccl in (False, True):
+            with pytest.raises(L.LbmError) as ei:
+                b.diagnostics(1, ccl)
+            assert ei.value.status == L.LBM_ERR_OOM
+            assert b.diagnostics(0) == want[0]
+        with pytest.raises(L.LbmError):
+            b.diagnostics(0, True)                                 # labels for the largest instance
+        monkeypatch.delenv("LBM_ALLOC_CAP_BYTES")
+        assert b.diagnostics(0, True) == want[1]
+        assert b.diagnostics(1, True)["numeric_ok"] == 1
