@@ -505,8 +505,9 @@ int ensure_labels(lbm_ctx* h) {
 }
 
 int ensure_ring(lbm_ctx* h) {
-  if (h->d_ring) return LBM_OK;
-  int rc = dev_alloc((void**)&h->d_ring, sizeof(double) * DIAG_STRIDE * lbm_ctx::kRing, "diagnostics ring");
+  if (h->d_ring_count) return LBM_OK;   // (allocated last)
+  int rc = h->d_ring ? LBM_OK
+                     : dev_alloc((void**)&h->d_ring, sizeof(double) * DIAG_STRIDE * lbm_ctx::kRing, "diagnostics ring");
   if (rc) return rc;
   rc = dev_alloc((void**)&h->d_ring_count, sizeof(unsigned long long), "ring counter");
   if (rc) return rc;

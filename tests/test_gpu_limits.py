@@ -105,3 +105,35 @@ def test_batch_diagnostics_after_a_failed_growth(L, monkeypatch):
         monkeypatch.delenv("LBM_ALLOC_CAP_BYTES")
         assert b.diagnostics(0, True) == want[1]
         assert b.diagnostics(1, True)["numeric_ok"] == 1
+
+
+# Asking for in-loop diagnostics with too little memory for the last of their
+# buffers fails; asked again with enough, they work.
+def test_in_loop_diagnostics_after_a_failed_start(L, monkeypatch):
+    gc.collect()
+    shape, f0 = (8, 6, 5), lbm_inputs.random_populations(8, 6, 5, seed=94)
+
+    def asked(cap):
+        monkeypatch.setenv("LBM_ALLOC_CAP_BYTES", str(cap))
+        lat = L.Lattice(*shape, 0.9, -5.5)
+        try:
+            lat.set_option("diag_interval", 1)
+            return lat, True
+        except L.LbmError as e:
+            assert e.status == L.LBM_ERR_OOM
+            return lat, False
+
+    lo, hi = 1 << 10, 1 << 20
+    while hi - lo > 1:
+        mid = (lo + hi) // 2
+        lat, ok = asked(mid)
+        lat.close()
+        lo, hi = (lo, mid) if ok else (mid, hi)
+    lat, ok = asked(lo)
+    assert not ok
+    monkeypatch.delenv("LBM_ALLOC_CAP_BYTES")
+    with lat:
+        lat.set_populations(f0)
+        lat.set_option("diag_interval", 1)
+        lat.step(3)
+        assert [r["step"] for r in lat.diag_history()] == [0, 1, 2]
