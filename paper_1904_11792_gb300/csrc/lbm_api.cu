@@ -2,10 +2,12 @@
 // life cycle, device memory, the stream, CUDA-graph replay of the time step,
 // kernel timing, checkpoints and the host side of diagnostics.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <string>
 
@@ -84,22 +86,56 @@ int cuda_fail(cudaError_t e, const char* where) {
     if (e_ != cudaSuccess) return cuda_fail(e_, #call); \
   } while (0)
 
-// Device allocation with an optional cap (environment LBM_ALLOC_CAP_BYTES)
-// so that out-of-memory handling can be exercised without exhausting a GPU.
-size_t g_alloc_total = 0;
-
-int dev_alloc(void** p, size_t bytes, const char* what) {
+// Bytes that the lattices hold, and whether `bytes` more exceed the optional cap
+// (environment LBM_ALLOC_CAP_BYTES: out-of-memory handling without exhausting a GPU).
+std::atomic<size_t> g_alloc_total{0};
+bool over_total_cap(size_t bytes) {
   const char* cap = std::getenv("LBM_ALLOC_CAP_BYTES");
-  if (cap && *cap) {
-    const unsigned long long c = std::strtoull(cap, nullptr, 10);
-    if (g_alloc_total + bytes > c)
-      return fail(LBM_ERR_OOM, std::string("allocation of ") + what + " exceeds LBM_ALLOC_CAP_BYTES");
+  return cap && *cap && g_alloc_total + bytes > std::strtoull(cap, nullptr, 10);
+}
+
+std::mutex g_spare_mu;
+Spare* g_spares = nullptr;   // those that hold memory
+
+// Takes s from the list and frees its memory (under the lock).
+void spare_drop(Spare& s) {
+  for (Spare** at = &g_spares; *at; at = &(*at)->next)
+    if (*at == &s) {
+      *at = s.next;
+      break;
+    }
+  if (s.p) cudaFree(s.p);
+  g_alloc_total -= s.bytes;
+  s.p = nullptr;
+  s.bytes = 0;
+}
+
+// Frees the idle Spares of the current device; whether there were any.
+bool spares_give_back() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  std::lock_guard<std::mutex> lock(g_spare_mu);
+  bool any = false;
+  for (Spare* s = g_spares; s;) {
+    Spare* const next = s->next;
+    if (!s->busy && s->device == dev) {
+      if (!any) cudaDeviceSynchronize();   // work of earlier calls may still use them
+      spare_drop(*s);
+      any = true;
+    }
+    s = next;
   }
-  cudaError_t e = cudaMalloc(p, bytes);
-  if (e != cudaSuccess) {
-    *p = nullptr;
-    return cuda_fail(e, what);
-  }
+  return any;
+}
+
+// A lattice's device allocation, under the cap.
+int dev_alloc(void** p, size_t bytes, const char* what) {
+  bool capped = over_total_cap(bytes);
+  if (capped && spares_give_back()) capped = over_total_cap(bytes);
+  *p = nullptr;
+  if (capped) return fail(LBM_ERR_OOM, std::string("allocation of ") + what + " exceeds LBM_ALLOC_CAP_BYTES");
+  const cudaError_t e = device_alloc(p, bytes);
+  if (e != cudaSuccess) return cuda_fail(e, what);
   g_alloc_total += bytes;
   return LBM_OK;
 }
@@ -537,22 +573,21 @@ void fill_diag(lbm_diag* out, const double* r, long long step) {
 }
 
 // Room for `planes` FP64 planes on their way to or from the host (fewer where
-// they exceed 64 MiB); end_transfer gives back what is larger than that.
+// they exceed 64 MiB or are refused), used until end_transfer, which gives back
+// what is larger than 64 MiB.
 int begin_transfer(lbm_ctx* h, int planes) {
-  const size_t need = transfer_doubles(h->g.N, planes);
-  if (h->transfer_n >= need) return LBM_OK;
-  dev_free(h->d_transfer, h->transfer_n * sizeof(double));
-  h->d_transfer = nullptr;
-  h->transfer_n = 0;
-  const int rc = dev_alloc((void**)&h->d_transfer, need * sizeof(double), "transfer planes");
-  if (rc == LBM_OK) h->transfer_n = need;
-  return rc;
+  spare_enter(h->transfer);
+  const cudaError_t e = transfer_room(h->transfer, h->g.N, planes, true);
+  if (e == cudaSuccess) return LBM_OK;
+  spare_leave(h->transfer);
+  if (e != cudaErrorMemoryAllocation) return cuda_fail(e, "transfer planes");
+  return fail(LBM_ERR_OOM, over_total_cap((size_t)h->g.N * sizeof(double))
+                               ? "allocation of transfer planes exceeds LBM_ALLOC_CAP_BYTES"
+                               : "transfer planes: out of memory");
 }
 void end_transfer(lbm_ctx* h) {
-  if (h->transfer_n <= ((size_t)8 << 20)) return;
-  dev_free(h->d_transfer, h->transfer_n * sizeof(double));
-  h->d_transfer = nullptr;
-  h->transfer_n = 0;
+  if (h->transfer.bytes > (size_t)64 << 20) spare_free(h->transfer);
+  spare_leave(h->transfer);
 }
 
 size_t trig_bytes(const Geom& g) { return sizeof(double2) * ((size_t)g.nx + g.ny + g.nz); }
@@ -640,7 +675,7 @@ void lbm_destroy(lbm_handle h) {
   dev_free(h->d_small, sizeof(double) * 64);
   dev_free(h->d_scratch, h->scratch_doubles * sizeof(double));
   for (void* p : h->pad) dev_free(p, h->pad_bytes);
-  dev_free(h->d_transfer, h->transfer_n * sizeof(double));
+  spare_free(h->transfer);
   dev_free(h->d_labels, (size_t)h->g.N * 2 * sizeof(int));
   dev_free(h->d_drop, h->drop_bytes);
   dev_free(h->d_trig, trig_bytes(h->g));
@@ -1086,11 +1121,12 @@ int lbm_moments(lbm_handle h, double* rho, double* ux, double* uy, double* uz) {
   if (rc) return rc;
   // the requested fields together where the planes hold them, else one by one
   const long long N = h->g.N;
-  const bool together = h->transfer_n >= (size_t)want * N;
+  double* const room = (double*)h->transfer.p;
+  const bool together = h->transfer.bytes >= (size_t)want * N * sizeof(double);
   cudaError_t e = cudaSuccess;
   double* dev[4] = {nullptr, nullptr, nullptr, nullptr};
   for (int k = 0, n = 0; k < 4; ++k)
-    if (outs[k]) dev[k] = h->d_transfer + (together ? (n++) * N : 0);
+    if (outs[k]) dev[k] = room + (together ? (n++) * N : 0);
   if (together)
     e = launch_moments(h->cfg.precision, layout, h->g, h->ph, f, h->psi, dev[0], dev[1], dev[2], dev[3], h->stream);
   for (int k = 0; k < 4 && e == cudaSuccess; ++k) {
@@ -1221,8 +1257,8 @@ int lbm_get_populations(lbm_handle h, double* host) {
   if (!h || !host) return fail(LBM_ERR_ARG, "null argument");
   int rc = begin_transfer(h, Q);
   if (rc) return rc;
-  const cudaError_t e = export_populations(h->cfg.precision, cur_layout(h), h->g, h->ph, cur_array(h), h->d_transfer,
-                                           h->transfer_n, host, h->stream);
+  const cudaError_t e = export_populations(h->cfg.precision, cur_layout(h), h->g, h->ph, cur_array(h),
+                                           (double*)h->transfer.p, h->transfer.bytes / sizeof(double), host, h->stream);
   end_transfer(h);
   return e == cudaSuccess ? LBM_OK : cuda_fail(e, "get_populations");
 }
@@ -1231,8 +1267,8 @@ int lbm_set_populations(lbm_handle h, const double* host) {
   if (!h || !host) return fail(LBM_ERR_ARG, "null argument");
   int rc = begin_transfer(h, Q);
   if (rc) return rc;
-  const cudaError_t e = import_populations(h->cfg.precision, cur_layout(h), h->g, h->ph, cur_array(h), h->d_transfer,
-                                           h->transfer_n, host, h->stream);
+  const cudaError_t e = import_populations(h->cfg.precision, cur_layout(h), h->g, h->ph, cur_array(h),
+                                           (double*)h->transfer.p, h->transfer.bytes / sizeof(double), host, h->stream);
   end_transfer(h);
   if (e != cudaSuccess) return cuda_fail(e, "set_populations");
   h->initialized = true;
@@ -1314,5 +1350,51 @@ bool alloc_over_cap(size_t bytes) {
   const char* cap = std::getenv("LBM_ALLOC_CAP_BYTES");
   return cap && *cap && bytes > std::strtoull(cap, nullptr, 10);
 }
-}  // namespace lbm
 
+void spare_enter(Spare& s) {
+  std::lock_guard<std::mutex> lock(g_spare_mu);
+  s.busy = true;
+}
+void spare_leave(Spare& s) {
+  std::lock_guard<std::mutex> lock(g_spare_mu);
+  s.busy = false;
+}
+void spare_free(Spare& s) {
+  std::lock_guard<std::mutex> lock(g_spare_mu);
+  spare_drop(s);
+}
+cudaError_t spare_alloc(Spare& s, size_t bytes, bool capped) {
+  std::lock_guard<std::mutex> lock(g_spare_mu);
+  spare_drop(s);
+  if (capped && over_total_cap(bytes)) return cudaErrorMemoryAllocation;
+  cudaError_t e = cudaGetDevice(&s.device);
+  if (e == cudaSuccess) e = cudaMalloc(&s.p, bytes);
+  if (e != cudaSuccess) {
+    (void)cudaGetLastError();
+    s.p = nullptr;
+    return e;
+  }
+  g_alloc_total += bytes;
+  s.bytes = bytes;
+  s.next = g_spares;
+  g_spares = &s;
+  return cudaSuccess;
+}
+cudaError_t transfer_room(Spare& s, long long N, int planes, bool capped) {
+  const size_t all = sizeof(double) * transfer_doubles(N, planes), one = sizeof(double) * (size_t)N;
+  if (s.bytes >= all) return cudaSuccess;
+  cudaError_t e = spare_alloc(s, all, true);
+  if (e == cudaErrorMemoryAllocation) e = spare_alloc(s, one, capped);
+  if (e == cudaErrorMemoryAllocation && spares_give_back()) e = spare_alloc(s, one, capped);
+  return e;
+}
+cudaError_t device_alloc(void** p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation && spares_give_back()) {
+    (void)cudaGetLastError();
+    e = cudaMalloc(p, bytes);
+  }
+  if (e != cudaSuccess) *p = nullptr;
+  return e;
+}
+}  // namespace lbm

@@ -280,7 +280,7 @@ struct lbm_batch_ctx {
   size_t scratch_doubles = 0;
   int* d_labels = nullptr;
   size_t labels_ints = 0;
-  double* d_plane = nullptr;
+  Spare planes;                    // FP64 planes on their way to the host
   long long max_nodes = 0, total_nodes = 0;
   int tiles = 0, psi_blocks = 0;
   dim3 block{32, 8, 1};
@@ -444,11 +444,11 @@ int ensure_padded(lbm_batch_ctx* b) {
       off += 2LL * Q * b->px[k] * g.ny * g.nz;   // a multiple of al: every instance starts on 16 bytes
     }
     if (alloc_over_cap((size_t)off * e)) return bfail(LBM_ERR_OOM, "the padded pool exceeds LBM_ALLOC_CAP_BYTES");
-    BCK(cudaMalloc(&b->pool_p, (size_t)off * e));
+    BCK(device_alloc((void**)&b->pool_p, (size_t)off * e));
     b->ttable_ok = false;
   }
   if (!b->d_ttable) {
-    BCK(cudaMalloc(&b->d_ttable, batch_tma_table_bytes(b->count)));
+    BCK(device_alloc((void**)&b->d_ttable, batch_tma_table_bytes(b->count)));
     b->ttable_ok = false;
   }
   if (!b->ttable_ok) {
@@ -535,7 +535,7 @@ cudaError_t grow(T** p, size_t* count, size_t n) {
   *p = nullptr;
   *count = 0;
   if (alloc_over_cap(sizeof(T) * n)) return cudaErrorMemoryAllocation;
-  const cudaError_t e = cudaMalloc(p, sizeof(T) * n);
+  const cudaError_t e = device_alloc((void**)p, sizeof(T) * n);
   if (e == cudaSuccess) *count = n;
   return e;
 }
@@ -647,7 +647,7 @@ void lbm_batch_destroy(lbm_batch b) {
   cudaFree(b->d_small);
   cudaFree(b->d_scratch);
   cudaFree(b->d_labels);
-  cudaFree(b->d_plane);
+  spare_free(b->planes);
   if (b->own_stream) cudaStreamDestroy(b->own_stream);
   delete b;
 }
@@ -709,25 +709,25 @@ lbm_batch lbm_batch_create(const lbm_instance* inst, int count, int precision, i
     err = cudaStreamCreateWithFlags(&b->own_stream, cudaStreamNonBlocking);
     b->stream = b->own_stream;
   }
-  if (err == cudaSuccess) err = cudaMalloc(&b->d_inst, sizeof(BatchInst) * count);
-  if (err == cudaSuccess) err = cudaMalloc(&b->d_ginst, sizeof(GInst) * count);
+  if (err == cudaSuccess) err = device_alloc((void**)&b->d_inst, sizeof(BatchInst) * count);
+  if (err == cudaSuccess) err = device_alloc((void**)&b->d_ginst, sizeof(GInst) * count);
   if (err == cudaSuccess && alloc_over_cap(b->pool_f_bytes + b->pool_psi_bytes)) {
     bfail(LBM_ERR_OOM, "the batch's pools exceed LBM_ALLOC_CAP_BYTES");
     lbm_batch_destroy(b);
     return nullptr;
   }
-  if (err == cudaSuccess) err = cudaMalloc(&b->pool_f, b->pool_f_bytes);
-  if (err == cudaSuccess) err = cudaMalloc(&b->pool_psi, b->pool_psi_bytes);
+  if (err == cudaSuccess) err = device_alloc((void**)&b->pool_f, b->pool_f_bytes);
+  if (err == cudaSuccess) err = device_alloc((void**)&b->pool_psi, b->pool_psi_bytes);
   // d_flag[0] the numeric flag, [2] the stochastic-rounding salt, [4] the
   // grid-barrier counter of the persistent step
-  if (err == cudaSuccess) err = cudaMalloc(&b->d_flag, sizeof(int) * 8);
-  if (err == cudaSuccess) err = cudaMalloc(&b->d_small, sizeof(double) * 64);
+  if (err == cudaSuccess) err = device_alloc((void**)&b->d_flag, sizeof(int) * 8);
+  if (err == cudaSuccess) err = device_alloc((void**)&b->d_small, sizeof(double) * 64);
   if (err == cudaSuccess) err = cudaMemsetAsync(b->d_flag, 0, sizeof(int) * 8, b->stream);
   // d_flag[2] (and [3]: the padded form's pair) is the stochastic-rounding step salt of every instance
   if (err == cudaSuccess)
     for (auto& I : b->inst) I.ph.salt = (const unsigned*)(b->d_flag + 2);
   if (err == cudaSuccess && precision == LBM_F64) {
-    err = cudaMalloc(&b->d_psi_tab, sizeof(double2) * kPsiTab);
+    err = device_alloc((void**)&b->d_psi_tab, sizeof(double2) * kPsiTab);
     if (err == cudaSuccess) err = psi_table_launch(b->d_psi_tab, b->stream);
     for (auto& I : b->inst) I.ph.psi_tab = b->d_psi_tab;
   }
@@ -866,7 +866,7 @@ int lbm_batch_step(lbm_batch b, int n) {
     // blocks, replayed from a graph (option graph, default on)
     const int m = std::min(n, kPersistSteps);
     if (!b->d_tickets) {
-      BCK(cudaMalloc(&b->d_tickets, sizeof(unsigned) * kPersistSteps));
+      BCK(device_alloc((void**)&b->d_tickets, sizeof(unsigned) * kPersistSteps));
       b->tickets_n = kPersistSteps;
     }
     if (b->use_graph) {
@@ -946,10 +946,11 @@ int lbm_batch_sync(lbm_batch b) {
 int lbm_batch_get_populations(lbm_batch b, int k, double* host) {
   if (!b || !host || k < 0 || k >= b->count) return bfail(LBM_ERR_ARG, "bad batch, instance or buffer");
   if (int rc = ensure_contig_instance(b, k)) return rc;
-  const size_t room = transfer_doubles(b->max_nodes, Q);
-  if (!b->d_plane) BCK(cudaMalloc(&b->d_plane, sizeof(double) * room));
   View v = view_of(b, k);
-  BCK(export_populations(b->precision, LAYOUT_LOCAL, v.g, v.ph, v.f, b->d_plane, room, host, b->stream));
+  const SpareUse use(b->planes);
+  BCK(transfer_room(b->planes, b->max_nodes, Q, false));
+  BCK(export_populations(b->precision, LAYOUT_LOCAL, v.g, v.ph, v.f, (double*)b->planes.p,
+                         b->planes.bytes / sizeof(double), host, b->stream));
   return LBM_OK;
 }
 

@@ -285,6 +285,35 @@ cudaError_t batch_tma_persist_launch(int precision, const void* d_table, const B
 // exceeds it (out-of-memory handling without exhausting a GPU).
 bool alloc_over_cap(size_t bytes);
 
+// Device memory that an object keeps between calls although it can do without
+// (planes of host transfers): whenever a device allocation of the library is
+// refused, every Spare on the device that no call is using is freed, and the
+// allocation tried again (device_alloc).  spare_alloc, spare_free and p belong to
+// the call between spare_enter and spare_leave.
+struct Spare {
+  void* p = nullptr;
+  size_t bytes = 0;
+  bool busy = false;
+  int device = 0;
+  Spare* next = nullptr;
+};
+void spare_enter(Spare& s);
+void spare_leave(Spare& s);
+struct SpareUse {
+  Spare& s;
+  explicit SpareUse(Spare& spare) : s(spare) { spare_enter(s); }
+  ~SpareUse() { spare_leave(s); }
+};
+// `bytes` in place of what s holds (nothing where they are refused; capped: also
+// by LBM_ALLOC_CAP_BYTES on all that the lattices hold); frees no other Spare.
+cudaError_t spare_alloc(Spare& s, size_t bytes, bool capped);
+void spare_free(Spare& s);
+// Room for FP64 planes of N nodes: transfer_doubles(N, planes) of them, one
+// plane where that many are refused.
+cudaError_t transfer_room(Spare& s, long long N, int planes, bool capped);
+// cudaMalloc, tried again once the idle Spares are freed.
+cudaError_t device_alloc(void** p, size_t bytes);
+
 }  // namespace lbm
 
 // ---- the handle -------------------------------------------------------------
@@ -317,8 +346,7 @@ struct lbm_ctx {
   double2* d_psi_tab = nullptr;   // FP64: table of psi_of<double>
   double* d_small = nullptr;      // small result buffer (diagnostics out etc.)
   double* d_scratch = nullptr;    // diagnostics partials
-  double* d_transfer = nullptr;   // FP64 planes on their way to or from the host (kept up to 64 MiB)
-  size_t transfer_n = 0;
+  lbm::Spare transfer;            // FP64 planes on their way to or from the host (kept up to 64 MiB)
   size_t scratch_doubles = 0;
   int* d_labels = nullptr;        // CCL labels and sizes (2 N ints)
   bool diag_ccl = false;          // label droplets at every in-loop diagnostic step

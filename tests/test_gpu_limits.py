@@ -83,6 +83,41 @@ def test_loaded_densities_reach_replayed_diagnostics(L, shape, fused, ccl):
     assert out[0][0]["liquid_volume_w"] != out[0][2]["liquid_volume_w"]
 
 
+# Where one plane of doubles fits beside the lattice, transfers work (all planes
+# together would not fit); what a handle keeps for the next transfer makes room
+# for other allocations, of the same handle or another.
+def test_transfers_where_one_plane_fits(L, monkeypatch):
+    gc.collect()
+    shape = (64, 64, 64)                             # a plane takes 2 MiB, 19 planes 38 MiB
+    f0 = lbm_inputs.random_populations(*shape, seed=91)
+    with L.Lattice(*shape, 0.9, -5.5, precision="f64") as lat:
+        monkeypatch.setenv("LBM_ALLOC_CAP_BYTES", str(3 << 20))
+        lat.set_populations(f0)
+        np.testing.assert_array_equal(lat.populations(), f0)
+        one = lat.moments()
+        monkeypatch.delenv("LBM_ALLOC_CAP_BYTES")
+        all_ = lat.moments()
+        np.testing.assert_array_equal(lat.populations(), f0)
+    for k in one:
+        np.testing.assert_array_equal(one[k], all_[k])
+
+
+def test_planes_kept_for_transfers_make_room(L, monkeypatch):
+    gc.collect()
+    shape = (64, 64, 64)
+    f0 = lbm_inputs.random_populations(*shape, seed=92)
+    with L.Lattice(*shape, 0.9, -5.5) as lat:
+        lat.set_populations(f0)
+        want = lat.populations()
+        monkeypatch.setenv("LBM_ALLOC_CAP_BYTES", str(10 << 20))
+        count, _ = lat.droplets()                    # labels: 2 MiB
+        lat.set_populations(f0)
+        with L.Lattice(32, 32, 32, 0.9, -5.5, torch_buffers=False) as other:   # 5 MiB
+            other.set_populations(lbm_inputs.random_populations(32, 32, 32, seed=93))
+        np.testing.assert_array_equal(lat.populations(), want)
+        assert lat.droplets()[0] == count
+
+
 # A growth of the diagnostics' scratch or labels that fails leaves the batch
 # without them, not with the size they had: smaller instances get their own.
 def test_batch_diagnostics_after_a_failed_growth(L, monkeypatch):
@@ -137,3 +172,27 @@ def test_in_loop_diagnostics_after_a_failed_start(L, monkeypatch):
         lat.set_option("diag_interval", 1)
         lat.step(3)
         assert [r["step"] for r in lat.diag_history()] == [0, 1, 2]
+
+
+def test_batch_planes_within_the_cap_and_given_back(L, monkeypatch):
+    import torch
+    gc.collect()
+    insts = [dict(nx=64, ny=64, nz=64, tau=0.9, G=-5.5, R0=16.0, lam=64.0, eps=0.1, phase=0.0, rho_l=2.5, rho_v=0.15,
+                  width=2.0)]
+    monkeypatch.setenv("LBM_ALLOC_CAP_BYTES", str(100 * 64 ** 3))   # pools 80 bytes a node, a plane 8, all planes 152
+    with L.Batch(insts, precision="f16dev") as b:
+        b.init()
+        b.step(2)
+        b.diagnostics(0)
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        one = b.populations(0)
+        assert free - torch.cuda.mem_get_info()[0] < 16 << 20
+        monkeypatch.delenv("LBM_ALLOC_CAP_BYTES")
+        np.testing.assert_array_equal(b.populations(0), one)
+        free = torch.cuda.mem_get_info()[0]
+        monkeypatch.setenv("LBM_ALLOC_CAP_BYTES", str(30 << 20))
+        with L.Lattice(48, 48, 48, 0.9, -5.5, torch_buffers=False) as lat:      # 17 MiB beside the planes' 38
+            lat.set_populations(lbm_inputs.random_populations(48, 48, 48, seed=95))
+        assert torch.cuda.mem_get_info()[0] - free > 30 << 20
+        np.testing.assert_array_equal(b.populations(0), one)
