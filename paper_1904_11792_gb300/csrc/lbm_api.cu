@@ -750,15 +750,14 @@ lbm_handle lbm_create_ex(const lbm_config* cfg) {
   }
   if (rc == LBM_OK) rc = dev_alloc((void**)&h->d_flag, sizeof(int) * 4, "flag");
   if (rc == LBM_OK) h->ph.salt = (const unsigned*)(h->d_flag + 2);
-  if (rc == LBM_OK && cfg->precision == LBM_F64) {
-    rc = dev_alloc((void**)&h->d_psi_tab, sizeof(double2) * kPsiTab, "psi table");
-    if (rc == LBM_OK) {
-      e = psi_table_launch(h->d_psi_tab, h->stream);
-      if (e != cudaSuccess) rc = cuda_fail(e, "psi table");
-    }
+  if (rc == LBM_OK) rc = dev_alloc((void**)&h->d_small, sizeof(double) * 64, "results");
+  // (where there is no room for the table, psi is computed by exp)
+  if (rc == LBM_OK && cfg->precision == LBM_F64 && !over_total_cap(sizeof(double2) * kPsiTab) &&
+      dev_alloc((void**)&h->d_psi_tab, sizeof(double2) * kPsiTab, "psi table") == LBM_OK) {
+    e = psi_table_launch(h->d_psi_tab, h->stream);
+    if (e != cudaSuccess) rc = cuda_fail(e, "psi table");
     h->ph.psi_tab = h->d_psi_tab;
   }
-  if (rc == LBM_OK) rc = dev_alloc((void**)&h->d_small, sizeof(double) * 64, "results");
   if (rc == LBM_OK) {
     e = cudaMemsetAsync(h->d_flag, 0, sizeof(int) * 4, h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->state, 0, h->state_bytes, h->stream);

@@ -726,9 +726,12 @@ lbm_batch lbm_batch_create(const lbm_instance* inst, int count, int precision, i
   // d_flag[2] (and [3]: the padded form's pair) is the stochastic-rounding step salt of every instance
   if (err == cudaSuccess)
     for (auto& I : b->inst) I.ph.salt = (const unsigned*)(b->d_flag + 2);
+  // (where there is no room for the table, psi is computed by exp)
   if (err == cudaSuccess && precision == LBM_F64) {
-    err = device_alloc((void**)&b->d_psi_tab, sizeof(double2) * kPsiTab);
-    if (err == cudaSuccess) err = psi_table_launch(b->d_psi_tab, b->stream);
+    if (device_alloc((void**)&b->d_psi_tab, sizeof(double2) * kPsiTab) == cudaSuccess)
+      err = psi_table_launch(b->d_psi_tab, b->stream);
+    else
+      (void)cudaGetLastError();
     for (auto& I : b->inst) I.ph.psi_tab = b->d_psi_tab;
   }
   if (err == cudaSuccess) err = cudaMemsetAsync(b->pool_f, 0, b->pool_f_bytes, b->stream);

@@ -196,3 +196,24 @@ def test_batch_planes_within_the_cap_and_given_back(L, monkeypatch):
             lat.set_populations(lbm_inputs.random_populations(48, 48, 48, seed=95))
         assert torch.cuda.mem_get_info()[0] - free > 30 << 20
         np.testing.assert_array_equal(b.populations(0), one)
+
+
+# A FP64 lattice in exactly the memory it needs: created without the table of
+# its pseudo-potential, it computes psi directly.
+@pytest.mark.parametrize("rho0", [1.0, 1.3])
+def test_f64_lattice_without_room_for_the_psi_table(L, monkeypatch, rho0):
+    gc.collect()
+    shape, f0 = (12, 9, 8), lbm_inputs.random_populations(12, 9, 8, seed=96)
+    cfg = L.lbm_config_default()
+    cfg.nx, cfg.ny, cfg.nz, cfg.precision = *shape, L.LBM_F64
+    monkeypatch.setenv("LBM_ALLOC_CAP_BYTES", str(sum(L.lbm_required_bytes(cfg)) + 16 + 512))
+    out = []
+    for cap in (1, 0):
+        with L.Lattice(*shape, 0.9, -5.5, precision="f64", rho0=rho0, torch_buffers=False) as lat:
+            monkeypatch.delenv("LBM_ALLOC_CAP_BYTES", raising=False)
+            lat.set_populations(f0)
+            lat.step(5)
+            out.append(lat.populations())
+    # psi differs by 2e-15 at most (each form's bound); |G| = 5.5 forces of ten
+    # psi products each, over 5 steps
+    np.testing.assert_allclose(out[0], out[1], rtol=1e-12, atol=1e-14)
