@@ -196,6 +196,7 @@ void drop_graphs(lbm_ctx* h) {
         cudaGraphExecDestroy(ge);
         ge = nullptr;
       }
+  h->pad_graphs = false;
 }
 
 cudaEvent_t take_event(lbm_ctx* h) {
@@ -370,28 +371,21 @@ bool ragged_form(const lbm_ctx* h) {
 bool ragged_direct(const lbm_ctx* h) {
   return ragged_form(h) && ragged_row(h->g, h->cfg.precision) == h->g.nx && ((uintptr_t)h->state & 15) == 0;
 }
-bool padded_form(const lbm_ctx* h) { return ragged_form(h) && !ragged_direct(h) && h->pad[1]; }
+bool padded_form(const lbm_ctx* h) { return ragged_form(h) && !ragged_direct(h) && h->pads.p; }
+void* pad_ptr(const lbm_ctx* h, int k) { return (char*)h->pads.p + k * h->pad_bytes; }
 
 // Allocates the padded arrays where they take at most a quarter of the free
-// memory; without them the steps stay on the two kernels.
+// memory; without them the steps stay on the two kernels.  Called only where
+// the steps at hand replay a chunk of several, whose later ones use them.
 void ensure_padded(lbm_ctx* h) {
-  if (h->pad[1] || h->pad_failed || !ragged_form(h) || ragged_direct(h)) return;
+  if (h->pads.p || h->pad_failed || !ragged_form(h) || ragged_direct(h)) return;
   const size_t bytes =
-      (size_t)Q * ragged_row(h->g, h->cfg.precision) * h->g.ny * h->g.nz * elem_size(h->cfg.precision);
+      ((size_t)Q * ragged_row(h->g, h->cfg.precision) * h->g.ny * h->g.nz * elem_size(h->cfg.precision) + 255) / 256 * 256;
   size_t free_b = 0, total_b = 0;
-  const std::string msg = g_last_error;
   h->pad_failed = cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || 8 * bytes > free_b ||
-                  dev_alloc(&h->pad[0], bytes, "padded rows") != LBM_OK;
-  if (!h->pad_failed) {
-    h->pad_bytes = bytes;
-    h->pad_failed = dev_alloc(&h->pad[1], bytes, "padded rows") != LBM_OK;
-  }
-  if (!h->pad_failed) return;
-  (void)cudaGetLastError();
-  g_last_error = msg;
-  dev_free(h->pad[0], h->pad_bytes);
-  h->pad[0] = h->pad[1] = nullptr;
-  h->pad_bytes = 0;
+                  spare_alloc(h->pads, 2 * bytes, true) != cudaSuccess;
+  if (h->pad_failed) (void)cudaGetLastError();
+  h->pad_bytes = bytes;
 }
 
 // Step k of a captured chunk of `steps` that starts on array `phase`, on
@@ -416,11 +410,11 @@ int enqueue_padded_step(lbm_ctx* h, cudaStream_t s, int k, int steps, int phase,
     } else {
       CK(launch_psi(prec, LAYOUT_LOCAL, h->vec, g, h->ph, src, h->psi, h->d_flag, s));
     }
-    CK(launch_collide_padded(prec, g, ph, src, h->pad[0], px, h->psi, auto_block(g, false, prec), s));
+    CK(launch_collide_padded(prec, g, ph, src, pad_ptr(h, 0), px, h->psi, auto_block(g, false, prec), s));
     return LBM_OK;
   }
   const bool last = k == steps - 1;
-  CK(launch_ragged(prec, g, ph, h->pad[(k - 1) & 1], px, last ? array_ptr(h, phase ^ (steps & 1)) : h->pad[k & 1],
+  CK(launch_ragged(prec, g, ph, pad_ptr(h, (k - 1) & 1), px, last ? array_ptr(h, phase ^ (steps & 1)) : pad_ptr(h, k & 1),
                    last ? g.nx : px, h->d_flag, h->fused_fz, h->fused_group, s));
   return LBM_OK;
 }
@@ -495,6 +489,7 @@ int capture_chunk(lbm_ctx* h, int phase, int steps, cudaGraphExec_t* exec) {
     // step numbers relative to a chunk start (a multiple of chunk_len()): the same
     // parity and the same diagnostic steps as every replay
     const bool padded = padded_form(h) && steps > 1;
+    h->pad_graphs |= padded;
     for (int k = 0; k < steps && rc == LBM_OK; ++k)
       rc = padded ? enqueue_padded_step(h, cs, k, steps, phase, side.join ? &side : nullptr)
                   : enqueue_step(h, cs, k, phase ^ (k & 1), false, side.join ? &side : nullptr);
@@ -674,7 +669,7 @@ void lbm_destroy(lbm_handle h) {
   dev_free(h->d_psi_tab, sizeof(double2) * kPsiTab);
   dev_free(h->d_small, sizeof(double) * 64);
   dev_free(h->d_scratch, h->scratch_doubles * sizeof(double));
-  for (void* p : h->pad) dev_free(p, h->pad_bytes);
+  spare_free(h->pads);
   spare_free(h->transfer);
   dev_free(h->d_labels, (size_t)h->g.N * 2 * sizeof(int));
   dev_free(h->d_drop, h->drop_bytes);
@@ -836,6 +831,11 @@ int lbm_set_option(lbm_handle h, const char* key, double v) {
   } else if (k == "fused") {
     h->fused = v == 0.0 ? 0 : (v == 2.0 ? 2 : 1);
     drop_graphs(h);
+    if (!h->fused && h->pads.p) {   // no step uses the padded arrays any more
+      CK(cudaStreamSynchronize(h->stream));
+      spare_free(h->pads);
+    }
+    h->pad_failed = false;
     if (h->diag_interval > 0) {
       int rc = ensure_scratch(h);
       if (rc) return rc;
@@ -1017,8 +1017,15 @@ int lbm_step(lbm_handle h, int n) {
   if (n < 0) return fail(LBM_ERR_ARG, "negative step count");
   if (!h->initialized) return fail(LBM_ERR_STATE, "lattice not initialised");
   const bool aa = h->cfg.pattern == LBM_AA;
-  if (h->use_graph && !h->kernel_timing && n > 1) ensure_padded(h);
-  const int base = chunk_len(h), longer = long_chunk_len(h);
+  const SpareUse use(h->pads);
+  if (h->pad_graphs && !h->pads.p) {   // given back since the last call
+    drop_graphs(h);
+    h->pad_failed = true;
+  }
+  const int base = chunk_len(h);
+  const long long first = (h->step + base - 1) / base * base;   // the first step a graph may start at
+  if (h->use_graph && !h->kernel_timing && base > 1 && h->step + n >= first + base) ensure_padded(h);
+  const int longer = long_chunk_len(h);
   const int k = h->diag_interval;
   if (h->graph_chunk != base) {
     drop_graphs(h);

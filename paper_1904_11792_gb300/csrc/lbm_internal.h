@@ -286,7 +286,7 @@ cudaError_t batch_tma_persist_launch(int precision, const void* d_table, const B
 bool alloc_over_cap(size_t bytes);
 
 // Device memory that an object keeps between calls although it can do without
-// (planes of host transfers): whenever a device allocation of the library is
+// (planes of host transfers, padded arrays): whenever a device allocation of the library is
 // refused, every Spare on the device that no call is using is freed, and the
 // allocation tried again (device_alloc).  spare_alloc, spare_free and p belong to
 // the call between spare_enter and spare_leave.
@@ -328,12 +328,13 @@ struct lbm_ctx {
   void* state = nullptr;  // populations: A-B = two arrays, AA = one
   size_t state_bytes = 0;
   bool own_state = false;
-  // two private arrays with rows padded to 16 bytes, between which the steps
-  // inside a captured chunk run where the lattice's own rows are not 16-byte
-  // multiples; pad_failed: there was no room for them
-  void* pad[2] = {nullptr, nullptr};
-  size_t pad_bytes = 0;           // of each
-  bool pad_failed = false;
+  // two private arrays of pad_bytes each with rows padded to 16 bytes, between
+  // which the steps inside a captured chunk run where the lattice's own rows are
+  // not 16-byte multiples; pad_graphs: the captured graphs use them; pad_failed:
+  // there was no room for them, or they were given back
+  lbm::Spare pads;
+  size_t pad_bytes = 0;
+  bool pad_graphs = false, pad_failed = false;
   void* psi = nullptr;
   size_t psi_bytes = 0;
   bool own_psi = false;
