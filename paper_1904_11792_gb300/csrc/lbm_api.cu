@@ -237,8 +237,19 @@ bool ragged_direct(const lbm_ctx* h);
 bool fused_form(const lbm_ctx* h) {
   const long long least = h->cfg.precision == LBM_F32 && h->ph.coll == COLL_SRT ? kFusedNodes : kFusedNodesLate;
   return h->fused && h->cfg.pattern == LBM_AB && fused_applicable(h->g, h->cfg.precision) &&
-         (h->fused > 0 || h->g.N > least || h->fused_fz || h->fused_group || h->fused_stall_test_ns);
+         (h->fused > 0 || h->g.N > least || h->fused_fz || h->fused_group || h->fused_stall_test_ns ||
+          (uintptr_t)h->state % 16);   // (TMA refuses such populations, on small lattices too)
 }
+
+// Whether node pairs move as vectors: not where the caller's buffers start at an
+// address that their loads and stores (and the psi pass's of four nodes, where nx
+// allows them) are not aligned to.
+bool buffers_aligned(const lbm_ctx* h) {
+  if (h->cfg.precision == LBM_F64) return true;   // one node at a time
+  const size_t unit = h->g.nx % 4 == 0 ? 4 : 2;
+  return (uintptr_t)h->state % (unit * elem_size(h->cfg.precision)) == 0 && (uintptr_t)h->psi % (unit * sizeof(float)) == 0;
+}
+bool vector_form(const lbm_ctx* h) { return h->vec && h->aligned; }
 
 // The psi pass of a diagnostic step of the two kernels: with the diagnostics,
 // and the droplet counts where they are on.
@@ -342,10 +353,10 @@ int enqueue_step(lbm_ctx* h, cudaStream_t s, long long step, int cur, bool timed
   if (diag_step) {
     if (int rc = enqueue_diagnostics(h, s, g, layout, src, aa ? nullptr : dst, side)) return rc;
   } else {
-    CK(launch_psi(prec, layout, h->vec, g, h->ph, src, h->psi, h->d_flag, s, aa ? nullptr : dst));
+    CK(launch_psi(prec, layout, vector_form(h), g, h->ph, src, h->psi, h->d_flag, s, aa ? nullptr : dst));
   }
   if (timed) CK(cudaEventRecord(e1, s));
-  const bool vec = node_pairs(prec, h->vec, h->g);
+  const bool vec = node_pairs(prec, vector_form(h), h->g);
   const int minb = h->minb ? h->minb : auto_minb(vec, mode, prec, h->g.N);
   const dim3 block = h->block_asked ? h->block : auto_block(h->g, vec, prec);
   if (h->ph.coll == COLL_MRT)
@@ -408,7 +419,7 @@ int enqueue_padded_step(lbm_ctx* h, cudaStream_t s, int k, int steps, int phase,
     if (h->diag_interval > 0) {
       if (int rc = enqueue_diagnostics(h, s, g, LAYOUT_LOCAL, src, nullptr, h->diag_ccl ? nullptr : side)) return rc;
     } else {
-      CK(launch_psi(prec, LAYOUT_LOCAL, h->vec, g, h->ph, src, h->psi, h->d_flag, s));
+      CK(launch_psi(prec, LAYOUT_LOCAL, vector_form(h), g, h->ph, src, h->psi, h->d_flag, s));
     }
     CK(launch_collide_padded(prec, g, ph, src, pad_ptr(h, 0), px, h->psi, auto_block(g, false, prec), s));
     return LBM_OK;
@@ -728,6 +739,8 @@ lbm_handle lbm_create_ex(const lbm_config* cfg) {
     if (cfg->ext_state) {
       if (cfg->ext_state_bytes < h->state_bytes)
         rc = fail(LBM_ERR_ARG, "ext_state_bytes smaller than required");
+      else if ((uintptr_t)cfg->ext_state % elem_size(cfg->precision))
+        rc = fail(LBM_ERR_ARG, "ext_state is not aligned to its elements");
       h->state = cfg->ext_state;
     } else {
       rc = dev_alloc(&h->state, h->state_bytes, "populations");
@@ -737,12 +750,15 @@ lbm_handle lbm_create_ex(const lbm_config* cfg) {
   if (rc == LBM_OK) {
     if (cfg->ext_psi) {
       if (cfg->ext_psi_bytes < h->psi_bytes) rc = fail(LBM_ERR_ARG, "ext_psi_bytes smaller than required");
+      else if ((uintptr_t)cfg->ext_psi % (cfg->precision == LBM_F64 ? 8 : 4))
+        rc = fail(LBM_ERR_ARG, "ext_psi is not aligned to its elements");
       h->psi = cfg->ext_psi;
     } else {
       rc = dev_alloc(&h->psi, h->psi_bytes, "psi");
       h->own_psi = rc == LBM_OK;
     }
   }
+  h->aligned = buffers_aligned(h);
   if (rc == LBM_OK) rc = dev_alloc((void**)&h->d_flag, sizeof(int) * 4, "flag");
   if (rc == LBM_OK) h->ph.salt = (const unsigned*)(h->d_flag + 2);
   if (rc == LBM_OK) rc = dev_alloc((void**)&h->d_small, sizeof(double) * 64, "results");
@@ -923,9 +939,9 @@ int lbm_get_option(lbm_handle h, const char* key, double* v) {
   else if (k == "diag_ccl") *v = h->diag_ccl;
   else if (k == "occupancy")
     *v = h->minb ? h->minb
-                 : auto_minb(node_pairs(h->cfg.precision, h->vec, h->g), h->cfg.pattern == LBM_AA ? MODE_AA_ODD : MODE_AB,
+                 : auto_minb(node_pairs(h->cfg.precision, vector_form(h), h->g), h->cfg.pattern == LBM_AA ? MODE_AA_ODD : MODE_AB,
                              h->cfg.precision, h->g.N);
-  else if (k == "vector") *v = h->vec && (h->g.nx % 2 == 0);
+  else if (k == "vector") *v = vector_form(h) && (h->g.nx % 2 == 0);
   else if (k == "stochastic_rounding") *v = h->ph.sr;
   else if (k == "fused")
     *v = h->fused && h->cfg.pattern == LBM_AB && fused_applicable(h->g, h->cfg.precision);
@@ -1119,7 +1135,7 @@ int lbm_moments(lbm_handle h, double* rho, double* ux, double* uy, double* uz) {
   if (!h->initialized) return fail(LBM_ERR_STATE, "lattice not initialised");
   const int layout = cur_layout(h);
   const void* f = cur_array(h);
-  CK(launch_psi(h->cfg.precision, layout, h->vec, h->g, h->ph, f, h->psi, h->d_flag, h->stream));
+  CK(launch_psi(h->cfg.precision, layout, vector_form(h), h->g, h->ph, f, h->psi, h->d_flag, h->stream));
   double* outs[4] = {rho, ux, uy, uz};
   int want = 0;
   for (double* o : outs) want += o != nullptr;

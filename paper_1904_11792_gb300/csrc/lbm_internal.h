@@ -365,6 +365,7 @@ struct lbm_ctx {
   bool block_asked = false;       // block was given (else auto_block is launched)
   int minb = 0;                   // collide kernel register budget variant (0 = auto)
   bool vec = true;                // two nodes per thread (when nx is even)
+  bool aligned = true;            // the buffers start where node pairs and groups of four may (own ones do)
   // single-pass A-B steps: -1 (until the option is set) where they apply and
   // pay, 0 never, 1 the 64-wide tiles where they apply and cut tiles where
   // they pay, 2 both where they apply

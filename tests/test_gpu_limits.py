@@ -73,3 +73,52 @@ def test_padded_arrays_only_where_steps_use_them(L, monkeypatch):
         lat.set_option("fused", 1)                                      # asked for again
         lat.step(2)
         assert held() > size // 2
+
+
+# Caller's buffers that start at any element: refused by the single pass (its
+# copies want 16 bytes; on small lattices too, which take the two kernels by
+# default), stepped by the two kernels one node at a time where pairs or groups
+# of four nodes would be misaligned.  Off its elements a buffer is refused.
+@pytest.mark.parametrize("precision,pattern", [("f64", "ab"), ("f32", "ab"), ("f32", "aa"), ("f16dev", "ab"),
+                                               ("f16dev", "aa"), ("bf16dev", "ab")])
+@pytest.mark.parametrize("shape", [(64, 8, 12), (66, 7, 9), (61, 7, 9)])
+def test_buffers_at_any_element(L, shape, precision, pattern):
+    import torch
+    f0 = lbm_inputs.random_populations(*shape, seed=97)
+    cfg = L.lbm_config_default()
+    cfg.nx, cfg.ny, cfg.nz = shape
+    cfg.tau, cfg.G, cfg.rho_ref = 0.9, -5.5, 0.1
+    cfg.precision, cfg.pattern = L.PRECISIONS[precision], L.PATTERNS[pattern]
+    elem = {"f64": 8, "f32": 4}.get(precision, 2)
+    psi_elem = 8 if precision == "f64" else 4
+    sb, pb = L.lbm_required_bytes(cfg)
+    state = torch.empty(sb + 16, dtype=torch.uint8, device="cuda")
+    psi = torch.empty(pb + 16, dtype=torch.uint8, device="cuda")
+    out = []
+    for a, b in ((0, 0), (elem, 0), (8, 0), (0, psi_elem), (4 if elem == 2 else elem, 8)):
+        cfg.ext_state, cfg.ext_state_bytes = state.data_ptr() + a, sb
+        cfg.ext_psi, cfg.ext_psi_bytes = psi.data_ptr() + b, pb
+        h = L.lbm_create_ex(cfg)
+        try:
+            L.lbm_set_option(h, "diag_interval", 2)
+            L.lbm_set_populations(h, f0)
+            if L.lbm_get_option(h, "fused") and pattern == "ab" and a % 16:
+                with pytest.raises(L.LbmError):
+                    L.lbm_step(h, 1)
+            L.lbm_set_option(h, "fused", 0)
+            L.lbm_set_populations(h, f0)
+            L.lbm_step(h, 6)
+            L.lbm_sync(h)
+            m = L.lbm_moments(h, shape[::-1])
+            out.append((L.lbm_get_populations(h, shape[::-1]), m, L.lbm_diagnostics(h, True).as_dict()["liquid_count"]))
+        finally:
+            L.lbm_destroy(h)
+    for f, m, n in out[1:]:
+        np.testing.assert_array_equal(f, out[0][0])
+        for k in m:
+            np.testing.assert_array_equal(m[k], out[0][1][k])
+        assert n == out[0][2]
+    for cfg.ext_state, cfg.ext_psi in ((state.data_ptr() + 1, psi.data_ptr()), (state.data_ptr(), psi.data_ptr() + 2)):
+        with pytest.raises(L.LbmError) as ei:
+            L.lbm_create_ex(cfg)
+        assert "aligned" in str(ei.value)
