@@ -390,6 +390,7 @@ void* pad_ptr(const lbm_ctx* h, int k) { return (char*)h->pads.p + k * h->pad_by
 // the steps at hand replay a chunk of several, whose later ones use them.
 void ensure_padded(lbm_ctx* h) {
   if (h->pads.p || h->pad_failed || !ragged_form(h) || ragged_direct(h)) return;
+  const CaptureAllowed allowed;
   const size_t bytes =
       ((size_t)Q * ragged_row(h->g, h->cfg.precision) * h->g.ny * h->g.nz * elem_size(h->cfg.precision) + 255) / 256 * 256;
   size_t free_b = 0, total_b = 0;
@@ -485,6 +486,7 @@ int long_chunk_len(const lbm_ctx* h) {
 // (capture is not allowed on the legacy default stream); the graph is
 // launched on the handle's stream.
 int capture_chunk(lbm_ctx* h, int phase, int steps, cudaGraphExec_t* exec) {
+  const CaptureAllowed allowed;
   cudaStream_t cs = nullptr;
   ReduceSide side{nullptr, nullptr, nullptr, false};
   cudaGraph_t graph = nullptr;

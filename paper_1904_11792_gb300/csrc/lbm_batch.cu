@@ -502,6 +502,7 @@ int enqueue_batch_step(lbm_batch_ctx* b, cudaStream_t s, int cur) {
 constexpr int kLongSteps = 16, kLongFrom = 64;
 
 int capture_steps(lbm_batch_ctx* b, int phase, int steps, cudaGraphExec_t* exec) {
+  const CaptureAllowed allowed;
   cudaStream_t cs;
   BCK(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
   cudaGraph_t g = nullptr;

@@ -285,6 +285,16 @@ cudaError_t batch_tma_persist_launch(int precision, const void* d_table, const B
 // exceeds it (out-of-memory handling without exhausting a GPU).
 bool alloc_over_cap(size_t bytes);
 
+// While a graph of steps is captured or memory for them allocated: calls that
+// the runtime forbids to a thread with a capture of its own under way (on
+// another stream, by the program that uses the library) do not void that
+// capture.  They touch none of its streams.
+struct CaptureAllowed {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  CaptureAllowed() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~CaptureAllowed() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 // Device memory that an object keeps between calls although it can do without
 // (planes of host transfers, padded arrays): whenever a device allocation of the library is
 // refused, every Spare on the device that no call is using is freed, and the

@@ -321,3 +321,62 @@ def test_buffers_at_any_element(L, shape, precision, pattern):
         with pytest.raises(L.LbmError) as ei:
             L.lbm_create_ex(cfg)
         assert "aligned" in str(ei.value)
+
+
+# Steps whose graph is captured, or whose longer graph is, while the program
+# captures a graph of its own on another stream: neither voids the other.
+@pytest.mark.parametrize("warm,n", [(0, 20), (20, 400)])
+@pytest.mark.parametrize("shape", [(64, 32, 32), (251, 64, 80)])
+def test_steps_beside_a_capture_of_the_program(L, shape, warm, n):
+    import torch
+    main, other = torch.cuda.Stream(), torch.cuda.Stream()
+    x = torch.zeros(1000, device="cuda")
+    out = []
+    for captured in (True, False):
+        with torch.cuda.stream(other):
+            lat = L.Lattice(*shape, 0.9, -5.5)
+        with lat:
+            lat.init_ligament(8.0, float(shape[0]), 0.1, 0.3, 2.1, 0.1, 2.0)
+            lat.step(warm)
+            torch.cuda.synchronize()
+            if captured:
+                g = torch.cuda.CUDAGraph()
+                with torch.cuda.graph(g, stream=main):
+                    x.add_(1)
+                    lat.step(n)
+                    x.add_(1)
+                g.replay()
+            else:
+                lat.step(n)
+            torch.cuda.synchronize()
+            out.append(lat.rho())
+    assert float(x.min()) == float(x.max()) == 2.0
+    np.testing.assert_array_equal(out[0], out[1])
+
+
+def test_batch_steps_beside_a_capture_of_the_program(L):
+    import torch
+    main, other = torch.cuda.Stream(), torch.cuda.Stream()
+    insts = [dict(nx=40, ny=20, nz=20, tau=0.9, G=-5.5, R0=5.0, lam=40.0, eps=0.1, phase=0.0, rho_l=2.5, rho_v=0.15,
+                  width=2.0)]
+    x = torch.zeros(1000, device="cuda")
+    out = []
+    for captured in (True, False):
+        with torch.cuda.stream(other):
+            b = L.Batch(insts)
+        with b:
+            b.init()
+            b.step(4)
+            torch.cuda.synchronize()
+            if captured:
+                g = torch.cuda.CUDAGraph()
+                with torch.cuda.graph(g, stream=main):
+                    x.add_(1)
+                    b.step(100)          # long enough for the longer graph
+                g.replay()
+            else:
+                b.step(100)
+            b.sync()
+            out.append(b.populations(0))
+    assert float(x.min()) == 1.0
+    np.testing.assert_array_equal(out[0], out[1])
