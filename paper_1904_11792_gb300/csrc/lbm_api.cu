@@ -60,6 +60,20 @@ dim3 auto_block(const Geom& g, bool pairs, int precision) {
   const dim3 b = small_block(g, pairs, precision);
   return (g.ny + b.y - 1) / b.y > 65535 ? default_block(g) : b;
 }
+
+// Default register budget of the collide-stream kernel (as blocks of 256
+// threads per SM), measured in the blocks of auto_block: 3 for the one-node
+// kernel and for the AA even step's two-node kernel (local loads and stores: no
+// spills at 80 registers); for the A-B step's two-node kernel 3 with 2-byte
+// storage above 2^21 nodes (512x256x256 FP16: 565 us per launch against 584
+// with 2; 150x80x80: 26.5 us per step against 25.6); 2 otherwise, with which
+// nothing spills (AA odd step of 512x256x256, FP16: 633 us per launch, with 3
+// 666; FP32: 783 against 930).
+int auto_minb(bool vec, int mode, int precision, long long N) {
+  if (precision == LBM_F64) return 2;   // 981 us per launch on 256x128x128 against 1009 with 3 (spills)
+  if (!vec || mode == MODE_AA_EVEN) return 3;
+  return mode == MODE_AB && precision != LBM_F32 && N > 2LL << 20 ? 3 : 2;
+}
 }  // namespace lbm
 
 namespace {
@@ -214,20 +228,6 @@ cudaEvent_t take_event(lbm_ctx* h) {
 // step parity for AA (whose graph chunks hold an even number of steps).
 int salt_word(const lbm_ctx* h, long long step, int cur) {
   return h->cfg.pattern == LBM_AA ? (int)(step & 1) : (cur & 1);
-}
-
-// Default register budget of the collide-stream kernel (as blocks of 256
-// threads per SM), measured in the blocks of auto_block: 3 for the one-node
-// kernel and for the AA even step's two-node kernel (local loads and stores: no
-// spills at 80 registers); for the A-B step's two-node kernel 3 with 2-byte
-// storage above 2^21 nodes (512x256x256 FP16: 565 us per launch against 584
-// with 2; 150x80x80: 26.5 us per step against 25.6); 2 otherwise, with which
-// nothing spills (AA odd step of 512x256x256, FP16: 633 us per launch, with 3
-// 666; FP32: 783 against 930).
-int auto_minb(bool vec, int mode, int precision, long long N) {
-  if (precision == LBM_F64) return 2;   // 981 us per launch on 256x128x128 against 1009 with 3 (spills)
-  if (!vec || mode == MODE_AA_EVEN) return 3;
-  return mode == MODE_AB && precision != LBM_F32 && N > 2LL << 20 ? 3 : 2;
 }
 
 bool ragged_direct(const lbm_ctx* h);

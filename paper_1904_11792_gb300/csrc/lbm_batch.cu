@@ -923,8 +923,8 @@ int lbm_batch_step_sequential(lbm_batch b, int n) {
       const bool vec = b->inst[k].vec != 0;
       BCK(launch_psi(b->precision, LAYOUT_LOCAL, vec, v.g, v.ph, v.f, v.psi, b->d_flag, b->stream, dst));
       // as a standalone lattice of this size runs by default
-      BCK(launch_collide(b->precision, MODE_AB, 0, vec, v.g, v.ph, v.f, dst, v.psi, auto_block(v.g, vec, b->precision),
-                         b->stream));
+      BCK(launch_collide(b->precision, MODE_AB, auto_minb(vec, MODE_AB, b->precision, v.g.N), vec, v.g, v.ph, v.f, dst,
+                         v.psi, auto_block(v.g, vec, b->precision), b->stream));
     }
     if (batch_sr(b)) BCK(launch_salt((unsigned*)(b->d_flag + 2), false, 0u, b->stream));
     b->cur ^= 1;

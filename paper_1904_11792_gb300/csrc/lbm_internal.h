@@ -86,6 +86,9 @@ constexpr int kSmCount = 152;
 // (lbm_api.cu).
 dim3 default_block(const Geom& g);
 dim3 auto_block(const Geom& g, bool pairs, int precision);
+// The register budget (minb of launch_collide) launched with where none was
+// asked for.
+int auto_minb(bool vec, int mode, int precision, long long N);
 
 // force + collision + streaming with the MRT collision (lbm_mrt.cu); the
 // same modes and layouts as launch_collide
