@@ -2,11 +2,12 @@
 
 For a lattice size and storage precision it times, on the GPU, the streaming
 pattern (A-B or AA), the collide-stream block shape and the register budget
-variant (blocks per SM) of the two-kernel step, and the single-pass fused step
-where it applies, picks the fastest whole step, and caches the choice in a
-JSON file keyed by device, size and precision.  For a batch it tunes the
-batched kernel's block shape.  All timing is CUDA events around real steps of
-the library (kernel_timing for per-kernel times).
+variant (blocks per SM) of the two-kernel step (those the library chooses by
+itself first), and the single pass where it applies, picks the fastest whole
+step, and caches the choice in a JSON file keyed by device, size and precision.
+For a batch it tunes the batched kernel's block shape.  All timing is CUDA events
+around real steps of the library (kernel_timing for per-kernel times; the single
+pass on cut tiles, which may run in replayed graphs only, over whole calls).
 """
 from __future__ import annotations
 
@@ -111,15 +112,35 @@ def tune_lattice(nx, ny, nz, precision="f32", patterns=("ab", "aa"), blocks=DEFA
                         best = t
                 lat.set_option("fused_fz", 0)
                 lat.set_option("fused_group", 0)
+            elif pattern == "ab" and precision != "f64":
+                # the step as it is chosen for other sizes: on larger ones a
+                # single pass (251x112x112: 106 us, two kernels 142)
+                step_ms = float("inf")
+                for _ in range(reps + 1):
+                    e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                    e0.record()
+                    lat.step(max(20, steps))
+                    e1.record()
+                    torch.cuda.synchronize()
+                    step_ms = min(step_ms, e0.elapsed_time(e1) / max(20, steps))
+                t = dict(pattern=pattern, fused=1, fused_fz=0, fused_group=0, block=[0, 0, 0], occupancy=0,
+                         step_ms=step_ms, glups=N / (step_ms * 1e-3) / 1e9)
+                trials.append(t)
+                if verbose:
+                    print(json.dumps(t))
+                if best is None or step_ms < best["step_ms"]:
+                    best = t
             lat.set_option("fused", 0)
-            for occ in occupancies:
-                for b in blocks:
-                    if not _fits(b, nx):
-                        continue
-                    for k, v in zip(("block_x", "block_y", "block_z"), (1, 1, 1)):
-                        lat.set_option(k, v)
-                    for k, v in zip(("block_x", "block_y", "block_z"), b):
-                        lat.set_option(k, v)
+            # (0, 0, 0) and 0: what the library chooses, until a block is set
+            for occ in (0,) + tuple(occupancies):
+                for b in (((0, 0, 0),) if occ == 0 else blocks):
+                    if any(b):
+                        if not _fits(b, nx):
+                            continue
+                        for k, v in zip(("block_x", "block_y", "block_z"), (1, 1, 1)):
+                            lat.set_option(k, v)
+                        for k, v in zip(("block_x", "block_y", "block_z"), b):
+                            lat.set_option(k, v)
                     lat.set_option("occupancy", occ)
                     lat.step(4)
                     torch.cuda.synchronize()
@@ -148,17 +169,19 @@ def tune_lattice(nx, ny, nz, precision="f32", patterns=("ab", "aa"), blocks=DEFA
 
 def apply(lat: "L.Lattice", choice: dict) -> None:
     """Applies a tuned choice to a lattice: the fused step, or the two-kernel
-    step with its block shape and occupancy (the pattern is fixed at
-    creation: create the lattice with choice['pattern'])."""
+    step with its block shape ([0, 0, 0]: the lattice keeps its own) and
+    occupancy (the pattern is fixed at creation: create the lattice with
+    choice['pattern'])."""
     lat.set_option("fused", int(choice.get("fused", 0)))
     if choice.get("fused"):
         lat.set_option("fused_fz", int(choice.get("fused_fz", 0)))
         lat.set_option("fused_group", int(choice.get("fused_group", 0)))
         return
-    for k, v in zip(("block_x", "block_y", "block_z"), (1, 1, 1)):
-        lat.set_option(k, v)
-    for k, v in zip(("block_x", "block_y", "block_z"), choice["block"]):
-        lat.set_option(k, v)
+    if any(choice["block"]):
+        for k, v in zip(("block_x", "block_y", "block_z"), (1, 1, 1)):
+            lat.set_option(k, v)
+        for k, v in zip(("block_x", "block_y", "block_z"), choice["block"]):
+            lat.set_option(k, v)
     lat.set_option("occupancy", choice["occupancy"])
 
 
