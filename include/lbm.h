@@ -88,7 +88,9 @@ typedef struct {
     int pattern;           /* LBM_AB or LBM_AA                                       */
     double rho_ref;        /* deviation reference density of the *DEV storage forms  */
     int block_x, block_y, block_z; /* collide-stream block shape (<= 256 threads), 0 = default */
-    void *ext_state;       /* optional caller device buffer for the populations      */
+    void *ext_state;       /* optional caller device buffer for the populations; any
+                              element-aligned address works, the single-pass step and
+                              vector accesses need 16 bytes (as CUDA allocates)       */
     size_t ext_state_bytes;
     void *ext_psi;         /* optional caller device buffer for psi                  */
     size_t ext_psi_bytes;
@@ -150,16 +152,18 @@ int lbm_set_stream(lbm_handle h, void *stream);
  * reduces the diagnostics of the state at t into a device ring, read with
  * lbm_diag_history; 0 = off, the default),
  * "kernel_timing" (0/1: record CUDA events around every kernel of lbm_step;
- * disables graphs), "block_x", "block_y", "block_z" (collide-stream block
+ * disables graphs, so lattices that run the single pass inside replayed graphs
+ * only, see "fused", are timed on the two kernels), "block_x", "block_y", "block_z" (collide-stream block
  * shape, at most 256 threads), "occupancy" (2, 3 or 4: 256-thread blocks
  * per SM the collide-stream kernel's register budget allows; 0 = auto,
  * the default: 3 for the one-node kernel and the AA even step's two-node
  * kernel and, above 2^21 nodes, for the A-B step's with 2-byte storage, 2
  * otherwise and in FP64; get answers the odd step's (AA) or
  * the A-B step's value),
- * "vector" (0/1, default 1: when nx is even each thread updates two
- * neighbouring nodes with 2-element vector loads and stores; block_x then
- * counts node pairs), "fused" (0, 1 or 2, default 1: A-B steps run as one
+ * "vector" (0/1, default 1: when nx is even and the storage 4- or 2-byte, each
+ * thread updates two neighbouring nodes with 2-element vector loads and stores,
+ * and block_x counts node pairs; get answers whether nx and the buffers allow
+ * it, FP64 takes one node per thread whatever it answers), "fused" (0, 1 or 2, default 1: A-B steps run as one
  * single-pass kernel that computes psi per tile in shared memory, reading
  * the populations once per step, with a variant that also reduces the
  * in-loop diagnostics on diagnostic steps; applies to FP32,
@@ -173,16 +177,16 @@ int lbm_set_stream(lbm_handle h, void *stream);
  * 2 all of them) run plain steps as a single pass on tiles cut at their edges: every
  * step where rows are a multiple of 16 bytes; otherwise the steps inside a
  * replayed graph but its first one, on two private arrays with padded rows
- * (allocated on the first such call if they take at most a quarter of the
- * free device memory, else not at all).  Everything else is the two-kernel
+ * (allocated on the first call that replays such a graph of several steps, if
+ * they take at most a quarter of the free device memory; freed with the value
+ * 0, and where another allocation of the library needs their room).  Everything else is the two-kernel
  * step; results equal it bitwise), "fused_fz" (z planes
  * each block of the fused step marches through; 0 = chosen from the lattice
  * size, the collision and the GPU, the default), "fused_group" (the fused step launches
  * its blocks in groups of this many consecutive z runs, the run varying
- * fastest inside a group, then the tile x, then the tile y; 0 = one run
- * per 4 tile columns of 64 nodes (FP32; one run for 2-byte storage), at
- * least one, the default; any value
- * gives the same results), "fused_fz_used" and "fused_group_used" (get
+ * fastest inside a group, then the tile x, then the tile y; 0, the
+ * default: 4 runs in FP32 on lattices at least 8 tiles wide, else one; any
+ * value gives the same results), "fused_fz_used" and "fused_group_used" (get
  * only: the run length and runs per group the fused step launches with for
  * the current options; 0 where the fused step does not apply),
  * "fused_stall_test" (a test hook of the
@@ -231,8 +235,8 @@ int lbm_init_profile(lbm_handle h, double R0, double lambda, double eps, double 
  * Eq. 5, the velocity shift of Eq. 6, the equilibrium of Eq. 2, the BGK
  * relaxation of Eq. 3 and streaming.  Where option "fused" applies (A-B
  * streaming, FP32 or 2-byte storage, nx % 64 == 0, ny % 4 == 0 for FP32 or
- * ny % 8 == 0 for 2-byte storage; the
- * default) a step is one single-pass kernel that computes psi per tile in
+ * ny % 8 == 0 for 2-byte storage; see it for the sizes that take it by
+ * default, and for other sizes) a step is one single-pass kernel that computes psi per tile in
  * shared memory (its diagnostic-step variant also reduces the in-loop
  * diagnostics); otherwise it is a psi pass followed by one kernel of force,
  * collision and streaming.  Steps are replayed from captured CUDA graphs
@@ -283,8 +287,8 @@ typedef struct {
  * receives the number of droplets, out the first min(*count, max_droplets)
  * of them (out may be NULL when max_droplets is 0).  The FP64 sums are
  * accumulated with atomics, so their last bits may differ between calls.
- * Device scratch: 8 N bytes of labels plus (80 + 4 ceil(nx/32)) bytes per
- * droplet.  Synchronises.  LBM_ERR_TIMEOUT if the labelling guard tripped. */
+ * Device scratch: 8 N bytes of labels, 16 (nx + ny + nz) bytes of angles and
+ * (80 + 4 ceil(nx/32)) bytes per droplet.  Synchronises.  LBM_ERR_TIMEOUT if the labelling guard tripped. */
 int lbm_droplets(lbm_handle h, lbm_droplet *out, int max_droplets, int *count);
 
 /* Canonical populations (see Conventions), host arrays of 19 * N doubles.

@@ -526,10 +526,12 @@ __device__ __forceinline__ void raise_flag(bool bad, int* flag) {
 }
 
 // 1 - exp(-r) in FP64 from a table: for 0 <= r < 8, X the multiple of 1/256
-// nearest r (0 below 1/256), k = 256 X and d = r - X (exact, |d| <= 1/256),
+// nearest r (from r = 1/256 on; below it X = 0), k = 256 X and d = r - X (exact,
+// |d| <= 1/512, below r = 1/256 up to 1/256),
 //   1 - exp(-r) = (1 - T_k) + T_k d q(d),  T_k = exp(-X),
-//   q(d) = 1 - d/2 + d^2/6 - d^3/24 + d^4/120  (Taylor; d^6/720 < 5e-18),
-// which keeps the relative error near 1e-16 where 1 - exp(-r) loses digits
+//   q(d) = 1 - d/2 + d^2/6 - d^3/24 + d^4/120  (Taylor),
+// which keeps the relative error near 1e-16 (1.3e-15, the remainder's d^5/720, at
+// most, just below r = 1/256: no density of a liquid or its vapour) where 1 - exp(-r) loses digits
 // for small r.  GB300's FP64 pipe issues about two lanes per clock and SM, so
 // an FP64 step costs what its FP64 instructions cost (the psi pass of
 // 256x128x128: 371 us with exp and the division, 222 us with the table): 7
